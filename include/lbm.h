@@ -367,9 +367,8 @@ int surr_predict(surr_ctx *ctx, const float *X, int32_t n, float *D_out, float *
 int surr_grad(surr_ctx *ctx, const float *X, const float *yD, const float *yB, int32_t n,
               float *grads, double *loss);
 /* `epochs` full-batch Adam steps on the n samples with learning rate lr;
- * loss_out (nullable): loss after the last step.  The step's launches are
- * captured once into a CUDA graph (kept for the next call with the same n
- * and lr) and the graph is replayed once per epoch. */
+ * loss_out (nullable): loss after the last step.  A step is two launches:
+ * the network forward and backward, then weight gradients and Adam. */
 int surr_train(surr_ctx *ctx, const float *X, const float *yD, const float *yB, int32_t n,
                int32_t epochs, float lr, double *loss_out);
 

@@ -3,18 +3,18 @@
 // accumulation, trained with Adam on FP32 master weights (the learned part
 // that picks capillary numbers near breakup).
 //
-// Forward, backward, loss and optimiser are hand-written kernels.  The
-// contractions are small (n x 128 x 128 per layer with n up to a few
-// thousand samples, ~1e7 multiply-adds per step): a tiled FMA kernel with the
-// weight tile and the input tile in shared memory finishes each in a few
-// microseconds, so the tensor cores would not change the step time.
-// Reductions over samples (weight gradients, loss) are deterministic: each
-// block owns its output tile and loops over all samples in a fixed order.
+// Forward, backward, loss and optimiser are hand-written kernels; a training
+// step is two launches (k_net, k_wgrad).  The network is 5e4 multiply-adds per
+// sample and pass, so at the sizes it is used at (1e3 to 1e4 samples) a step
+// is bound by the latency of its dependent layers and sums, not by
+// arithmetic.  All sums are single FP32 chains in a fixed order.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <cuda_bf16.h>
 #include <new>
+#include <type_traits>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -23,25 +23,17 @@
 namespace surr {
 
 constexpr int NLAYER = 5;
-constexpr int WIDTH[NLAYER + 1] = {5, 128, 128, 128, 128, 2};
 constexpr int MAXW = 128;
+// Layer widths 5, 128, 128, 128, 128, 2.
+__host__ __device__ constexpr int width(int l) { return l == 0 ? 5 : (l == NLAYER ? 2 : MAXW); }
 
 // Parameter offsets in the flat FP32 vector: layer l holds W [fout][fin]
 // then b [fout].
-struct Offsets {
-    int w[NLAYER], b[NLAYER], total;
-    constexpr Offsets() : w(), b(), total(0) {
-        int o = 0;
-        for (int l = 0; l < NLAYER; ++l) {
-            w[l] = o;
-            o += WIDTH[l + 1] * WIDTH[l];
-            b[l] = o;
-            o += WIDTH[l + 1];
-        }
-        total = o;
-    }
-};
-constexpr Offsets OFF{};
+__host__ __device__ constexpr int w_off(int l) {
+    return l == 0 ? 0 : 6 * MAXW + (l - 1) * (MAXW + 1) * MAXW;
+}
+__host__ __device__ constexpr int b_off(int l) { return w_off(l) + width(l + 1) * width(l); }
+constexpr int NPARAM = b_off(NLAYER - 1) + width(NLAYER);
 
 __device__ __forceinline__ float silu(float z) { return z / (1.0f + expf(-z)); }
 __device__ __forceinline__ float silu_grad(float z) {
@@ -49,64 +41,413 @@ __device__ __forceinline__ float silu_grad(float z) {
     return s * (1.0f + z * (1.0f - s));
 }
 
-// out_pre[n][fout] = in[n][fin] W^T + b; out_act = SiLU(out_pre) (hidden) or
-// out_pre (last layer).  Block: 32 samples x 32 outputs, 256 threads, each
-// thread 4 outputs of one sample.
-constexpr int FT_S = 32, FT_O = 32;
+// ---------------------------------------------------------------------------
+// A training step is two launches: k_net (forward and backward through all
+// layers, one block per tile of TILE samples) and k_wgrad (weight gradients,
+// Adam and the BF16 copies).  Every output is one chain of FMAs in a fixed
+// order (over the inputs, the outputs or the samples), so results do not
+// depend on the tiling or the grid.
+// ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) k_linear_fwd(const float* __restrict__ in, int fin,
-                                                    const __nv_bfloat16* __restrict__ W,
-                                                    const float* __restrict__ b, int fout, int n,
-                                                    float* __restrict__ pre,
-                                                    float* __restrict__ act, int hidden) {
-    __shared__ float sx[FT_S][MAXW + 1];
-    __shared__ float sw[FT_O][MAXW + 1];
-    const int s0 = blockIdx.x * FT_S, o0 = blockIdx.y * FT_O;
-    for (int k = threadIdx.x; k < FT_S * fin; k += blockDim.x) {
-        const int s = k / fin, i = k % fin;
-        sx[s][i] = (s0 + s < n) ? in[(int64_t)(s0 + s) * fin + i] : 0.0f;
-    }
-    for (int k = threadIdx.x; k < FT_O * fin; k += blockDim.x) {
-        const int o = k / fin, i = k % fin;
-        sw[o][i] = (o0 + o < fout) ? __bfloat162float(W[(int64_t)(o0 + o) * fin + i]) : 0.0f;
-    }
-    __syncthreads();
-    const int s = threadIdx.x / 8, og = threadIdx.x % 8;  // outputs og, og+8, og+16, og+24
-    float acc[4];
+// Row pitch (BF16 values) of a hidden layer's weights in shared memory: 66
+// words, so the 8-byte loads of 16 neighbouring rows fall in distinct banks.
+constexpr int WPITCH = 132;
+
+struct NetArgs {
+    const float* x;            // inputs [n][5]
+    const float* params;       // FP32 masters (the biases are read from here)
+    const __nv_bfloat16* wq;   // BF16 weights
+    const float *yD, *yB;      // targets (backward only)
+    float* out;                // outputs [n][2]
+    float* act[NLAYER - 1];    // hidden activations [n][128] (backward only)
+    float* gpre[NLAYER];       // loss gradients by pre-activation [n][fout] (backward only)
+    double* term;              // loss of each sample [n], or null
+    long long* tick;           // Adam step counter to advance, or null
+    float* corr;               // Adam's bias corrections of that step [2]
+    float b1, b2;
+    int n;
+};
+
+// Shared memory of a block that carries S samples at a time.
+// Rows of samples are padded so that neighbouring rows start in different
+// banks (and stay aligned for the pair loads of an even RS).
+template <int S, int RS, bool BACKWARD>
+struct NetSmem {
+    static constexpr int SP = S + (RS % 2 ? 1 - S % 2 : 2);
+    alignas(16) float x[MAXW][SP];                      // activations, later gradients, of a layer
+    alignas(16) float pre[BACKWARD ? 4 : 1][BACKWARD ? MAXW : 1][SP];  // pre-activations
+    alignas(16) __nv_bfloat16 w[3][MAXW * WPITCH];     // hidden layers 1..3
+    float w0[MAXW * 5], w4[2 * MAXW];                  // first and last layer
+    float b[4 * MAXW + 2];
+    float xin[5][S], out[2][S];
+};
+
+// Asynchronous copy of 4, 8 or 16 bytes into shared memory; zeros where !ok.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool ok = true) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int have = ok ? BYTES : 0;
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(have) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(have)
+                     : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// N consecutive floats of shared memory, in pairs where N is even.
+template <int N>
+__device__ __forceinline__ void lds(const float* p, float (&v)[N]) {
+    if constexpr (N % 2 == 0) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] = 0.0f;
-    for (int i = 0; i < fin; ++i) {
-        const float x = sx[s][i];
+        for (int j = 0; j < N; j += 2) {
+            const float2 q = *reinterpret_cast<const float2*>(p + j);
+            v[j] = q.x, v[j + 1] = q.y;
+        }
+    } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j] = fmaf(x, sw[og + 8 * j][i], acc[j]);
-    }
-    if (s0 + s >= n) return;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int o = o0 + og + 8 * j;
-        if (o >= fout) continue;
-        const float z = acc[j] + b[o];
-        pre[(int64_t)(s0 + s) * fout + o] = z;
-        act[(int64_t)(s0 + s) * fout + o] = hidden ? silu(z) : z;
+        for (int j = 0; j < N; ++j) v[j] = p[j];
     }
 }
 
-// Gradient of the loss  mean((D - yD)^2) + mean(BCE(z, yB))  with respect to
-// the two outputs, and the loss itself (one block, fixed-order reduction).
-__global__ void k_loss_grad(const float* __restrict__ out, const float* __restrict__ yD,
-                            const float* __restrict__ yB, int n, float* __restrict__ gout,
-                            double* __restrict__ loss) {
+// All layers of S = NT RO RS / 128 samples in one block, activations in shared
+// memory, the weights loaded once per block.  A thread owns RO outputs (RO
+// rows of the weights, 8 bytes = 4 inputs per load) and RS samples.
+//
+// What bounds it: issue and shared-memory bandwidth (a broadcast load returns
+// 128 bytes a cycle like any other, so a k costs (2 RO + 4 RS) / 4 cycles of
+// the SM for RO RS / 4 cycles of FMAs), at the few warps these sizes give an
+// SM.  Measured on GB300: an epoch of 1024 samples (this kernel and k_wgrad)
+// 40 us with <2, 2, 256> (8 samples a block, 128 blocks), 44 with <4, 2, 128>
+// and <4, 1, 256>, 504 before with one launch per layer and direction; a scan
+// of 11,776 samples, copies included, 70 us with <4, 5, 512>, 74 with
+// <8, 5, 256>, 193 before.
+template <int RO, int RS, int NT, bool BACKWARD>
+__global__ void __launch_bounds__(NT) k_net(const NetArgs a) {
+    constexpr int OG = MAXW / RO;          // threads along the outputs
+    constexpr int S = NT / OG * RS;        // samples of the block
+    extern __shared__ __align__(16) unsigned char smem_net[];
+    auto& M = *reinterpret_cast<NetSmem<S, RS, BACKWARD>*>(smem_net);
+    const int t = threadIdx.x;
+    if (BACKWARD && a.tick && blockIdx.x == gridDim.x - 1) {
+        // the last block has no samples: it counts the Adam step k_wgrad will
+        // take (two FP64 powers, a microsecond that nothing else waits for)
+        if (t < 2) {
+            const double step = (double)(*a.tick + 1);
+            a.corr[t] = (float)(1.0 - pow((double)(t ? a.b2 : a.b1), step));
+            __syncwarp(3u);
+            if (t == 0) *a.tick += 1;
+        }
+        return;
+    }
+    const int nblocks = gridDim.x - (BACKWARD && a.tick ? 1 : 0);
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        const __nv_bfloat16* src = a.wq + w_off(l + 1);
+        for (int k = t; k < MAXW * 32; k += NT)
+            cp_async<8>(&M.w[l][(k >> 5) * WPITCH + 4 * (k & 31)], src + 4 * k);
+    }
+    cp_async_commit();
+    for (int k = t; k < MAXW * 5; k += NT) M.w0[k] = __bfloat162float(a.wq[w_off(0) + k]);
+    for (int k = t; k < 2 * MAXW; k += NT) M.w4[k] = __bfloat162float(a.wq[w_off(4) + k]);
+    for (int k = t; k < 4 * MAXW + 2; k += NT) M.b[k] = a.params[b_off(k / MAXW) + k % MAXW];
+
+    const int ntile = (a.n + S - 1) / S;
+    const int og = t % OG, sb = t / OG * RS;  // outputs og + OG r, samples sb + j
+    for (int tile = blockIdx.x; tile < ntile; tile += nblocks) {
+        const int s0 = tile * S;
+        __syncthreads();  // the previous tile is done
+        for (int k = t; k < 5 * S; k += NT) {
+            const int s = k / 5, i = k % 5;
+            M.xin[i][s] = s0 + s < a.n ? a.x[(int64_t)(s0 + s) * 5 + i] : 0.0f;
+        }
+        __syncthreads();
+        // ---- forward, hidden layers (layer 0 runs while the others' weights arrive)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            float acc[RO][RS];
+#pragma unroll
+            for (int r = 0; r < RO; ++r)
+#pragma unroll
+                for (int j = 0; j < RS; ++j) acc[r][j] = 0.0f;
+            if (l == 0) {
+#pragma unroll
+                for (int i = 0; i < 5; ++i)
+#pragma unroll
+                    for (int r = 0; r < RO; ++r) {
+                        const float w = M.w0[(og + OG * r) * 5 + i];
+#pragma unroll
+                        for (int j = 0; j < RS; ++j) acc[r][j] = fmaf(M.xin[i][sb + j], w, acc[r][j]);
+                    }
+            } else {
+                const __nv_bfloat16* row = &M.w[l > 0 ? l - 1 : 0][og * WPITCH];
+#pragma unroll 4
+                for (int k = 0; k < MAXW; k += 4) {
+                    uint2 wv[RO];
+#pragma unroll
+                    for (int r = 0; r < RO; ++r)
+                        wv[r] = *reinterpret_cast<const uint2*>(row + OG * r * WPITCH + k);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float v[RS];
+                        lds<RS>(&M.x[k + q][sb], v);
+#pragma unroll
+                        for (int r = 0; r < RO; ++r) {
+                            const uint32_t h = q < 2 ? wv[r].x : wv[r].y;
+                            const float w = q & 1 ? bf_hi(h) : bf_lo(h);
+#pragma unroll
+                            for (int j = 0; j < RS; ++j) acc[r][j] = fmaf(v[j], w, acc[r][j]);
+                        }
+                    }
+                }
+                __syncthreads();  // every thread has read the layer's inputs
+            }
+#pragma unroll
+            for (int r = 0; r < RO; ++r) {
+                const int o = og + OG * r;
+                const float bias = M.b[l * MAXW + o];
+#pragma unroll
+                for (int j = 0; j < RS; ++j) {
+                    const float z = acc[r][j] + bias, y = silu(z);
+                    M.x[o][sb + j] = y;
+                    if constexpr (BACKWARD) {
+                        M.pre[l][o][sb + j] = z;
+                        if (s0 + sb + j < a.n) a.act[l][(int64_t)(s0 + sb + j) * MAXW + o] = y;
+                    }
+                }
+            }
+            if (l == 0) cp_async_wait<0>();
+            __syncthreads();
+        }
+        // ---- last layer: two outputs per sample
+        for (int k = t; k < 2 * S; k += NT) {
+            const int oo = k / S, s = k % S;
+            float acc = 0.0f;
+#pragma unroll 16
+            for (int i = 0; i < MAXW; ++i) acc = fmaf(M.x[i][s], M.w4[oo * MAXW + i], acc);
+            const float z = acc + M.b[4 * MAXW + oo];
+            if constexpr (BACKWARD) M.out[oo][s] = z;
+            if (s0 + s < a.n) a.out[(int64_t)(s0 + s) * 2 + oo] = z;
+        }
+        if constexpr (BACKWARD) {
+            __syncthreads();
+            // gradient of  mean((D - yD)^2) + mean(BCE(z, yB))  by the outputs
+            if (t < S) {
+                const int s = s0 + t;
+                float g0 = 0.0f, g1 = 0.0f;
+                if (s < a.n) {
+                    const float d = M.out[0][t] - a.yD[s];
+                    const float z = M.out[1][t];
+                    const float y = a.yB[s];
+                    g0 = 2.0f * d / a.n;
+                    g1 = (1.0f / (1.0f + expf(-z)) - y) / a.n;
+                    a.gpre[4][2 * (int64_t)s] = g0;
+                    a.gpre[4][2 * (int64_t)s + 1] = g1;
+                    if (a.term) {
+                        const double bce =
+                            fmax((double)z, 0.0) - (double)z * y + log1p(exp(-fabs((double)z)));
+                        a.term[s] = (double)d * d + bce;
+                    }
+                }
+                M.out[0][t] = g0;
+                M.out[1][t] = g1;
+            }
+            __syncthreads();
+            // gradient by the pre-activations of the last hidden layer, then
+            // of the others: RO neighbouring inputs per thread
+            static_assert(!BACKWARD || RO == 2 || RO == 4, "one load holds a thread's inputs");
+            const int i0 = RO * og;
+#pragma unroll
+            for (int l = 4; l > 0; --l) {
+                float acc[RO][RS];
+#pragma unroll
+                for (int r = 0; r < RO; ++r)
+#pragma unroll
+                    for (int j = 0; j < RS; ++j) acc[r][j] = 0.0f;
+                if (l == 4) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+#pragma unroll
+                        for (int r = 0; r < RO; ++r)
+#pragma unroll
+                            for (int j = 0; j < RS; ++j)
+                                acc[r][j] = fmaf(M.out[k][sb + j], M.w4[k * MAXW + i0 + r], acc[r][j]);
+                } else {
+                    const __nv_bfloat16* col = &M.w[l < 4 ? l - 1 : 0][i0];
+#pragma unroll 16
+                    for (int k = 0; k < MAXW; ++k) {
+                        float w[RO];
+                        if constexpr (RO == 4) {
+                            const uint2 wv = *reinterpret_cast<const uint2*>(col + k * WPITCH);
+                            w[2] = bf_lo(wv.y), w[3] = bf_hi(wv.y);
+                            w[0] = bf_lo(wv.x), w[1] = bf_hi(wv.x);
+                        } else {
+                            const uint32_t wv = *reinterpret_cast<const uint32_t*>(col + k * WPITCH);
+                            w[0] = bf_lo(wv), w[1] = bf_hi(wv);
+                        }
+                        float g[RS];
+                        lds<RS>(&M.x[k][sb], g);
+#pragma unroll
+                        for (int r = 0; r < RO; ++r)
+#pragma unroll
+                            for (int j = 0; j < RS; ++j) acc[r][j] = fmaf(g[j], w[r], acc[r][j]);
+                    }
+                    __syncthreads();  // every thread has read the layer's gradients
+                }
+#pragma unroll
+                for (int j = 0; j < RS; ++j) {
+#pragma unroll
+                    for (int r = 0; r < RO; ++r) {
+                        acc[r][j] *= silu_grad(M.pre[l - 1][i0 + r][sb + j]);
+                        M.x[i0 + r][sb + j] = acc[r][j];
+                    }
+                    if (s0 + sb + j < a.n) {
+                        float* g = a.gpre[l - 1] + (int64_t)(s0 + sb + j) * MAXW + i0;
+#pragma unroll
+                        for (int r = 0; r < RO; r += 2)
+                            *reinterpret_cast<float2*>(g + r) = make_float2(acc[r][j], acc[r + 1][j]);
+                    }
+                }
+                __syncthreads();
+            }
+        }
+    }
+}
+
+// Weight gradients gW[o][i] = sum_s gpre[s][o] in[s][i], gb[o] = sum_s gpre[s][o],
+// and (ADAM) the Adam update with bias correction of the same weights and
+// their BF16 copies, by the threads that hold the sums.
+//
+// One warp per WO x WI tile of one layer's weights, 2 x 2 weights per thread;
+// the samples pass through a ring of WST shared-memory chunks of WCH samples
+// filled by cp.async.  Each sum is one chain over the samples in order, so at
+// 1024 samples the chain (4 cycles a sample) and the shared-memory reads (4
+// cycles a sample and warp) bound the kernel, and small tiles are what keeps
+// all SMs busy: 408 warps, about one per scheduler.
+constexpr int WO = 16, WI = 8, WCH = 64, WST = 4;
+
+struct WgradArgs {
+    const float* in[NLAYER];    // inputs of each layer [n][fin]
+    const float* gpre[NLAYER];  // gradients by its pre-activations [n][fout]
+    float *grads, *params, *m, *v;
+    __nv_bfloat16* wq;
+    const float* corr;          // Adam's bias corrections
+    float lr, b1, b2, eps;
+    int n;
+};
+
+// Blocks of layer l: ceil(fout / WO) x ceil(fin / WI), layer after layer.
+__host__ __device__ constexpr int wg_tiles(int l) {
+    return ((width(l + 1) + WO - 1) / WO) * ((width(l) + WI - 1) / WI);
+}
+constexpr int WG_BLOCKS = wg_tiles(0) + wg_tiles(1) + wg_tiles(2) + wg_tiles(3) + wg_tiles(4);
+
+template <bool ADAM>
+__global__ void __launch_bounds__(32) k_wgrad(const WgradArgs a) {
+    __shared__ __align__(16) float sg[WST][WCH][WO], sx[WST][WCH][WI];
+    int l = 0, tile = blockIdx.x;
+    while (tile >= wg_tiles(l)) tile -= wg_tiles(l++);
+    const int fin = width(l), fout = width(l + 1);
+    const int ni = (fin + WI - 1) / WI;
+    const int o0 = tile / ni * WO, i0 = tile % ni * WI;
+    const float *in = a.in[l], *gp = a.gpre[l];
+    const int t = threadIdx.x;
+    // Chunk c of one operand: W columns from col0 of rows of `width` floats.
+    // Samples beyond n and columns beyond the layer are zeros (their copies
+    // read nothing; the source address stays inside the buffer).
+    auto load_one = [&](float* dst, int W, const float* src, int width, int col0, int c) {
+        const int left = a.n - c * WCH;
+        src += (int64_t)c * WCH * width;
+        if (width >= MAXW) {
+            const int per = W / 4;
+            for (int k = t; k < WCH * per; k += 32) {
+                const int s = k / per, q = 4 * (k % per);
+                const bool ok = s < left;
+                cp_async<16>(dst + s * W + q, ok ? src + (int64_t)s * width + col0 + q : src, ok);
+            }
+        } else {
+            for (int k = t; k < WCH * W; k += 32) {
+                const int s = k / W, q = k % W;
+                const bool ok = s < left && q < width;
+                cp_async<4>(dst + s * W + q, ok ? src + (int64_t)s * width + q : src, ok);
+            }
+        }
+    };
+    const int nchunk = (a.n + WCH - 1) / WCH;
+    auto load = [&](int c) {
+        if (c < nchunk) {
+            load_one(&sg[c % WST][0][0], WO, gp, fout, o0, c);
+            load_one(&sx[c % WST][0][0], WI, in, fin, i0, c);
+        }
+        cp_async_commit();
+    };
+    const int oi = 2 * (t / 4), ig = 2 * (t % 4);  // outputs o0 + oi, + 1; inputs i0 + ig, + 1
+#pragma unroll
+    for (int c = 0; c < WST - 1; ++c) load(c);
+    float acc[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}}, accb[2] = {0.0f, 0.0f};
+    auto sum = [&](auto bias) {
+        for (int c = 0; c < nchunk; ++c) {
+            cp_async_wait<WST - 2>();
+            __syncwarp();
+            load(c + WST - 1);  // into the chunk read before this one
+            const float(*pg)[WO] = sg[c % WST];
+            const float(*px)[WI] = sx[c % WST];
+#pragma unroll 16
+            for (int s = 0; s < WCH; ++s) {
+                const float2 g = *reinterpret_cast<const float2*>(&pg[s][oi]);
+                const float2 x = *reinterpret_cast<const float2*>(&px[s][ig]);
+                acc[0][0] = fmaf(g.x, x.x, acc[0][0]);
+                acc[0][1] = fmaf(g.x, x.y, acc[0][1]);
+                acc[1][0] = fmaf(g.y, x.x, acc[1][0]);
+                acc[1][1] = fmaf(g.y, x.y, acc[1][1]);
+                if constexpr (decltype(bias)::value) {
+                    accb[0] += g.x;
+                    accb[1] += g.y;
+                }
+            }
+            __syncwarp();
+        }
+    };
+    if (i0 == 0) sum(std::true_type{});
+    else sum(std::false_type{});
+    const float c1 = ADAM ? a.corr[0] : 1.0f, c2 = ADAM ? a.corr[1] : 1.0f;
+    auto finish = [&](int k, float gk) {
+        if constexpr (!ADAM) {
+            a.grads[k] = gk;
+        } else {
+            // (written out: 64 steps amplify another rounding of these two to 1e-4)
+            const float mk = __fmaf_rn(1.0f - a.b1, gk, __fmul_rn(a.b1, a.m[k]));
+            const float vk = __fmaf_rn(__fmul_rn(1.0f - a.b2, gk), gk, __fmul_rn(a.b2, a.v[k]));
+            a.m[k] = mk;
+            a.v[k] = vk;
+            const float mh = mk / c1, vh = vk / c2;
+            const float p = a.params[k] - a.lr * mh / (sqrtf(vh) + a.eps);
+            a.params[k] = p;
+            a.wq[k] = __float2bfloat16_rn(p);
+        }
+    };
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int o = o0 + oi + e;
+        if (o >= fout) continue;
+        if (i0 + ig < fin) finish(w_off(l) + o * fin + i0 + ig, acc[e][0]);
+        if (i0 + ig + 1 < fin) finish(w_off(l) + o * fin + i0 + ig + 1, acc[e][1]);
+        if (i0 == 0 && ig == 0) finish(b_off(l) + o, accb[e]);
+    }
+}
+
+// The mean of the samples' losses (one block, fixed-order reduction).
+__global__ void k_loss(const double* __restrict__ term, int n, double* __restrict__ loss) {
     __shared__ double red[256];
     double acc = 0.0;
-    for (int s = threadIdx.x; s < n; s += blockDim.x) {
-        const float d = out[2 * s] - yD[s];
-        const float z = out[2 * s + 1];
-        const float y = yB[s];
-        gout[2 * s] = 2.0f * d / n;
-        gout[2 * s + 1] = (1.0f / (1.0f + expf(-z)) - y) / n;
-        const double bce = fmax((double)z, 0.0) - (double)z * y + log1p(exp(-fabs((double)z)));
-        acc += (double)d * d + bce;
-    }
+    for (int s = threadIdx.x; s < n; s += blockDim.x) acc += term[s];
     red[threadIdx.x] = acc;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -116,115 +457,10 @@ __global__ void k_loss_grad(const float* __restrict__ out, const float* __restri
     if (threadIdx.x == 0) *loss = red[0] / n;
 }
 
-// gin[n][fin] = (gpre[n][fout] W) * SiLU'(pre_in[n][fin])  (pre_in NULL: no
-// activation factor).  Block: 32 samples x 32 inputs.
-__global__ void __launch_bounds__(256) k_linear_bwd_in(const float* __restrict__ gpre, int fout,
-                                                       const __nv_bfloat16* __restrict__ W,
-                                                       int fin, int n,
-                                                       const float* __restrict__ pre_in,
-                                                       float* __restrict__ gin) {
-    __shared__ float sg[FT_S][MAXW + 1];
-    __shared__ float sw[MAXW][FT_O + 1];
-    const int s0 = blockIdx.x * FT_S, i0 = blockIdx.y * FT_O;
-    for (int k = threadIdx.x; k < FT_S * fout; k += blockDim.x) {
-        const int s = k / fout, o = k % fout;
-        sg[s][o] = (s0 + s < n) ? gpre[(int64_t)(s0 + s) * fout + o] : 0.0f;
-    }
-    for (int k = threadIdx.x; k < fout * FT_O; k += blockDim.x) {
-        const int o = k / FT_O, i = k % FT_O;
-        sw[o][i] = (i0 + i < fin) ? __bfloat162float(W[(int64_t)o * fin + i0 + i]) : 0.0f;
-    }
-    __syncthreads();
-    const int s = threadIdx.x / 8, ig = threadIdx.x % 8;
-    float acc[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] = 0.0f;
-    for (int o = 0; o < fout; ++o) {
-        const float g = sg[s][o];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j] = fmaf(g, sw[o][ig + 8 * j], acc[j]);
-    }
-    if (s0 + s >= n) return;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int i = i0 + ig + 8 * j;
-        if (i >= fin) continue;
-        float v = acc[j];
-        if (pre_in) v *= silu_grad(pre_in[(int64_t)(s0 + s) * fin + i]);
-        gin[(int64_t)(s0 + s) * fin + i] = v;
-    }
-}
-
-// gW[fout][fin] = sum_s gpre[s][o] in[s][i]; gb[o] = sum_s gpre[s][o].
-// Block: 32 outputs x 32 inputs (plus the bias column), loops over all
-// samples in chunks of 64 (fixed order: deterministic).
-constexpr int GT = 32, GCH = 64;
-
-__global__ void __launch_bounds__(256) k_linear_bwd_w(const float* __restrict__ gpre, int fout,
-                                                      const float* __restrict__ in, int fin,
-                                                      int n, float* __restrict__ gW,
-                                                      float* __restrict__ gb) {
-    __shared__ float sg[GCH][GT + 1];
-    __shared__ float sx[GCH][GT + 1];
-    const int o0 = blockIdx.x * GT, i0 = blockIdx.y * GT;
-    const int oi = threadIdx.x / 8;         // output row in the tile (0..31)
-    const int ig = threadIdx.x % 8;         // inputs ig, ig+8, ig+16, ig+24
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    float accb = 0.0f;
-    for (int c0 = 0; c0 < n; c0 += GCH) {
-        for (int k = threadIdx.x; k < GCH * GT; k += blockDim.x) {
-            const int s = k / GT, j = k % GT;
-            const bool ok = c0 + s < n;
-            sg[s][j] = (ok && o0 + j < fout) ? gpre[(int64_t)(c0 + s) * fout + o0 + j] : 0.0f;
-            sx[s][j] = (ok && i0 + j < fin) ? in[(int64_t)(c0 + s) * fin + i0 + j] : 0.0f;
-        }
-        __syncthreads();
-        for (int s = 0; s < GCH; ++s) {
-            const float g = sg[s][oi];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[j] = fmaf(g, sx[s][ig + 8 * j], acc[j]);
-            accb += g;
-        }
-        __syncthreads();
-    }
-    const int o = o0 + oi;
-    if (o >= fout) return;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int i = i0 + ig + 8 * j;
-        if (i < fin) gW[(int64_t)o * fin + i] = acc[j];
-    }
-    if (blockIdx.y == 0 && ig == 0) gb[o] = accb;
-}
-
-// Adam with bias correction on the FP32 master parameters, then their BF16
-// copies (weights only are used in BF16; biases stay FP32).  The step number
-// is *t + 1, read on the device (k_to_bf16 advances *t after the step), so
-// that one captured step can be replayed.
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int count, float lr, float b1, float b2, float eps,
-                       const long long* __restrict__ t) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    const double step = (double)(*t + 1);
-    const float c1 = (float)(1.0 - pow((double)b1, step));
-    const float c2 = (float)(1.0 - pow((double)b2, step));
-    const float gk = g[k];
-    const float mk = b1 * m[k] + (1.0f - b1) * gk;
-    const float vk = b2 * v[k] + (1.0f - b2) * gk * gk;
-    m[k] = mk;
-    v[k] = vk;
-    const float mh = mk / c1, vh = vk / c2;
-    p[k] -= lr * mh / (sqrtf(vh) + eps);
-}
-
-// BF16 copies of the parameters; `tick` (nullable): the Adam step counter,
-// advanced by one.
-__global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ q, int count,
-                          long long* __restrict__ tick) {
+// BF16 copies of the parameters.
+__global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ q, int count) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < count) q[k] = __float2bfloat16_rn(p[k]);
-    if (tick && k == 0) *tick += 1;
 }
 
 }  // namespace surr
@@ -238,19 +474,16 @@ struct surr_ctx {
     float* m = nullptr;
     float* v = nullptr;
     long long* adam_t = nullptr;      // Adam steps taken (device counter)
-    // one captured training step (forward, backward, Adam, BF16 copies),
-    // valid for n samples and learning rate lr with the current buffers
-    cudaGraphExec_t step_graph = nullptr;
-    int graph_n = 0;
-    float graph_lr = 0.0f;
-    cudaStream_t cap_stream = nullptr;
-    int cap = 0;                      // samples the activation buffers hold
+    float* corr = nullptr;            // bias corrections of the current Adam step [2]
+    int sms = 0;
+    int cap = 0;                      // samples the batch buffers hold
     float* x = nullptr;               // inputs [cap][5]
-    float* pre[NLAYER] = {};          // pre-activations per layer [cap][fout]
-    float* act[NLAYER] = {};          // activations per layer [cap][fout]
-    float* gbuf[2] = {nullptr, nullptr};  // gradient ping-pong [cap][128]
+    float* out = nullptr;             // outputs [cap][2]
+    float* act[NLAYER - 1] = {};      // hidden activations [cap][128]
+    float* gpre[NLAYER] = {};         // gradients by pre-activation [cap][fout]
     float* yD = nullptr;
     float* yB = nullptr;
+    double* term = nullptr;           // loss of each sample [cap]
     double* loss = nullptr;
     cudaStream_t stream = nullptr;
 };
@@ -263,38 +496,38 @@ int fail(cudaError_t e) {
     return LBM_ERR_CUDA;
 }
 
-void drop_step_graph(surr_ctx* c) {
-    if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
-    c->step_graph = nullptr;
-}
-
 void free_batch(surr_ctx* c) {
-    drop_step_graph(c);  // it refers to the activation buffers
     cudaFree(c->x);
-    for (int l = 0; l < NLAYER; ++l) {
-        cudaFree(c->pre[l]);
+    cudaFree(c->out);
+    for (int l = 0; l < NLAYER - 1; ++l) {
         cudaFree(c->act[l]);
-        c->pre[l] = c->act[l] = nullptr;
+        c->act[l] = nullptr;
     }
-    cudaFree(c->gbuf[0]);
-    cudaFree(c->gbuf[1]);
+    for (int l = 0; l < NLAYER; ++l) {
+        cudaFree(c->gpre[l]);
+        c->gpre[l] = nullptr;
+    }
     cudaFree(c->yD);
     cudaFree(c->yB);
-    c->x = c->gbuf[0] = c->gbuf[1] = c->yD = c->yB = nullptr;
+    cudaFree(c->term);
+    c->x = c->out = c->yD = c->yB = nullptr;
+    c->term = nullptr;
     c->cap = 0;
 }
 
 int ensure_batch(surr_ctx* c, int n) {
     if (n <= c->cap) return LBM_OK;
     free_batch(c);
-    bool ok = cudaMalloc(&c->x, sizeof(float) * n * WIDTH[0]) == cudaSuccess &&
-              cudaMalloc(&c->gbuf[0], sizeof(float) * n * MAXW) == cudaSuccess &&
-              cudaMalloc(&c->gbuf[1], sizeof(float) * n * MAXW) == cudaSuccess &&
-              cudaMalloc(&c->yD, sizeof(float) * n) == cudaSuccess &&
-              cudaMalloc(&c->yB, sizeof(float) * n) == cudaSuccess;
+    const size_t m = (size_t)n;
+    bool ok = cudaMalloc(&c->x, sizeof(float) * m * width(0)) == cudaSuccess &&
+              cudaMalloc(&c->out, sizeof(float) * m * 2) == cudaSuccess &&
+              cudaMalloc(&c->yD, sizeof(float) * m) == cudaSuccess &&
+              cudaMalloc(&c->yB, sizeof(float) * m) == cudaSuccess &&
+              cudaMalloc(&c->term, sizeof(double) * m) == cudaSuccess;
+    for (int l = 0; l < NLAYER - 1 && ok; ++l)
+        ok = cudaMalloc(&c->act[l], sizeof(float) * m * MAXW) == cudaSuccess;
     for (int l = 0; l < NLAYER && ok; ++l)
-        ok = cudaMalloc(&c->pre[l], sizeof(float) * n * WIDTH[l + 1]) == cudaSuccess &&
-             cudaMalloc(&c->act[l], sizeof(float) * n * WIDTH[l + 1]) == cudaSuccess;
+        ok = cudaMalloc(&c->gpre[l], sizeof(float) * m * width(l + 1)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_batch(c);
@@ -304,82 +537,108 @@ int ensure_batch(surr_ctx* c, int n) {
     return LBM_OK;
 }
 
-void refresh_bf16(surr_ctx* c, bool tick = false) {
-    k_to_bf16<<<(OFF.total + 255) / 256, 256, 0, c->stream>>>(c->params, c->wq, OFF.total,
-                                                              tick ? c->adam_t : nullptr);
+void refresh_bf16(surr_ctx* c) {
+    k_to_bf16<<<(NPARAM + 255) / 256, 256, 0, c->stream>>>(c->params, c->wq, NPARAM);
 }
 
-void forward(surr_ctx* c, int n) {
-    const float* in = c->x;
+constexpr float ADAM_B1 = 0.9f, ADAM_B2 = 0.999f, ADAM_EPS = 1e-8f;
+constexpr int TRAIN_RO = 2, TRAIN_RS = 2, TRAIN_NT = 256;
+constexpr int TRAIN_S = TRAIN_NT * TRAIN_RO / MAXW * TRAIN_RS;  // samples a block: 8
+constexpr int PRED_RO = 4, PRED_NT = 512;
+constexpr int PRED_SG = PRED_NT * PRED_RO / MAXW;
+using TrainSmem = NetSmem<TRAIN_S, TRAIN_RS, true>;
+template <int RS>
+using PredSmem = NetSmem<PRED_SG * RS, RS, false>;
+
+// Calls f with the samples per thread of an inference launch, 1 to 5, as a
+// compile-time constant: the fewest that let one wave of blocks (one per SM
+// by shared memory) take all n samples; beyond that (12,160 samples on 152
+// SMs) blocks walk several tiles of 80.
+template <class F>
+auto with_pred_rs(int n, int sms, F&& f) {
+    using std::integral_constant;
+    const int per = (n + sms - 1) / sms;
+    if (per <= 1 * PRED_SG) return f(integral_constant<int, 1>{});
+    if (per <= 2 * PRED_SG) return f(integral_constant<int, 2>{});
+    if (per <= 3 * PRED_SG) return f(integral_constant<int, 3>{});
+    if (per <= 4 * PRED_SG) return f(integral_constant<int, 4>{});
+    return f(integral_constant<int, 5>{});
+}
+
+cudaError_t configure_net() {
+    cudaError_t e = cudaFuncSetAttribute(k_net<TRAIN_RO, TRAIN_RS, TRAIN_NT, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(TrainSmem));
+    for (int n = PRED_SG; n <= 5 * PRED_SG && e == cudaSuccess; n += PRED_SG)
+        e = with_pred_rs(n, 1, [](auto R) {
+            return cudaFuncSetAttribute(k_net<PRED_RO, R(), PRED_NT, false>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sizeof(PredSmem<R()>));
+        });
+    return e;
+}
+
+// The network over the n samples in the buffers: outputs, and (backward) the
+// activations and gradients k_wgrad reads, the samples' losses, and the count
+// of the Adam step that follows.
+void run_net(surr_ctx* c, int n, bool backward, bool loss, bool tick) {
+    NetArgs a{};
+    a.x = c->x;
+    a.params = c->params;
+    a.wq = c->wq;
+    a.yD = c->yD;
+    a.yB = c->yB;
+    a.out = c->out;
+    for (int l = 0; l < NLAYER - 1; ++l) a.act[l] = c->act[l];
+    for (int l = 0; l < NLAYER; ++l) a.gpre[l] = c->gpre[l];
+    a.term = loss ? c->term : nullptr;
+    a.tick = tick ? c->adam_t : nullptr;
+    a.corr = c->corr;
+    a.b1 = ADAM_B1;
+    a.b2 = ADAM_B2;
+    a.n = n;
+    auto blocks = [&](int samples) { return std::min((n + samples - 1) / samples, c->sms); };
+    if (backward)
+        k_net<TRAIN_RO, TRAIN_RS, TRAIN_NT, true>
+            <<<blocks(TRAIN_S) + (tick ? 1 : 0), TRAIN_NT, sizeof(TrainSmem), c->stream>>>(a);
+    else
+        with_pred_rs(n, c->sms, [&](auto R) {
+            k_net<PRED_RO, R(), PRED_NT, false>
+                <<<blocks(PRED_SG * R()), PRED_NT, sizeof(PredSmem<R()>), c->stream>>>(a);
+            return 0;
+        });
+    if (loss) k_loss<<<1, 256, 0, c->stream>>>(c->term, n, c->loss);
+}
+
+// Weight gradients of the n samples run_net left in the buffers: into
+// c->grads, or (adam) straight into an Adam step.
+void run_wgrad(surr_ctx* c, int n, bool adam, float lr) {
+    WgradArgs a{};
     for (int l = 0; l < NLAYER; ++l) {
-        const int fin = WIDTH[l], fout = WIDTH[l + 1];
-        dim3 grid((n + FT_S - 1) / FT_S, (fout + FT_O - 1) / FT_O);
-        k_linear_fwd<<<grid, 256, 0, c->stream>>>(in, fin, c->wq + OFF.w[l], c->params + OFF.b[l],
-                                                  fout, n, c->pre[l], c->act[l], l < NLAYER - 1);
-        in = c->act[l];
+        a.in[l] = l == 0 ? c->x : c->act[l - 1];
+        a.gpre[l] = c->gpre[l];
     }
-}
-
-// Gradients of the loss for the n samples in the activation buffers into
-// c->grads (needs forward first and yD, yB on the device).
-void backward(surr_ctx* c, int n) {
-    k_loss_grad<<<1, 256, 0, c->stream>>>(c->act[NLAYER - 1], c->yD, c->yB, n, c->gbuf[0], c->loss);
-    int cur = 0;
-    for (int l = NLAYER - 1; l >= 0; --l) {
-        const int fin = WIDTH[l], fout = WIDTH[l + 1];
-        const float* in = l == 0 ? c->x : c->act[l - 1];
-        dim3 gw((fout + GT - 1) / GT, (fin + GT - 1) / GT);
-        k_linear_bwd_w<<<gw, 256, 0, c->stream>>>(c->gbuf[cur], fout, in, fin, n,
-                                                  c->grads + OFF.w[l], c->grads + OFF.b[l]);
-        if (l > 0) {
-            dim3 gi((n + FT_S - 1) / FT_S, (fin + FT_O - 1) / FT_O);
-            k_linear_bwd_in<<<gi, 256, 0, c->stream>>>(c->gbuf[cur], fout, c->wq + OFF.w[l], fin,
-                                                        n, c->pre[l - 1], c->gbuf[1 - cur]);
-            cur = 1 - cur;
-        }
-    }
-}
-
-// One Adam step on the n samples in the buffers.
-void train_step(surr_ctx* c, int n, float lr) {
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    forward(c, n);
-    backward(c, n);
-    k_adam<<<(OFF.total + 255) / 256, 256, 0, c->stream>>>(c->params, c->grads, c->m, c->v,
-                                                           OFF.total, lr, b1, b2, eps, c->adam_t);
-    refresh_bf16(c, true);
-}
-
-// The step as a graph (captured on the private stream; replayed on c->stream).
-int build_step_graph(surr_ctx* c, int n, float lr) {
-    drop_step_graph(c);
-    if (!c->cap_stream &&
-        cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
-        return fail(cudaGetLastError());
-    const cudaStream_t saved = c->stream;
-    c->stream = c->cap_stream;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        train_step(c, n, lr);
-        e = cudaStreamEndCapture(c->cap_stream, &g);
-    }
-    c->stream = saved;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->step_graph, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        c->step_graph = nullptr;
-        return fail(e);
-    }
-    c->graph_n = n;
-    c->graph_lr = lr;
-    return LBM_OK;
+    a.grads = c->grads;
+    a.params = c->params;
+    a.m = c->m;
+    a.v = c->v;
+    a.wq = c->wq;
+    a.corr = c->corr;
+    a.lr = lr;
+    a.b1 = ADAM_B1;
+    a.b2 = ADAM_B2;
+    a.eps = ADAM_EPS;
+    a.n = n;
+    if (adam)
+        k_wgrad<true><<<WG_BLOCKS, 32, 0, c->stream>>>(a);
+    else
+        k_wgrad<false><<<WG_BLOCKS, 32, 0, c->stream>>>(a);
 }
 
 int upload_batch(surr_ctx* c, const float* X, const float* yD, const float* yB, int n) {
     int rc = ensure_batch(c, n);
     if (rc != LBM_OK) return rc;
-    cudaError_t e = cudaMemcpyAsync(c->x, X, sizeof(float) * n * WIDTH[0], cudaMemcpyHostToDevice,
+    cudaError_t e = cudaMemcpyAsync(c->x, X, sizeof(float) * n * width(0), cudaMemcpyHostToDevice,
                                     c->stream);
     if (e == cudaSuccess && yD)
         e = cudaMemcpyAsync(c->yD, yD, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream);
@@ -393,19 +652,14 @@ int train_epochs(surr_ctx* c, const float* X, const float* yD, const float* yB, 
                  float lr, double* loss_out) {
     int rc = upload_batch(c, X, yD, yB, n);
     if (rc != LBM_OK) return rc;
-    // the step's launches are captured once and the graph replayed per epoch
-    if (epochs > 0 && (!c->step_graph || c->graph_n != n || c->graph_lr != lr)) {
-        rc = build_step_graph(c, n, lr);
-        if (rc != LBM_OK) return rc;
+    for (int ep = 0; ep < epochs; ++ep) {
+        run_net(c, n, true, false, true);
+        run_wgrad(c, n, true, lr);
     }
-    cudaError_t e = cudaSuccess;
-    for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep)
-        e = cudaGraphLaunch(c->step_graph, c->stream);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && loss_out) {
         // loss of the parameters after the last update
-        forward(c, n);
-        backward(c, n);
+        run_net(c, n, true, true, false);
         e = cudaMemcpyAsync(loss_out, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -416,7 +670,7 @@ int train_epochs(surr_ctx* c, const float* X, const float* yD, const float* yB, 
 
 extern "C" {
 
-int32_t surr_param_count(void) { return OFF.total; }
+int32_t surr_param_count(void) { return NPARAM; }
 
 int surr_create(uint64_t seed, void* stream, surr_ctx** out) {
     if (!out) return LBM_ERR_INVALID_ARG;
@@ -424,20 +678,29 @@ int surr_create(uint64_t seed, void* stream, surr_ctx** out) {
     surr_ctx* c = new (std::nothrow) surr_ctx();
     if (!c) return LBM_ERR_NOMEM;
     c->stream = (cudaStream_t)stream;
-    const size_t pb = sizeof(float) * OFF.total;
+    const size_t pb = sizeof(float) * NPARAM;
     if (cudaMalloc(&c->params, pb) != cudaSuccess || cudaMalloc(&c->grads, pb) != cudaSuccess ||
         cudaMalloc(&c->m, pb) != cudaSuccess || cudaMalloc(&c->v, pb) != cudaSuccess ||
-        cudaMalloc(&c->wq, sizeof(__nv_bfloat16) * OFF.total) != cudaSuccess ||
+        cudaMalloc(&c->wq, sizeof(__nv_bfloat16) * NPARAM) != cudaSuccess ||
         cudaMalloc(&c->loss, sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&c->corr, sizeof(float) * 2) != cudaSuccess ||
         cudaMalloc(&c->adam_t, sizeof(long long)) != cudaSuccess) {
         cudaGetLastError();
         surr_destroy(c);
         return LBM_ERR_NOMEM;
     }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        configure_net() != cudaSuccess) {
+        cudaGetLastError();
+        surr_destroy(c);
+        return LBM_ERR_CUDA;
+    }
     // He initialisation W ~ N(0, 2 / fan_in), b = 0, from a seeded host
     // generator (SplitMix64, Steele, Lea and Flood 2014, and the Box-Muller
     // transform) so that runs are reproducible
-    float* host = new (std::nothrow) float[OFF.total];
+    float* host = new (std::nothrow) float[NPARAM];
     if (!host) {
         surr_destroy(c);
         return LBM_ERR_NOMEM;
@@ -451,13 +714,13 @@ int surr_create(uint64_t seed, void* stream, surr_ctx** out) {
     };
     auto uniform = [&]() { return ((next() >> 11) + 0.5) * (1.0 / 9007199254740992.0); };
     for (int l = 0; l < NLAYER; ++l) {
-        const double sd = std::sqrt(2.0 / WIDTH[l]);
-        for (int k = 0; k < WIDTH[l + 1] * WIDTH[l]; ++k) {
+        const double sd = std::sqrt(2.0 / width(l));
+        for (int k = 0; k < width(l + 1) * width(l); ++k) {
             const double u1 = uniform(), u2 = uniform();
-            host[OFF.w[l] + k] = (float)(sd * std::sqrt(-2.0 * std::log(u1)) *
+            host[w_off(l) + k] = (float)(sd * std::sqrt(-2.0 * std::log(u1)) *
                                          std::cos(6.283185307179586 * u2));
         }
-        for (int k = 0; k < WIDTH[l + 1]; ++k) host[OFF.b[l] + k] = 0.0f;
+        for (int k = 0; k < width(l + 1); ++k) host[b_off(l) + k] = 0.0f;
     }
     const int rc = surr_set_params(c, host);
     delete[] host;
@@ -481,13 +744,13 @@ void surr_destroy(surr_ctx* c) {
     cudaFree(c->wq);
     cudaFree(c->loss);
     cudaFree(c->adam_t);
-    if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+    cudaFree(c->corr);
     delete c;
 }
 
 int surr_set_params(surr_ctx* c, const float* params) {
     if (!c || !params) return LBM_ERR_INVALID_ARG;
-    const size_t pb = sizeof(float) * OFF.total;
+    const size_t pb = sizeof(float) * NPARAM;
     cudaError_t e = cudaMemcpyAsync(c->params, params, pb, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->m, 0, pb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->v, 0, pb, c->stream);
@@ -499,7 +762,7 @@ int surr_set_params(surr_ctx* c, const float* params) {
 
 int surr_get_params(surr_ctx* c, float* params) {
     if (!c || !params) return LBM_ERR_INVALID_ARG;
-    cudaError_t e = cudaMemcpyAsync(params, c->params, sizeof(float) * OFF.total,
+    cudaError_t e = cudaMemcpyAsync(params, c->params, sizeof(float) * NPARAM,
                                     cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     return fail(e);
@@ -509,10 +772,10 @@ int surr_predict(surr_ctx* c, const float* X, int32_t n, float* D_out, float* lo
     if (!c || !X || n < 1) return LBM_ERR_INVALID_ARG;
     int rc = upload_batch(c, X, nullptr, nullptr, n);
     if (rc != LBM_OK) return rc;
-    forward(c, n);
+    run_net(c, n, false, false, false);
     float* out = new (std::nothrow) float[2 * (size_t)n];
     if (!out) return LBM_ERR_NOMEM;
-    cudaError_t e = cudaMemcpyAsync(out, c->act[NLAYER - 1], sizeof(float) * 2 * n,
+    cudaError_t e = cudaMemcpyAsync(out, c->out, sizeof(float) * 2 * n,
                                     cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess)
@@ -529,11 +792,11 @@ int surr_grad(surr_ctx* c, const float* X, const float* yD, const float* yB, int
     if (!c || !X || !yD || !yB || n < 1) return LBM_ERR_INVALID_ARG;
     int rc = upload_batch(c, X, yD, yB, n);
     if (rc != LBM_OK) return rc;
-    forward(c, n);
-    backward(c, n);
-    cudaError_t e = cudaSuccess;
-    if (grads)
-        e = cudaMemcpyAsync(grads, c->grads, sizeof(float) * OFF.total, cudaMemcpyDeviceToHost,
+    run_net(c, n, true, loss != nullptr, false);
+    if (grads) run_wgrad(c, n, false, 0.0f);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && grads)
+        e = cudaMemcpyAsync(grads, c->grads, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost,
                             c->stream);
     if (e == cudaSuccess && loss)
         e = cudaMemcpyAsync(loss, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
