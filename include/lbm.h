@@ -196,7 +196,11 @@ int lbm_launches_per_step(const lbm_ctx *ctx);
 /* Launch shape of the sweep kernels: threads per block (tile_x; the block
  * owns tile_x - 4 columns; 128 for FUSED; 128 or 192 for TMA with 16-bit
  * storage; 64, 128 or 192 for TMA with FP32 storage) and rows per block
- * (seg_y >= 4).
+ * (seg_y >= 4).  Until one is set (here, or cells per thread or store mode
+ * below), a TMA context takes the shape the library chooses for its grid: on
+ * small grids a step that holds all rows of 32-column tiles in flight at once
+ * instead of sweeping them (same bits), else the sweep with strips that fill
+ * the chip; the getter reports the sweep's shape either way.
  * 0 keeps the current value.
  * Errors: INVALID_ARG, UNSUPPORTED (split kernel, or tile_x not available). */
 int lbm_set_launch_shape(lbm_ctx *ctx, int32_t tile_x, int32_t seg_y);
@@ -247,7 +251,8 @@ int lbm_debug_stall_next_step(lbm_ctx *ctx);
  * and keeps the fastest shape.  Candidates (TMA kernel): (tile_x, cells per
  * thread) in {(128, 1), (192, 1), (64, 1), (128, 2), (192, 2)} with both
  * store modes for FP32 storage, and (128 or 192, 1 or 2) staged for 16-bit
- * storage; FUSED: tile_x 128.  seg_y in {8, 16, 32, 64, 128} plus the values
+ * storage, and the small-grid step (kept with the fastest sweep
+ * shape, which is what is reported); FUSED: tile_x 128.  seg_y in {8, 16, 32, 64, 128} plus the values
  * that fill one and two waves of resident blocks.  Needs one extra device buffer the size of a population
  * buffer while it runs.  Outputs (nullable): chosen shape and its time per
  * step in milliseconds.  Synchronous.

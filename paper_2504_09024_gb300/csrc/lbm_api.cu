@@ -60,6 +60,7 @@ struct lbm_ctx {
     cudaGraphExec_t graph[GRAPH_CHUNKS][2] = {};  // [log2(32 / steps)][parity]
     CUtensorMap tmaps[2];   // bulk-tensor load maps over the two population buffers
     lbm::StoreMaps smaps[2];  // bulk-tensor store maps over the same buffers
+    CUtensorMap tile_maps[2];  // load maps of the tile-parallel step
     // 16-bit storage: the state lives in pop16 (word planes, lbm_store16.cuh);
     // the FP32 buffers stage initialisation and field output
     int st = lbm::ST_F32;
@@ -200,6 +201,49 @@ lbm::KParams make_kparams(const lbm_params& p) {
     return k;
 }
 
+int sm_count() {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm > 0 ? nsm : 1;
+}
+
+// Launch shape of a run whose user has not set one.
+//  * Up to 14 tiles of 32 x 8 per SM: the tile-parallel step, 4 rows a tile
+//    while those fit the chip at once (three blocks per SM), else 8.  Measured
+//    on GB300 (FP32 coupled, us per step, against 128-wide strips of 32 rows
+//    before and the best sweep shape): 128 x 128 4.9 / 57.0 / 10.9, 512 x 256
+//    13.3 / 58.4 / 14.6, 1024 x 512 36.9 / 59.0 / 35.6; 2048 x 1024 128 / 136
+//    / 96, so larger grids take the sweep.
+//  * The sweep: the height that fills the chip with one wave of strips, of the
+//    width whose (rows + 5) x (time of a row at full residency) is least
+//    (row times in us, measured; 5 rows of each strip are halo and lag).  The
+//    widths are those that one and two cells per thread both have.
+//    2048 x 1024: FP32 136 -> 96, FP16 114 -> 91.
+lbm::FusedShape default_shape(const lbm::KParams& kp, int st) {
+    const int nsm = sm_count();
+    lbm::FusedShape best{192, 32, 1, st == lbm::ST_F32 ? lbm::OUT_DIRECT : lbm::OUT_STAGED};
+    double best_t = 1e300;
+    const struct { int bx; double row; } cand[2] = {{192, 2.15}, {128, 2.4}};
+    for (const auto& c : cand) {
+        const int slots = nsm * lbm::sweep2_blocks_per_sm(c.bx, 1, best.out, kp.coupled, st);
+        const int strips = (kp.nx + c.bx - 5) / (c.bx - 4);
+        const int nseg = std::max(1, slots / strips);
+        const int seg = std::max(4, (kp.ny + nseg - 1) / nseg);
+        const double waves = std::ceil((double)strips * ((kp.ny + seg - 1) / seg) / slots);
+        const double t = waves * (seg + 5) * c.row;
+        if (t < best_t) {
+            best_t = t;
+            best.bx = c.bx;
+            best.seg = seg;
+        }
+    }
+    const int64_t strips = (kp.nx + 31) / 32;
+    if (strips * ((kp.ny + 7) / 8) <= 14 * (int64_t)nsm)
+        best.tile = strips * ((kp.ny + 3) / 4) <= 3 * (int64_t)nsm ? 4 : 8;
+    return best;
+}
+
 // One time step from buffer src; step_off is the launch's offset within a
 // captured graph (the step counter of the stochastic roundings).
 void launch_one_step(lbm_ctx* ctx, int src, cudaStream_t st, int step_off = 0) {
@@ -208,7 +252,12 @@ void launch_one_step(lbm_ctx* ctx, int src, cudaStream_t st, int step_off = 0) {
     if (ctx->kernel == LBM_KERNEL_TMA) {
         float* dst = ctx->st == lbm::ST_F32 ? ctx->ds.pop[1 - src]
                                             : ctx->pop16_alloc[1 - src] + lbm::XGHOST;
-        lbm::launch_step_sweep2(kp, dst, ctx->ds.fields, ctx->shape, ctx->tmaps[src],
+        // (the stall hook is the sweep's)
+        if (ctx->shape.tile && !kp.stall_test)
+            lbm::launch_step_tile(kp, dst, ctx->ds.fields, ctx->shape.tile, ctx->tile_maps[src], ctx->st,
+                                  ctx->derr, st);
+        else
+            lbm::launch_step_sweep2(kp, dst, ctx->ds.fields, ctx->shape, ctx->tmaps[src],
                                 ctx->smaps[1 - src], ctx->st, ctx->derr, st);
     } else if (ctx->kernel == LBM_KERNEL_SPLIT) {
         lbm::launch_step_split(kp, ctx->ds, src, st);
@@ -223,7 +272,8 @@ int build_tensor_maps(lbm_ctx* ctx) {
     for (int b = 0; b < 2; ++b) {
         float* base = ctx->st == lbm::ST_F32 ? ctx->pop_alloc[b] : ctx->pop16_alloc[b];
         if (!lbm::make_tensor_map(&ctx->tmaps[b], base, ctx->kp, nplanes, ctx->shape.bx) ||
-            !lbm::make_store_maps(&ctx->smaps[b], base, ctx->kp, ctx->st, ctx->shape.bx))
+            !lbm::make_store_maps(&ctx->smaps[b], base, ctx->kp, ctx->st, ctx->shape.bx) ||
+            !lbm::make_tensor_map(&ctx->tile_maps[b], base, ctx->kp, nplanes, lbm::tile_map_bx()))
             return LBM_ERR_UNSUPPORTED;
     }
     return LBM_OK;
@@ -342,8 +392,6 @@ int lbm_create(const lbm_params* p, void* stream, lbm_ctx** out) {
                                                                        : LBM_KERNEL_FUSED)
                                                : p->kernel;
     ctx->st = p->dtype == LBM_F16S ? lbm::ST_F16 : (p->dtype == LBM_BF16S ? lbm::ST_BF16 : lbm::ST_F32);
-    // 16-bit rows leave through the staging area (staged bulk-tensor stores)
-    ctx->shape.out = ctx->st == lbm::ST_F32 ? lbm::OUT_DIRECT : lbm::OUT_STAGED;
     if (ctx->kernel == LBM_KERNEL_TMA && !lbm::tma_available()) {
         delete ctx;
         return LBM_ERR_UNSUPPORTED;
@@ -362,11 +410,13 @@ int lbm_create(const lbm_params* p, void* stream, lbm_ctx** out) {
         lbm_destroy(ctx);
         return LBM_ERR_CUDA;
     }
-    if (lbm::configure_fused_smem() != cudaSuccess || lbm::configure_sweep2_smem() != cudaSuccess) {
+    if (lbm::configure_fused_smem() != cudaSuccess || lbm::configure_sweep2_smem() != cudaSuccess ||
+        lbm::configure_tile_smem() != cudaSuccess) {
         cudaGetLastError();
         lbm_destroy(ctx);
         return LBM_ERR_CUDA;
     }
+    if (ctx->kernel == LBM_KERNEL_TMA) ctx->shape = default_shape(ctx->kp, ctx->st);
     ctx->ds.nlat = ctx->kp.coupled ? 3 : 2;
     const size_t pop_bytes = sizeof(float) * (size_t)ctx->ds.nlat * 9 * (size_t)ctx->kp.plane;
     const size_t fld_bytes = sizeof(float) * (size_t)lbm::FP_COUNT * (size_t)ctx->kp.plane;
@@ -681,6 +731,7 @@ int lbm_set_launch_shape(lbm_ctx* ctx, int32_t tile_x, int32_t seg_y) {
     if (!ok_bx) return LBM_ERR_UNSUPPORTED;
     if (tile_x) ctx->shape.bx = tile_x;
     if (seg_y) ctx->shape.seg = seg_y;
+    if (tile_x || seg_y) ctx->shape.tile = 0;
     drop_graphs(ctx);
     return build_tensor_maps(ctx);
 }
@@ -697,6 +748,7 @@ int lbm_set_cells_per_thread(lbm_ctx* ctx, int32_t cells) {
     if (ctx->kernel != LBM_KERNEL_TMA) return cells == 1 ? LBM_OK : LBM_ERR_UNSUPPORTED;
     if (!lbm::sweep2_shape_ok(ctx->shape.bx, cells, ctx->st)) return LBM_ERR_UNSUPPORTED;
     ctx->shape.cpt = cells;
+    ctx->shape.tile = 0;
     drop_graphs(ctx);
     return LBM_OK;
 }
@@ -709,6 +761,7 @@ int lbm_set_store_mode(lbm_ctx* ctx, int32_t mode) {
     if (!ctx || (mode != LBM_STORE_DIRECT && mode != LBM_STORE_STAGED)) return LBM_ERR_INVALID_ARG;
     if (ctx->kernel != LBM_KERNEL_TMA) return mode == LBM_STORE_DIRECT ? LBM_OK : LBM_ERR_UNSUPPORTED;
     ctx->shape.out = mode;
+    ctx->shape.tile = 0;
     drop_graphs(ctx);
     return LBM_OK;
 }
@@ -1326,13 +1379,6 @@ int lbm_batch_get_launch_shape(const lbm_batch* b, int32_t* tile_x, int32_t* seg
 
 namespace {
 
-int sm_count() {
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm > 0 ? nsm : 1;
-}
-
 // Rows per block worth trying for a grid of nx x ny: a fixed ladder plus the
 // values that fill one or two waves of resident blocks.
 int seg_candidates(int nx, int ny, int bx, int per_sm, int* out, int cap) {
@@ -1396,6 +1442,25 @@ int lbm_autotune(lbm_ctx* ctx, int32_t steps, int32_t* tile_x, int32_t* seg_y,
                     ++ncand;
                 }
     }
+    // ms per step of shape sh on the live state, which is put back afterwards
+    auto time_shape = [&](const lbm::FusedShape& sh) -> double {
+        float ms = 1e30f;
+        rc = set_shape(ctx, sh);
+        if (rc != LBM_OK) return ms;
+        // twice the timed count first: captures the graphs the timed steps
+        // replay, from either buffer parity
+        rc = lbm_step(ctx, 2 * (int64_t)steps);
+        if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventRecord(e0, ctx->stream));
+        if (rc == LBM_OK) rc = lbm_step(ctx, steps);
+        if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventRecord(e1, ctx->stream));
+        if (rc == LBM_OK) rc = lbm_synchronize(ctx);
+        if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventElapsedTime(&ms, e0, e1));
+        ce = cudaMemcpy(state_alloc(ctx, cur0), snap, pop_bytes, cudaMemcpyDeviceToDevice);
+        ctx->cur = cur0;
+        ctx->step = step0;
+        sync_step_ctr(ctx);
+        return ms / steps;
+    };
     for (int a = 0; a < ncand && ce == cudaSuccess && rc == LBM_OK; ++a) {
         const int bx = cand[a][0], cpt = cand[a][1], out = cand[a][2];
         const int per_sm = ctx->kernel != LBM_KERNEL_TMA
@@ -1403,28 +1468,25 @@ int lbm_autotune(lbm_ctx* ctx, int32_t steps, int32_t* tile_x, int32_t* seg_y,
                                : lbm::sweep2_blocks_per_sm(bx, cpt, out, ctx->kp.coupled, ctx->st);
         int segs[8];
         const int ns = seg_candidates(ctx->kp.nx, ctx->kp.ny, bx, per_sm, segs, 8);
-        for (int k = 0; k < ns && rc == LBM_OK; ++k) {
-            rc = set_shape(ctx, lbm::FusedShape{bx, segs[k], cpt, out});
-            if (rc != LBM_OK) break;
-            // twice the timed count first: captures the graphs the timed
-            // steps replay, from either buffer parity
-            rc = lbm_step(ctx, 2 * (int64_t)steps);
-            if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventRecord(e0, ctx->stream));
-            if (rc == LBM_OK) rc = lbm_step(ctx, steps);
-            if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventRecord(e1, ctx->stream));
-            if (rc == LBM_OK) rc = lbm_synchronize(ctx);
-            float ms = 0.0f;
-            if (rc == LBM_OK) rc = cuda_fail(ctx, cudaEventElapsedTime(&ms, e0, e1));
-            if (rc == LBM_OK && ms / steps < best) {
-                best = ms / steps;
-                best_shape = lbm::FusedShape{bx, segs[k], cpt, out};
+        for (int k = 0; k < ns && ce == cudaSuccess && rc == LBM_OK; ++k) {
+            const lbm::FusedShape sh{bx, segs[k], cpt, out};
+            const double ms = time_shape(sh);
+            if (rc == LBM_OK && ms < best) {
+                best = ms;
+                best_shape = sh;
             }
-            // put the state back before the next candidate
-            ce = cudaMemcpy(state_alloc(ctx, cur0), snap, pop_bytes, cudaMemcpyDeviceToDevice);
-            ctx->cur = cur0;
-            ctx->step = step0;
-            sync_step_ctr(ctx);
-            if (ce != cudaSuccess) break;
+        }
+    }
+    // the tile-parallel step, beside the best sweep shape (which is what the
+    // shape getters report and what setting it again selects: the same bits)
+    for (int tile : {4, 8}) {
+        if (ctx->kernel != LBM_KERNEL_TMA || ce != cudaSuccess || rc != LBM_OK) break;
+        lbm::FusedShape sh = best_shape;
+        sh.tile = tile;
+        const double ms = time_shape(sh);
+        if (rc == LBM_OK && ms < best) {
+            best = ms;
+            best_shape = sh;
         }
     }
     if (e0) cudaEventDestroy(e0);

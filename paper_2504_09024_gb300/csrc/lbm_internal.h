@@ -32,6 +32,7 @@ struct FusedShape {
     int seg;      // rows per block
     int cpt = 1;  // cells (adjacent columns) per thread of the bulk-tensor sweep
     int out = 0;  // its store mode: 0 direct stores, 1 staged bulk-tensor stores
+    int tile = 0; // rows per tile of the tile-parallel step (lbm_tile.cuh); 0: the sweep
 };
 
 // Bulk-tensor store maps of one population buffer (bulk-tensor sweep): the
@@ -105,6 +106,12 @@ bool make_store_maps(StoreMaps* m, float* alloc, const KParams& p, int st, int b
 void launch_step_sweep2(const KParams& p, float* dst, const float* fields, const FusedShape& sh,
                         const CUtensorMap& load_map, const StoreMaps& store_maps, int st,
                         int* err, cudaStream_t s);
+// Tile-parallel step (lbm_tile.cuh), every storage format: seg rows per tile,
+// load map with boxes of tile_map_bx() + 4 columns.
+int tile_map_bx();
+cudaError_t configure_tile_smem();
+void launch_step_tile(const KParams& p, float* dst, const float* fields, int seg, const CUtensorMap& load_map,
+                      int st, int* err, cudaStream_t s);
 // (per storage format)
 bool sweep2_f32_shape_ok(int bx, int cpt);
 size_t sweep2_f32_smem_bytes(int bx, int cpt, int out, bool coupled);

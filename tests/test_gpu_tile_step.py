@@ -1,0 +1,49 @@
+"""The tile-parallel step, which contexts with no launch shape set take on
+small grids, gives the bits of the sweep at every launch shape."""
+import numpy as np
+import pytest
+
+from paper_2504_09024_gb300 import lbm, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def run(nx, ny, dtype, walls, fixed_u, ratio, steps, shape=None):
+    phys = W.Physics(nx=nx, ny=ny, walls_y=walls, mode=int(fixed_u), u_wall=0.02 * walls, M_phi=0.02,
+                     D_s=0.02, nu_a=0.1 * ratio, rho_a=ratio, sigma_o=5e-3, beta=0.3)
+    phi, c = W.drop_fields(nx, ny, max(1.5, min(nx, ny) / 3.0), 4.0, xc=nx / 2 + 0.31, yc=ny / 2 + 0.17,
+                           c_of_theta=lambda t: 0.3 + 0.15 * np.cos(t))
+    ux = W.shear_profile(nx, ny, 0.02)[0] if walls else np.full_like(phi, 0.01)
+    s = lbm.Sim(phys, dtype=dtype, kernel=lbm.LBM_KERNEL_TMA)
+    if shape:
+        s.set_launch_shape(*shape)
+    s.init(phi, c, ux, np.full_like(phi, 0.004 * (1 - walls)))
+    s.step(steps)
+    out = s.pops()
+    s.close()
+    return out
+
+
+# tiles of 32 columns and of 4 rows, or 8 where the 4-row tiles outnumber the
+# resident blocks (1031 x 61: 528 of them): whole and ragged in both
+# directions, narrower than a tile, shorter than the halo
+@pytest.mark.parametrize("nx,ny", [(4, 4), (5, 7), (32, 8), (33, 17), (63, 4), (100, 61), (1031, 61)])
+@pytest.mark.parametrize("walls", [0, 1])
+@pytest.mark.parametrize("dtype,fixed_u,ratio", [
+    (lbm.LBM_F32, False, 1.0), (lbm.LBM_F32, False, 2.0), (lbm.LBM_F32, True, 1.0),
+    (lbm.LBM_F16S, False, 1.0), (lbm.LBM_BF16S, True, 1.0)])
+def test_tile_step_equals_sweep(nx, ny, walls, dtype, fixed_u, ratio):
+    a = run(nx, ny, dtype, walls, fixed_u, ratio, 41)
+    b = run(nx, ny, dtype, walls, fixed_u, ratio, 41, shape=(128, 16))
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+
+
+def test_library_shape_fills_one_wave():
+    """Beyond the tile-parallel range the chosen sweep shape covers the grid
+    in one wave of resident blocks."""
+    s = lbm.Sim(W.Physics(nx=2048, ny=1024))
+    bx, seg = lbm.lbm_get_launch_shape(s.ctx)
+    assert bx in (64, 128, 192) and seg >= 4
+    assert -(-2048 // (bx - 4)) * -(-1024 // seg) <= 152 * 6
+    s.close()
