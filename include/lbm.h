@@ -265,9 +265,9 @@ int lbm_autotune(lbm_ctx *ctx, int32_t steps, int32_t *tile_x, int32_t *seg_y,
  * Batches (ensembles of independent runs, e.g. drops in shear at different
  * grid sizes and parameters).  A batch owns one context per run and steps
  * them in one of two forms:
- *   LBM_BATCH_PERSISTENT  every time step is one launch of a persistent TMA
- *       sweep over the tiles of all runs, one launch per 64 runs; all runs
- *       share block width, cells per thread and rows per tile.  The runs'
+ *   LBM_BATCH_PERSISTENT  every time step is one launch over the tiles of all
+ *       runs (one block per tile), one launch per 64 runs; all runs share
+ *       block width, cells per thread and rows per tile.  The runs'
  *       parameters live in a bank in constant memory of 256 runs per
  *       device; a batch that finds no room there has the chains form only;
  *   LBM_BATCH_CHAINS      every run is stepped by its own single-run
@@ -315,9 +315,10 @@ int32_t lbm_batch_get_form(const lbm_batch *b);
  * tile (>= 4), cells per thread (1 or 2, see lbm_set_cells_per_thread) and
  * store mode (see lbm_set_store_mode) of the persistent form; 0 keeps the
  * current width and rows.  Setting them also sets
- * every run's own shape (chains form).  The getter also reports the
- * persistent grid size (blocks of all launches of a step) and the number of
- * tiles.  Errors: INVALID_ARG, UNSUPPORTED. */
+ * every run's own shape (chains form).  Until one is set the library chooses
+ * from the sizes of the runs (64-wide tiles; for small batches the small-grid
+ * step of lbm_set_launch_shape).  The getter also reports the number of blocks
+ * and of tiles of a step.  Errors: INVALID_ARG, UNSUPPORTED. */
 int lbm_batch_set_launch_shape(lbm_batch *b, int32_t tile_x, int32_t seg_y);
 int lbm_batch_set_cells_per_thread(lbm_batch *b, int32_t cells);
 int lbm_batch_set_store_mode(lbm_batch *b, int32_t mode);
@@ -327,7 +328,7 @@ int lbm_batch_get_launch_shape(const lbm_batch *b, int32_t *tile_x, int32_t *seg
 /* Autotuner of the batched step: the persistent form over (tile_x, cells
  * per thread, store mode) in {(64, 1, direct), (128, 1, direct), (192, 1,
  * direct), (64, 1, staged), (128, 1, staged), (128, 2, staged)} x seg_y in
- * {24, 32, 40, 48, 56, 64, 80}; the chains form with every run's shape from
+ * {16, 24, 32, 40, 48, 56, 64, 80} and the small-grid step; the chains form with every run's shape from
  * lbm_autotune on one run of each grid size, and with the shapes (192, 38,
  * 1, direct), (128, 32, 1, direct) and (192, 38, 2, direct) for every run;
  * the fastest form and shapes are kept.  Every candidate is timed over `steps` rounded up to whole 32-step

@@ -52,6 +52,7 @@ struct lbm_ctx {
     int64_t step = 0;
     int kernel = LBM_KERNEL_FUSED;
     lbm::FusedShape shape{128, 32};
+    bool width_set = false;  // the block width was set or tuned by the user, not by the library
     double* stage = nullptr;
     size_t stage_bytes = 0;
     double* dpartial = nullptr;
@@ -244,6 +245,15 @@ lbm::FusedShape default_shape(const lbm::KParams& kp, int st) {
     return best;
 }
 
+// The run's step by bulk-tensor loads, at its launch shape.
+void launch_tma_step(lbm_ctx* ctx, const lbm::KParams& kp, float* dst, int src, int* err, cudaStream_t st) {
+    if (ctx->shape.tile)
+        lbm::launch_step_tile(kp, dst, ctx->ds.fields, ctx->shape.tile, ctx->tile_maps[src], ctx->st, err, st);
+    else
+        lbm::launch_step_sweep2(kp, dst, ctx->ds.fields, ctx->shape, ctx->tmaps[src], ctx->smaps[1 - src],
+                                ctx->st, err, st);
+}
+
 // One time step from buffer src; step_off is the launch's offset within a
 // captured graph (the step counter of the stochastic roundings).
 void launch_one_step(lbm_ctx* ctx, int src, cudaStream_t st, int step_off = 0) {
@@ -252,13 +262,7 @@ void launch_one_step(lbm_ctx* ctx, int src, cudaStream_t st, int step_off = 0) {
     if (ctx->kernel == LBM_KERNEL_TMA) {
         float* dst = ctx->st == lbm::ST_F32 ? ctx->ds.pop[1 - src]
                                             : ctx->pop16_alloc[1 - src] + lbm::XGHOST;
-        // (the stall hook is the sweep's)
-        if (ctx->shape.tile && !kp.stall_test)
-            lbm::launch_step_tile(kp, dst, ctx->ds.fields, ctx->shape.tile, ctx->tile_maps[src], ctx->st,
-                                  ctx->derr, st);
-        else
-            lbm::launch_step_sweep2(kp, dst, ctx->ds.fields, ctx->shape, ctx->tmaps[src],
-                                ctx->smaps[1 - src], ctx->st, ctx->derr, st);
+        launch_tma_step(ctx, kp, dst, src, ctx->derr, st);
     } else if (ctx->kernel == LBM_KERNEL_SPLIT) {
         lbm::launch_step_split(kp, ctx->ds, src, st);
     } else {
@@ -729,7 +733,10 @@ int lbm_set_launch_shape(lbm_ctx* ctx, int32_t tile_x, int32_t seg_y) {
     const bool ok_bx = tile_x == 0 || (tma ? lbm::sweep2_shape_ok(tile_x, ctx->shape.cpt, ctx->st)
                                            : tile_x == 128);
     if (!ok_bx) return LBM_ERR_UNSUPPORTED;
-    if (tile_x) ctx->shape.bx = tile_x;
+    if (tile_x) {
+        ctx->shape.bx = tile_x;
+        ctx->width_set = true;
+    }
     if (seg_y) ctx->shape.seg = seg_y;
     if (tile_x || seg_y) ctx->shape.tile = 0;
     drop_graphs(ctx);
@@ -746,11 +753,14 @@ int lbm_get_launch_shape(const lbm_ctx* ctx, int32_t* tile_x, int32_t* seg_y) {
 int lbm_set_cells_per_thread(lbm_ctx* ctx, int32_t cells) {
     if (!ctx || cells < 1 || cells > 2) return LBM_ERR_INVALID_ARG;
     if (ctx->kernel != LBM_KERNEL_TMA) return cells == 1 ? LBM_OK : LBM_ERR_UNSUPPORTED;
-    if (!lbm::sweep2_shape_ok(ctx->shape.bx, cells, ctx->st)) return LBM_ERR_UNSUPPORTED;
-    ctx->shape.cpt = cells;
-    ctx->shape.tile = 0;
-    drop_graphs(ctx);
-    return LBM_OK;
+    lbm::FusedShape sh = ctx->shape;
+    if (!lbm::sweep2_shape_ok(sh.bx, cells, ctx->st)) {
+        if (ctx->width_set) return LBM_ERR_UNSUPPORTED;
+        sh.bx = 192;  // a width the library chose gives way to the user's cells
+    }
+    sh.cpt = cells;
+    sh.tile = 0;
+    return set_shape(ctx, sh);
 }
 
 int32_t lbm_get_cells_per_thread(const lbm_ctx* ctx) {
@@ -865,8 +875,8 @@ int lbm_load_state(lbm_ctx* ctx, const char* path) {
 
 // ---------------------------------------------------------------------------
 // Batches: many runs advanced together, in one of two forms.
-//  * persistent: every step is one launch of the persistent batch kernel over
-//    the tiles of all runs (one launch per table of BATCH_TABLE_RUNS runs);
+//  * persistent: every step is one launch of the batch kernel over the tiles
+//    of all runs (one launch per table of BATCH_TABLE_RUNS runs);
 //    all runs share the block width, cells per thread and rows per tile.
 //  * chains: every run is stepped by its own single-run launches, each run
 //    with its own launch shape, the runs' chains spread over side streams.
@@ -883,11 +893,11 @@ struct lbm_batch {
     cudaStream_t cap_stream = nullptr;
     bool coupled = true;
     int form = LBM_BATCH_PERSISTENT;
-    lbm::FusedShape shape{192, 32, 1};  // shape of the persistent form
+    lbm::FusedShape shape{64, 32, 1};   // shape of the persistent form
+    bool width_set = false;             // its block width was set or tuned by the user
     // persistent form: tables of run parameters and tilings, grids
     int ntab = 0;
     lbm::BatchTable* htab = nullptr;    // [ntab]
-    int* tab_blocks = nullptr;          // [ntab] grid sizes
     int nitems = 0;                     // tiles of a step
     lbm::RunDesc* hdesc = nullptr;      // host copy of the run table
     lbm::RunDesc* ddesc = nullptr;
@@ -925,22 +935,71 @@ int batch_fail(lbm_batch* b, cudaError_t e) {
     return LBM_ERR_CUDA;
 }
 
+// Launch shape of a batch whose user has not set one: the tile-parallel step up
+// to 14 tiles of 32 x 8 per SM (as for one run), else 64-wide strips, the
+// fastest width of the batch kernel at every size measured, of the height with
+// the least (waves of resident blocks, and a third for the last) x (rows + 5).
+// us per step (192 x 32 before, now): 10 runs of 768 x 256 146 -> 109, 128 of
+// 384 x 128 569 -> 358, 10 of 256 x 128 73 -> 27.  The 64-wide form has no two
+// cells per thread: setting that takes the 192-wide one.
+lbm::FusedShape batch_default_shape(const lbm_params* params, int nruns) {
+    const int nsm = sm_count();
+    lbm::FusedShape best{64, 32, 1, lbm::OUT_DIRECT};
+    const double slots = (double)nsm * lbm::batch_blocks_per_sm(params[0].mode == LBM_COUPLED);
+    double best_t = 1e300;
+    for (int seg : {8, 12, 16, 20, 24, 28, 32, 40, 48, 64}) {
+        double blocks = 0;
+        for (int r = 0; r < nruns; ++r)
+            blocks += (double)((params[r].nx + 59) / 60) * ((params[r].ny + seg - 1) / seg);
+        const double t = (std::max(1.0, blocks / slots) + 0.3) * (seg + 5);
+        if (t < best_t) {
+            best_t = t;
+            best.seg = seg;
+        }
+    }
+    int64_t tiles4 = 0, tiles8 = 0;
+    for (int r = 0; r < nruns; ++r) {
+        const int64_t strips = (params[r].nx + 31) / 32;
+        tiles4 += strips * ((params[r].ny + 3) / 4);
+        tiles8 += strips * ((params[r].ny + 7) / 8);
+    }
+    if (tiles8 <= 14 * (int64_t)nsm) best.tile = tiles4 <= 3 * (int64_t)nsm ? 4 : 8;
+    return best;
+}
+
+// Shape of the runs of a batch in the chains form, while the user has not set
+// one: that of the persistent form, but strips of the height that gives the
+// side streams' concurrent launches 1.3 times the resident blocks (a chain
+// pays (rows + 5) per launch, so where the blocks in flight do not fill the
+// chip shorter strips win).  us per step at the persistent form's height and
+// now: 128 runs of 384 x 128 478 -> 381, 32 of them 109 -> 96, 24 of 600 x 200
+// 148 -> 143; ten of 768 x 256 88 at 32 rows either way.
+lbm::FusedShape batch_chain_shape(const lbm_batch* b, int r) {
+    lbm::FusedShape sh = b->shape;
+    if (sh.tile) return sh;
+    const lbm::KParams& kp = b->runs[r]->kp;
+    const double want = 1.3 * sm_count() * lbm::batch_blocks_per_sm(b->coupled);
+    const int at_once = std::min(b->nruns, BATCH_SIDE_STREAMS);
+    const int strips = (kp.nx + sh.bx - 5) / (sh.bx - 4);
+    const int nseg = std::max(1, (int)(want / ((double)at_once * strips)));
+    sh.seg = std::max(8, (kp.ny + nseg - 1) / nseg);
+    return sh;
+}
+
 // Tensor maps, parameter tables, tilings and grids of the persistent form
 // for its current launch shape; run tables to the device.
 int batch_build_tiles(lbm_batch* b) {
     batch_drop_graphs(b);
-    const int bx = b->shape.bx, tx = bx - 4;
+    // tiles of the sweep, or of the tile-parallel step
+    const int bx = b->shape.tile ? lbm::tile_map_bx() : b->shape.bx;
+    const int tx = bx - 4, seg = b->shape.tile ? b->shape.tile : b->shape.seg;
     const int nl = b->coupled ? 3 : 2;
     int64_t total = 0;
     for (int r = 0; r < b->nruns; ++r) {
         const lbm_ctx* c = b->runs[r];
-        total += (int64_t)((c->kp.nx + tx - 1) / tx) * ((c->kp.ny + b->shape.seg - 1) / b->shape.seg);
+        total += (int64_t)((c->kp.nx + tx - 1) / tx) * ((c->kp.ny + seg - 1) / seg);
     }
     if (total > (int64_t)1 << 30) return LBM_ERR_INVALID_ARG;
-    const int per_sm = lbm::sweep2_batch_blocks_per_sm(bx, b->shape.cpt, b->shape.out, b->coupled);
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     for (int r = 0; r < b->nruns; ++r) {
         lbm_ctx* c = b->runs[r];
         lbm::RunDesc& d = b->hdesc[r];
@@ -951,7 +1010,7 @@ int batch_build_tiles(lbm_batch* b) {
             d.pop[k] = c->ds.pop[k];
         }
         d.fields = c->ds.fields;
-        d.seg = b->shape.seg;
+        d.seg = seg;
         d.flip = c->cur ^ b->parity;
         b->hkp[r] = c->kp;
     }
@@ -965,7 +1024,7 @@ int batch_build_tiles(lbm_batch* b) {
             const lbm_ctx* c = b->runs[r];
             const lbm::RunDesc& d = b->hdesc[r];
             lbm::BatchEntry& en = tab.e[r - r0];
-            const int nsx = (c->kp.nx + tx - 1) / tx, nsy = (c->kp.ny + b->shape.seg - 1) / b->shape.seg;
+            const int nsx = (c->kp.nx + tx - 1) / tx, nsy = (c->kp.ny + seg - 1) / seg;
             for (int k = 0; k < 2; ++k) {
                 en.tmap[k] = &b->ddesc[r].tmap[k];
                 en.smap[k] = &b->ddesc[r].smap[k];
@@ -981,7 +1040,6 @@ int batch_build_tiles(lbm_batch* b) {
         tab.nentries = r1 - r0;
         tab.ntiles = first;
         tab.slot0 = b->slot0 + r0;
-        b->tab_blocks[t] = std::min(first, per_sm * (nsm > 0 ? nsm : 1));
     }
     cudaError_t e = cudaMemcpy(b->ddesc, b->hdesc, sizeof(lbm::RunDesc) * b->nruns,
                                cudaMemcpyHostToDevice);
@@ -1025,9 +1083,7 @@ int batch_sync_desc(lbm_batch* b) {
 void batch_persistent_steps(lbm_batch* b, int parity, int n, cudaStream_t st) {
     for (int s = 0; s < n; ++s)
         for (int t = 0; t < b->ntab; ++t) {
-            lbm::BatchTable& tab = b->htab[t];
-            lbm::launch_sweep2_batch(tab, b->tab_blocks[t], b->shape, b->coupled,
-                                     parity ^ (s & 1), s, b->derr, st);
+            lbm::launch_batch(b->htab[t], b->shape, b->coupled, parity ^ (s & 1), s, b->derr, st);
         }
     lbm::launch_step_advance_many(b->dctrs, b->nruns, (unsigned)n, st);
 }
@@ -1063,8 +1119,7 @@ cudaError_t batch_chain_steps(lbm_batch* b, int parity, int n, cudaStream_t st) 
             lbm::KParams kp = c->kp;
             kp.step_off = s;
             float* dst = c->ds.pop[1 - src];
-            lbm::launch_step_sweep2(kp, dst, c->ds.fields, c->shape, c->tmaps[src],
-                                    c->smaps[1 - src], lbm::ST_F32, b->derr, b->side[k]);
+            launch_tma_step(c, kp, dst, src, b->derr, b->side[k]);
             src ^= 1;
         }
         lbm::launch_step_advance(c->dstep, (unsigned)n, b->side[k]);
@@ -1135,8 +1190,7 @@ int lbm_batch_create(const lbm_params* params, int32_t nruns, void* stream, lbm_
     b->hdesc = (lbm::RunDesc*)std::calloc((size_t)nruns, sizeof(lbm::RunDesc));
     b->hkp = (lbm::KParams*)std::calloc((size_t)nruns, sizeof(lbm::KParams));
     b->htab = (lbm::BatchTable*)std::calloc((size_t)b->ntab, sizeof(lbm::BatchTable));
-    b->tab_blocks = (int*)std::calloc((size_t)b->ntab, sizeof(int));
-    if (!b->runs || !b->hdesc || !b->hkp || !b->htab || !b->tab_blocks) {
+    if (!b->runs || !b->hdesc || !b->hkp || !b->htab) {
         lbm_batch_destroy(b);
         return LBM_ERR_NOMEM;
     }
@@ -1186,9 +1240,9 @@ int lbm_batch_create(const lbm_params* params, int32_t nruns, void* stream, lbm_
         return LBM_ERR_NOMEM;
     }
     cudaMemset(b->derr, 0, sizeof(int));
-    // the runs' own shapes (chains form) follow the persistent shape until tuned
+    b->shape = batch_default_shape(params, nruns);
     for (int r = 0; r < nruns; ++r) {
-        const int rc = set_shape(b->runs[r], b->shape);
+        const int rc = set_shape(b->runs[r], batch_chain_shape(b, r));
         if (rc != LBM_OK) {
             lbm_batch_destroy(b);
             return rc;
@@ -1213,7 +1267,6 @@ void lbm_batch_destroy(lbm_batch* b) {
     std::free(b->hdesc);
     std::free(b->hkp);
     std::free(b->htab);
-    std::free(b->tab_blocks);
     cudaFree(b->ddesc);
     cudaFree(b->dctrs);
     cudaFree(b->derr);
@@ -1324,8 +1377,13 @@ int lbm_batch_set_launch_shape(lbm_batch* b, int32_t tile_x, int32_t seg_y) {
     if (seg_y != 0 && seg_y < 4) return LBM_ERR_INVALID_ARG;
     const int rc = lbm_batch_synchronize(b);
     if (rc != LBM_OK) return rc;
-    if (tile_x) b->shape.bx = tile_x;
+    if (tile_x) {
+        b->shape.bx = tile_x;
+        b->width_set = true;
+        for (int r = 0; r < b->nruns; ++r) b->runs[r]->width_set = true;
+    }
     if (seg_y) b->shape.seg = seg_y;
+    if (tile_x || seg_y) b->shape.tile = 0;
     for (int r = 0; r < b->nruns; ++r) {
         const int rr = set_shape(b->runs[r], b->shape);
         if (rr != LBM_OK) return rr;
@@ -1338,6 +1396,7 @@ int lbm_batch_set_store_mode(lbm_batch* b, int32_t mode) {
     const int rc = lbm_batch_synchronize(b);
     if (rc != LBM_OK) return rc;
     b->shape.out = mode;
+    b->shape.tile = 0;
     for (int r = 0; r < b->nruns; ++r) {
         const int rr = set_shape(b->runs[r], b->shape);
         if (rr != LBM_OK) return rr;
@@ -1347,10 +1406,13 @@ int lbm_batch_set_store_mode(lbm_batch* b, int32_t mode) {
 
 int lbm_batch_set_cells_per_thread(lbm_batch* b, int32_t cells) {
     if (!b || cells < 1 || cells > 2) return LBM_ERR_INVALID_ARG;
-    if (!lbm::sweep2_shape_ok(b->shape.bx, cells, lbm::ST_F32)) return LBM_ERR_UNSUPPORTED;
+    const bool fits = lbm::sweep2_shape_ok(b->shape.bx, cells, lbm::ST_F32);
+    if (!fits && b->width_set) return LBM_ERR_UNSUPPORTED;
     const int rc = lbm_batch_synchronize(b);
     if (rc != LBM_OK) return rc;
+    if (!fits) b->shape.bx = 192;  // a width the library chose gives way to the user's cells
     b->shape.cpt = cells;
+    b->shape.tile = 0;
     for (int r = 0; r < b->nruns; ++r) {
         const int rr = set_shape(b->runs[r], b->shape);
         if (rr != LBM_OK) return rr;
@@ -1363,9 +1425,7 @@ int lbm_batch_get_launch_shape(const lbm_batch* b, int32_t* tile_x, int32_t* seg
     if (!b) return LBM_ERR_INVALID_ARG;
     if (tile_x) *tile_x = b->shape.bx;
     if (seg_y) *seg_y = b->shape.seg;
-    int nb = 0;
-    for (int t = 0; t < b->ntab; ++t) nb += b->tab_blocks[t];
-    if (blocks) *blocks = nb;
+    if (blocks) *blocks = b->nitems;  // one block per tile
     if (tiles) *tiles = b->nitems;
     return LBM_OK;
 }
@@ -1494,6 +1554,7 @@ int lbm_autotune(lbm_ctx* ctx, int32_t steps, int32_t* tile_x, int32_t* seg_y,
     cudaFree(snap);
     if (ce != cudaSuccess) return cuda_fail(ctx, ce);
     const int rc2 = set_shape(ctx, best_shape);
+    ctx->width_set = true;
     if (rc != LBM_OK) return rc;
     if (rc2 != LBM_OK) return rc2;
     if (tile_x) *tile_x = best_shape.bx;
@@ -1571,9 +1632,9 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
     // tile heights (the tile count against the grid decides the last wave)
     const int ncand = b->slot0 >= 0 ? 6 : 0;
     const int cand[6][3] = {{64, 1, 0}, {128, 1, 0}, {192, 1, 0}, {64, 1, 1}, {128, 1, 1}, {128, 2, 1}};
-    const int segs[7] = {24, 32, 40, 48, 56, 64, 80};
+    const int segs[8] = {16, 24, 32, 40, 48, 56, 64, 80};
     for (int a = 0; a < ncand && ce == cudaSuccess && rc == LBM_OK; ++a) {
-        for (int k = 0; k < 7 && ce == cudaSuccess && rc == LBM_OK; ++k) {
+        for (int k = 0; k < 8 && ce == cudaSuccess && rc == LBM_OK; ++k) {
             b->shape = lbm::FusedShape{cand[a][0], segs[k], cand[a][1], cand[a][2]};
             rc = batch_build_tiles(b);
             double ms = 0.0;
@@ -1583,6 +1644,20 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
                 best_form = LBM_BATCH_PERSISTENT;
                 best_shape = b->shape;
             }
+        }
+    }
+    // the tile-parallel step, kept with the best sweep shape (reported)
+    for (int tile : {4, 8}) {
+        if (ncand == 0 || ce != cudaSuccess || rc != LBM_OK) break;
+        const lbm::FusedShape sweep = best_shape;
+        b->shape = sweep;
+        b->shape.tile = tile;
+        rc = batch_build_tiles(b);
+        double ms = 0.0;
+        if (rc == LBM_OK) rc = time_it(ms);
+        if (rc == LBM_OK && ms < best) {
+            best = ms;
+            best_shape = b->shape;
         }
     }
     // chains form: every grid size tuned on its first run (the shape shared
@@ -1638,6 +1713,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
     // persistent shape
     b->form = best_form;
     b->shape = best_shape;
+    b->width_set = true;
     for (int r = 0; r < b->nruns && rc == LBM_OK; ++r)
         rc = set_shape(b->runs[r], best_form == LBM_BATCH_CHAINS ? best_runs[r] : best_shape);
     std::free(best_runs);

@@ -43,7 +43,7 @@ struct StoreMaps {
 };
 
 // One run of a batch: its tensor maps (in global memory, where the
-// persistent batch kernel reads them), buffers and buffer parity.
+// batch kernels read them), buffers and buffer parity.
 struct alignas(128) RunDesc {
     CUtensorMap tmap[2];    // bulk-tensor load maps over the run's two population buffers
     StoreMaps smap[2];      // bulk-tensor store maps over the same buffers
@@ -53,8 +53,8 @@ struct alignas(128) RunDesc {
     int flip;               // the run reads buffer (parity ^ flip) at batch parity `parity`
 };
 
-// Tiling of up to BATCH_TABLE_RUNS runs, passed to the persistent batch
-// kernel as one kernel parameter; larger batches take one launch per table
+// Tiling of up to BATCH_TABLE_RUNS runs, passed to a batch kernel as one
+// kernel parameter; larger batches take one launch per table
 // per step.  Entry e covers the tiles first .. first + tiles - 1 of the
 // launch, strip-major within its run (tile t: strip (t - first) % nsx,
 // segment (t - first) / nsx); the run's parameters are slot slot0 + e of the
@@ -78,7 +78,7 @@ struct BatchTable {
 };
 static_assert(sizeof(BatchTable) <= 32764, "kernel parameters are limited to 32764 bytes");
 
-// The batch parameter bank: run parameters of the persistent batch kernel in
+// The batch parameter bank: run parameters of the batch kernels in
 // constant memory, BATCH_PARAM_SLOTS slots per device, handed out in
 // contiguous ranges (a kernel reads them with indexed constant loads, which
 // the constant cache serves as it serves kernel parameters).
@@ -127,12 +127,12 @@ cudaError_t configure_sweep2_16_smem();
 void launch_sweep2_16(const KParams& p, float* dst, const float* fields, const FusedShape& sh,
                       const CUtensorMap& load_map, const StoreMaps& store_maps, int st, int* err,
                       cudaStream_t s);
-// Batched step: one persistent launch over the tab.ntiles tiles of the runs
-// in `tab`, which share the launch shape (FP32 storage); step_off is the
-// launch's offset within its graph (the stochastic roundings' step).
-void launch_sweep2_batch(const BatchTable& tab, int blocks, const FusedShape& sh, bool coupled,
-                         int parity, int step_off, int* err, cudaStream_t st);
-int sweep2_batch_blocks_per_sm(int bx, int cpt, int out, bool coupled);
+// Batched step: one launch over the tab.ntiles tiles of the runs in `tab`,
+// which share the launch shape (FP32 storage); step_off is the launch's offset
+// within its graph (the stochastic roundings' step).
+int batch_blocks_per_sm(bool coupled);  // resident blocks of the 64-wide form
+void launch_batch(const BatchTable& tab, const FusedShape& sh, bool coupled, int parity, int step_off,
+                  int* err, cudaStream_t st);
 // Advance the device step counter of the stochastic roundings by n (one
 // counter, or the counters of nctr runs).
 void launch_step_advance(unsigned* ctr, unsigned n, cudaStream_t s);

@@ -1,6 +1,5 @@
 // Fused step with bulk-tensor (TMA) loads and stores, FP32 populations: the
-// step kernels (single run, and the persistent kernel over the tiles of a
-// batch of runs), tensor maps and launchers.  The sweep of one tile is in
+// step kernels (single run, and one launch over the tiles of a batch of runs), tensor maps and launchers.  The sweep of one tile is in
 // lbm_sweep2.cuh.
 #include <cstdio>
 #include <cstring>
@@ -10,31 +9,49 @@
 #include <cudaTypedefs.h>
 
 #include "lbm_sweep2.cuh"
+#include "lbm_tile.cuh"
 
 namespace lbm {
 
-// Run parameters of the persistent batch kernel (the batch parameter bank).
+// Run parameters of the batch kernels (the batch parameter bank).
 __constant__ KParams c_batch_params[BATCH_PARAM_SLOTS];
 
-// One time step of every run of a batch in one launch: each block walks the
-// tiles of the table with a stride of the grid size.  Runs may differ in size
-// and parameters; the entry of a tile is found by bisection over the table's
-// first tiles.  A run's parameters come from the parameter bank, the
-// addresses of its buffers and tensor maps from the table (a kernel
-// parameter); the maps themselves are in global memory.
-// Register budget of the persistent batch kernel.  A run's parameters come
-// from the bank by an index known only at run time, so the compiler holds
-// them in registers where the single-run kernel takes them as constant
-// operands: the one-cell form needs 130-160 registers a thread instead of 80
-// (held to 80 it spilled 200-300 bytes a thread and ran 1.6 times slower).
+// Register budget of the batch kernels.  A run's parameters come from the bank
+// by an index known only at run time, so they are no constant operands: what
+// does not fit the registers is loaded again at each use.  128- and 192-wide
+// blocks held to the 80 registers of the single-run kernel ran 1.3 times
+// slower than at 128 (198 against 146 us for ten runs of 768 x 256); 64-wide
+// ones take 96 and are the fastest.
 template <int BX, int CPT, bool COUPLED, int OUT>
 constexpr int batch_min_blocks() {
     constexpr int threads = 2 * BX / CPT;
-    constexpr int regs = CPT == 1 ? 128 : 168;
+    constexpr int regs = CPT == 1 ? (BX == 64 ? 96 : 128) : 168;
     constexpr int by_regs = 65536 / (regs * threads);
     return by_regs < 1 ? 1 : by_regs;
 }
 
+// The entry of tile `it` of a batch launch, by bisection over the table's
+// first tiles.  `it` is the block index, so the compiler sees that the entry
+// is the same for the whole block and takes its parameters and addresses from
+// the constant bank through uniform registers.
+__device__ __forceinline__ int batch_entry(const BatchTable& tab, int it) {
+    int lo = 0, hi = tab.nentries;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (tab.e[mid].first <= it) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// One time step of every run of a batch in one launch, one block per tile of
+// the table.  Runs may differ in size and parameters; a run's parameters come
+// from the parameter bank, the addresses of its buffers and tensor maps from
+// the table (a kernel parameter), the maps themselves are in global memory.
+// (Blocks that walked the tiles with a grid stride held the parameters in 130
+// to 160 registers, 16 warps per SM; here the 64-wide blocks need 96, five per
+// SM.)  Measured, us per step with the library's shapes before and now: ten
+// runs of 768 x 256 146 and 109, 128 runs of 384 x 128 569 and 358.
 template <int BX, int CPT, bool COUPLED, int OUT>
 __global__ void __launch_bounds__(2 * BX / CPT, (batch_min_blocks<BX, CPT, COUPLED, OUT>()))
     k_sweep2_batch(const __grid_constant__ BatchTable tab, int parity, int step_off,
@@ -52,24 +69,30 @@ __global__ void __launch_bounds__(2 * BX / CPT, (batch_min_blocks<BX, CPT, COUPL
         fence_barrier_init();
     }
     __syncthreads();
+    const int lo = batch_entry(tab, blockIdx.x);
+    const BatchEntry& en = tab.e[lo];
+    const KParams& p = c_batch_params[tab.slot0 + lo];
+    const int local = blockIdx.x - en.first;
+    const int sy = local / en.nsx, sx = local - sy * en.nsx;
+    const int src = parity ^ en.flip;
     uint32_t issued = 0;
-    for (int it = blockIdx.x; it < tab.ntiles; it += gridDim.x) {
-        int lo = 0, hi = tab.nentries;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (tab.e[mid].first <= it) lo = mid;
-            else hi = mid;
-        }
-        const BatchEntry& en = tab.e[lo];
-        const KParams& p = c_batch_params[tab.slot0 + lo];
-        const int local = it - en.first;
-        const int sy = local / en.nsx, sx = local - sy * en.nsx;
-        const int src = parity ^ en.flip;
-        const bool ok = sweep_tile2<BX, CPT, COUPLED, ST_F32, OUT>(
-            en.tmap[src], en.smap[1 - src], p, en.pop[1 - src], en.fields, en.seg, sx, sy, S,
-            step_seed_at(p, step_off), issued, err);
-        if (!ok) break;
-    }
+    sweep_tile2<BX, CPT, COUPLED, ST_F32, OUT>(en.tmap[src], en.smap[1 - src], p, en.pop[1 - src],
+                                               en.fields, en.seg, sx, sy, S, step_seed_at(p, step_off),
+                                               issued, err);
+}
+
+// The same over the tiles of the tile-parallel step (lbm_tile.cuh).
+template <bool COUPLED>
+__global__ void __launch_bounds__(TILE_NT, 3)
+    k_tile_batch(const __grid_constant__ BatchTable tab, int parity, int step_off, int* __restrict__ err) {
+    const int lo = batch_entry(tab, blockIdx.x);
+    const BatchEntry& en = tab.e[lo];
+    const KParams& p = c_batch_params[tab.slot0 + lo];
+    const int local = blockIdx.x - en.first;
+    const int sy = local / en.nsx, sx = local - sy * en.nsx;
+    const int src = parity ^ en.flip;
+    tile_step<COUPLED, ST_F32>(en.tmap[src], p, en.pop[1 - src], en.fields, en.seg, sx, sy,
+                               step_seed_at(p, step_off), err);
 }
 
 // ---------------------------------------------------------------------------
@@ -167,6 +190,10 @@ cudaError_t configure_sweep2_f32_smem() {
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, bf);
                 return 0;
             });
+    cudaFuncSetAttribute(k_tile_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)TileLayout<true, ST_F32>::bytes(TILE_SEG));
+    cudaFuncSetAttribute(k_tile_batch<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)TileLayout<false, ST_F32>::bytes(TILE_SEG));
     return cudaGetLastError();
 }
 
@@ -199,27 +226,33 @@ void launch_sweep2_f32(const KParams& p, float* dst, const float* fields, const 
     });
 }
 
-int sweep2_batch_blocks_per_sm(int bx, int cpt, int out, bool coupled) {
+int batch_blocks_per_sm(bool coupled) {
     int n = 0;
-    const size_t smem = sweep2_f32_smem_bytes(bx, cpt, out, coupled);
-    const cudaError_t e = with_shape_f32(bx, cpt, out, [&](auto B, auto C, auto O) {
-        return coupled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                             &n, k_sweep2_batch<B(), C(), true, O()>, 2 * B() / C(), smem)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                             &n, k_sweep2_batch<B(), C(), false, O()>, 2 * B() / C(), smem);
-    });
+    const size_t smem = sweep2_f32_smem_bytes(64, 1, OUT_DIRECT, coupled);
+    const cudaError_t e =
+        coupled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep2_batch<64, 1, true, OUT_DIRECT>, 128, smem)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep2_batch<64, 1, false, OUT_DIRECT>, 128, smem);
     return e == cudaSuccess && n > 0 ? n : 1;
 }
 
-void launch_sweep2_batch(const BatchTable& tab, int blocks, const FusedShape& sh, bool coupled,
-                         int parity, int step_off, int* err, cudaStream_t st) {
+void launch_batch(const BatchTable& tab, const FusedShape& sh, bool coupled, int parity, int step_off,
+                  int* err, cudaStream_t st) {
+    if (sh.tile) {
+        if (coupled)
+            k_tile_batch<true><<<tab.ntiles, TILE_NT, TileLayout<true, ST_F32>::bytes(sh.tile), st>>>(
+                tab, parity, step_off, err);
+        else
+            k_tile_batch<false><<<tab.ntiles, TILE_NT, TileLayout<false, ST_F32>::bytes(sh.tile), st>>>(
+                tab, parity, step_off, err);
+        return;
+    }
     const size_t smem = sweep2_f32_smem_bytes(sh.bx, sh.cpt, sh.out, coupled);
     with_shape_f32(sh.bx, sh.cpt, sh.out, [&](auto B, auto C, auto O) {
         if (coupled)
-            k_sweep2_batch<B(), C(), true, O()><<<blocks, 2 * B() / C(), smem, st>>>(
+            k_sweep2_batch<B(), C(), true, O()><<<tab.ntiles, 2 * B() / C(), smem, st>>>(
                 tab, parity, step_off, err);
         else
-            k_sweep2_batch<B(), C(), false, O()><<<blocks, 2 * B() / C(), smem, st>>>(
+            k_sweep2_batch<B(), C(), false, O()><<<tab.ntiles, 2 * B() / C(), smem, st>>>(
                 tab, parity, step_off, err);
         return 0;
     });

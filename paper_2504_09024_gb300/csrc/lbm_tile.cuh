@@ -43,11 +43,12 @@ struct TileLayout {
     static_assert((ST == ST_F32 ? 18 : 10) * TILE_W >= 3 * TILE_WW, "room for nx, ny, |grad phi|");
 };
 
-// seg: rows per tile (4 .. TILE_SEG).  err: device flag of the bounded wait.
+// Tile (bxi, byi) of a run.  seg: rows per tile (4 .. TILE_SEG); seed: the hash
+// of the step (step_seed); err: device flag of the bounded wait.
 template <bool COUPLED, int ST>
-__global__ void __launch_bounds__(TILE_NT, 3)
-    k_tile(const __grid_constant__ CUtensorMap tmap, KParams p, float* __restrict__ dst,
-           const float* __restrict__ F, int seg, int* __restrict__ err) {
+__device__ __forceinline__ void tile_step(const CUtensorMap* tmap, const KParams& p, float* __restrict__ dst,
+                                          const float* __restrict__ F, int seg, int bxi, int byi,
+                                          uint32_t seed, int* __restrict__ err) {
     using L = TileLayout<COUPLED, ST>;
     constexpr int W = TILE_W, WW = TILE_WW, TX = TILE_TX, SLOT = L::SLOT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -63,22 +64,24 @@ __global__ void __launch_bounds__(TILE_NT, 3)
     float* mom = reinterpret_cast<float*>(s_phi) + L::NFIELD * (seg + 4) * WW;  // [5][seg * TX]
 
     const int t = threadIdx.x;
-    const int x0 = blockIdx.x * TX, xend = min(x0 + TX, p.nx);
-    const int y0 = blockIdx.y * seg, y1 = min(y0 + seg, p.ny);
+    const int x0 = bxi * TX, xend = min(x0 + TX, p.nx);
+    const int y0 = byi * seg, y1 = min(y0 + seg, p.ny);
     const int rows = y1 - y0;
     if (t == 0) {
         mbar_init(bar, 1);
+        mbar_init(bar + 1, 1);  // the failure-path test hook
         fence_barrier_init();
         mbar_arrive_expect_tx(bar, (uint32_t)((rows + 6) * L::NL * W * sizeof(float)));
         for (int k = 0; k < rows + 6; ++k) {
             const int row = y0 - 3 + k;  // staged row k; rows beyond walls read fill values
             const int y = p.walls ? row : wrap_i(row, p.ny);
-            tma_load_3d(raw + k * SLOT, &tmap, x0 - 4 + XGHOST, y, 0, bar);
+            tma_load_3d(raw + k * SLOT, tmap, x0 - 4 + XGHOST, y, 0, bar);
         }
     }
-    const uint32_t seed = step_seed(p);
     __syncthreads();  // the barrier is initialised
-    const bool ok = mbar_wait_bounded(bar, 0);
+    bool ok = mbar_wait_bounded(bar, 0);
+    // failure-path test: wait on a barrier that no copy completes
+    if (p.stall_test) ok = mbar_wait_bounded(bar + 1, 0, 4096) && ok;
 
     // ---------------- A: moments of the window ----------------
     if (ok) {
@@ -249,6 +252,13 @@ __global__ void __launch_bounds__(TILE_NT, 3)
             });
         }
     }
+}
+
+template <bool COUPLED, int ST>
+__global__ void __launch_bounds__(TILE_NT, 3)
+    k_tile(const __grid_constant__ CUtensorMap tmap, KParams p, float* __restrict__ dst,
+           const float* __restrict__ F, int seg, int* __restrict__ err) {
+    tile_step<COUPLED, ST>(&tmap, p, dst, F, seg, blockIdx.x, blockIdx.y, step_seed(p), err);
 }
 
 }  // namespace lbm

@@ -47,3 +47,69 @@ def test_library_shape_fills_one_wave():
     assert bx in (64, 128, 192) and seg >= 4
     assert -(-2048 // (bx - 4)) * -(-1024 // seg) <= 152 * 6
     s.close()
+
+
+@pytest.mark.parametrize("grids", [[(100, 60), (72, 44), (64, 5)], [(1031, 61)] * 6 + [(300, 40)] * 3])
+@pytest.mark.parametrize("fixed_u", [False, True])
+def test_batch_shapes_agree_bitwise(grids, fixed_u):
+    """Batches at the library's shape (the tile-parallel step here: 4 and 8
+    rows a tile), in both forms, give the bits of the sweep at a set shape."""
+    out = []
+    for form, shape in ((lbm.LBM_BATCH_PERSISTENT, None), (lbm.LBM_BATCH_CHAINS, None),
+                        (lbm.LBM_BATCH_PERSISTENT, (192, 24)), (lbm.LBM_BATCH_PERSISTENT, (64, 16))):
+        physics = [W.Physics(nx=nx, ny=ny, walls_y=0 if fixed_u else k % 2, mode=int(fixed_u), M_phi=0.02,
+                             D_s=0.02 + 0.01 * k, sigma_o=5e-3, beta=0.05 * k)
+                   for k, (nx, ny) in enumerate(grids)]
+        b = lbm.Batch(physics)
+        b.set_form(form)
+        if shape:
+            b.set_launch_shape(*shape)
+        for r, (nx, ny) in zip(b.runs, grids):
+            phi, c = W.drop_fields(nx, ny, max(1.5, min(nx, ny) / 3.0), 4.0, xc=nx / 2 + 0.31, c0=0.3)
+            r.init(phi, c, np.full_like(phi, 0.01), np.zeros_like(phi))
+        b.step(37)
+        b.sync()
+        out.append([r.pops() for r in b.runs])
+        b.close()
+    for other in out[1:]:
+        for p, q in zip(out[0], other):
+            for k in p:
+                np.testing.assert_array_equal(p[k], q[k], err_msg=k)
+
+
+def test_two_cells_per_thread_on_the_librarys_shape():
+    """A width the library chose gives way where two cells per thread do not
+    have it; one the user set does not."""
+    phys = W.Physics(nx=100, ny=60)
+    b = lbm.Batch([phys, phys])
+    lbm.lbm_set_cells_per_thread(b.runs[0].ctx, 2)
+    b.set_cells_per_thread(2)
+    assert b.launch_shape()[0] in (128, 192)
+    b.set_cells_per_thread(1)
+    b.set_launch_shape(64, 16)
+    with pytest.raises(lbm.LBMError):
+        b.set_cells_per_thread(2)
+    b.close()
+
+
+def test_batch_stall_hook_on_the_tile_step():
+    """The bounded wait of the tile-parallel step, in a batch and alone."""
+    phys = W.Physics(nx=100, ny=60)
+    phi, c = W.drop_fields(100, 60, 14.0, 4.0, c0=0.3)
+    z = np.zeros_like(phi)
+    b = lbm.Batch([phys, phys])
+    s = lbm.Sim(phys, kernel=lbm.LBM_KERNEL_TMA)
+    for r in (b.runs[0], b.runs[1], s):
+        r.init(phi, c, z, z)
+    for r, obj in ((b.runs[1], b), (s, s)):
+        lbm.lbm_debug_stall_next_step(r.ctx)
+        obj.step(1)
+        with pytest.raises(lbm.LBMError) as e:
+            obj.sync()
+        assert e.value.code == lbm.LBM_ERR_TIMEOUT
+        r.init(phi, c, z, z)
+        obj.step(3)
+        obj.sync()
+        assert np.isfinite(r.fields()["phi"]).all()
+    s.close()
+    b.close()
