@@ -517,11 +517,11 @@ def ensemble_comparison(args, stream):
             "timing": f"median of 3 regions of {k} steps, CUDA events"}
 
 
-# The D3Q27 phase-field + surfactant step (include/lbm3.h): 27 fixed-point
-# words per lattice read and written once per cell update, two lattices.
-BYTES_PER_CELL_3D = 432
+# The D3Q27 phase-field + surfactant step (include/lbm3.h): the four moments
+# that are kept of each lattice, read and written once per cell update.
+BYTES_PER_CELL_3D = 64
 SPHERE3D_N = {"sphere3d": 256, "sphere3d-384": 384,
-              "sphere3d-128": 128}  # 128^3 (0.9 GB, above L2): the profiler's small case
+              "sphere3d-128": 128}  # 128^3 (134 MB of states, just above L2)
 
 
 def sphere3d_case(n):
@@ -623,7 +623,8 @@ def run_sphere3d(args, rank, world, local_rank):
                    "kernel": "k3_step", "launch_shape": r["launch_shape"],
                    "launch_shape_from": "command line" if (args.rows or args.seg_z) else "lbm3_autotune",
                    "timed_regions": f"median of {args.repeats} regions of {args.steps} steps",
-                   "l2": f"populations (2 x {ncell * 216 / 1e9:.1f} GB) exceed the 129 MB L2; no flush",
+                   "l2": f"states (2 x {ncell * 32 / 1e9:.2f} GB) "
+                         f"{'exceed' if ncell * 64 > 129e6 else 'fit'} the 129 MB L2; no flush",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "roofline": r["roofline"],
         "e2e": {"value": whole_job_mlups(world, ncell, args.steps, r["e2e_s"]), "unit": UNIT,

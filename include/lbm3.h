@@ -27,14 +27,15 @@
  *   - Population arrays are [27][nz][ny][nx] float64.  Population a has
  *     velocity (E[a % 3], E[(a / 3) % 3], E[a / 9]) with E = {0, +1, -1};
  *     lbm3_velocities() returns the list.
- *   - Populations are stored on the device as int32 fixed point in units of
- *     2^-28 (range +-8), plane by plane ([nz][27][ny][nx] words per lattice),
- *     two buffers of 2 x 27 x nx ny nz words (ping-pong);
- *     the collision arithmetic is FP32.  The pull sums are exact integer sums
- *     and each collision gives its rest population the integer remainder of
- *     the cell's zeroth moment, so sum phi and sum c are conserved exactly.
- *     A cell whose phi or c leaves (-4, 4) marks its populations invalid;
- *     outputs show them as NaN and lbm3_sums counts them.
+ *   - Populations are int32 fixed point in units of 2^-28 (range +-8) and
+ *     the collision arithmetic is FP32.  Between steps the device holds only
+ *     the four sums of them that a collision reads, s and j of each lattice
+ *     ([nz][4][ny][nx][2] words, two buffers), and the initial fields; the
+ *     populations are formed again when they are asked for.  The sums are
+ *     exact in integers and each collision gives its rest population the
+ *     integer remainder of the cell's zeroth moment, so sum phi and sum c are
+ *     conserved exactly.  A cell whose phi or c leaves (-4, 4) marks its
+ *     populations invalid; outputs show them as NaN and lbm3_sums counts them.
  *   - Work runs on the stream given to lbm3_create (NULL: the library's own
  *     non-blocking stream).  lbm3_step is asynchronous; calls that return data
  *     to the host synchronise that stream.
@@ -50,9 +51,9 @@
 extern "C" {
 #endif
 
-/* nx * ny * nz may not exceed this (populations of 2^31 cells would need
- * 464 GB; 2^30 cells need 232 GB of the GPU's memory), and 27 * nx * ny must
- * stay below 2^31 (offsets inside a plane's 27 populations are 32-bit). */
+/* nx * ny * nz may not exceed this (2^30 cells need 86 GB of the GPU's memory,
+ * 129 GB with a velocity field), and 27 * nx * ny must stay below 2^31 (offsets
+ * inside a plane are 32-bit). */
 #define LBM3_MAX_CELLS 1073741824LL
 
 typedef struct lbm3_params {
@@ -71,8 +72,9 @@ typedef struct lbm3_ctx lbm3_ctx;
 int lbm3_params_default(lbm3_params *p);
 
 /* Validate *p and create a context on the current CUDA device.
- * stream: a cudaStream_t or NULL.  Allocates the two population buffers, the
- * velocity field (velocity_field = 1) and reduction scratch.
+ * stream: a cudaStream_t or NULL.  Allocates the two state buffers, room for
+ * the initial fields, the velocity field (velocity_field = 1) and reduction
+ * scratch.
  * Errors: INVALID_ARG (NULL, a size < 1, too many cells, 27 nx ny >= 2^31, phi_a == phi_b,
  * |phi_a| or |phi_b| > 2, a uniform |u_i| >= 1/2, W <= 0, a non-finite
  * value), RATE (M_phi or D_s <= 0), NOMEM, CUDA. */
@@ -94,7 +96,7 @@ int lbm3_init_fields_device(lbm3_ctx *ctx, const double *phi, const double *c,
                             const double *ux, const double *uy, const double *uz);
 
 /* Advance nsteps >= 0 time steps, one kernel launch per step: streaming
- * (pull), phi and c, the normal and theta, theta_c, and both collisions.
+ * phi and c, the normal and theta, theta_c, both collisions and streaming.
  * Asynchronous. */
 int lbm3_step(lbm3_ctx *ctx, int64_t nsteps);
 
@@ -130,7 +132,8 @@ int64_t lbm3_get_step(const lbm3_ctx *ctx);
 /* Launch shape of the step kernel: rows = tile height in cells including the
  * one-cell halo on each side (one warp per row, 32 columns of which 30 are
  * updated), one of 6, 10, 18; seg_z = planes a block marches through, >= 1.
- * 0 keeps the current value.  INVALID_ARG otherwise. */
+ * 0 keeps the current value.  INVALID_ARG otherwise.  A new context has a
+ * shape chosen by its grid and kind of velocity. */
 int lbm3_set_launch_shape(lbm3_ctx *ctx, int32_t rows, int32_t seg_z);
 int lbm3_get_launch_shape(const lbm3_ctx *ctx, int32_t *rows, int32_t *seg_z);
 

@@ -84,11 +84,11 @@ SOURCES_3D = ["lbm3d.cu"]
 def source_hash(which: str = "2d") -> str:
     """Hash of the sources of one kernel family, keying profiler records:
     "2d" -- the coupled D2Q9 sweeps, their headers and include/lbm.h;
-    "3d" -- the D3Q27 step (lbm3d.cu) and include/lbm3.h."""
+    "3d" -- the D3Q27 step (lbm3d.cu, lbm_vec.cuh) and include/lbm3.h."""
     import hashlib
     h = hashlib.sha256()
     if which == "3d":
-        for f in SOURCES_3D:
+        for f in SOURCES_3D + ["lbm_vec.cuh"]:
             h.update(open(os.path.join(CSRC, f), "rb").read())
         h.update(open(os.path.join(ROOT, "include", "lbm3.h"), "rb").read())
         return h.hexdigest()[:16]

@@ -15,32 +15,45 @@
 //     A = central (1, 0, cs^2) -> (1 - cs^2 - u^2, (cs^2 + u^2 + u)/2, (cs^2 + u^2 - u)/2)
 //     B = central (0, 1, 0)    -> (-2u, u + 1/2, u - 1/2)
 //     C = central (1, 0, 0)    -> (1 - u^2, (u^2 + u)/2, (u^2 - u)/2).
-// A collision therefore needs only s = sum a and j = sum e a of the incoming
-// populations: the pull loads are summed as they arrive.
 //
-// Storage in fixed point.  Populations are int32 in units of 2^-28 (range
-// +-8), plane by plane: word (z, q, y, x) of a lattice is at
-// ((z * 27 + q) * ny + y) * nx + x, so every offset inside a plane's 27
-// populations fits 32 bits (27 nx ny < 2^31) and only the plane base is 64-bit.  The pull sums are exact integer sums; the collision runs in FP32 on
-// those moments, its 26 moving outputs are rounded to the grid, and the rest
-// population takes the integer remainder s - sum(others), so every collision
-// conserves sum f and sum h exactly.  (With FP32 storage every cell of a
-// uniform region makes the same rounding error in every step and the region's
-// phi drifts coherently; in integers a uniform region is an exact fixed
-// point.)  A cell whose zeroth moment leaves (-4, 4) stores FX_BAD in all its
-// populations; the reductions count them.
+// State: four words a lattice and cell.  A collision therefore needs only
+// s = sum a and j = sum e a of the incoming populations, and those four sums
+// are all that is kept between steps: int32 fixed point in units of 2^-28,
+// words 2 (((z * 4 + m) * ny + y) * nx + x) (f) and the next (h), m = s, jx, jy, jz.
+// A step forms the 27 outgoing populations of a cell in registers, rounds each
+// to the 2^-28 grid (the rest population takes the integer remainder of s, so
+// sum f and sum h are conserved exactly) and adds them into the sums of the
+// cells they stream to; the sums are exact in integers, so the state is the
+// one that storing all 54 populations gives, at 64 bytes a cell and step
+// instead of 432.  (With FP32 storage every cell of a uniform region makes the
+// same rounding error in every step and the region's phi drifts coherently; in
+// integers a uniform region is an exact fixed point.)
 //
-// Step kernel.  A block owns a 30 x (ROWS - 2) column tile with a one-cell
-// halo (one warp per row of 32 columns) and marches through seg_z planes.
-// At plane k it pulls the f populations of plane k + 1 for every tile and
-// halo cell (phi into a four-plane shared ring, the first moments of the
-// tile cells kept in registers for the next plane) and the h populations of
-// plane k for the tile cells, waits at one barrier, then updates the tile
-// cells of plane k: gradient of phi from the ring, normal, theta, theta_c,
-// both collisions, 54 coalesced stores.  With four ring slots the slot
-// written at plane k + 1 is one no thread still reads, and the one written at
-// plane k + 2 was last read before the barrier of plane k + 1, so one barrier
-// per plane suffices.
+// A cell whose zeroth moment leaves (-4, 4) sends FX_BAD in all its
+// populations.  Populations are formed again when they are asked for: those of
+// the state from the moments one step back (the other buffer), those of the
+// initial state from the fields it was made of, which the context keeps.  The
+// sums alone say phi, c and the totals, unless a population may have been out
+// of range; the step that saw such a cell raises the context's `wild` word,
+// and the outputs then look at every population.
+//
+// Step kernel.  A block owns a 30 x (ROWS - 2) column of cells with a one-cell
+// halo (one warp per row of 32 columns) and marches through seg_z planes.  At
+// plane k each thread forms the populations of its cell; along x they are
+// added by shuffles, along y through shared memory, along z in registers, and
+// the moments of plane k - 1 are then complete and stored.  phi of plane k + 2
+// (with a second halo cell for the gradient) is on its way to shared memory and
+// the moments of plane k + 1 are on their way to registers meanwhile.  The
+// exchange buffer and the phi plane alternate between two copies, so one
+// barrier per plane suffices.  Halo rows form only the populations that enter
+// the tile.
+//
+// What bounds it: instruction issue (66-73 % of the slots, DRAM at a fifth of
+// its rate).  256^3 at the library's shape, uniform u: 1980 us a step with all
+// populations stored, 575 us now (the 64 bytes a cell take 160 us); with a
+// velocity field 740 us.  f and h share packed FP32 instructions (lane x: f,
+// lane y: h), and what crosses rows goes as one 16-byte word per population
+// group: together 600 to 575 us (784 to 724 us with a field).
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -48,11 +61,15 @@
 #include <cstdint>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "lbm3.h"
+#include "lbm_vec.cuh"
 
 namespace {
+
+using lbm::f2;
 
 constexpr int Q27 = 27;
 constexpr int TILE_W = 32;   // columns of a tile row, halo included
@@ -63,6 +80,7 @@ constexpr double FX_ONE_D = 268435456.0;
 constexpr double FX_INV_D = 1.0 / 268435456.0;
 constexpr int FX_BAD = (-2147483647 - 1);       // invalid population marker
 constexpr float S_MAX = 4.0f;                   // valid |zeroth moment|
+constexpr float K_TAME = 0.3f * FX_ONE;         // sum of |k'| up to which no population leaves the range
 constexpr int SUM_BLOCKS = 1024;
 constexpr int SUM_THREADS = 256;
 
@@ -77,8 +95,10 @@ struct K3Params {
     float w_kappa, w_chi, M_phi, D_s;
     float c4W, c8W, phi_a, phi_b, phim, inv_dphi;
     float u[3];
-    float fac[3][3][3];  // uniform u: [axis][A, B, C][e = 0, +1, -1] factors
-    const float* uf;     // per-cell velocity [3][N], or null for the uniform u
+    // uniform u: factors A, B, C along x by e = 0, +1, -1, and the products of
+    // those along y and z, [c][b]: Ay Az, Cy Cz, By Cz, Cy Bz; in both lanes
+    float2 fx[3][3], aa[3][3], cc[3][3], bc[3][3], cb[3][3];
+    const float* uf;  // per-cell velocity [3][N], or null for the uniform u
 };
 
 __host__ __device__ __forceinline__ int wrapi(int v, int n) {
@@ -88,7 +108,7 @@ __host__ __device__ __forceinline__ int wrapi(int v, int n) {
 
 // One-dimensional factors of P^-1 F^-1(u) (index 0: e = 0, 1: e = +1, 2: e = -1).
 template <class T>
-__device__ __forceinline__ void axis_factors(T u, T* A, T* B, T* C) {
+__host__ __device__ __forceinline__ void axis_factors(T u, T* A, T* B, T* C) {
     const T u2 = u * u;
     const T t = T(1) / T(3) + u2;
     A[0] = T(1) - t;
@@ -121,309 +141,542 @@ __device__ __forceinline__ void emit27(const T (&Ax)[3], const T (&Bx)[3], const
     }
 }
 
-// Zeroth and first raw moments of the 27 populations pulled into a cell:
-// population (a, b, c) comes from (x - e_a, y - e_b, z - e_c).  Exact integer
-// sums (two's complement wrap-around is harmless: the true sums are in range).
-struct Moments {
-    uint32_t s, jx, jy, jz;
+__device__ __forceinline__ float fx_to_f(int v) { return (float)v * FX_INV; }
+
+// What the gradient needs of one plane of phi around a cell: phi smoothed over
+// the plane, and its smoothed differences along x and y (twice the derivative).
+// Differences of equal values are exactly zero.
+struct Plane {
+    float g0, gx, gy;
 };
 
-__device__ __forceinline__ Moments pull_moments(const int* __restrict__ base, long long pstride, int nxny,
-                                                const int (&zs)[3], const int (&ys)[3], const int (&xs)[3]) {
-    Moments m{0u, 0u, 0u, 0u};
-    const int x1 = nxny + xs[1], x2 = 2 * nxny + xs[2];
+template <class At>
+__device__ __forceinline__ Plane plane_of(At at) {
+    float m[3], d[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int* q0 = base + zs[c] * pstride + 9 * c * nxny;  // population (0, 0, c) of the plane
+    for (int r = 0; r < 3; ++r) {
+        const float l = at(r - 1, -1), o = at(r - 1, 0), h = at(r - 1, 1);
+        m[r] = __fmaf_rn(__fadd_rn(l, h), 1.0f / 6.0f, __fmul_rn(o, 2.0f / 3.0f));
+        d[r] = __fsub_rn(h, l);
+    }
+    return Plane{__fmaf_rn(__fadd_rn(m[0], m[2]), 1.0f / 6.0f, __fmul_rn(m[1], 2.0f / 3.0f)),
+                 __fmaf_rn(__fadd_rn(d[0], d[2]), 1.0f / 6.0f, __fmul_rn(d[1], 2.0f / 3.0f)),
+                 __fsub_rn(m[2], m[0])};
+}
+
+// A collision of both lattices (lane x: f, lane y: h), in fixed-point units:
+// zeroth moments, relaxed first-order central moments and the velocity.  Every
+// operation is written out (no contraction left to the compiler), so that the
+// step and the kernels that form populations again agree to the last bit.
+struct Collision {
+    int2 s_fx;
+    f2 s, k[3];
+    float u[3];
+    bool ok;    // both zeroth moments inside (-4, 4)
+    bool tame;  // no population can leave the fixed-point range, nor their sums 32 bits
+};
+
+template <bool UFIELD>
+__device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[4], const Plane& lo,
+                                             const Plane& mid, const Plane& hi, const float (&u)[3]) {
+    Collision r;
+    const float g[3] = {0.5f * __fmaf_rn(__fadd_rn(lo.gx, hi.gx), 1.0f / 6.0f, __fmul_rn(mid.gx, 2.0f / 3.0f)),
+                        0.5f * __fmaf_rn(__fadd_rn(lo.gy, hi.gy), 1.0f / 6.0f, __fmul_rn(mid.gy, 2.0f / 3.0f)),
+                        0.5f * __fsub_rn(hi.g0, lo.g0)};
+    const float g2 = __fmaf_rn(g[2], g[2], __fmaf_rn(g[1], g[1], __fmul_rn(g[0], g[0])));
+    const float inv = g2 > 1e-24f ? rsqrtf(g2) : 0.f;
+    r.s_fx = m[0];
+    r.s = f2((float)m[0].x, (float)m[0].y);
+    const float phi = __fmul_rn(r.s.x, FX_INV), c = __fmul_rn(r.s.y, FX_INV);
+    // theta (Eq. theta) and theta_c (Eq. ISS), times M_phi and D_s
+    const float theta =
+        __fmul_rn(__fmul_rn(__fmul_rn(p.c4W, __fsub_rn(p.phi_a, phi)), __fsub_rn(phi, p.phi_b)), p.inv_dphi);
+    const float thetac = __fmul_rn(__fmul_rn(__fmul_rn(p.c8W, c), __fsub_rn(p.phim, phi)), p.inv_dphi);
+    const f2 q(__fmul_rn(p.M_phi, theta) * FX_ONE, __fmul_rn(p.D_s, thetac) * FX_ONE);
+    const f2 w(p.w_kappa, p.w_chi);
+    float big = 0.f;
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int* row = q0 + ys[b];
-            q0 += 3 * nxny;
-            const uint32_t v0 = (uint32_t)__ldg(row + xs[0]);
-            const uint32_t v1 = (uint32_t)__ldg(row + x1);
-            const uint32_t v2 = (uint32_t)__ldg(row + x2);
-            const uint32_t sx = v0 + v1 + v2;
-            m.s += sx;
-            m.jx += v1 - v2;
-            if (b == 1) m.jy += sx;
-            if (b == 2) m.jy -= sx;
-            if (c == 1) m.jz += sx;
-            if (c == 2) m.jz -= sx;
+    for (int i = 0; i < 3; ++i) {
+        const f2 a = lbm::vfma(f2(-u[i]), r.s, f2((float)m[i + 1].x, (float)m[i + 1].y));
+        r.u[i] = u[i];
+        r.k[i] = lbm::vfma(w, lbm::vfma(q, f2(__fmul_rn(g[i], inv)), -a), a);
+        big += fabsf(r.k[i].x) + fabsf(r.k[i].y);  // NaN stays NaN
+    }
+    r.ok = fabsf(phi) < S_MAX && fabsf(c) < S_MAX;
+    // Uniform |u| < 1/2: over the 27 neighbours the A products add up to 1 and those of
+    // B and C to at most 3.2 a component, so |sum| < 4 + 3.2 * 0.3.  A field with
+    // |u| <= 1/4, each neighbour its own: 2.3 and 3.5, so |sum| < 2 * 2.3 + 3.5 * 0.3.
+    r.tame = r.ok && big < K_TAME;
+    if (UFIELD)
+        r.tame = r.tame && fmaxf(fabsf(phi), fabsf(c)) < 2.0f &&
+                 fmaxf(fmaxf(fabsf(u[0]), fabsf(u[1])), fabsf(u[2])) <= 0.25f;
+    return r;
+}
+
+// Populations (0, b, c), (1, b, c), (2, b, c) of both lattices, c = 0, 1, 2,
+// rounded to the grid: row(c, v0, v1, v2).  UFIELD takes the factors from the
+// cell's velocity, otherwise they come with the parameters.  The rest population
+// is left to the caller (v0 of b = c = 0).
+template <bool UFIELD, bool BAD, class Row>
+__device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r, int b, Row row) {
+    float A[3][3], B[3][3], C[3][3];
+    if constexpr (UFIELD) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float v = r.u[i], u2 = __fmul_rn(v, v), t = __fadd_rn(1.0f / 3.0f, u2);
+            A[i][0] = __fsub_rn(1.0f, t);
+            A[i][1] = __fmul_rn(0.5f, __fadd_rn(t, v));
+            A[i][2] = __fmul_rn(0.5f, __fsub_rn(t, v));
+            B[i][0] = -2.0f * v;
+            B[i][1] = __fadd_rn(v, 0.5f);
+            B[i][2] = __fsub_rn(v, 0.5f);
+            C[i][0] = __fsub_rn(1.0f, u2);
+            C[i][1] = __fmul_rn(0.5f, __fadd_rn(u2, v));
+            C[i][2] = __fmul_rn(0.5f, __fsub_rn(u2, v));
         }
     }
-    return m;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        f2 P, X, R;
+        if constexpr (UFIELD) {
+            P = r.s * f2(__fmul_rn(A[1][b], A[2][c]));
+            X = r.k[0] * f2(__fmul_rn(C[1][b], C[2][c]));
+            R = lbm::vfma(r.k[1], f2(__fmul_rn(B[1][b], C[2][c])), r.k[2] * f2(__fmul_rn(C[1][b], B[2][c])));
+        } else {
+            P = r.s * lbm::from_f2(p.aa[c][b]);
+            X = r.k[0] * lbm::from_f2(p.cc[c][b]);
+            R = lbm::vfma(r.k[1], lbm::from_f2(p.bc[c][b]), r.k[2] * lbm::from_f2(p.cb[c][b]));
+        }
+        uint2 v[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const f2 ax = UFIELD ? f2(A[0][a]) : lbm::from_f2(p.fx[0][a]),
+                     bx = UFIELD ? f2(B[0][a]) : lbm::from_f2(p.fx[1][a]),
+                     cx = UFIELD ? f2(C[0][a]) : lbm::from_f2(p.fx[2][a]);
+            const f2 t = lbm::vfma(R, cx, lbm::vfma(X, bx, P * ax));
+            int2 w = make_int2(__float2int_rn(t.x), __float2int_rn(t.y));
+            if (BAD && !r.ok) w = make_int2(FX_BAD, FX_BAD);
+            v[a] = make_uint2((uint32_t)w.x, (uint32_t)w.y);
+        }
+        row(c, v[0], v[1], v[2]);
+    }
 }
 
-__device__ __forceinline__ float fx_to_f(uint32_t v) { return (float)(int)v * FX_INV; }
-
-// Round the 26 moving outputs to the grid and give the rest population the
-// remainder of the exact zeroth moment s_fx (or FX_BAD everywhere).
-__device__ __forceinline__ void store_collision(int* __restrict__ o, int nxny, bool ok, uint32_t s_fx,
-                                                const float (&Ax)[3], const float (&Bx)[3], const float (&Cx)[3],
-                                                const float (&Ay)[3], const float (&By)[3], const float (&Cy)[3],
-                                                const float (&Az)[3], const float (&Bz)[3], const float (&Cz)[3],
-                                                float s, const float (&k)[3]) {
-    uint32_t moved = 0u;
-    emit27(Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, s, k[0], k[1], k[2], [&](int q, float v) {
-        if (q == 0) return;
-        const int iv = ok ? __float2int_rn(v * FX_ONE) : FX_BAD;
-        moved += (uint32_t)iv;
-        o[q * nxny] = iv;
-    });
-    o[0] = ok ? (int)(s_fx - moved) : FX_BAD;
+__device__ __forceinline__ uint2 operator+(uint2 a, uint2 b) { return make_uint2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ uint2 operator-(uint2 a, uint2 b) { return make_uint2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ uint2 from_left(uint2 v) {
+    return make_uint2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
+}
+__device__ __forceinline__ uint2 from_right(uint2 v) {
+    return make_uint2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
 }
 
-// Resident blocks per SM the register budget is sized for: 96 registers a
-// thread at 10 and 18 rows, 80 at 6 rows (four blocks of six warps; the
-// uniform-velocity variant spills 40 bytes there and is still the fastest
-// shape measured).
+// Resident blocks per SM the register budget is sized for: 80 registers a
+// thread at 6 rows, 96 at 10 and 18 (up to 190 bytes of spill at 6 rows, 84 at
+// 10 and 18 with a velocity field, 40 without).
 template <int ROWS>
 constexpr int k3_min_blocks() { return ROWS == 6 ? 4 : ROWS == 10 ? 2 : 1; }
 
+constexpr int RING_W = TILE_W + 2;
+template <int ROWS>
+constexpr int k3_ring_words() { return (ROWS + 2) * RING_W; }
+template <int ROWS>
+constexpr int k3_xchg_words() { return 24 * ROWS * TILE_W; }  // 6 x uint4 a cell
+template <int ROWS>
+constexpr int k3_smem() { return 4 * 2 * (k3_ring_words<ROWS>() + k3_xchg_words<ROWS>()); }
+
 template <int ROWS, bool UFIELD>
-__global__ void __launch_bounds__(ROWS * 32, k3_min_blocks<ROWS>()) k3_step(const K3Params p, const int* __restrict__ fa,
-                                                     const int* __restrict__ ha, int* __restrict__ fb,
-                                                     int* __restrict__ hb) {
-    __shared__ float ring[4][ROWS][TILE_W];
+__global__ void __launch_bounds__(ROWS * 32, k3_min_blocks<ROWS>())
+k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __restrict__ dst,
+        int* __restrict__ wild) {
+    extern __shared__ __align__(16) float smem[];
+    constexpr int RING = k3_ring_words<ROWS>(), XCHG = k3_xchg_words<ROWS>(), NT = ROWS * 32;
+    constexpr int PLANE = ROWS * TILE_W;
+    // per (c, b = 1, 2): sums and differences along x of f, then of h, [2][6][ROWS][TILE_W]
+    uint4* xchg = reinterpret_cast<uint4*>(smem);
+    float* ring = smem + 2 * XCHG;  // [2][ROWS + 2][RING_W]
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int gx = blockIdx.x * TILE_IN + tx - 1;
-    const int gy = blockIdx.y * (ROWS - 2) + ty - 1;
-    const bool inner = tx >= 1 && tx <= TILE_IN && ty >= 1 && ty <= ROWS - 2 && gx < p.nx && gy < p.ny;
-    const int x = wrapi(gx, p.nx), y = wrapi(gy, p.ny);
-    // source column / row of the velocity component e = 0, +1, -1
-    const int xs[3] = {x, wrapi(gx - 1, p.nx), wrapi(gx + 1, p.nx)};
-    const int ys[3] = {y * p.nx, wrapi(gy - 1, p.ny) * p.nx, wrapi(gy + 1, p.ny) * p.nx};
-    const long long N = p.N;
+    const int bx = blockIdx.x * TILE_IN, by = blockIdx.y * (ROWS - 2);
+    const int last = min(ROWS - 2, p.ny - by);  // last tile row that is updated
+    const bool inner = ty >= 1 && ty <= last;
+    const bool store = inner && tx >= 1 && tx <= TILE_IN && bx + tx - 1 < p.nx;
     const int nxny = (int)p.nxny;
-    const long long pstride = 27LL * nxny;  // words of one plane's 27 populations
+    const int cell = wrapi(by + ty - 1, p.ny) * p.nx + wrapi(bx + tx - 1, p.nx);  // inside a plane
+    // the two cells of the phi plane that this thread fetches
+    static_assert(RING <= 2 * NT, "two phi cells a thread");
+    const int i1 = threadIdx.x + NT;
+    const int o0 = wrapi(by + (int)threadIdx.x / RING_W - 2, p.ny) * p.nx +
+                   wrapi(bx + (int)threadIdx.x % RING_W - 2, p.nx);
+    const int o1 = i1 < RING ? wrapi(by + i1 / RING_W - 2, p.ny) * p.nx + wrapi(bx + i1 % RING_W - 2, p.nx) : 0;
+    const long long pstride = 8LL * nxny;  // words of one plane of the state
     const int z0 = blockIdx.z * p.seg_z;
     const int z1 = min(p.nz, z0 + p.seg_z);
+    auto next = [&](int z) { return z + 1 == p.nz ? 0 : z + 1; };
 
-    // source plane of the velocity component e = 0, +1, -1
-    auto planes = [&](int z, int (&zs)[3]) {
-        zs[0] = z;
-        zs[1] = wrapi(z - 1, p.nz);
-        zs[2] = wrapi(z + 1, p.nz);
+    auto fetch = [&](int z, int slot) {
+        const int* q = src + z * pstride;
+        ring[slot * RING + threadIdx.x] = fx_to_f(__ldg(q + 2 * o0));
+        if (i1 < RING) ring[slot * RING + i1] = fx_to_f(__ldg(q + 2 * o1));
+    };
+    auto plane = [&](int slot) {
+        const float* at = ring + slot * RING + (ty + 1) * RING_W + tx + 1;
+        return plane_of([&](int dy, int dx) { return at[dy * RING_W + dx]; });
+    };
+    auto moments = [&](int z, int2 (&m)[4]) {
+        const int2* q = reinterpret_cast<const int2*>(src + z * pstride);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m[i] = __ldg(q + (size_t)i * nxny + cell);
+    };
+    auto velocity = [&](int z, float (&u)[3]) {
+        const float* q = p.uf + (long long)z * nxny + cell;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[i] = UFIELD ? __ldg(q + i * p.N) : p.u[i];
     };
 
-    int sm = 0, sc = 1, sp = 2, sf = 3;  // ring slots of planes k - 1, k, k + 1 (sf: free)
-    int zs[3];
-    planes(wrapi(z0 - 1, p.nz), zs);
-    ring[sm][ty][tx] = fx_to_f(pull_moments(fa, pstride, nxny, zs, ys, xs).s);
-    planes(z0, zs);
-    Moments cur = pull_moments(fa, pstride, nxny, zs, ys, xs);
-    ring[sc][ty][tx] = fx_to_f(cur.s);
+    int zc = wrapi(z0 - 1, p.nz);  // the plane of k
+    fetch(wrapi(z0 - 2, p.nz), 0);
+    fetch(zc, 1);
+    int2 m[4];
+    float u[3];
+    moments(zc, m);
+    velocity(zc, u);
+    __syncthreads();
+    Plane lo = plane(0), mid = plane(1);
+    __syncthreads();
+    int zn = next(zc), zp = next(zn);
+    fetch(zn, 0);
+    __syncthreads();
 
-    const float w1[3] = {1.0f / 6.0f, 2.0f / 3.0f, 1.0f / 6.0f};  // offsets -1, 0, +1
+    // Sums on their way, of f and h: `part` of plane k - 1 (complete but for what
+    // comes from plane k), `up` of plane k (what came from plane k - 1).
+    uint2 part[4] = {}, up[3] = {};
+    int slot = 0;
+    for (int k = z0 - 1; k <= z1; ++k) {
+        int2 mn[4];
+        float un[3];
+        moments(zn, mn);
+        velocity(zn, un);
+        const int* q = src + zp * pstride;
+        const int f0 = __ldg(q + 2 * o0), f1 = __ldg(q + 2 * o1);
 
-    int zc[3];  // planes of the current k (for the h pull)
-    planes(z0, zc);
-    for (int k = z0; k < z1; ++k) {
-        planes(wrapi(k + 1, p.nz), zs);
-        const Moments nxt = pull_moments(fa, pstride, nxny, zs, ys, xs);
-        ring[sp][ty][tx] = fx_to_f(nxt.s);
-        Moments hm{0u, 0u, 0u, 0u};
-        if (inner) hm = pull_moments(ha, pstride, nxny, zc, ys, xs);
+        uint4* x = xchg + slot * (XCHG / 4) + ty * TILE_W + tx;
+        uint2 s0[3], d0[3];  // sums and differences along x of the populations that stay in the row
+        Plane hi{0.f, 0.f, 0.f};
+        if (ty <= last + 1) {
+            hi = plane(slot);
+            const Collision r = collide<UFIELD>(p, m, lo, mid, hi, u);
+            if (!r.tame) *wild = 1;
+            auto emit = [&](auto bad) {
+                constexpr bool BAD = decltype(bad)::value;
+                uint2 moved = make_uint2(0u, 0u);
+                // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
+                auto across = [&](int b) {
+                    emit_rows<UFIELD, BAD>(p, r, b, [&](int c, uint2 v0, uint2 v1, uint2 v2) {
+                        moved = moved + (v0 + v1 + v2);
+                        const uint2 t1 = from_left(v1), t2 = from_right(v2);
+                        const uint2 s = v0 + t1 + t2, d = t1 - t2;
+                        x[(2 * c + b - 1) * PLANE] = make_uint4(s.x, d.x, s.y, d.y);
+                    });
+                };
+                if (ty <= last) across(1);
+                if (ty >= 1) across(2);
+                if (inner) {
+                    uint2 r1, r2;
+                    emit_rows<UFIELD, BAD>(p, r, 0, [&](int c, uint2 v0, uint2 v1, uint2 v2) {
+                        const uint2 t1 = from_left(v1), t2 = from_right(v2);
+                        if (c == 0) {  // the rest population, once the other 26 are known
+                            moved = moved + (v1 + v2);
+                            r1 = t1;
+                            r2 = t2;
+                        } else {
+                            moved = moved + (v0 + v1 + v2);
+                            s0[c] = v0 + t1 + t2;
+                            d0[c] = t1 - t2;
+                        }
+                    });
+                    uint2 rest = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
+                    if (BAD && !r.ok) rest = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
+                    s0[0] = rest + r1 + r2;
+                    d0[0] = r1 - r2;
+                }
+            };
+            if (__all_sync(0xffffffffu, r.ok))
+                emit(std::false_type{});
+            else
+                emit(std::true_type{});
+        }
+        ring[(slot ^ 1) * RING + threadIdx.x] = fx_to_f(f0);
+        if (i1 < RING) ring[(slot ^ 1) * RING + i1] = fx_to_f(f1);
         __syncthreads();
         if (inner) {
-            // gradient d_i phi = (1/cs2) sum_a w_a e_ai phi(x + e_a), accumulated
-            // value by value from the ring (weights (1/2) w1 w1 on the two
-            // transverse offsets)
-            float gxv = 0.f, gyv = 0.f, gzv = 0.f;
+            uint2 S[3], JX[3], JY[3];
 #pragma unroll
-            for (int dz = 0; dz < 3; ++dz) {
-                const float(*plane)[TILE_W] = ring[dz == 0 ? sm : dz == 1 ? sc : sp];
-#pragma unroll
-                for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-                    for (int dx = 0; dx < 3; ++dx) {
-                        if (dx == 1 && dy == 1 && dz == 1) continue;
-                        const float v = plane[ty + dy - 1][tx + dx - 1];
-                        if (dx != 1) gxv += (dx == 2 ? w1[dy] * w1[dz] : -w1[dy] * w1[dz]) * v;
-                        if (dy != 1) gyv += (dy == 2 ? w1[dx] * w1[dz] : -w1[dx] * w1[dz]) * v;
-                        if (dz != 1) gzv += (dz == 2 ? w1[dx] * w1[dy] : -w1[dx] * w1[dy]) * v;
-                    }
+            for (int c = 0; c < 3; ++c) {
+                const uint4 dn = x[2 * c * PLANE - TILE_W];        // from y - 1
+                const uint4 ab = x[(2 * c + 1) * PLANE + TILE_W];  // from y + 1
+                S[c] = s0[c] + make_uint2(dn.x, dn.z) + make_uint2(ab.x, ab.z);
+                JX[c] = d0[c] + make_uint2(dn.y, dn.w) + make_uint2(ab.y, ab.w);
+                JY[c] = make_uint2(dn.x, dn.z) - make_uint2(ab.x, ab.z);
             }
-            gxv *= 0.5f;
-            gyv *= 0.5f;
-            gzv *= 0.5f;
-            const float g2 = gxv * gxv + gyv * gyv + gzv * gzv;
-            const float inv = g2 > 1e-24f ? rsqrtf(g2) : 0.f;
-            const float n3[3] = {gxv * inv, gyv * inv, gzv * inv};
-
-            const int co = ys[0] + x;                       // offset inside the plane
-            const long long cell = (long long)k * nxny + co;  // cell index (velocity field)
-            // velocity factors: from the parameters (uniform u) or per cell
-            float u3[3] = {p.u[0], p.u[1], p.u[2]};
-            float F[3][3][3];
-            if constexpr (UFIELD) {
-                u3[0] = p.uf[cell];
-                u3[1] = p.uf[N + cell];
-                u3[2] = p.uf[2 * N + cell];
-#pragma unroll
-                for (int ax = 0; ax < 3; ++ax) axis_factors(u3[ax], F[ax][0], F[ax][1], F[ax][2]);
+            if (store && k > z0) {
+                uint2* out = reinterpret_cast<uint2*>(dst + (k - 1) * pstride) + cell;
+                out[0] = part[0] + S[2];
+                out[(size_t)nxny] = part[1] + JX[2];
+                out[2 * (size_t)nxny] = part[2] + JY[2];
+                out[3 * (size_t)nxny] = part[3] - S[2];
             }
-            const float(*Fx)[3][3] = UFIELD ? F : p.fac;
-            const float(&Ax)[3] = Fx[0][0], (&Bx)[3] = Fx[0][1], (&Cx)[3] = Fx[0][2];
-            const float(&Ay)[3] = Fx[1][0], (&By)[3] = Fx[1][1], (&Cy)[3] = Fx[1][2];
-            const float(&Az)[3] = Fx[2][0], (&Bz)[3] = Fx[2][1], (&Cz)[3] = Fx[2][2];
-            // theta (Eq. theta) and theta_c (Eq. ISS)
-            const float phi = fx_to_f(cur.s), c = fx_to_f(hm.s);
-            const float theta = p.c4W * (p.phi_a - phi) * (phi - p.phi_b) * p.inv_dphi;
-            const float thetac = p.c8W * c * (p.phim - phi) * p.inv_dphi;
-            const float qf = p.M_phi * theta, qh = p.D_s * thetac;
-            // first-order central moments k = j - u s, relaxed towards K theta n
-            const float jf[3] = {fx_to_f(cur.jx), fx_to_f(cur.jy), fx_to_f(cur.jz)};
-            const float jh[3] = {fx_to_f(hm.jx), fx_to_f(hm.jy), fx_to_f(hm.jz)};
-            float kf[3], kh[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const float a = jf[i] - u3[i] * phi;
-                kf[i] = a + p.w_kappa * (qf * n3[i] - a);
-                const float b = jh[i] - u3[i] * c;
-                kh[i] = b + p.w_chi * (qh * n3[i] - b);
-            }
-            const bool ok = fabsf(phi) < S_MAX && fabsf(c) < S_MAX;
-            store_collision(fb + k * pstride + co, nxny, ok, cur.s, Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, phi, kf);
-            store_collision(hb + k * pstride + co, nxny, ok, hm.s, Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, c, kh);
+            part[0] = up[0] + S[0];
+            part[1] = up[1] + JX[0];
+            part[2] = up[2] + JY[0];
+            part[3] = up[0];
+            up[0] = S[1];
+            up[1] = JX[1];
+            up[2] = JY[1];
         }
-        const int t = sm;
-        sm = sc;
-        sc = sp;
-        sp = sf;
-        sf = t;
-        cur = nxt;
+        slot ^= 1;
+        lo = mid;
+        mid = hi;
+        zn = zp;
+        zp = next(zp);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) zc[i] = zs[i];
+        for (int i = 0; i < 4; ++i) m[i] = mn[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[i] = un[i];
     }
 }
 
-// Discrete equilibria of the given fields, written where the pull of the
-// first step reads them: the pull gives cell x population a from x - e_a of
-// buffer A, so population a of cell x is stored at x - e_a and the state (the
-// pulled populations) is the equilibrium at every cell.  FP64 arithmetic,
-// FP32 storage.
-__global__ void k3_init(const K3Params p, const double* __restrict__ phi, const double* __restrict__ c,
-                        const double* __restrict__ ux, const double* __restrict__ uy,
-                        const double* __restrict__ uz, double W, double phi_a, double phi_b,
-                        double M_phi, double D_s, int* __restrict__ fa, int* __restrict__ ha,
-                        float* __restrict__ uf) {
-    const long long N = p.N;
-    for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < N;
-         cell += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(cell % p.nx);
-        const int y = (int)((cell / p.nx) % p.ny);
-        const int z = (int)(cell / p.nxny);
-        const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
-        double g[3] = {0.0, 0.0, 0.0};
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const double v = phi[((long long)wrapi(z + dz, p.nz) * p.ny + wrapi(y + dy, p.ny)) * p.nx +
-                                         wrapi(x + dx, p.nx)];
-                    const double w = 3.0 * w1[dx + 1] * w1[dy + 1] * w1[dz + 1];
-                    g[0] += w * dx * v;
-                    g[1] += w * dy * v;
-                    g[2] += w * dz * v;
-                }
-        const double m = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-        double n[3];
-        for (int i = 0; i < 3; ++i) n[i] = m > 1e-12 ? g[i] / m : 0.0;
-        const double ph = phi[cell], cc = c[cell];
-        const double dphi = phi_a - phi_b;
-        const double theta = (4.0 / W) * (phi_a - ph) * (ph - phi_b) / dphi;
-        const double thetac = (8.0 * cc / W) * (0.5 * (phi_a + phi_b) - ph) / dphi;
-        double u[3] = {p.u[0], p.u[1], p.u[2]};
-        if (ux) {
-            u[0] = ux[cell];
-            u[1] = uy[cell];
-            u[2] = uz[cell];
-            uf[cell] = (float)u[0];
-            uf[N + cell] = (float)u[1];
-            uf[2 * N + cell] = (float)u[2];
-        }
-        double Ax[3], Bx[3], Cx[3], Ay[3], By[3], Cy[3], Az[3], Bz[3], Cz[3];
-        axis_factors(u[0], Ax, Bx, Cx);
-        axis_factors(u[1], Ay, By, Cy);
-        axis_factors(u[2], Az, Bz, Cz);
-        // destination of population (a, b, c): the cell x - e
-        const int xd[3] = {x, wrapi(x - 1, p.nx), wrapi(x + 1, p.nx)};
-        const int yd[3] = {y, wrapi(y - 1, p.ny), wrapi(y + 1, p.ny)};
-        const int zd[3] = {z, wrapi(z - 1, p.nz), wrapi(z + 1, p.nz)};
-        auto dest = [&](int q) {
-            const int a = q % 3, b = (q / 3) % 3, cq = q / 9;
-            return ((long long)zd[cq] * Q27 + q) * p.nxny + (long long)yd[b] * p.nx + xd[a];
-        };
-        const double qf = M_phi * theta, qh = D_s * thetac;
-        // non-finite or out-of-range values become FX_BAD
-        const bool ok = fabs(ph) < (double)S_MAX && fabs(cc) < (double)S_MAX;
-        auto fx = [&](double v) { return ok && fabs(v) < 8.0 ? (int)__double2ll_rn(v * FX_ONE_D) : FX_BAD; };
-        emit27(Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, ph, qf * n[0], qf * n[1], qf * n[2],
-               [&](int q, double v) { fa[dest(q)] = fx(v); });
-        emit27(Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, cc, qh * n[0], qh * n[1], qh * n[2],
-               [&](int q, double v) { ha[dest(q)] = fx(v); });
-    }
-}
+// The fields an initial state is made of (velocity null: uniform u).
+struct Seed {
+    const double *phi, *c, *u[3];
+    double W, phi_a, phi_b, M_phi, D_s;
+};
 
-// State of cell x: population a is buffer A's value at x - e_a (plane-major
-// word index, see the storage note at the top).
-__device__ __forceinline__ long long pull_src(const K3Params& p, long long cell, int q) {
+// Discrete equilibria of the given fields at one cell, in FP64, rounded to the
+// grid (FX_BAD for what is not finite or out of range): out(q, f, h).
+template <class Out>
+__device__ __forceinline__ void equilibrium(const K3Params& p, const Seed& in, long long cell, Out out) {
     const int x = (int)(cell % p.nx);
     const int y = (int)((cell / p.nx) % p.ny);
     const int z = (int)(cell / p.nxny);
-    const int E[3] = {0, 1, -1};
-    const int a = q % 3, b = (q / 3) % 3, c = q / 9;
-    return ((long long)wrapi(z - E[c], p.nz) * Q27 + q) * p.nxny + (long long)wrapi(y - E[b], p.ny) * p.nx +
-           wrapi(x - E[a], p.nx);
+    const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
+    double g[3] = {0.0, 0.0, 0.0};
+    for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const double v = in.phi[((long long)wrapi(z + dz, p.nz) * p.ny + wrapi(y + dy, p.ny)) * p.nx +
+                                        wrapi(x + dx, p.nx)];
+                const double w = 3.0 * w1[dx + 1] * w1[dy + 1] * w1[dz + 1];
+                g[0] += w * dx * v;
+                g[1] += w * dy * v;
+                g[2] += w * dz * v;
+            }
+    const double m = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    double n[3];
+    for (int i = 0; i < 3; ++i) n[i] = m > 1e-12 ? g[i] / m : 0.0;
+    const double ph = in.phi[cell], cc = in.c[cell];
+    const double dphi = in.phi_a - in.phi_b;
+    const double theta = (4.0 / in.W) * (in.phi_a - ph) * (ph - in.phi_b) / dphi;
+    const double thetac = (8.0 * cc / in.W) * (0.5 * (in.phi_a + in.phi_b) - ph) / dphi;
+    double u[3] = {p.u[0], p.u[1], p.u[2]};
+    if (in.u[0])
+        for (int i = 0; i < 3; ++i) u[i] = in.u[i][cell];
+    double Ax[3], Bx[3], Cx[3], Ay[3], By[3], Cy[3], Az[3], Bz[3], Cz[3];
+    axis_factors(u[0], Ax, Bx, Cx);
+    axis_factors(u[1], Ay, By, Cy);
+    axis_factors(u[2], Az, Bz, Cz);
+    const double qf = in.M_phi * theta, qh = in.D_s * thetac;
+    const bool ok = fabs(ph) < (double)S_MAX && fabs(cc) < (double)S_MAX;
+    auto fx = [&](double v) { return ok && fabs(v) < 8.0 ? (int)__double2ll_rn(v * FX_ONE_D) : FX_BAD; };
+    int f[Q27];
+    emit27(Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, ph, qf * n[0], qf * n[1], qf * n[2],
+           [&](int q, double v) { f[q] = fx(v); });
+    emit27(Ax, Bx, Cx, Ay, By, Cy, Az, Bz, Cz, cc, qh * n[0], qh * n[1], qh * n[2],
+           [&](int q, double v) { out(q, f[q], fx(v)); });
 }
 
-// phi = sum f and c = sum h of the state: exact integer sums, then FP64
-// (NaN where a pulled population is FX_BAD).
-__global__ void k3_fields(const K3Params p, const int* __restrict__ fa, const int* __restrict__ ha,
+// The state of the given fields, and a copy of the fields (see `Seed`).
+__global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state, double* __restrict__ keep,
+                        float* __restrict__ uf, int* __restrict__ wild) {
+    const long long N = p.N;
+    for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < N;
+         cell += (long long)gridDim.x * blockDim.x) {
+        keep[cell] = in.phi[cell];
+        keep[N + cell] = in.c[cell];
+        if (in.u[0])
+            for (int i = 0; i < 3; ++i) {
+                const double v = in.u[i][cell];
+                keep[(2 + i) * N + cell] = v;
+                uf[i * N + cell] = (float)v;
+            }
+        uint2 m[4] = {};
+        bool bad = false;
+        equilibrium(p, in, cell, [&](int q, int f, int h) {
+            bad |= f == FX_BAD || h == FX_BAD;
+            const int e[3] = {q % 3, (q / 3) % 3, q / 9};
+            const uint2 v = make_uint2((uint32_t)f, (uint32_t)h);
+            m[0] = m[0] + v;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if (e[i] == 1) m[1 + i] = m[1 + i] + v;
+                if (e[i] == 2) m[1 + i] = m[1 + i] - v;
+            }
+        });
+        uint2* o = reinterpret_cast<uint2*>(state) + (cell / p.nxny) * 4 * p.nxny + cell % p.nxny;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i * p.nxny] = m[i];
+        if (bad) *wild = 1;
+    }
+}
+
+// The populations that a cell of a state sends out in a step: out(q, f, h).
+template <class Out>
+__device__ __forceinline__ void outgoing(const K3Params& p, const int* __restrict__ state, int x, int y, int z,
+                                         Out out) {
+    Plane pl[3];
+#pragma unroll
+    for (int dz = 0; dz < 3; ++dz) {
+        const int* q = state + 8 * p.nxny * wrapi(z + dz - 1, p.nz);
+        pl[dz] = plane_of([&](int dy, int dx) {
+            return fx_to_f(q[2 * ((long long)wrapi(y + dy, p.ny) * p.nx + wrapi(x + dx, p.nx))]);
+        });
+    }
+    const long long in = (long long)y * p.nx + x;
+    int2 m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = reinterpret_cast<const int2*>(state)[(4LL * z + i) * p.nxny + in];
+    float u[3] = {p.u[0], p.u[1], p.u[2]};
+    if (p.uf)
+        for (int i = 0; i < 3; ++i) u[i] = p.uf[i * p.N + z * p.nxny + in];
+    const Collision r = collide<true>(p, m, pl[0], pl[1], pl[2], u);
+    uint2 v[Q27], moved = make_uint2(0u, 0u);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        auto row = [&](int c, uint2 v0, uint2 v1, uint2 v2) {
+            const int q = 3 * b + 9 * c;
+            v[q] = v0;
+            v[q + 1] = v1;
+            v[q + 2] = v2;
+            if (q) moved = moved + v0;
+            moved = moved + v1 + v2;
+        };
+        if (p.uf)
+            emit_rows<true, true>(p, r, b, row);
+        else
+            emit_rows<false, true>(p, r, b, row);
+    }
+    v[0] = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
+    if (!r.ok) v[0] = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
+#pragma unroll
+    for (int q = 0; q < Q27; ++q) out(q, (int)v[q].x, (int)v[q].y);
+}
+
+__device__ __forceinline__ int vel(int a) { return a == 0 ? 0 : a == 1 ? 1 : -1; }
+
+// phi and c of a cell from its 27 incoming populations (NaN where one is
+// FX_BAD): of the initial fields (prev null), or sent by the state before.
+__device__ __forceinline__ void fields_of_populations(const K3Params& p, const Seed& seed, const int* prev,
+                                                   long long cell, double* phi, double* c) {
+    long long sf = 0, sh = 0;
+    bool bf = false, bh = false;
+    auto add = [&](int f, int h) {
+        bf |= f == FX_BAD;
+        bh |= h == FX_BAD;
+        sf += f;
+        sh += h;
+    };
+    if (!prev) {
+        equilibrium(p, seed, cell, [&](int, int f, int h) { add(f, h); });
+    } else {
+        const int x = (int)(cell % p.nx), y = (int)((cell / p.nx) % p.ny), z = (int)(cell / p.nxny);
+        for (int want = 0; want < Q27; ++want)
+            outgoing(p, prev, wrapi(x - vel(want % 3), p.nx), wrapi(y - vel((want / 3) % 3), p.ny),
+                     wrapi(z - vel(want / 9), p.nz), [&](int q, int f, int h) {
+                         if (q == want) add(f, h);
+                     });
+    }
+    if (phi) phi[cell] = bf ? nan("") : (double)sf * FX_INV_D;
+    if (c) c[cell] = bh ? nan("") : (double)sh * FX_INV_D;
+}
+
+// phi and c of the state: exact integer sums, then FP64.
+__global__ void k3_fields(const K3Params p, const int* __restrict__ state, const int* __restrict__ wild,
                           double* __restrict__ phi, double* __restrict__ c) {
+    if (*wild) return;
+    const int nxny = (int)p.nxny;
     for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < p.N;
          cell += (long long)gridDim.x * blockDim.x) {
-        long long sf = 0, sh = 0;
-        bool bf = false, bh = false;
-        for (int q = 0; q < Q27; ++q) {
-            const long long src = pull_src(p, cell, q);
-            const int a = fa[src], b = ha[src];
-            bf |= a == FX_BAD;
-            bh |= b == FX_BAD;
-            sf += a;
-            sh += b;
+        const int2 s = reinterpret_cast<const int2*>(state)[cell + cell / nxny * 3 * nxny];
+        if (phi) phi[cell] = (double)s.x * FX_INV_D;
+        if (c) c[cell] = (double)s.y * FX_INV_D;
+    }
+}
+
+// The same where a population may be invalid.  A kernel of its own: the code
+// that forms populations takes three times the registers.
+__global__ void k3_fields_wild(const K3Params p, const Seed seed, const int* prev, const int* __restrict__ wild,
+                               double* __restrict__ phi, double* __restrict__ c) {
+    if (!*wild) return;
+    for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < p.N;
+         cell += (long long)gridDim.x * blockDim.x)
+        fields_of_populations(p, seed, prev, cell, phi, c);
+}
+
+// The state's populations as float64 [27][N] (NaN for FX_BAD): of the initial
+// fields (prev null), or sent by the state before to the cells they reached.
+__global__ void k3_pops(const K3Params p, const Seed seed, const int* prev, double* __restrict__ f,
+                        double* __restrict__ h) {
+    for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < p.N;
+         cell += (long long)gridDim.x * blockDim.x) {
+        auto put = [&](long long i, int a, int b) {
+            if (f) f[i] = a == FX_BAD ? nan("") : (double)a * FX_INV_D;
+            if (h) h[i] = b == FX_BAD ? nan("") : (double)b * FX_INV_D;
+        };
+        if (!prev) {
+            equilibrium(p, seed, cell, [&](int q, int a, int b) { put(q * p.N + cell, a, b); });
+            continue;
         }
-        if (phi) phi[cell] = bf ? nan("") : (double)sf * FX_INV_D;
-        if (c) c[cell] = bh ? nan("") : (double)sh * FX_INV_D;
+        const int x = (int)(cell % p.nx), y = (int)((cell / p.nx) % p.ny), z = (int)(cell / p.nxny);
+        outgoing(p, prev, x, y, z, [&](int q, int a, int b) {
+            const int tx = wrapi(x + vel(q % 3), p.nx), ty = wrapi(y + vel((q / 3) % 3), p.ny),
+                      tz = wrapi(z + vel(q / 9), p.nz);
+            put(q * p.N + ((long long)tz * p.ny + ty) * p.nx + tx, a, b);
+        });
     }
 }
 
-// The state's populations as float64 [27][N] (NaN for FX_BAD).
-__global__ void k3_pops(const K3Params p, const int* __restrict__ fa, const int* __restrict__ ha,
-                        double* __restrict__ f, double* __restrict__ h) {
-    const long long total = Q27 * p.N;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int q = (int)(i / p.N);
-        const long long src = pull_src(p, i % p.N, q);
-        const int a = fa[src], b = ha[src];
-        if (f) f[i] = a == FX_BAD ? nan("") : (double)a * FX_INV_D;
-        if (h) h[i] = b == FX_BAD ? nan("") : (double)b * FX_INV_D;
-    }
+// Invalid populations of a cell (out of those it sent in the last step, or of
+// its initial ones) and the sums of its valid ones.
+__device__ __noinline__ void totals_of_populations(const K3Params& p, const Seed& seed, const int* prev,
+                                                   long long cell, long long& sf, long long& sh, long long& bad) {
+    auto add = [&](int, int f, int h) {
+        if (f != FX_BAD) sf += f; else bad += 1;
+        if (h != FX_BAD) sh += h; else bad += 1;
+    };
+    if (!prev)
+        equilibrium(p, seed, cell, add);
+    else
+        outgoing(p, prev, (int)(cell % p.nx), (int)((cell / p.nx) % p.ny), (int)(cell / p.nxny), add);
 }
 
-// Totals: sum f, sum h (exact, in integer units) and the FX_BAD count over the
-// whole buffer (the pull is a permutation, so the state's totals are the
-// buffer's).  Fixed grid and reduction order.
-__global__ void __launch_bounds__(SUM_THREADS) k3_sum1(long long total, const int* __restrict__ fa,
-                                                       const int* __restrict__ ha,
+// Totals: sum f, sum h (exact, in integer units) and the FX_BAD count of the
+// state's populations (streaming is a permutation: those sent are those that
+// arrived).  Fixed grid and reduction order.
+__global__ void __launch_bounds__(SUM_THREADS) k3_sum1(const K3Params p, const Seed seed,
+                                                       const int* __restrict__ state, const int* prev,
+                                                       const int* __restrict__ wild,
                                                        long long* __restrict__ partial) {
     long long sf = 0, sh = 0, bad = 0;
-    for (long long i = blockIdx.x * (long long)SUM_THREADS + threadIdx.x; i < total;
-         i += (long long)SUM_BLOCKS * SUM_THREADS) {
-        const int a = fa[i], b = ha[i];
-        if (a != FX_BAD) sf += a; else bad += 1;
-        if (b != FX_BAD) sh += b; else bad += 1;
+    const bool each = *wild != 0;
+    const int nxny = (int)p.nxny;
+    for (long long cell = blockIdx.x * (long long)SUM_THREADS + threadIdx.x; cell < p.N;
+         cell += (long long)SUM_BLOCKS * SUM_THREADS) {
+        if (each) {
+            totals_of_populations(p, seed, prev, cell, sf, sh, bad);
+            continue;
+        }
+        const int2 s = reinterpret_cast<const int2*>(state)[cell + cell / nxny * 3 * nxny];
+        sf += s.x;
+        sh += s.y;
     }
     __shared__ long long red[3][SUM_THREADS];
     red[0][threadIdx.x] = sf;
@@ -462,8 +715,10 @@ struct lbm3_ctx {
     K3Params kp;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    int* buf[2] = {nullptr, nullptr};    // each: f [nz][27][ny][nx] then h, fixed point
+    int* buf[2] = {nullptr, nullptr};    // states, [nz][4][ny][nx][2] fixed point: now and one step back
     float* uf = nullptr;                 // [3][N] prescribed velocity (velocity_field = 1)
+    double* keep = nullptr;              // the initial fields, [2][N] or [5][N] with the velocity
+    int* wild = nullptr;                 // a population may have been out of range since the last init
     long long* partial = nullptr;        // 3 x SUM_BLOCKS partial sums
     double* result = nullptr;            // 3 totals
     int cur = 0;
@@ -482,12 +737,31 @@ int fail(lbm3_ctx* ctx, cudaError_t e) {
 
 double rate_of(double coeff) { return 1.0 / (coeff * 3.0 + 0.5); }
 
-int* fbuf(lbm3_ctx* ctx, int which) { return ctx->buf[which]; }
-int* hbuf(lbm3_ctx* ctx, int which) { return ctx->buf[which] + (size_t)Q27 * ctx->kp.N; }
+// The initial fields kept by the context.
+Seed seed_of(const lbm3_ctx* ctx) {
+    const lbm3_params& p = ctx->p;
+    const long long N = ctx->kp.N;
+    Seed s{ctx->keep, ctx->keep + N, {nullptr, nullptr, nullptr}, p.W, p.phi_a, p.phi_b, p.M_phi, p.D_s};
+    if (p.velocity_field)
+        for (int i = 0; i < 3; ++i) s.u[i] = ctx->keep + (2 + i) * N;
+    return s;
+}
+
+// The state one step back, or null if the state is the initial one.
+const int* before(const lbm3_ctx* ctx) { return ctx->step ? ctx->buf[1 - ctx->cur] : nullptr; }
 
 int grid_1d(long long n, int threads) {
     long long b = (n + threads - 1) / threads;
     return (int)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
+}
+
+// Shared memory above 48 KB has to be asked for, once per kernel and device.
+template <int ROWS>
+cudaError_t allow_smem(bool field) {
+    return field ? cudaFuncSetAttribute(k3_step<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        k3_smem<ROWS>())
+                 : cudaFuncSetAttribute(k3_step<ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        k3_smem<ROWS>());
 }
 
 int launch_step(lbm3_ctx* ctx) {
@@ -499,18 +773,18 @@ int launch_step(lbm3_ctx* ctx) {
               (kp.nz + ctx->seg_z - 1) / ctx->seg_z);
     const int src = ctx->cur, dst = 1 - ctx->cur;
     const bool field = kp.uf != nullptr;
-    auto go = [&](auto kern, int threads) {
-        kern<<<grid, threads, 0, ctx->stream>>>(p, fbuf(ctx, src), hbuf(ctx, src), fbuf(ctx, dst), hbuf(ctx, dst));
+    auto go = [&](auto kern, int threads, int smem) {
+        kern<<<grid, threads, smem, ctx->stream>>>(p, ctx->buf[src], ctx->buf[dst], ctx->wild);
     };
     switch (rows) {
         case 6:
-            field ? go(k3_step<6, true>, 6 * 32) : go(k3_step<6, false>, 6 * 32);
+            field ? go(k3_step<6, true>, 6 * 32, k3_smem<6>()) : go(k3_step<6, false>, 6 * 32, k3_smem<6>());
             break;
         case 10:
-            field ? go(k3_step<10, true>, 10 * 32) : go(k3_step<10, false>, 10 * 32);
+            field ? go(k3_step<10, true>, 10 * 32, k3_smem<10>()) : go(k3_step<10, false>, 10 * 32, k3_smem<10>());
             break;
         case 18:
-            field ? go(k3_step<18, true>, 18 * 32) : go(k3_step<18, false>, 18 * 32);
+            field ? go(k3_step<18, true>, 18 * 32, k3_smem<18>()) : go(k3_step<18, false>, 18 * 32, k3_smem<18>());
             break;
         default:
             return LBM_ERR_INVALID_ARG;
@@ -520,6 +794,31 @@ int launch_step(lbm3_ctx* ctx) {
     ctx->cur = dst;
     ctx->step += 1;
     return LBM_OK;
+}
+
+// The launch shape of a context whose user sets none.  A block spends seg_z + 3
+// planes' time (the halo planes and the first loads), so the segments that are
+// best make the blocks of an SM times that the smallest.  At 18 rows an SM holds
+// one block; at 10 rows two, which then take 1.45 times as long as one alone.
+// With a uniform velocity 18 rows win where both fill the chip (fewer halo
+// rows: 256^3 575 against 622 us, 150x97x61 43 against 45 us); a velocity field
+// needs the second block to hide the longer chains (256^3 791 against 724 us,
+// 220x200x180 425 against 355 us, 150x97x61 55 against 53 us).
+void default_shape(const lbm3_params* p, int* rows, int* seg_z) {
+    *rows = p->velocity_field ? 10 : 18;
+    const long long tiles = (long long)((p->nx + TILE_IN - 1) / TILE_IN) * ((p->ny + *rows - 3) / (*rows - 2));
+    double best = -1.0;
+    for (int n = 1; n <= p->nz; ++n) {
+        const int seg = (p->nz + n - 1) / n;
+        if (n > 1 && seg == (p->nz + n - 2) / (n - 1)) continue;
+        const long long blocks = tiles * ((p->nz + seg - 1) / seg), per_sm = (blocks + 151) / 152;
+        const double load = p->velocity_field ? 1.45 * (double)(per_sm / 2) + (double)(per_sm % 2) : (double)per_sm;
+        const double cost = load * (seg + 3);
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            *seg_z = seg;
+        }
+    }
 }
 
 bool finite_all(const double* v, int n) {
@@ -565,7 +864,6 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
     kp.nz = p->nz;
     kp.nxny = (long long)p->nx * p->ny;
     kp.N = kp.nxny * p->nz;
-    kp.seg_z = ctx->seg_z;
     kp.w_kappa = (float)rate_of(p->M_phi);
     kp.w_chi = (float)rate_of(p->D_s);
     kp.M_phi = (float)p->M_phi;
@@ -576,18 +874,23 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
     kp.phi_b = (float)p->phi_b;
     kp.phim = (float)(0.5 * (p->phi_a + p->phi_b));
     kp.inv_dphi = (float)(1.0 / (p->phi_a - p->phi_b));
+    double fac[3][3][3];  // [axis][A, B, C][e = 0, +1, -1]
     for (int i = 0; i < 3; ++i) {
         kp.u[i] = (float)p->u[i];
-        // the one-dimensional factors A, B, C of P^-1 F^-1(u) (see axis_factors)
-        const double u = p->u[i], u2 = u * u, t = 1.0 / 3.0 + u2;
-        const double f[3][3] = {{1.0 - t, 0.5 * (t + u), 0.5 * (t - u)},
-                                {-2.0 * u, u + 0.5, u - 0.5},
-                                {1.0 - u2, 0.5 * (u2 + u), 0.5 * (u2 - u)}};
-        for (int k = 0; k < 3; ++k)
-            for (int e = 0; e < 3; ++e) kp.fac[i][k][e] = (float)f[k][e];
+        axis_factors(p->u[i], fac[i][0], fac[i][1], fac[i][2]);
     }
+    auto both = [](double v) { return make_float2((float)v, (float)v); };
+    for (int k = 0; k < 3; ++k)
+        for (int e = 0; e < 3; ++e) kp.fx[k][e] = both(fac[0][k][e]);
+    for (int c = 0; c < 3; ++c)
+        for (int b = 0; b < 3; ++b) {
+            kp.aa[c][b] = both(fac[1][0][b] * fac[2][0][c]);
+            kp.cc[c][b] = both(fac[1][2][b] * fac[2][2][c]);
+            kp.bc[c][b] = both(fac[1][1][b] * fac[2][2][c]);
+            kp.cb[c][b] = both(fac[1][2][b] * fac[2][1][c]);
+        }
     kp.uf = nullptr;
-    ctx->seg_z = p->nz < 64 ? p->nz : 64;
+    default_shape(p, &ctx->rows, &ctx->seg_z);
     cudaError_t e = cudaSuccess;
     if (stream) {
         ctx->stream = (cudaStream_t)stream;
@@ -595,14 +898,23 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
         e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
         ctx->own_stream = e == cudaSuccess;
     }
-    const size_t pop_bytes = sizeof(int) * 2 * Q27 * (size_t)kp.N;
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&ctx->buf[i], pop_bytes);
+    const size_t state_bytes = sizeof(int) * 8 * (size_t)kp.N;
+    const size_t keep_bytes = sizeof(double) * (p->velocity_field ? 5 : 2) * (size_t)kp.N;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&ctx->buf[i], state_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->keep, keep_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->wild, sizeof(int));
     if (e == cudaSuccess && p->velocity_field) e = cudaMalloc(&ctx->uf, sizeof(float) * 3 * (size_t)kp.N);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->partial, sizeof(long long) * 3 * SUM_BLOCKS);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->result, sizeof(double) * 3);
     // defined contents before the first init (the autotuner may step them)
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMemsetAsync(ctx->buf[i], 0, pop_bytes, ctx->stream);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMemsetAsync(ctx->buf[i], 0, state_bytes, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->keep, 0, keep_bytes, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->wild, 0, sizeof(int), ctx->stream);
     if (e == cudaSuccess && ctx->uf) e = cudaMemsetAsync(ctx->uf, 0, sizeof(float) * 3 * (size_t)kp.N, ctx->stream);
+    const bool field = p->velocity_field != 0;
+    if (e == cudaSuccess) e = allow_smem<6>(field);
+    if (e == cudaSuccess) e = allow_smem<10>(field);
+    if (e == cudaSuccess) e = allow_smem<18>(field);
     if (e != cudaSuccess) {
         const int rc = fail(nullptr, e);
         lbm3_destroy(ctx);
@@ -619,6 +931,8 @@ void lbm3_destroy(lbm3_ctx* ctx) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     for (int i = 0; i < 2; ++i) cudaFree(ctx->buf[i]);
     cudaFree(ctx->uf);
+    cudaFree(ctx->keep);
+    cudaFree(ctx->wild);
     cudaFree(ctx->partial);
     cudaFree(ctx->result);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
@@ -632,10 +946,17 @@ int lbm3_init_fields_device(lbm3_ctx* ctx, const double* phi, const double* c, c
     if (field && (!ux || !uy || !uz)) return LBM_ERR_INVALID_ARG;
     Nvtx r("lbm3_init_fields");
     const lbm3_params& p = ctx->p;
+    Seed in{phi, c, {nullptr, nullptr, nullptr}, p.W, p.phi_a, p.phi_b, p.M_phi, p.D_s};
+    if (field) {
+        in.u[0] = ux;
+        in.u[1] = uy;
+        in.u[2] = uz;
+    }
+    const cudaError_t e = cudaMemsetAsync(ctx->wild, 0, sizeof(int), ctx->stream);
+    if (e != cudaSuccess) return fail(ctx, e);
     ctx->cur = 0;
-    k3_init<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(
-        ctx->kp, phi, c, field ? ux : nullptr, field ? uy : nullptr, field ? uz : nullptr, p.W, p.phi_a,
-        p.phi_b, p.M_phi, p.D_s, fbuf(ctx, 0), hbuf(ctx, 0), ctx->uf);
+    k3_init<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, in, ctx->buf[0], ctx->keep, ctx->uf,
+                                                              ctx->wild);
     ctx->step = 0;
     return fail(ctx, cudaGetLastError());
 }
@@ -677,8 +998,9 @@ int lbm3_step(lbm3_ctx* ctx, int64_t nsteps) {
 int lbm3_get_fields_device(lbm3_ctx* ctx, double* phi, double* c) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     if (!phi && !c) return LBM_OK;
-    k3_fields<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, fbuf(ctx, ctx->cur),
-                                                                 hbuf(ctx, ctx->cur), phi, c);
+    k3_fields<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, ctx->buf[ctx->cur], ctx->wild, phi, c);
+    k3_fields_wild<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), before(ctx), ctx->wild,
+                                                                      phi, c);
     return fail(ctx, cudaGetLastError());
 }
 
@@ -700,8 +1022,7 @@ int lbm3_get_fields(lbm3_ctx* ctx, double* phi, double* c) {
 int lbm3_get_populations_device(lbm3_ctx* ctx, double* f, double* h) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     if (!f && !h) return LBM_OK;
-    const long long n = (long long)Q27 * ctx->kp.N;
-    k3_pops<<<grid_1d(n, 256), 256, 0, ctx->stream>>>(ctx->kp, fbuf(ctx, ctx->cur), hbuf(ctx, ctx->cur), f, h);
+    k3_pops<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), before(ctx), f, h);
     return fail(ctx, cudaGetLastError());
 }
 
@@ -722,9 +1043,8 @@ int lbm3_get_populations(lbm3_ctx* ctx, double* f, double* h) {
 
 int lbm3_sums(lbm3_ctx* ctx, double out[3]) {
     if (!ctx || !out) return LBM_ERR_INVALID_ARG;
-    const long long total = Q27 * ctx->kp.N;
-    k3_sum1<<<SUM_BLOCKS, SUM_THREADS, 0, ctx->stream>>>(total, fbuf(ctx, ctx->cur), hbuf(ctx, ctx->cur),
-                                                         ctx->partial);
+    k3_sum1<<<SUM_BLOCKS, SUM_THREADS, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), ctx->buf[ctx->cur], before(ctx),
+                                                         ctx->wild, ctx->partial);
     k3_sum2<<<1, SUM_THREADS, 0, ctx->stream>>>(ctx->partial, ctx->result);
     int rc = fail(ctx, cudaGetLastError());
     if (rc == LBM_OK)
