@@ -55,9 +55,8 @@ struct lbm_ctx {
     bool width_set = false;  // the block width was set or tuned by the user, not by the library
     double* stage = nullptr;
     size_t stage_bytes = 0;
-    double* dpartial = nullptr;
+    unsigned long long* dwords = nullptr;  // scratch of the diagnostics
     double* dresult = nullptr;
-    int diag_nb = 0;
     cudaGraphExec_t graph[GRAPH_CHUNKS][2] = {};  // [log2(32 / steps)][parity]
     CUtensorMap tmaps[2];   // bulk-tensor load maps over the two population buffers
     lbm::StoreMaps smaps[2];  // bulk-tensor store maps over the same buffers
@@ -424,11 +423,10 @@ int lbm_create(const lbm_params* p, void* stream, lbm_ctx** out) {
     ctx->ds.nlat = ctx->kp.coupled ? 3 : 2;
     const size_t pop_bytes = sizeof(float) * (size_t)ctx->ds.nlat * 9 * (size_t)ctx->kp.plane;
     const size_t fld_bytes = sizeof(float) * (size_t)lbm::FP_COUNT * (size_t)ctx->kp.plane;
-    ctx->diag_nb = lbm::diag_blocks(ctx->kp);
     if (cudaMalloc(&ctx->pop_alloc[0], pop_bytes) != cudaSuccess ||
         cudaMalloc(&ctx->pop_alloc[1], pop_bytes) != cudaSuccess ||
         cudaMalloc(&ctx->fields_alloc, fld_bytes) != cudaSuccess ||
-        cudaMalloc(&ctx->dpartial, sizeof(double) * lbm::DIAG_NSUM * ctx->diag_nb) != cudaSuccess ||
+        cudaMalloc(&ctx->dwords, sizeof(unsigned long long) * lbm::diag_words(ctx->kp)) != cudaSuccess ||
         cudaMalloc(&ctx->dresult, sizeof(double) * 16) != cudaSuccess ||
         cudaMalloc(&ctx->derr, sizeof(int)) != cudaSuccess ||
         cudaMalloc(&ctx->dstep, sizeof(unsigned)) != cudaSuccess ||
@@ -470,7 +468,7 @@ void lbm_destroy(lbm_ctx* ctx) {
     cudaFree(ctx->pop_alloc[1]);
     cudaFree(ctx->fields_alloc);
     cudaFree(ctx->stage);
-    cudaFree(ctx->dpartial);
+    cudaFree(ctx->dwords);
     cudaFree(ctx->dresult);
     cudaFree(ctx->derr);
     cudaFree(ctx->pop16_alloc[0]);
@@ -556,7 +554,6 @@ int lbm_get_fields_device(lbm_ctx* ctx, double* phi, double* c, double* ux, doub
                           double* P) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     const int b = fp32_view(ctx);
-    lbm::launch_fields(ctx->kp, ctx->ds, b, ctx->stream);
     lbm::launch_macro_out(ctx->kp, ctx->ds, b, phi, c, ux, uy, P, ctx->stream);
     return check_launch(ctx);
 }
@@ -627,13 +624,11 @@ int lbm_diagnostics(lbm_ctx* ctx, lbm_diag* out) {
     if (!ctx || !out) return LBM_ERR_INVALID_ARG;
     NvtxRange range("lbm_diagnostics");
     const int64_t n = cells(ctx);
-    int rc = ensure_stage(ctx, sizeof(double) * 5 * (size_t)n);
+    int rc = ensure_stage(ctx, sizeof(int) * (size_t)n);
     if (rc != LBM_OK) return rc;
-    double* d = ctx->stage;
-    rc = lbm_get_fields_device(ctx, d, d + n, d + 2 * n, d + 3 * n, nullptr);
-    if (rc != LBM_OK) return rc;
-    lbm::launch_diag(ctx->kp, d, d + n, d + 2 * n, d + 3 * n, ctx->dpartial, ctx->diag_nb,
-                     ctx->dresult, ctx->stream);
+    const cudaError_t e = lbm::launch_diag(ctx->kp, ctx->ds, fp32_view(ctx), reinterpret_cast<int*>(ctx->stage),
+                                           ctx->dwords, ctx->dresult, ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
     rc = check_launch(ctx);
     if (rc != LBM_OK) return rc;
     double res[16];
@@ -661,35 +656,19 @@ int lbm_diagnostics(lbm_ctx* ctx, lbm_diag* out) {
 int lbm_count_components(lbm_ctx* ctx, double level, int32_t* count) {
     if (!ctx || !count) return LBM_ERR_INVALID_ARG;
     const int64_t n = cells(ctx);
-    // labels and flags live in the staging buffer (int32 per cell, then 2 ints)
-    int rc = ensure_stage(ctx, sizeof(int) * (size_t)(n + 2) + sizeof(double));
+    // the labels and the count live in the staging buffer
+    int rc = ensure_stage(ctx, sizeof(int) * (size_t)(n + 1) + sizeof(double));
     if (rc != LBM_OK) return rc;
     int* label = reinterpret_cast<int*>(ctx->stage);
-    int* flag = label + n;  // [0]: changed, [1]: root count
-    const int b = fp32_view(ctx);
-    lbm::launch_fields(ctx->kp, ctx->ds, b, ctx->stream);
-    lbm::launch_label_init(ctx->kp, ctx->ds.fields, (float)level, label, ctx->stream);
-    // each sweep moves every label at least one cell and halves pointer
-    // chains, so n sweeps always suffice
-    for (int64_t it = 0; it < n + 1; ++it) {
-        int changed = 0;
-        cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream);
-        if (e == cudaSuccess) {
-            lbm::launch_label_step(ctx->kp, label, flag, ctx->stream);
-            e = cudaMemcpyAsync(&changed, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e);
-        if (!changed) break;
-    }
-    int roots = 0;
-    cudaError_t e = cudaMemsetAsync(flag + 1, 0, sizeof(int), ctx->stream);
-    if (e == cudaSuccess) {
-        lbm::launch_label_roots(ctx->kp, label, flag + 1, ctx->stream);
-        e = cudaMemcpyAsync(&roots, flag + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    cudaError_t e = lbm::launch_components(ctx->kp, ctx->ds, fp32_view(ctx), (float)level, label, label + n,
+                                           ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
+    rc = check_launch(ctx);
+    if (rc != LBM_OK) return rc;
+    int roots = 0;
+    e = cudaMemcpyAsync(&roots, label + n, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return cuda_fail(ctx, cudaGetLastError());
     *count = roots;
     return lbm_synchronize(ctx);
 }

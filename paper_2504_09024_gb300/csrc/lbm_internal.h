@@ -145,7 +145,7 @@ void launch_unpack16(const KParams& p, const float* src16_alloc, float* dst32_al
                      cudaStream_t s);
 // Fill the field planes (phi, c, dP*, sigma, n, |grad phi|) of the current state.
 void launch_fields(const KParams& p, const DevState& s, int src, cudaStream_t st);
-// Macroscopic outputs (float64, dense [ny][nx]) of the current state; needs launch_fields first.
+// Macroscopic outputs (float64, dense [ny][nx]) of the current state.
 void launch_macro_out(const KParams& p, const DevState& s, int src, double* phi, double* c,
                       double* ux, double* uy, double* P, cudaStream_t st);
 // Initialisation from float64 fields (dense); writes buffer `dst` (uses the other as scratch).
@@ -160,17 +160,19 @@ void launch_set_pops(const KParams& p, const DevState& s, int dst, const double*
                      const double* h, const double* g, cudaStream_t st);
 
 // Connected components of {phi > level} (4-neighbour, periodic in x, and in
-// y without walls) on the FP_PHI field plane: label init, one propagation
-// sweep (sets *changed when a label moved), root count.
-void launch_label_init(const KParams& p, const float* fields, float level, int* label,
-                       cudaStream_t st);
-void launch_label_step(const KParams& p, int* label, int* changed, cudaStream_t st);
-void launch_label_roots(const KParams& p, const int* label, int* count, cudaStream_t st);
-// FP64 reductions: partial sums per block into `partial`, then a fixed-order finish.
-constexpr int DIAG_NSUM = 12;
-int diag_blocks(const KParams& p);
-void launch_diag(const KParams& p, const double* phi, const double* c, const double* ux,
-                 const double* uy, double* partial, int nblocks, double* result,
-                 cudaStream_t st);
+// y without walls) of the current state into *count; label: nx * ny words.
+cudaError_t launch_components(const KParams& p, const DevState& s, int src, float level, int* label, int* count,
+                              cudaStream_t st);
+// FP64 reductions of given fields: partial sums per block into `partial`, then a
+// fixed-order finish into result[0 .. 12].
+constexpr int STATS_NSUM = 12;
+int stats_blocks(const KParams& p);
+void launch_field_stats(const KParams& p, const double* phi, const double* c, const double* ux,
+                        const double* uy, double* partial, int nblocks, double* result, cudaStream_t st);
+// Diagnostics of the current state into result[0 .. 13] (layout at k_diag1);
+// wmap: nx * ny words, words: diag_words(p) 64-bit words of scratch.
+size_t diag_words(const KParams& p);
+cudaError_t launch_diag(const KParams& p, const DevState& s, int src, int* wmap, unsigned long long* words,
+                        double* result, cudaStream_t st);
 
 }  // namespace lbm

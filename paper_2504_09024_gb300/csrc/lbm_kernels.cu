@@ -8,9 +8,10 @@
 //    stencils read from the rings.  Populations are read once per cell (plus
 //    the halo columns and the segment ends) and written once.
 //  * k_fields / k_normals / k_collide -- the same step as a three-kernel chain
-//    with the fields materialised in global memory; used as a cross-check, for
-//    the macroscopic outputs and for initialisation.
-//  * initialisation, population import/export and FP64 reductions.
+//    with the fields materialised in global memory; used as a cross-check and
+//    for initialisation.
+//  * macroscopic outputs and diagnostics (macro_tile), initialisation,
+//    population import/export and the count of drops.
 #include <cmath>
 
 #include "lbm_cell.cuh"
@@ -119,32 +120,135 @@ __global__ void k_collide(KParams p, const float* __restrict__ src, float* __res
     if (COUPLED) store9(dst + 18 * p.plane, p, idx, i, gg);
 }
 
-template <bool COUPLED>
-__global__ void k_macro_out(KParams p, const float* __restrict__ src, const float* __restrict__ F,
-                            double* __restrict__ ophi, double* __restrict__ oc,
-                            double* __restrict__ oux, double* __restrict__ ouy,
-                            double* __restrict__ oP) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (i >= p.nx) return;
-    const int64_t idx = (int64_t)j * p.pitch + i;
-    const int64_t o = (int64_t)j * p.nx + i;
-    CellGeom g = gather_geom<COUPLED>(p, F, i, j);
-    float gg[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    float ufx = 0.0f, ufy = 0.0f;
-    if (COUPLED) {
-        pull9(src + 18 * p.plane, p, i, j, gg);
+// FP64 instructions issue at two lanes a cycle and SM; these conversions are
+// integer arithmetic.  Same values as the conversion instructions.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v), e = (b >> 23) & 255u;
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    if (e == 0u || e == 255u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + (896u << 20))), (int)(b << 29));
+}
+
+// s / scale for a power of two `scale` (NaN for the invalid marker).
+__device__ __forceinline__ double fx_widen(int s, float scale) {
+    const int k = (int)(__float_as_uint(scale) >> 23) - 127;
+    if (s == FX_INVALID || k < -126) return fx_to_double(s, scale);
+    if (s == 0) return 0.0;
+    const uint32_t m = (uint32_t)abs(s);
+    const int lz = __clz(m);
+    const uint32_t f = m << lz << 1;  // the bits below the leading one
+    const uint32_t hi = ((uint32_t)s & 0x80000000u) | ((uint32_t)(1023 + 31 - lz - k) << 20) | (f >> 12);
+    return __hiloint2double((int)hi, (int)(f << 20));
+}
+
+// Macroscopic state of the cells of a 32 x 8 tile, one per thread: out(i, j,
+// phi_fx, c_fx, ux, uy, dP) for those inside the grid (dP: P - P0).  The block
+// forms phi, sigma and P* of the tile and two cells around it in shared memory,
+// then the normals of the tile and one cell around it, then each cell's forces,
+// with the operations of the three-kernel chain in their order (same bits).
+//
+// Bound by the pulls (1.69 times the tile's, from L2) and their latency.  As
+// three kernels through global field planes the fields of 128 runs of 384 x 128
+// took 23 us a run, now 13.
+constexpr int MT_X = 32, MT_Y = 8;
+template <bool COUPLED, class Out>
+__device__ __forceinline__ void macro_tile(const KParams& p, const float* __restrict__ src,
+                                           const float* __restrict__ F, Out out) {
+    constexpr int WX = MT_X + 4, WY = MT_Y + 4, NX = MT_X + 2, NY = MT_Y + 2;
+    const int x0 = blockIdx.x * MT_X, y0 = blockIdx.y * MT_Y;
+    const int rows = min(MT_Y, p.ny - y0), cols = min(MT_X, p.nx - x0);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i = x0 + tx, j = y0 + ty;
+    const bool own = tx < cols && ty < rows;
+    const uint32_t seed = step_seed(p);
+    if constexpr (!COUPLED) {
+        if (!own) return;
+        const uint32_t bits = moment_bits(seed, i, j, p.nx);
+        const ScalarMoments f = pull_scalar(src, p, 0, i, j), h = pull_scalar(src + 9 * p.plane, p, 1, i, j);
+        const int64_t idx = (int64_t)j * p.pitch + i;
+        out(i, j, fx_add_sr(f.s0, f.inc, p.fx_scale[0], bits),
+            fx_add_sr(h.s0, h.inc, p.fx_scale[1], second_bits(bits)), F[FP_UX * p.plane + idx],
+            F[FP_UY * p.plane + idx], 0.0f);
     } else {
-        ufx = F[FP_UX * p.plane + idx];
-        ufy = F[FP_UY * p.plane + idx];
+        __shared__ int s_phi[WY * WX], s_c[MT_Y * MT_X];
+        __shared__ float s_sig[WY * WX], s_dps[WY * WX], s_nx[NY * NX], s_ny[NY * NX], s_gm[NY * NX];
+        for (int k = threadIdx.x; k < (rows + 4) * WX; k += MT_X * MT_Y) {
+            const int r = k / WX, w = k - r * WX;
+            if (w >= cols + 4) continue;
+            const int gi = wrap_i(x0 + w - 2, p.nx), gj = ext_row(y0 + r - 2, p.ny, p.walls);
+            const uint32_t bits = moment_bits(seed, gi, gj, p.nx);
+            const ScalarMoments f = pull_scalar(src, p, 0, gi, gj);
+            const ScalarMoments h = pull_scalar(src + 9 * p.plane, p, 1, gi, gj);
+            float a[9];
+            pull9(src + 18 * p.plane, p, gi, gj, a);
+            const int c_fx = fx_add_sr(h.s0, h.inc, p.fx_scale[1], second_bits(bits));
+            s_phi[k] = fx_add_sr(f.s0, f.inc, p.fx_scale[0], bits);
+            s_sig[k] = sigma_of_c(p, (float)c_fx * p.fx_inv[1]);
+            s_dps[k] = sum9(a);
+            if (r >= 2 && r < rows + 2 && w >= 2 && w < cols + 2) s_c[(r - 2) * MT_X + w - 2] = c_fx;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < (rows + 2) * NX; k += MT_X * MT_Y) {
+            const int r = k / NX, w = k - r * NX;
+            if (w >= cols + 2) continue;
+            int v[3][3];
+            for (int a = 0; a < 3; ++a)
+                for (int b = 0; b < 3; ++b) v[a][b] = s_phi[(r + a) * WX + w + b];
+            float gx, gy;
+            iso_grad_fx(v, p.fx_inv[0], gx, gy);
+            unit_normal(gx, gy, s_nx[k], s_ny[k], s_gm[k]);
+        }
+        __syncthreads();
+        if (!own) return;
+        auto around = [&](const auto* s, int stride, int at, auto(&v)[3][3]) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) v[a][b] = s[at + (a - 1) * stride + b - 1];
+        };
+        const int at = (ty + 2) * WX + tx + 2, an = (ty + 1) * NX + tx + 1;
+        CellGeom g;
+        float vx[3][3], vy[3][3], v[3][3];
+        g.phi_fx = s_phi[at];
+        g.phi = (float)g.phi_fx * p.fx_inv[0];
+        g.c = (float)s_c[ty * MT_X + tx] * p.fx_inv[1];
+        g.nx = s_nx[an];
+        g.ny = s_ny[an];
+        g.gm = s_gm[an];
+        g.sig = s_sig[at];
+        g.dps = s_dps[at];
+        around(s_nx, NX, an, vx);
+        around(s_ny, NX, an, vy);
+        g.kappa = iso_div(vx, vy);
+        around(s_sig, WX, at, v);
+        iso_grad(v, g.sgx, g.sgy);
+        around(s_dps, WX, at, v);
+        iso_grad(v, g.pgx, g.pgy);
+        g.fgx = g.fgy = 0.0f;
+        if (!p.rho_uniform) {
+            int vi[3][3];
+            around(s_phi, WX, at, vi);
+            iso_grad_fx(vi, p.fx_inv[0], g.fgx, g.fgy);
+        }
+        float gg[9];
+        pull9(src + 18 * p.plane, p, i, j, gg);
+        const CellOut r = collide_flow_cell(p, g, j, gg, false);
+        out(i, j, g.phi_fx, s_c[ty * MT_X + tx], r.ux, r.uy, r.dP);
     }
-    CellOut r = collide_cell<COUPLED>(p, g, j, ufx, ufy, 0.0f, 0.0f, 0.0f, 0.0f, gg, nullptr,
-                                      nullptr, false);
-    if (ophi) ophi[o] = fx_to_double(g.phi_fx, p.fx_scale[0]);
-    if (oc) oc[o] = fx_to_double(__float_as_int(F[FP_C * p.plane + idx]), p.fx_scale[1]);
-    if (oux) oux[o] = r.ux;
-    if (ouy) ouy[o] = r.uy;
-    if (oP) oP[o] = COUPLED ? (double)p.P0 + (double)r.dP : 0.0;
+}
+
+template <bool COUPLED>
+__global__ void __launch_bounds__(MT_X * MT_Y)
+k_macro_out(KParams p, const float* __restrict__ src, const float* __restrict__ F, double* __restrict__ ophi,
+            double* __restrict__ oc, double* __restrict__ oux, double* __restrict__ ouy, double* __restrict__ oP) {
+    macro_tile<COUPLED>(p, src, F, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float dP) {
+        const int64_t o = (int64_t)j * p.nx + i;
+        if (ophi) ophi[o] = fx_widen(phi_fx, p.fx_scale[0]);
+        if (oc) oc[o] = fx_widen(c_fx, p.fx_scale[1]);
+        if (oux) oux[o] = widen(ux);
+        if (ouy) ouy[o] = widen(uy);
+        if (oP) oP[o] = COUPLED ? (double)p.P0 + widen(dP) : 0.0;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -377,6 +481,47 @@ __global__ void k_init_pre(KParams p, const float* __restrict__ F, float* __rest
     }
 }
 
+// a + b = s + e exactly (Knuth's TwoSum).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// Deviation form of nine slots: returns their sum S rounded to fixed point (scale:
+// a power of two, inv its reciprocal) and d_q = u_q - w_q S.  In pairs of floats,
+// 48 bits: FP64 instructions issue at two lanes a cycle and SM, and ninety of them
+// a cell made the kernel 140 us at 1024 x 512; now 27.5.
+__device__ __forceinline__ int deviations(const float (&u)[9], float scale, float inv, float (&d)[9]) {
+    float hi = 0.0f, lo = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        float e;
+        two_sum(hi, u[q], hi, e);
+        lo += e;
+    }
+    // hi + lo to the nearest unit, ties to even
+    const float A = hi * scale;
+    int S = FX_INVALID;
+    if (fabsf(A) <= (float)FX_RANGE) {
+        const int iA = __float2int_rn(A);
+        const float rem = __fadd_rn(__fsub_rn(A, (float)iA), lo * scale), fl = floorf(rem);
+        const int n = iA + (int)fl;
+        S = n + (rem - fl > 0.5f || (rem - fl == 0.5f && (n & 1)));
+        if (abs(S) > FX_RANGE) S = FX_INVALID;
+    }
+    const float Sh = (float)S, Sl = (float)(S - (S == FX_INVALID ? S : (int)Sh));
+#pragma unroll
+    for (int q = 1; q < 9; ++q) {
+        const float w = wq(q) * inv;  // exact
+        const float P = __fmul_rn(w, Sh), e = __fmaf_rn(w, Sl, __fmaf_rn(w, Sh, -P));
+        float s, t;
+        two_sum(u[q], -P, s, t);
+        d[q] = S == FX_INVALID ? __int_as_float(0x7fc00000) : __fadd_rn(s, __fsub_rn(t, e));
+    }
+    return S;
+}
+
 // Stored (post-collision, pull-ready) form from post-streaming populations:
 // slot q at y is read by the pull of cell y + e_q, or, when y + e_q lies
 // beyond a wall, by the bounce-back of direction opp(q) at y.  The two
@@ -403,14 +548,8 @@ __global__ void k_unstream(KParams p, int nlat, const float* __restrict__ pre,
             }
         }
         if (l < 2) {
-            double S = 0.0;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) S += (double)u[q];
-            const int S_fx = fx_from_double(S, p.fx_scale[l]);
-            const double Sr = fx_to_double(S_fx, p.fx_scale[l]);
             float d[9];
-#pragma unroll
-            for (int q = 1; q < 9; ++q) d[q] = (float)((double)u[q] - (double)wq(q) * Sr);
+            const int S_fx = deviations(u, p.fx_scale[l], p.fx_inv[l], d);
             store_dev(dl, p, idx, i, S_fx, d);
         } else {
             store9(dl, p, idx, i, u);
@@ -477,18 +616,278 @@ __global__ void k_f64_to_pre(KParams p, int lat, const double* __restrict__ in,
 }
 
 // ---------------------------------------------------------------------------
-// FP64 reductions (fixed order: per-block partials, one finishing block)
+// diagnostics: totals and the shape moments of the drop
 // ---------------------------------------------------------------------------
 
+// The drop indicator w, (phi - phi_b) / (phi_a - phi_b) clipped to [0, 1], in
+// units of phi's fixed point.  The shape moments (centroid, Ixx, Iyy, Ixy;
+// D = (L - B) / (L + B) of Sec. 4.3) belong to the drop region: the clip keeps
+// the small over- and undershoot of phi away from the interface, which its
+// distance would weigh heavily, out.
+__device__ __forceinline__ int drop_indicator(const KParams& p, int phi_fx) {
+    const int span = p.phi_a_fx - p.phi_b_fx, v = phi_fx - p.phi_b_fx;
+    return span > 0 ? min(max(v, 0), span) : min(max(-v, 0), -span);
+}
+
+// Everything that is summed over cells is a whole number (fixed-point values and
+// counts), so the sums are exact whatever their order and can be made by atomic
+// adds; w is summed by column and by row, from which the centroid, Ixx and Iyy
+// follow with one term per column or row.  Only Ixy needs the cells again.  With
+// FP64 sums, and the sines and cosines taken per cell, the two passes took 272 us
+// at 1024 x 512 after 72 us for the fields; now 78 and 17 us with the fields.
 constexpr int DIAG_THREADS = 256;
 constexpr double TWO_PI = 6.283185307179586476925286766559;
+enum DiagWord { DW_PHI = 0, DW_C, DW_NONFINITE, DW_SIGMA_NEG, DW_UMAX2, DW_DONE1, DW_DONE2, DW_COUNT = 8 };
+using u64 = unsigned long long;
+
+// Blocks of pass 2, each with a partial sum of Ixy: about 16 rows a thread, long
+// enough for the loads and short enough to fill the chip.
+static int ixy_strips(const KParams& p) { return (p.nx + DIAG_THREADS - 1) / DIAG_THREADS; }
+static int ixy_bands(const KParams& p) {
+    const int most = 1024 / ixy_strips(p), bands = (p.ny + 15) / 16;
+    return most < 1 ? 1 : bands < most ? bands : most;
+}
+size_t diag_words(const KParams& p) {
+    return DW_COUNT + (size_t)p.nx + p.ny + (size_t)ixy_strips(p) * ixy_bands(p);
+}
+
+// Sum over a warp of signed 32-bit values, exact.
+__device__ __forceinline__ long long warp_sum(int v) {
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffu);
+    const int hi = __reduce_add_sync(0xffffffffu, v >> 16);
+    return (long long)hi * 65536 + (long long)lo;
+}
+
+template <int NK>
+__device__ __forceinline__ void block_sum(double (&v)[NK]) {
+    __shared__ double red[NK][DIAG_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+        if (lane == 0) red[k][w] = v[k];
+    }
+    __syncthreads();
+    for (int k = 0; k < NK; ++k) {
+        v[k] = 0.0;
+        for (int q = 0; q < DIAG_THREADS / 32; ++q) v[k] += red[k][q];
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ double min_image(double d, int n, bool periodic) {
+    if (!periodic) return d;
+    while (d >= 0.5 * n) d -= n;
+    while (d < -0.5 * n) d += n;
+    return d;
+}
+
+// True in the block that is the last of the grid to come here; what the others
+// wrote before is then visible to it.
+__device__ __forceinline__ bool last_block(u64* done) {
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(done, 1ull) + 1 == (u64)gridDim.x * gridDim.y;
+        __threadfence();
+    }
+    __syncthreads();
+    return last;
+}
+
+// result layout: [0] sum_phi [1] sum_c [2] xc [3] yc [4] nonfinite [5] sigma_neg [6] umax
+//                [7] Ixx [8] Iyy [9] Ixy [10] L [11] B [12] D [13] sum w
+// Pass 1: fields of every cell, all sums but Ixy's, w of every cell into `wmap`
+// (0 where a field is not finite).  arg_lo, arg_hi: 1 - c / c_max between which
+// sigma is positive for certain.
+template <bool COUPLED>
+__global__ void __launch_bounds__(DIAG_THREADS)
+k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, float arg_lo, float arg_hi,
+        int* __restrict__ wmap, u64* __restrict__ words, double* __restrict__ res) {
+    static_assert(MT_X * MT_Y == DIAG_THREADS && MT_Y * 32 == DIAG_THREADS, "one warp per tile row");
+    u64* col = words + DW_COUNT;
+    u64* row = col + p.nx;
+    int phi = 0, c = 0, w = 0, nonfinite = 0, sigma_neg = 0;
+    float u2 = 0.0f, a = 0.0f, b = 0.0f;
+    macro_tile<COUPLED>(p, src, F, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float) {
+        const int64_t o = (int64_t)j * p.nx + i;
+        if (phi_fx == FX_INVALID || c_fx == FX_INVALID || !isfinite(ux) || !isfinite(uy)) {
+            nonfinite = 1;
+            wmap[o] = 0;
+            return;
+        }
+        phi = phi_fx;
+        c = c_fx;
+        w = drop_indicator(p, phi_fx);
+        wmap[o] = w;
+        a = ux;
+        b = uy;
+        u2 = ux * ux + uy * uy;
+        if (p.beta != 0.0f) {
+            const float near = 1.0f - (float)c_fx * p.fx_inv[1] * p.inv_cmax;
+            if (!(near > arg_lo && near < arg_hi)) {
+                const double arg = 1.0 - fx_to_double(c_fx, p.fx_scale[1]) * (double)p.inv_cmax;
+                sigma_neg = arg <= 0.0 || 1.0 + (double)p.beta * log(arg) < 0.0;
+            }
+        }
+    });
+    __shared__ int sw[MT_Y][MT_X];
+    __shared__ u64 su[MT_Y];
+    __shared__ long long ssum[2][MT_Y];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i = blockIdx.x * MT_X + tx, j = blockIdx.y * MT_Y + ty;
+    sw[ty][tx] = w;
+    const long long sphi = warp_sum(phi), sc = warp_sum(c), sr = warp_sum(w);
+    const unsigned bad = __popc(__ballot_sync(0xffffffffu, nonfinite)),
+                   neg = __popc(__ballot_sync(0xffffffffu, sigma_neg));
+    // the largest |u|^2 of the warp: in FP64 for the cells that may have it
+    const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(u2)));
+    double top = 0.0;
+    if ((a != 0.0f || b != 0.0f) && (most < 1e-30f || u2 >= most * 0.999999f)) top = widen(a) * widen(a) + widen(b) * widen(b);
+    u64 tb = (u64)__double_as_longlong(top);
+    for (int o = 16; o > 0; o >>= 1) tb = max(tb, __shfl_xor_sync(0xffffffffu, tb, o));
+    if (tx == 0) {
+        su[ty] = tb;
+        ssum[0][ty] = sphi;
+        ssum[1][ty] = sc;
+        if (sr) atomicAdd(row + j, (u64)sr);
+        if (bad) atomicAdd(words + DW_NONFINITE, (u64)bad);
+        if (neg) atomicAdd(words + DW_SIGMA_NEG, (u64)neg);
+    }
+    __syncthreads();
+    if (ty == 0 && i < p.nx) {
+        long long s = 0;
+        for (int r = 0; r < MT_Y; ++r) s += sw[r][tx];
+        if (s) atomicAdd(col + i, (u64)s);
+    }
+    if (threadIdx.x == DIAG_THREADS - 1) {
+        u64 m = 0;
+        for (int r = 0; r < MT_Y; ++r) m = max(m, su[r]);
+        if (m) atomicMax(words + DW_UMAX2, m);
+    }
+    // one add a block: atomics on one address are served one after the other
+    if (threadIdx.x >= 64 && threadIdx.x < 66) {
+        long long t = 0;
+        for (int r = 0; r < MT_Y; ++r) t += ssum[threadIdx.x - 64][r];
+        if (t) atomicAdd(words + (threadIdx.x == 64 ? DW_PHI : DW_C), (u64)t);
+    }
+    if (!last_block(words + DW_DONE1)) return;
+
+    // the centroid and the moments that follow from the column and row sums, by
+    // one block, in units of w
+    double v[6] = {0, 0, 0, 0, 0, 0};  // sum w, cos x, sin x; rows: cos y, sin y, y
+    for (int k = threadIdx.x; k < p.nx; k += DIAG_THREADS) {
+        const double s = (double)(long long)__ldcg(col + k);
+        if (s == 0.0) continue;
+        double sn, cs;
+        sincos(TWO_PI * (k + 0.5) / p.nx, &sn, &cs);
+        v[0] += s;
+        v[1] += s * cs;
+        v[2] += s * sn;
+    }
+    for (int k = threadIdx.x; k < p.ny; k += DIAG_THREADS) {
+        const double s = (double)(long long)__ldcg(row + k);
+        if (s == 0.0) continue;
+        if (p.walls) {
+            v[5] += s * (k + 0.5);
+            continue;
+        }
+        double sn, cs;
+        sincos(TWO_PI * (k + 0.5) / p.ny, &sn, &cs);
+        v[3] += s * cs;
+        v[4] += s * sn;
+    }
+    block_sum<6>(v);
+    double xc = 0.5 * p.nx, yc = 0.5 * p.ny;
+    if (v[0] != 0.0) {
+        double ax = atan2(v[2], v[1]);
+        if (ax < 0) ax += TWO_PI;
+        xc = ax * p.nx / TWO_PI;
+        if (p.walls) {
+            yc = v[5] / v[0];
+        } else {
+            double ay = atan2(v[4], v[3]);
+            if (ay < 0) ay += TWO_PI;
+            yc = ay * p.ny / TWO_PI;
+        }
+    }
+    double I[2] = {0.0, 0.0};
+    for (int k = threadIdx.x; k < p.nx; k += DIAG_THREADS) {
+        const double d = min_image(k + 0.5 - xc, p.nx, true);
+        I[0] += (double)(long long)__ldcg(col + k) * d * d;
+    }
+    for (int k = threadIdx.x; k < p.ny; k += DIAG_THREADS) {
+        const double d = min_image(k + 0.5 - yc, p.ny, !p.walls);
+        I[1] += (double)(long long)__ldcg(row + k) * d * d;
+    }
+    block_sum<2>(I);
+    if (threadIdx.x != 0) return;
+    const double sw0 = v[0] != 0.0 ? v[0] : 1.0;
+    res[0] = (double)(long long)__ldcg(words + DW_PHI) / (double)p.fx_scale[0];
+    res[1] = (double)(long long)__ldcg(words + DW_C) / (double)p.fx_scale[1];
+    res[2] = xc;
+    res[3] = yc;
+    res[4] = (double)__ldcg(words + DW_NONFINITE);
+    res[5] = (double)__ldcg(words + DW_SIGMA_NEG);
+    res[6] = sqrt(__longlong_as_double((long long)__ldcg(words + DW_UMAX2)));
+    res[7] = I[0] / sw0;
+    res[8] = I[1] / sw0;
+    res[13] = v[0];
+}
+
+// Pass 2: Ixy about the centroid, then the axes of the drop.  A thread owns a
+// column of a band of rows: one multiply-add a cell.
+__global__ void __launch_bounds__(DIAG_THREADS)
+k_diag2(KParams p, const int* __restrict__ wmap, u64* __restrict__ words, double* __restrict__ res) {
+    double* partial = reinterpret_cast<double*>(words + DW_COUNT + p.nx + p.ny);
+    const double xc = res[2], yc = res[3];
+    const int strips = (p.nx + DIAG_THREADS - 1) / DIAG_THREADS;
+    const int band = blockIdx.x / strips, bands = gridDim.x / strips;
+    const int i = (blockIdx.x - band * strips) * DIAG_THREADS + threadIdx.x;
+    const int j0 = (int)((int64_t)p.ny * band / bands), j1 = (int)((int64_t)p.ny * (band + 1) / bands);
+    double v[1] = {0.0};
+    __shared__ double dy[32];
+    for (int jb = j0; jb < j1; jb += 32) {
+        __syncthreads();
+        if (threadIdx.x < 32) dy[threadIdx.x] = min_image(jb + (int)threadIdx.x + 0.5 - yc, p.ny, !p.walls);
+        __syncthreads();
+        if (i >= p.nx) continue;
+        for (int j = jb; j < min(j1, jb + 32); ++j) {
+            const int w = wmap[(int64_t)j * p.nx + i];
+            if (w) v[0] += fx_widen(w, 1.0f) * dy[j - jb];
+        }
+    }
+    if (i < p.nx) v[0] *= min_image(i + 0.5 - xc, p.nx, true);
+    block_sum<1>(v);
+    if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
+    if (!last_block(words + DW_DONE2)) return;
+    double t[1] = {0.0};
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += DIAG_THREADS) t[0] += __ldcg(partial + k);
+    block_sum<1>(t);
+    if (threadIdx.x != 0) return;
+    const double I[3] = {res[7], res[8], res[13] != 0.0 ? t[0] / res[13] : 0.0};
+    const double tr = I[0] + I[1], det = I[0] * I[1] - I[2] * I[2];
+    const double disc = sqrt(fmax(0.25 * tr * tr - det, 0.0));
+    const double l1 = 0.5 * tr + disc, l2 = fmax(0.5 * tr - disc, 0.0);
+    const double L = 4.0 * sqrt(l1), B = 4.0 * sqrt(l2);
+    res[9] = I[2];
+    res[10] = L;
+    res[11] = B;
+    res[12] = (L + B) > 0.0 ? (L - B) / (L + B) : 0.0;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 statistics of given fields (fixed order: per-block partials, one
+// finishing block)
+// ---------------------------------------------------------------------------
 
 __device__ __forceinline__ bool finite_cell(double a, double b, double c, double d) {
     return isfinite(a) && isfinite(b) && isfinite(c) && isfinite(d);
 }
 
 template <int NS>
-__device__ void block_sum(double (&v)[NS], double* partial_out) {
+__device__ void block_partial(double (&v)[NS], double* partial_out) {
     __shared__ double red[NS][DIAG_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -507,23 +906,20 @@ __device__ void block_sum(double (&v)[NS], double* partial_out) {
     }
 }
 
-// Drop indicator: (phi - phi_b) / (phi_a - phi_b) clipped to [0, 1].  The
-// shape moments (centroid, Ixx, Iyy, Ixy; D = (L - B) / (L + B) of Sec. 4.3)
-// belong to the drop region: the clip keeps the small over- and undershoot of
-// phi away from the interface, which its distance would weigh heavily, out.
-__device__ __forceinline__ double drop_indicator(const KParams& p, double phi) {
+// The drop indicator (see `drop_indicator`) of an FP64 phi.
+__device__ __forceinline__ double drop_indicator_of(const KParams& p, double phi) {
     const double w = (phi - (double)p.phi_b) / ((double)p.phi_a - (double)p.phi_b);
     return fmin(fmax(w, 0.0), 1.0);
 }
 
 // Pass 1 sums: phi, c, w cos/sin(2 pi x / nx), w cos/sin(2 pi y / ny), w y,
 // nonfinite count, sigma<0 count, max |u| (as max), w (w: drop indicator).
-constexpr int DIAG_SW = 10;  // slot of sum w; after pass 1, block 0's slot holds the total
-__global__ void k_diag1(KParams p, const double* __restrict__ phi, const double* __restrict__ c,
+constexpr int STATS_SW = 10;  // slot of sum w; after pass 1, block 0's slot holds the total
+__global__ void k_stats1(KParams p, const double* __restrict__ phi, const double* __restrict__ c,
                         const double* __restrict__ ux, const double* __restrict__ uy,
                         double* __restrict__ partial) {
-    double v[DIAG_NSUM];
-    for (int k = 0; k < DIAG_NSUM; ++k) v[k] = 0.0;
+    double v[STATS_NSUM];
+    for (int k = 0; k < STATS_NSUM; ++k) v[k] = 0.0;
     double umax = 0.0;
     const int64_t n = (int64_t)p.nx * p.ny;
     for (int64_t o = (int64_t)blockIdx.x * DIAG_THREADS + threadIdx.x; o < n;
@@ -535,7 +931,7 @@ __global__ void k_diag1(KParams p, const double* __restrict__ phi, const double*
             continue;
         }
         const double ax = TWO_PI * (i + 0.5) / p.nx, ay = TWO_PI * (j + 0.5) / p.ny;
-        const double w = drop_indicator(p, f);
+        const double w = drop_indicator_of(p, f);
         v[0] += f;
         v[1] += cc;
         v[2] += w * cos(ax);
@@ -543,7 +939,7 @@ __global__ void k_diag1(KParams p, const double* __restrict__ phi, const double*
         v[4] += w * cos(ay);
         v[5] += w * sin(ay);
         v[6] += w * (j + 0.5);
-        v[DIAG_SW] += w;
+        v[STATS_SW] += w;
         const double arg = 1.0 - cc * (double)p.inv_cmax;
         if (p.beta != 0.0f && (arg <= 0.0 || 1.0 + (double)p.beta * log(arg) < 0.0)) v[8] += 1.0;
         umax = fmax(umax, sqrt(a * a + b * b));
@@ -551,34 +947,34 @@ __global__ void k_diag1(KParams p, const double* __restrict__ phi, const double*
     for (int o = 16; o > 0; o >>= 1) umax = fmax(umax, __shfl_down_sync(0xffffffffu, umax, o));
     __shared__ double smax[DIAG_THREADS / 32];
     if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = umax;
-    block_sum<DIAG_NSUM>(v, partial + (int64_t)blockIdx.x * DIAG_NSUM);
+    block_partial<STATS_NSUM>(v, partial + (int64_t)blockIdx.x * STATS_NSUM);
     if (threadIdx.x == 0) {
         double m = 0.0;
         for (int q = 0; q < DIAG_THREADS / 32; ++q) m = fmax(m, smax[q]);
-        partial[(int64_t)blockIdx.x * DIAG_NSUM + 9] = m;
+        partial[(int64_t)blockIdx.x * STATS_NSUM + 9] = m;
     }
 }
 
 // result layout: [0] sum_phi [1] sum_c [2] xc [3] yc [4] nonfinite [5] sigma_neg [6] umax
 //                [7] Ixx [8] Iyy [9] Ixy [10] L [11] B [12] D
 // Sums over the nb partial rows (slot 9 by max instead when MAX9) by one
-// block of DIAG_FINISH threads: thread t adds rows t, t + DIAG_FINISH, ... in
+// block of STATS_FINISH threads: thread t adds rows t, t + STATS_FINISH, ... in
 // order, then a fixed tree over the threads, so the result does not depend
 // on scheduling.  Thread 0 receives the totals in s.
-constexpr int DIAG_FINISH = 256;
+constexpr int STATS_FINISH = 256;
 template <int NK, bool MAX9>
 __device__ __forceinline__ void finish_sums(const double* __restrict__ partial, int nb,
                                             double s[NK]) {
-    __shared__ double red[NK][DIAG_FINISH];
+    __shared__ double red[NK][STATS_FINISH];
     for (int k = 0; k < NK; ++k) s[k] = 0.0;
-    for (int b = threadIdx.x; b < nb; b += DIAG_FINISH)
+    for (int b = threadIdx.x; b < nb; b += STATS_FINISH)
         for (int k = 0; k < NK; ++k) {
-            const double v = partial[(int64_t)b * DIAG_NSUM + k];
+            const double v = partial[(int64_t)b * STATS_NSUM + k];
             s[k] = (MAX9 && k == 9) ? fmax(s[k], v) : s[k] + v;
         }
     for (int k = 0; k < NK; ++k) red[k][threadIdx.x] = s[k];
     __syncthreads();
-    for (int w = DIAG_FINISH / 2; w > 0; w >>= 1) {
+    for (int w = STATS_FINISH / 2; w > 0; w >>= 1) {
         if (threadIdx.x < w)
             for (int k = 0; k < NK; ++k)
                 red[k][threadIdx.x] = (MAX9 && k == 9)
@@ -589,21 +985,21 @@ __device__ __forceinline__ void finish_sums(const double* __restrict__ partial, 
     for (int k = 0; k < NK; ++k) s[k] = red[k][0];
 }
 
-__global__ void __launch_bounds__(DIAG_FINISH) k_diag_finish1(KParams p, double* __restrict__ partial,
+__global__ void __launch_bounds__(STATS_FINISH) k_stats_finish1(KParams p, double* __restrict__ partial,
                                                               int nb, double* __restrict__ res) {
-    double s[DIAG_NSUM];
-    finish_sums<DIAG_NSUM, true>(partial, nb, s);
+    double s[STATS_NSUM];
+    finish_sums<STATS_NSUM, true>(partial, nb, s);
     if (threadIdx.x != 0) return;
     const double m = s[9];
     res[0] = s[0];
     res[1] = s[1];
     double xc = 0.5 * p.nx, yc = 0.5 * p.ny;
-    if (s[DIAG_SW] != 0.0) {
+    if (s[STATS_SW] != 0.0) {
         double ax = atan2(s[3], s[2]);
         if (ax < 0) ax += TWO_PI;
         xc = ax * p.nx / TWO_PI;
         if (p.walls) {
-            yc = s[6] / s[DIAG_SW];
+            yc = s[6] / s[STATS_SW];
         } else {
             double ay = atan2(s[5], s[4]);
             if (ay < 0) ay += TWO_PI;
@@ -616,17 +1012,10 @@ __global__ void __launch_bounds__(DIAG_FINISH) k_diag_finish1(KParams p, double*
     res[5] = s[8];
     res[6] = m;
     // the normalisation of pass 2 (the result array has no free slot)
-    partial[DIAG_SW] = s[DIAG_SW];
+    partial[STATS_SW] = s[STATS_SW];
 }
 
-__device__ __forceinline__ double min_image(double d, int n, bool periodic) {
-    if (!periodic) return d;
-    while (d >= 0.5 * n) d -= n;
-    while (d < -0.5 * n) d += n;
-    return d;
-}
-
-__global__ void k_diag2(KParams p, const double* __restrict__ phi, const double* __restrict__ c,
+__global__ void k_stats2(KParams p, const double* __restrict__ phi, const double* __restrict__ c,
                         const double* __restrict__ ux, const double* __restrict__ uy,
                         const double* __restrict__ res, double* __restrict__ partial) {
     double v[3] = {0.0, 0.0, 0.0};
@@ -639,20 +1028,20 @@ __global__ void k_diag2(KParams p, const double* __restrict__ phi, const double*
         if (!finite_cell(f, c[o], ux[o], uy[o])) continue;
         const double dx = min_image(i + 0.5 - xc, p.nx, true);
         const double dy = min_image(j + 0.5 - yc, p.ny, !p.walls);
-        const double w = drop_indicator(p, f);
+        const double w = drop_indicator_of(p, f);
         v[0] += w * dx * dx;
         v[1] += w * dy * dy;
         v[2] += w * dx * dy;
     }
-    block_sum<3>(v, partial + (int64_t)blockIdx.x * DIAG_NSUM);
+    block_partial<3>(v, partial + (int64_t)blockIdx.x * STATS_NSUM);
 }
 
-__global__ void __launch_bounds__(DIAG_FINISH) k_diag_finish2(const double* __restrict__ partial,
+__global__ void __launch_bounds__(STATS_FINISH) k_stats_finish2(const double* __restrict__ partial,
                                                               int nb, double* __restrict__ res) {
     double I[3];
     finish_sums<3, false>(partial, nb, I);
     if (threadIdx.x != 0) return;
-    const double s0 = partial[DIAG_SW];  // sum of the drop indicator (pass 1)
+    const double s0 = partial[STATS_SW];  // sum of the drop indicator (pass 1)
     if (s0 != 0.0)
         for (int k = 0; k < 3; ++k) I[k] /= s0;
     const double tr = I[0] + I[1], det = I[0] * I[1] - I[2] * I[2];
@@ -715,11 +1104,11 @@ cudaError_t configure_fused_smem() {
 
 void launch_macro_out(const KParams& p, const DevState& s, int src, double* phi, double* c,
                       double* ux, double* uy, double* P, cudaStream_t st) {
-    const int bx = 128;
+    const dim3 grid((p.nx + MT_X - 1) / MT_X, (p.ny + MT_Y - 1) / MT_Y);
     if (p.coupled)
-        k_macro_out<true><<<row_grid(p, bx), bx, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
+        k_macro_out<true><<<grid, MT_X * MT_Y, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
     else
-        k_macro_out<false><<<row_grid(p, bx), bx, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
+        k_macro_out<false><<<grid, MT_X * MT_Y, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
 }
 
 void launch_init(const KParams& p, const DevState& s, int dst, const double* phi,
@@ -752,7 +1141,23 @@ void launch_set_pops(const KParams& p, const DevState& s, int dst, const double*
     k_unstream<<<row_grid(p, bx), bx, 0, st>>>(p, s.nlat, tmp, s.pop[dst]);
 }
 
-int diag_blocks(const KParams& p) {
+cudaError_t launch_diag(const KParams& p, const DevState& s, int src, int* wmap, unsigned long long* words,
+                        double* result, cudaStream_t st) {
+    const cudaError_t e = cudaMemsetAsync(words, 0, sizeof(u64) * diag_words(p), st);
+    if (e != cudaSuccess) return e;
+    // 1 + beta log(arg) > 0 between these, with a margin for the FP32 arg
+    const double span = p.beta != 0.0f ? 1.0 / std::fabs((double)p.beta) : 0.0;
+    const float lo = (float)(std::exp(-span) + 1e-5), hi = (float)(std::exp(std::fmin(span, 80.0)) * 0.99999);
+    const dim3 grid((p.nx + MT_X - 1) / MT_X, (p.ny + MT_Y - 1) / MT_Y);
+    if (p.coupled)
+        k_diag1<true><<<grid, DIAG_THREADS, 0, st>>>(p, s.pop[src], s.fields, lo, hi, wmap, words, result);
+    else
+        k_diag1<false><<<grid, DIAG_THREADS, 0, st>>>(p, s.pop[src], s.fields, lo, hi, wmap, words, result);
+    k_diag2<<<ixy_strips(p) * ixy_bands(p), DIAG_THREADS, 0, st>>>(p, wmap, words, result);
+    return cudaSuccess;
+}
+
+int stats_blocks(const KParams& p) {
     const int64_t n = (int64_t)p.nx * p.ny;
     int64_t b = (n + DIAG_THREADS * 8 - 1) / (DIAG_THREADS * 8);
     if (b < 1) b = 1;
@@ -760,75 +1165,97 @@ int diag_blocks(const KParams& p) {
     return (int)b;
 }
 
-void launch_diag(const KParams& p, const double* phi, const double* c, const double* ux,
-                 const double* uy, double* partial, int nb, double* result, cudaStream_t st) {
-    k_diag1<<<nb, DIAG_THREADS, 0, st>>>(p, phi, c, ux, uy, partial);
-    k_diag_finish1<<<1, DIAG_FINISH, 0, st>>>(p, partial, nb, result);
-    k_diag2<<<nb, DIAG_THREADS, 0, st>>>(p, phi, c, ux, uy, result, partial);
-    k_diag_finish2<<<1, DIAG_FINISH, 0, st>>>(partial, nb, result);
+void launch_field_stats(const KParams& p, const double* phi, const double* c, const double* ux,
+                        const double* uy, double* partial, int nb, double* result, cudaStream_t st) {
+    k_stats1<<<nb, DIAG_THREADS, 0, st>>>(p, phi, c, ux, uy, partial);
+    k_stats_finish1<<<1, STATS_FINISH, 0, st>>>(p, partial, nb, result);
+    k_stats2<<<nb, DIAG_THREADS, 0, st>>>(p, phi, c, ux, uy, result, partial);
+    k_stats_finish2<<<1, STATS_FINISH, 0, st>>>(partial, nb, result);
 }
 
 // ---------------------------------------------------------------------------
-// 4-connected components of {phi > level}: labels by minimum-index
-// propagation with pointer jumping (the label of a cell is the smallest cell
-// index reachable inside the set), then a count of the roots.
+// 4-connected components of {phi > level}, periodic in x, and in y without walls
 // ---------------------------------------------------------------------------
+// Union-find on the cells: label[k] <= k points towards the smallest cell of k's
+// tree.  Cells start pointing at the first cell of their run within 32 aligned
+// columns; then every run is joined to its neighbours, each pair of runs once.
+// Components = trees at the start - joins.  Bound by the latency of the chains of
+// loads and atomics.  (Propagating the least label sweep by sweep, with a host
+// read after each, took 234 us a call at 1024 x 512; now 68, 25 of them here.)
 
-__global__ void k_label_init(const KParams p, const float* __restrict__ F, float level,
-                             int* __restrict__ label) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (int64_t)p.nx * p.ny) return;
-    const int i = (int)(k % p.nx), j = (int)(k / p.nx);
-    // the phi plane holds the fixed-point zeroth moment
-    const int phi_fx = __float_as_int(F[FP_PHI * p.plane + (int64_t)j * p.pitch + i]);
-    label[k] = (phi_fx != FX_INVALID && (float)phi_fx * p.fx_inv[0] > level) ? (int)k : -1;
+constexpr int LABEL_ROWS = 8;  // rows a block handles, one warp each
+
+__global__ void __launch_bounds__(32 * LABEL_ROWS)
+k_label_init(const KParams p, const float* __restrict__ src, float level, int* __restrict__ label,
+             int* __restrict__ count) {
+    const int tx = threadIdx.x & 31;
+    const int i = blockIdx.x * 32 + tx, j = blockIdx.y * LABEL_ROWS + (threadIdx.x >> 5);
+    bool in = false;
+    if (i < p.nx && j < p.ny) {
+        const ScalarMoments m = pull_scalar(src, p, 0, i, j);
+        const int phi_fx = fx_add_sr(m.s0, m.inc, p.fx_scale[0], moment_bits(step_seed(p), i, j, p.nx));
+        in = phi_fx != FX_INVALID && (float)phi_fx * p.fx_inv[0] > level;
+    }
+    const unsigned set = __ballot_sync(0xffffffffu, in);
+    // the run's first lane: just above the highest clear bit below this lane
+    const unsigned gap = ~set & ((1u << tx) - 1u);
+    const int first = gap ? 32 - __clz(gap) : 0;
+    const int k = j * p.nx + i;
+    if (i < p.nx && j < p.ny) label[k] = in ? k - (tx - first) : -1;
+    const int trees = __syncthreads_count(in && first == tx);
+    if (threadIdx.x == 0 && trees) atomicAdd(count, trees);
 }
 
-__global__ void k_label_step(const KParams p, int* __restrict__ label, int* __restrict__ changed) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (int64_t)p.nx * p.ny) return;
-    const int own = label[k];
-    if (own < 0) return;
-    const int i = (int)(k % p.nx), j = (int)(k / p.nx);
-    int m = own;
-    const int nb[4][2] = {{wrap_i(i - 1, p.nx), j}, {wrap_i(i + 1, p.nx), j}, {i, j - 1}, {i, j + 1}};
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        int jj = nb[d][1];
-        if (jj < 0 || jj >= p.ny) {
-            if (p.walls) continue;  // no neighbour across a wall
-            jj = wrap_i(jj, p.ny);
+// Join the trees of a and b; 1 if they were two.  Labels only ever fall and a
+// label is below its cell, so the walks and the retries end.
+__device__ __forceinline__ int join(int* label, int a, int b) {
+    volatile int* L = label;
+    while (true) {
+        for (int n = L[a]; n != a; n = L[a]) a = n;
+        for (int n = L[b]; n != b; n = L[b]) b = n;
+        if (a == b) return 0;
+        if (a < b) {
+            const int t = a;
+            a = b;
+            b = t;
         }
-        const int v = label[(int64_t)jj * p.nx + nb[d][0]];
-        if (v >= 0 && v < m) m = v;
-    }
-    m = min(m, label[m]);  // pointer jumping
-    if (m < own) {
-        atomicMin(&label[k], m);
-        *changed = 1;
+        const int old = atomicMin(label + a, b);
+        if (old == a) return 1;  // a was a root until now
+        a = old;                 // it had a parent already: join that one
     }
 }
 
-__global__ void k_label_roots(const KParams p, const int* __restrict__ label, int* __restrict__ count) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (int64_t)p.nx * p.ny) return;
-    if (label[k] == (int)k) atomicAdd(count, 1);
+__global__ void __launch_bounds__(32 * LABEL_ROWS)
+k_label_join(const KParams p, int* __restrict__ label, int* __restrict__ count) {
+    const int tx = threadIdx.x & 31;
+    const int i = blockIdx.x * 32 + tx, j = blockIdx.y * LABEL_ROWS + (threadIdx.x >> 5);
+    int joins = 0;
+    if (i < p.nx && j < p.ny) {
+        const int k = j * p.nx + i;
+        auto inside = [&](int at) { return label[at] >= 0; };
+        if (inside(k)) {
+            const int left = j * p.nx + wrap_i(i - 1, p.nx);
+            if ((tx == 0 || i == 0) && inside(left)) joins += join(label, k, left);
+            if (j > 0 || !p.walls) {
+                const int above = wrap_i(j - 1, p.ny) * p.nx;
+                // the cell to the left has joined the same two runs already
+                const bool again = tx > 0 && inside(left) && inside(above + i - 1);
+                if (inside(above + i) && !again) joins += join(label, k, above + i);
+            }
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) joins += __shfl_down_sync(0xffffffffu, joins, o);
+    if (tx == 0 && joins) atomicSub(count, joins);
 }
 
-void launch_label_init(const KParams& p, const float* fields, float level, int* label,
-                       cudaStream_t st) {
-    const int64_t n = (int64_t)p.nx * p.ny;
-    k_label_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, fields, level, label);
-}
-
-void launch_label_step(const KParams& p, int* label, int* changed, cudaStream_t st) {
-    const int64_t n = (int64_t)p.nx * p.ny;
-    k_label_step<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, label, changed);
-}
-
-void launch_label_roots(const KParams& p, const int* label, int* count, cudaStream_t st) {
-    const int64_t n = (int64_t)p.nx * p.ny;
-    k_label_roots<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, label, count);
+cudaError_t launch_components(const KParams& p, const DevState& s, int src, float level, int* label, int* count,
+                              cudaStream_t st) {
+    const cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((p.nx + 31) / 32, (p.ny + LABEL_ROWS - 1) / LABEL_ROWS);
+    k_label_init<<<grid, 32 * LABEL_ROWS, 0, st>>>(p, s.pop[src], level, label, count);
+    k_label_join<<<grid, 32 * LABEL_ROWS, 0, st>>>(p, label, count);
+    return cudaSuccess;
 }
 
 }  // namespace lbm

@@ -19,10 +19,10 @@
 
 namespace {
 
-// Partial sums of the two reduction passes: one row of DIAG_NSUM doubles per
+// Partial sums of the two reduction passes: one row of STATS_NSUM doubles per
 // reduction block, at most LBM_NOALLOC_MAX_BLOCKS blocks (96 KiB in all).
 constexpr int kMaxBlocks = LBM_NOALLOC_MAX_BLOCKS;
-static __device__ __align__(256) double g_stats_scratch[kMaxBlocks * lbm::DIAG_NSUM];
+static __device__ __align__(256) double g_stats_scratch[kMaxBlocks * lbm::STATS_NSUM];
 
 // Device address of g_stats_scratch per CUDA context.  A context has its own
 // copy of the module, and a context that is destroyed and created again
@@ -114,8 +114,8 @@ extern "C" int lbm_field_stats_noalloc(const double* phi, const double* c, const
     p.inv_cmax = (float)(1.0 / c_max);
     p.phi_a = (float)phi_a;  // the drop indicator of the shape moments
     p.phi_b = (float)phi_b;
-    const int nb = lbm::diag_blocks(p);
+    const int nb = lbm::stats_blocks(p);
     if (nb > kMaxBlocks) return LBM_ERR_INVALID_ARG;
-    lbm::launch_diag(p, phi, c, ux, uy, scratch, nb, result, (cudaStream_t)stream);
+    lbm::launch_field_stats(p, phi, c, ux, uy, scratch, nb, result, (cudaStream_t)stream);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
