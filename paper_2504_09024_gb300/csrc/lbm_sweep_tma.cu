@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(TILE_NT, 3)
     const int sy = local / en.nsx, sx = local - sy * en.nsx;
     const int src = parity ^ en.flip;
     tile_step<COUPLED, ST_F32>(en.tmap[src], p, en.pop[1 - src], en.fields, en.seg, sx, sy,
-                               step_seed_at(p, step_off), err);
+                               [&] { return step_seed_at(p, step_off); }, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -239,11 +239,11 @@ void launch_batch(const BatchTable& tab, const FusedShape& sh, bool coupled, int
                   int* err, cudaStream_t st) {
     if (sh.tile) {
         if (coupled)
-            k_tile_batch<true><<<tab.ntiles, TILE_NT, TileLayout<true, ST_F32>::bytes(sh.tile), st>>>(
-                tab, parity, step_off, err);
+            launch_after(k_tile_batch<true>, dim3(tab.ntiles), TileLayout<true, ST_F32>::bytes(sh.tile), st, tab,
+                         parity, step_off, err);
         else
-            k_tile_batch<false><<<tab.ntiles, TILE_NT, TileLayout<false, ST_F32>::bytes(sh.tile), st>>>(
-                tab, parity, step_off, err);
+            launch_after(k_tile_batch<false>, dim3(tab.ntiles), TileLayout<false, ST_F32>::bytes(sh.tile), st, tab,
+                         parity, step_off, err);
         return;
     }
     const size_t smem = sweep2_f32_smem_bytes(sh.bx, sh.cpt, sh.out, coupled);

@@ -38,7 +38,7 @@ void launch_step_tile(const KParams& p, float* dst, const float* fields, int seg
                       int st, int* err, cudaStream_t s) {
     const dim3 grid((p.nx + TILE_TX - 1) / TILE_TX, (p.ny + seg - 1) / seg);
     with_tile(p.coupled, st, [&](auto C, auto S) {
-        k_tile<C(), S()><<<grid, TILE_NT, TileLayout<C(), S()>::bytes(seg), s>>>(load_map, p, dst, fields, seg, err);
+        launch_after(k_tile<C(), S()>, grid, TileLayout<C(), S()>::bytes(seg), s, load_map, p, dst, fields, seg, err);
         return 0;
     });
 }
