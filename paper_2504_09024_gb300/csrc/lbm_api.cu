@@ -317,6 +317,20 @@ int fp32_view(lbm_ctx* ctx) {
     return 0;
 }
 
+// The current state as the source of its macroscopic fields.
+lbm::MacroSource macro_source(lbm_ctx* ctx) {
+    const bool tma = ctx->kernel == LBM_KERNEL_TMA;
+    return lbm::MacroSource{tma ? &ctx->tile_maps[ctx->cur] : nullptr, ctx->st,
+                            tma ? nullptr : ctx->ds.pop[fp32_view(ctx)], ctx->ds.fields, ctx->derr};
+}
+
+// The run's parameters without the test hook, which is for the next step.
+lbm::KParams unstalled(const lbm_ctx* ctx) {
+    lbm::KParams kp = ctx->kp;
+    kp.stall_test = 0;
+    return kp;
+}
+
 // Graph of GRAPH_STEPS >> chunk steps starting from buffer `parity`.
 int build_graph(lbm_ctx* ctx, int parity, int chunk) {
     const int n = GRAPH_STEPS >> chunk;
@@ -414,7 +428,7 @@ int lbm_create(const lbm_params* p, void* stream, lbm_ctx** out) {
         return LBM_ERR_CUDA;
     }
     if (lbm::configure_fused_smem() != cudaSuccess || lbm::configure_sweep2_smem() != cudaSuccess ||
-        lbm::configure_tile_smem() != cudaSuccess) {
+        lbm::configure_tile_smem() != cudaSuccess || lbm::configure_macro_smem() != cudaSuccess) {
         cudaGetLastError();
         lbm_destroy(ctx);
         return LBM_ERR_CUDA;
@@ -553,8 +567,7 @@ int lbm_step(lbm_ctx* ctx, int64_t nsteps) {
 int lbm_get_fields_device(lbm_ctx* ctx, double* phi, double* c, double* ux, double* uy,
                           double* P) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
-    const int b = fp32_view(ctx);
-    lbm::launch_macro_out(ctx->kp, ctx->ds, b, phi, c, ux, uy, P, ctx->stream);
+    lbm::launch_macro_out(unstalled(ctx), macro_source(ctx), phi, c, ux, uy, P, ctx->stream);
     return check_launch(ctx);
 }
 
@@ -626,7 +639,7 @@ int lbm_diagnostics(lbm_ctx* ctx, lbm_diag* out) {
     const int64_t n = cells(ctx);
     int rc = ensure_stage(ctx, sizeof(int) * (size_t)n);
     if (rc != LBM_OK) return rc;
-    const cudaError_t e = lbm::launch_diag(ctx->kp, ctx->ds, fp32_view(ctx), reinterpret_cast<int*>(ctx->stage),
+    const cudaError_t e = lbm::launch_diag(unstalled(ctx), macro_source(ctx), reinterpret_cast<int*>(ctx->stage),
                                            ctx->dwords, ctx->dresult, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     rc = check_launch(ctx);

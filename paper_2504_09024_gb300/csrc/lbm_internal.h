@@ -145,9 +145,19 @@ void launch_unpack16(const KParams& p, const float* src16_alloc, float* dst32_al
                      cudaStream_t s);
 // Fill the field planes (phi, c, dP*, sigma, n, |grad phi|) of the current state.
 void launch_fields(const KParams& p, const DevState& s, int src, cudaStream_t st);
-// Macroscopic outputs (float64, dense [ny][nx]) of the current state.
-void launch_macro_out(const KParams& p, const DevState& s, int src, double* phi, double* c,
-                      double* ux, double* uy, double* P, cudaStream_t st);
+// Where the macroscopic fields of a state come from: its tile load map and storage
+// format, or (map null) the FP32 populations `pop`; err: flag of the bounded waits.
+struct MacroSource {
+    const CUtensorMap* map;
+    int st;
+    const float* pop;
+    const float* fields;
+    int* err;
+};
+cudaError_t configure_macro_smem();
+// Macroscopic outputs (float64, dense [ny][nx]) of a state.
+void launch_macro_out(const KParams& p, const MacroSource& m, double* phi, double* c, double* ux, double* uy,
+                      double* P, cudaStream_t st);
 // Initialisation from float64 fields (dense); writes buffer `dst` (uses the other as scratch).
 void launch_init(const KParams& p, const DevState& s, int dst, const double* phi,
                  const double* c, const double* ux, const double* uy, const double* P,
@@ -169,10 +179,10 @@ constexpr int STATS_NSUM = 12;
 int stats_blocks(const KParams& p);
 void launch_field_stats(const KParams& p, const double* phi, const double* c, const double* ux,
                         const double* uy, double* partial, int nblocks, double* result, cudaStream_t st);
-// Diagnostics of the current state into result[0 .. 13] (layout at k_diag1);
+// Diagnostics of a state into result[0 .. 13] (layout at k_diag1);
 // wmap: nx * ny words, words: diag_words(p) 64-bit words of scratch.
 size_t diag_words(const KParams& p);
-cudaError_t launch_diag(const KParams& p, const DevState& s, int src, int* wmap, unsigned long long* words,
+cudaError_t launch_diag(const KParams& p, const MacroSource& m, int* wmap, unsigned long long* words,
                         double* result, cudaStream_t st);
 
 }  // namespace lbm

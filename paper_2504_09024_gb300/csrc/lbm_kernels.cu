@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "lbm_cell.cuh"
+#include "lbm_tile.cuh"
 
 namespace lbm {
 
@@ -147,9 +148,9 @@ __device__ __forceinline__ double fx_widen(int s, float scale) {
 // then the normals of the tile and one cell around it, then each cell's forces,
 // with the operations of the three-kernel chain in their order (same bits).
 //
-// Bound by the pulls (1.69 times the tile's, from L2) and their latency.  As
-// three kernels through global field planes the fields of 128 runs of 384 x 128
-// took 23 us a run, now 13.
+// Bound by the pulls (1.69 times the tile's, from L2) and their latency.  Serves
+// the kernels without bulk-tensor loads; the others have the tile staged as the
+// step does (tile_step with an `out`), from their own storage format.
 constexpr int MT_X = 32, MT_Y = 8;
 template <bool COUPLED, class Out>
 __device__ __forceinline__ void macro_tile(const KParams& p, const float* __restrict__ src,
@@ -237,11 +238,29 @@ __device__ __forceinline__ void macro_tile(const KParams& p, const float* __rest
     }
 }
 
-template <bool COUPLED>
+// ST: storage format of the state that `tmap` loads, or ST_NONE: plain pulls from
+// the FP32 state `src`.
+constexpr int ST_NONE = -1;
+template <bool COUPLED, int ST, class Out>
+__device__ __forceinline__ void macro_cells(const CUtensorMap* tmap, const KParams& p, const float* __restrict__ src,
+                                            const float* __restrict__ F, int* err, Out out) {
+    if constexpr (ST == ST_NONE) {
+        macro_tile<COUPLED>(p, src, F, out);
+    } else {
+        static_assert(MT_X == TILE_TX && MT_X * MT_Y == TILE_NT && MT_Y == TILE_SEG, "one cell per thread");
+        tile_step<COUPLED, ST>(tmap, p, nullptr, F, MT_Y, blockIdx.x, blockIdx.y, [&] { return step_seed(p); }, err,
+                               out);
+    }
+}
+
+// Fields as three kernels through global planes, then as plain pulls, then by
+// staged tiles: 128 runs of 384 x 128 23, 13 and 10 us a run, 768 x 256 16 us.
+template <bool COUPLED, int ST>
 __global__ void __launch_bounds__(MT_X * MT_Y)
-k_macro_out(KParams p, const float* __restrict__ src, const float* __restrict__ F, double* __restrict__ ophi,
-            double* __restrict__ oc, double* __restrict__ oux, double* __restrict__ ouy, double* __restrict__ oP) {
-    macro_tile<COUPLED>(p, src, F, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float dP) {
+k_macro_out(const __grid_constant__ CUtensorMap tmap, KParams p, const float* __restrict__ src,
+            const float* __restrict__ F, int* __restrict__ err, double* __restrict__ ophi, double* __restrict__ oc,
+            double* __restrict__ oux, double* __restrict__ ouy, double* __restrict__ oP) {
+    macro_cells<COUPLED, ST>(&tmap, p, src, F, err, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float dP) {
         const int64_t o = (int64_t)j * p.nx + i;
         if (ophi) ophi[o] = fx_widen(phi_fx, p.fx_scale[0]);
         if (oc) oc[o] = fx_widen(c_fx, p.fx_scale[1]);
@@ -648,7 +667,7 @@ static int ixy_bands(const KParams& p) {
     return most < 1 ? 1 : bands < most ? bands : most;
 }
 size_t diag_words(const KParams& p) {
-    return DW_COUNT + (size_t)p.nx + p.ny + (size_t)ixy_strips(p) * ixy_bands(p);
+    return DW_COUNT + 3 * ((size_t)p.nx + p.ny) + (size_t)ixy_strips(p) * ixy_bands(p);
 }
 
 // Sum over a warp of signed 32-bit values, exact.
@@ -701,16 +720,21 @@ __device__ __forceinline__ bool last_block(u64* done) {
 // Pass 1: fields of every cell, all sums but Ixy's, w of every cell into `wmap`
 // (0 where a field is not finite).  arg_lo, arg_hi: 1 - c / c_max between which
 // sigma is positive for certain.
-template <bool COUPLED>
+template <bool COUPLED, int ST>
 __global__ void __launch_bounds__(DIAG_THREADS)
-k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, float arg_lo, float arg_hi,
-        int* __restrict__ wmap, u64* __restrict__ words, double* __restrict__ res) {
+k_diag1(const __grid_constant__ CUtensorMap tmap, KParams p, const float* __restrict__ src,
+        const float* __restrict__ F, int* __restrict__ err, float arg_lo, float arg_hi, int* __restrict__ wmap,
+        u64* __restrict__ words, double* __restrict__ res) {
     static_assert(MT_X * MT_Y == DIAG_THREADS && MT_Y * 32 == DIAG_THREADS, "one warp per tile row");
-    u64* col = words + DW_COUNT;
+    // cosines and sines of the columns and rows: formed by the blocks at the grid's
+    // edges, spread over the SMs (FP64 on the finishing block's one SM is slow)
+    double2* xtrig = reinterpret_cast<double2*>(words + DW_COUNT);
+    double2* ytrig = xtrig + p.nx;
+    u64* col = reinterpret_cast<u64*>(ytrig + p.ny);
     u64* row = col + p.nx;
     int phi = 0, c = 0, w = 0, nonfinite = 0, sigma_neg = 0;
     float u2 = 0.0f, a = 0.0f, b = 0.0f;
-    macro_tile<COUPLED>(p, src, F, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float) {
+    macro_cells<COUPLED, ST>(&tmap, p, src, F, err, [&](int i, int j, int phi_fx, int c_fx, float ux, float uy, float) {
         const int64_t o = (int64_t)j * p.nx + i;
         if (phi_fx == FX_INVALID || c_fx == FX_INVALID || !isfinite(ux) || !isfinite(uy)) {
             nonfinite = 1;
@@ -772,6 +796,10 @@ k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, f
         for (int r = 0; r < MT_Y; ++r) t += ssum[threadIdx.x - 64][r];
         if (t) atomicAdd(words + (threadIdx.x == 64 ? DW_PHI : DW_C), (u64)t);
     }
+    if (blockIdx.y == 0 && ty == 0 && i < p.nx) sincos(TWO_PI * (i + 0.5) / p.nx, &xtrig[i].y, &xtrig[i].x);
+    const int jt = blockIdx.y * MT_Y + tx;
+    if (blockIdx.x == 0 && ty == 1 && tx < MT_Y && jt < p.ny && !p.walls)
+        sincos(TWO_PI * (jt + 0.5) / p.ny, &ytrig[jt].y, &ytrig[jt].x);
     if (!last_block(words + DW_DONE1)) return;
 
     // the centroid and the moments that follow from the column and row sums, by
@@ -780,11 +808,10 @@ k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, f
     for (int k = threadIdx.x; k < p.nx; k += DIAG_THREADS) {
         const double s = (double)(long long)__ldcg(col + k);
         if (s == 0.0) continue;
-        double sn, cs;
-        sincos(TWO_PI * (k + 0.5) / p.nx, &sn, &cs);
+        const double2 t = __ldcg(xtrig + k);
         v[0] += s;
-        v[1] += s * cs;
-        v[2] += s * sn;
+        v[1] += s * t.x;
+        v[2] += s * t.y;
     }
     for (int k = threadIdx.x; k < p.ny; k += DIAG_THREADS) {
         const double s = (double)(long long)__ldcg(row + k);
@@ -793,25 +820,31 @@ k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, f
             v[5] += s * (k + 0.5);
             continue;
         }
-        double sn, cs;
-        sincos(TWO_PI * (k + 0.5) / p.ny, &sn, &cs);
-        v[3] += s * cs;
-        v[4] += s * sn;
+        const double2 t = __ldcg(ytrig + k);
+        v[3] += s * t.x;
+        v[4] += s * t.y;
     }
     block_sum<6>(v);
-    double xc = 0.5 * p.nx, yc = 0.5 * p.ny;
-    if (v[0] != 0.0) {
-        double ax = atan2(v[2], v[1]);
-        if (ax < 0) ax += TWO_PI;
-        xc = ax * p.nx / TWO_PI;
-        if (p.walls) {
-            yc = v[5] / v[0];
-        } else {
-            double ay = atan2(v[4], v[3]);
-            if (ay < 0) ay += TWO_PI;
-            yc = ay * p.ny / TWO_PI;
+    __shared__ double centre[2];
+    if (threadIdx.x == 0) {  // (one thread: FP64 by all 256 would take the SM 12 us)
+        double xc = 0.5 * p.nx, yc = 0.5 * p.ny;
+        if (v[0] != 0.0) {
+            double ax = atan2(v[2], v[1]);
+            if (ax < 0) ax += TWO_PI;
+            xc = ax * p.nx / TWO_PI;
+            if (p.walls) {
+                yc = v[5] / v[0];
+            } else {
+                double ay = atan2(v[4], v[3]);
+                if (ay < 0) ay += TWO_PI;
+                yc = ay * p.ny / TWO_PI;
+            }
         }
+        centre[0] = xc;
+        centre[1] = yc;
     }
+    __syncthreads();
+    const double xc = centre[0], yc = centre[1];
     double I[2] = {0.0, 0.0};
     for (int k = threadIdx.x; k < p.nx; k += DIAG_THREADS) {
         const double d = min_image(k + 0.5 - xc, p.nx, true);
@@ -840,7 +873,7 @@ k_diag1(KParams p, const float* __restrict__ src, const float* __restrict__ F, f
 // column of a band of rows: one multiply-add a cell.
 __global__ void __launch_bounds__(DIAG_THREADS)
 k_diag2(KParams p, const int* __restrict__ wmap, u64* __restrict__ words, double* __restrict__ res) {
-    double* partial = reinterpret_cast<double*>(words + DW_COUNT + p.nx + p.ny);
+    double* partial = reinterpret_cast<double*>(words + DW_COUNT + 3 * ((size_t)p.nx + p.ny));
     const double xc = res[2], yc = res[3];
     const int strips = (p.nx + DIAG_THREADS - 1) / DIAG_THREADS;
     const int band = blockIdx.x / strips, bands = gridDim.x / strips;
@@ -1102,13 +1135,48 @@ cudaError_t configure_fused_smem() {
                                 maxb);
 }
 
-void launch_macro_out(const KParams& p, const DevState& s, int src, double* phi, double* c,
-                      double* ux, double* uy, double* P, cudaStream_t st) {
-    const dim3 grid((p.nx + MT_X - 1) / MT_X, (p.ny + MT_Y - 1) / MT_Y);
-    if (p.coupled)
-        k_macro_out<true><<<grid, MT_X * MT_Y, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
-    else
-        k_macro_out<false><<<grid, MT_X * MT_Y, 0, st>>>(p, s.pop[src], s.fields, phi, c, ux, uy, P);
+namespace {
+
+// f(coupled, storage format) as constants, and the shared memory of that form.
+template <typename F>
+cudaError_t with_macro(bool coupled, int st, F&& f) {
+    using std::integral_constant;
+    auto go = [&](auto C) {
+        if (st == ST_F32) return f(C, integral_constant<int, ST_F32>{}, TileLayout<C(), ST_F32>::bytes(MT_Y));
+        if (st == ST_F16) return f(C, integral_constant<int, ST_F16>{}, TileLayout<C(), ST_F16>::bytes(MT_Y));
+        if (st == ST_BF16) return f(C, integral_constant<int, ST_BF16>{}, TileLayout<C(), ST_BF16>::bytes(MT_Y));
+        return f(C, integral_constant<int, ST_NONE>{}, (size_t)0);
+    };
+    return coupled ? go(std::true_type{}) : go(std::false_type{});
+}
+
+dim3 macro_grid(const KParams& p) { return dim3((p.nx + MT_X - 1) / MT_X, (p.ny + MT_Y - 1) / MT_Y); }
+
+}  // namespace
+
+cudaError_t configure_macro_smem() {
+    cudaError_t e = cudaSuccess;
+    for (bool coupled : {false, true})
+        for (int st : {ST_F32, ST_F16, ST_BF16})
+            if (e == cudaSuccess)
+                e = with_macro(coupled, st, [](auto C, auto S, size_t smem) {
+                    cudaError_t a = cudaFuncSetAttribute(k_macro_out<C(), S()>,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                    return a != cudaSuccess ? a
+                                            : cudaFuncSetAttribute(k_diag1<C(), S()>,
+                                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                                   (int)smem);
+                });
+    return e;
+}
+
+void launch_macro_out(const KParams& p, const MacroSource& m, double* phi, double* c, double* ux, double* uy,
+                      double* P, cudaStream_t st) {
+    with_macro(p.coupled, m.map ? m.st : ST_NONE, [&](auto C, auto S, size_t smem) {
+        k_macro_out<C(), S()><<<macro_grid(p), MT_X * MT_Y, smem, st>>>(m.map ? *m.map : CUtensorMap{}, p, m.pop,
+                                                                        m.fields, m.err, phi, c, ux, uy, P);
+        return cudaSuccess;
+    });
 }
 
 void launch_init(const KParams& p, const DevState& s, int dst, const double* phi,
@@ -1141,18 +1209,18 @@ void launch_set_pops(const KParams& p, const DevState& s, int dst, const double*
     k_unstream<<<row_grid(p, bx), bx, 0, st>>>(p, s.nlat, tmp, s.pop[dst]);
 }
 
-cudaError_t launch_diag(const KParams& p, const DevState& s, int src, int* wmap, unsigned long long* words,
+cudaError_t launch_diag(const KParams& p, const MacroSource& m, int* wmap, unsigned long long* words,
                         double* result, cudaStream_t st) {
     const cudaError_t e = cudaMemsetAsync(words, 0, sizeof(u64) * diag_words(p), st);
     if (e != cudaSuccess) return e;
     // 1 + beta log(arg) > 0 between these, with a margin for the FP32 arg
     const double span = p.beta != 0.0f ? 1.0 / std::fabs((double)p.beta) : 0.0;
     const float lo = (float)(std::exp(-span) + 1e-5), hi = (float)(std::exp(std::fmin(span, 80.0)) * 0.99999);
-    const dim3 grid((p.nx + MT_X - 1) / MT_X, (p.ny + MT_Y - 1) / MT_Y);
-    if (p.coupled)
-        k_diag1<true><<<grid, DIAG_THREADS, 0, st>>>(p, s.pop[src], s.fields, lo, hi, wmap, words, result);
-    else
-        k_diag1<false><<<grid, DIAG_THREADS, 0, st>>>(p, s.pop[src], s.fields, lo, hi, wmap, words, result);
+    with_macro(p.coupled, m.map ? m.st : ST_NONE, [&](auto C, auto S, size_t smem) {
+        k_diag1<C(), S()><<<macro_grid(p), DIAG_THREADS, smem, st>>>(m.map ? *m.map : CUtensorMap{}, p, m.pop,
+                                                                     m.fields, m.err, lo, hi, wmap, words, result);
+        return cudaSuccess;
+    });
     k_diag2<<<ixy_strips(p) * ixy_bands(p), DIAG_THREADS, 0, st>>>(p, wmap, words, result);
     return cudaSuccess;
 }

@@ -72,11 +72,15 @@ void launch_after(void (*kernel)(P...), dim3 grid, size_t smem, cudaStream_t st,
 }
 
 // Tile (bxi, byi) of a run.  seg: rows per tile (4 .. TILE_SEG); seed_of(): the
-// hash of the step (step_seed); err: device flag of the bounded wait.
-template <bool COUPLED, int ST, class Seed>
+// hash of the step (step_seed); err: device flag of the bounded wait.  With an
+// `out` the block takes no step: it hands out(i, j, phi_fx, c_fx, ux, uy, P - P0)
+// of its cells to it, one cell per thread at 8 rows.
+struct TakeStep {};
+template <bool COUPLED, int ST, class Seed, class Out = TakeStep>
 __device__ __forceinline__ void tile_step(const CUtensorMap* tmap, const KParams& p, float* __restrict__ dst,
                                           const float* __restrict__ F, int seg, int bxi, int byi,
-                                          Seed seed_of, int* __restrict__ err) {
+                                          Seed seed_of, int* __restrict__ err, Out out = Out()) {
+    constexpr bool STEP = std::is_same<Out, TakeStep>::value;
     using L = TileLayout<COUPLED, ST>;
     constexpr int W = TILE_W, WW = TILE_WW, TX = TILE_TX, SLOT = L::SLOT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -243,7 +247,11 @@ __device__ __forceinline__ void tile_step(const CUtensorMap* tmap, const KParams
             else
                 pull_flow16_v<1, ST, W>(R0 - SLOT, R0, R0 + SLOT, w + 2, bot, top, p.qinv[2], gg);
             const CellOutT<float> o =
-                collide_flow_cell(p, g, jc, gg, true, ST == ST_F32 ? 1.0f : p.qs[2]);
+                collide_flow_cell(p, g, jc, gg, STEP, ST == ST_F32 ? 1.0f : p.qs[2]);
+            if constexpr (!STEP) {
+                out(i, jc, phi_fx, c_fx, o.ux, o.uy, o.dP);
+                continue;
+            }
             ux = o.ux;
             uy = o.uy;
             nx = g.nx;
@@ -261,11 +269,15 @@ __device__ __forceinline__ void tile_step(const CUtensorMap* tmap, const KParams
                                     [&](int m) { return __uint_as_float(wv[m]); });
             }
         } else {
-            float gm;
-            normal_at(r, w, nx, ny, gm);
             const int64_t idx = (int64_t)jc * p.pitch + i;
             ux = F[FP_UX * p.plane + idx];
             uy = F[FP_UY * p.plane + idx];
+            if constexpr (!STEP) {
+                out(i, jc, phi_fx, c_fx, ux, uy, 0.0f);
+                continue;
+            }
+            float gm;
+            normal_at(r, w, nx, ny, gm);
         }
         float df[9], dh[9];
         collide_scalars_pair(p, phi_fx, phi, (float)c_fx * p.fx_inv[1], nx, ny, ux, uy,
