@@ -125,7 +125,7 @@ __device__ __forceinline__ void lds(const float* p, float (&v)[N]) {
 // 128 bytes a cycle like any other, so a k costs (2 RO + 4 RS) / 4 cycles of
 // the SM for RO RS / 4 cycles of FMAs), at the few warps these sizes give an
 // SM.  Measured on GB300: an epoch of 1024 samples (this kernel and k_wgrad)
-// 40 us with <2, 2, 256> (8 samples a block, 128 blocks), 44 with <4, 2, 128>
+// 37 us with <2, 2, 256> (8 samples a block, 128 blocks), 41 with <4, 2, 128>
 // and <4, 1, 256>, 504 before with one launch per layer and direction; a scan
 // of 11,776 samples, copies included, 70 us with <4, 5, 512>, 74 with
 // <8, 5, 256>, 193 before.
@@ -349,6 +349,29 @@ __host__ __device__ constexpr int wg_tiles(int l) {
 }
 constexpr int WG_BLOCKS = wg_tiles(0) + wg_tiles(1) + wg_tiles(2) + wg_tiles(3) + wg_tiles(4);
 
+// A whole chunk of one operand, W columns of rows of WIDTH floats: what differs
+// between a thread's copies is an immediate.  With the row, the column and the
+// bounds worked out for each copy they were a third of the kernel's instructions
+// (64 epochs of 1024 samples 2.70 ms, now 2.34).
+// Columns beyond a narrow layer stay the zeros they were set to at the start.
+template <int W, int WIDTH>
+__device__ __forceinline__ void load_chunk(float* dst, const float* src, int t) {
+    if constexpr (WIDTH >= MAXW) {
+        constexpr int PER = W / 4, STEP = 32 / PER;
+        dst += t / PER * W + 4 * (t % PER);
+        src += t / PER * WIDTH + 4 * (t % PER);
+#pragma unroll
+        for (int i = 0; i < WCH / STEP; ++i) cp_async<16>(dst + i * STEP * W, src + i * STEP * WIDTH);
+    } else {
+        constexpr int PER = WIDTH <= 2 ? 2 : 8, STEP = 32 / PER;
+        dst += t / PER * W + t % PER;
+        src += t / PER * WIDTH + t % PER;
+        if (t % PER < WIDTH)
+#pragma unroll
+            for (int i = 0; i < WCH / STEP; ++i) cp_async<4>(dst + i * STEP * W, src + i * STEP * WIDTH);
+    }
+}
+
 template <bool ADAM>
 __global__ void __launch_bounds__(32) k_wgrad(const WgradArgs a) {
     __shared__ __align__(16) float sg[WST][WCH][WO], sx[WST][WCH][WI];
@@ -359,7 +382,12 @@ __global__ void __launch_bounds__(32) k_wgrad(const WgradArgs a) {
     const int o0 = tile / ni * WO, i0 = tile % ni * WI;
     const float *in = a.in[l], *gp = a.gpre[l];
     const int t = threadIdx.x;
-    // Chunk c of one operand: W columns from col0 of rows of `width` floats.
+    if (fout < WO || fin < WI) {
+        for (int k = t; k < WST * WCH * WO; k += 32) (&sg[0][0][0])[k] = 0.0f;
+        for (int k = t; k < WST * WCH * WI; k += 32) (&sx[0][0][0])[k] = 0.0f;
+        __syncwarp();
+    }
+    // The last, partial chunk of one operand: W columns from col0 of rows of `width` floats.
     // Samples beyond n and columns beyond the layer are zeros (their copies
     // read nothing; the source address stays inside the buffer).
     auto load_one = [&](float* dst, int W, const float* src, int width, int col0, int c) {
@@ -382,9 +410,16 @@ __global__ void __launch_bounds__(32) k_wgrad(const WgradArgs a) {
     };
     const int nchunk = (a.n + WCH - 1) / WCH;
     auto load = [&](int c) {
-        if (c < nchunk) {
-            load_one(&sg[c % WST][0][0], WO, gp, fout, o0, c);
-            load_one(&sx[c % WST][0][0], WI, in, fin, i0, c);
+        float *dg = &sg[c % WST][0][0], *dx = &sx[c % WST][0][0];
+        if ((c + 1) * WCH <= a.n) {
+            const float *g = gp + (int64_t)c * WCH * fout + o0, *x = in + (int64_t)c * WCH * fin + i0;
+            if (fout == MAXW) load_chunk<WO, MAXW>(dg, g, t);
+            else load_chunk<WO, width(NLAYER)>(dg, g, t);
+            if (fin == MAXW) load_chunk<WI, MAXW>(dx, x, t);
+            else load_chunk<WI, width(0)>(dx, x, t);
+        } else if (c < nchunk) {
+            load_one(dg, WO, gp, fout, o0, c);
+            load_one(dx, WI, in, fin, i0, c);
         }
         cp_async_commit();
     };
