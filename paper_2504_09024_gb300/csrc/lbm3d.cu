@@ -48,12 +48,13 @@
 // barrier per plane suffices.  Halo rows form only the populations that enter
 // the tile.
 //
-// What bounds it: instruction issue (66-73 % of the slots, DRAM at a fifth of
-// its rate).  256^3 at the library's shape, uniform u: 1980 us a step with all
-// populations stored, 575 us now (the 64 bytes a cell take 160 us); with a
-// velocity field 740 us.  f and h share packed FP32 instructions (lane x: f,
-// lane y: h), and what crosses rows goes as one 16-byte word per population
-// group: together 600 to 575 us (784 to 724 us with a field).
+// What bounds it: instruction issue (58-73 % of the slots, DRAM at a fifth of its
+// rate) at the 18 to 20 warps an SM that the registers allow.  256^3 at the library's
+// shape: 1980 us a step with all populations stored; in moments 600 us with a
+// uniform velocity and 784 with a field; f and h in packed FP32 instructions (lane
+// x: f, lane y: h) and 16-byte words across rows 575 and 724; a row's two moving
+// populations and its sum instead of three populations (emit_rows) 504 and 655.
+// The 64 bytes a cell take 160 us.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -95,9 +96,10 @@ struct K3Params {
     float w_kappa, w_chi, M_phi, D_s;
     float c4W, c8W, phi_a, phi_b, phim, inv_dphi;
     float u[3];
-    // uniform u: factors A, B, C along x by e = 0, +1, -1, and the products of
-    // those along y and z, [c][b]: Ay Az, Cy Cz, By Cz, Cy Bz; in both lanes
-    float2 fx[3][3], aa[3][3], cc[3][3], bc[3][3], cb[3][3];
+    // uniform u: the factors along x of emit_rows (t/2, 2u, u^2/2, u/2), and the
+    // products of those along y and z, [c][b]: Ay Az, Cy Cz / 2, By Cz, Cy Bz; in
+    // both lanes
+    float2 fx[4], aa[3][3], cc[3][3], bc[3][3], cb[3][3];
     const float* uf;  // per-cell velocity [3][N], or null for the uniform u
 };
 
@@ -213,16 +215,20 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
     return r;
 }
 
-// Populations (0, b, c), (1, b, c), (2, b, c) of both lattices, c = 0, 1, 2,
-// rounded to the grid: row(c, v0, v1, v2).  UFIELD takes the factors from the
-// cell's velocity, otherwise they come with the parameters.  The rest population
-// is left to the caller (v0 of b = c = 0).
+// Populations (0, b, c), (1, b, c), (2, b, c) of both lattices, c = 0, 1, 2, as
+// row(c, total, v1, v2): v1 and v2 and the row's sum are rounded to the grid, and
+// v0 = total - v1 - v2.  With P = s A A, X = kx C C, R = ky B C + kz C B the row is
+//     total = P + R,  v1, v2 = E +- O,
+//     E = P (cs^2 + u^2)/2 + X u + R u^2/2,  O = (P + R) u/2 + X/2.
+// UFIELD takes the factors from the cell's velocity, otherwise they come with the
+// parameters.  The rest population is the caller's (v0 of b = c = 0).
 template <bool UFIELD, bool BAD, class Row>
 __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r, int b, Row row) {
-    float A[3][3], B[3][3], C[3][3];
+    float A[3][3], B[3][3], C[3][3];  // along y and z
+    f2 th, u2x, uh2, uh;              // along x
     if constexpr (UFIELD) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 1; i < 3; ++i) {
             const float v = r.u[i], u2 = __fmul_rn(v, v), t = __fadd_rn(1.0f / 3.0f, u2);
             A[i][0] = __fsub_rn(1.0f, t);
             A[i][1] = __fmul_rn(0.5f, __fadd_rn(t, v));
@@ -234,31 +240,35 @@ __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r,
             C[i][1] = __fmul_rn(0.5f, __fadd_rn(u2, v));
             C[i][2] = __fmul_rn(0.5f, __fsub_rn(u2, v));
         }
+        const float v = r.u[0], h2 = __fmul_rn(0.5f * v, v);
+        th = f2(__fadd_rn(0.5f / 3.0f, h2));
+        u2x = f2(2.0f * v);
+        uh2 = f2(h2);
+        uh = f2(0.5f * v);
+    } else {
+        th = lbm::from_f2(p.fx[0]);
+        u2x = lbm::from_f2(p.fx[1]);
+        uh2 = lbm::from_f2(p.fx[2]);
+        uh = lbm::from_f2(p.fx[3]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        f2 P, X, R;
+        f2 P, X, R;  // X: half of the above
         if constexpr (UFIELD) {
             P = r.s * f2(__fmul_rn(A[1][b], A[2][c]));
-            X = r.k[0] * f2(__fmul_rn(C[1][b], C[2][c]));
+            X = r.k[0] * f2(__fmul_rn(0.5f * C[1][b], C[2][c]));
             R = lbm::vfma(r.k[1], f2(__fmul_rn(B[1][b], C[2][c])), r.k[2] * f2(__fmul_rn(C[1][b], B[2][c])));
         } else {
             P = r.s * lbm::from_f2(p.aa[c][b]);
             X = r.k[0] * lbm::from_f2(p.cc[c][b]);
             R = lbm::vfma(r.k[1], lbm::from_f2(p.bc[c][b]), r.k[2] * lbm::from_f2(p.cb[c][b]));
         }
-        uint2 v[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const f2 ax = UFIELD ? f2(A[0][a]) : lbm::from_f2(p.fx[0][a]),
-                     bx = UFIELD ? f2(B[0][a]) : lbm::from_f2(p.fx[1][a]),
-                     cx = UFIELD ? f2(C[0][a]) : lbm::from_f2(p.fx[2][a]);
-            const f2 t = lbm::vfma(R, cx, lbm::vfma(X, bx, P * ax));
-            int2 w = make_int2(__float2int_rn(t.x), __float2int_rn(t.y));
-            if (BAD && !r.ok) w = make_int2(FX_BAD, FX_BAD);
-            v[a] = make_uint2((uint32_t)w.x, (uint32_t)w.y);
-        }
-        row(c, v[0], v[1], v[2]);
+        const f2 W = P + R, O = lbm::vfma(W, uh, X), E = lbm::vfma(P, th, lbm::vfma(X, u2x, R * uh2));
+        auto grid = [&](f2 v) {
+            return BAD && !r.ok ? make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD)
+                                : make_uint2((uint32_t)__float2int_rn(v.x), (uint32_t)__float2int_rn(v.y));
+        };
+        row(c, grid(W), grid(E + O), grid(E - O));
     }
 }
 
@@ -272,8 +282,7 @@ __device__ __forceinline__ uint2 from_right(uint2 v) {
 }
 
 // Resident blocks per SM the register budget is sized for: 80 registers a
-// thread at 6 rows, 96 at 10 and 18 (up to 190 bytes of spill at 6 rows, 84 at
-// 10 and 18 with a velocity field, 40 without).
+// thread at 6 rows (80 to 176 bytes of spill), 96 at 10 and 18 (up to 44).
 template <int ROWS>
 constexpr int k3_min_blocks() { return ROWS == 6 ? 4 : ROWS == 10 ? 2 : 1; }
 
@@ -371,10 +380,10 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
                 uint2 moved = make_uint2(0u, 0u);
                 // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
                 auto across = [&](int b) {
-                    emit_rows<UFIELD, BAD>(p, r, b, [&](int c, uint2 v0, uint2 v1, uint2 v2) {
-                        moved = moved + (v0 + v1 + v2);
+                    emit_rows<UFIELD, BAD>(p, r, b, [&](int c, uint2 total, uint2 v1, uint2 v2) {
+                        moved = moved + total;
                         const uint2 t1 = from_left(v1), t2 = from_right(v2);
-                        const uint2 s = v0 + t1 + t2, d = t1 - t2;
+                        const uint2 s = (total - v1 - v2) + t1 + t2, d = t1 - t2;
                         x[(2 * c + b - 1) * PLANE] = make_uint4(s.x, d.x, s.y, d.y);
                     });
                 };
@@ -382,15 +391,15 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
                 if (ty >= 1) across(2);
                 if (inner) {
                     uint2 r1, r2;
-                    emit_rows<UFIELD, BAD>(p, r, 0, [&](int c, uint2 v0, uint2 v1, uint2 v2) {
+                    emit_rows<UFIELD, BAD>(p, r, 0, [&](int c, uint2 total, uint2 v1, uint2 v2) {
                         const uint2 t1 = from_left(v1), t2 = from_right(v2);
                         if (c == 0) {  // the rest population, once the other 26 are known
                             moved = moved + (v1 + v2);
                             r1 = t1;
                             r2 = t2;
                         } else {
-                            moved = moved + (v0 + v1 + v2);
-                            s0[c] = v0 + t1 + t2;
+                            moved = moved + total;
+                            s0[c] = (total - v1 - v2) + t1 + t2;
                             d0[c] = t1 - t2;
                         }
                     });
@@ -551,13 +560,12 @@ __device__ __forceinline__ void outgoing(const K3Params& p, const int* __restric
     uint2 v[Q27], moved = make_uint2(0u, 0u);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        auto row = [&](int c, uint2 v0, uint2 v1, uint2 v2) {
+        auto row = [&](int c, uint2 total, uint2 v1, uint2 v2) {
             const int q = 3 * b + 9 * c;
-            v[q] = v0;
+            v[q] = total - v1 - v2;
             v[q + 1] = v1;
             v[q + 2] = v2;
-            if (q) moved = moved + v0;
-            moved = moved + v1 + v2;
+            moved = moved + (q ? total : v1 + v2);
         };
         if (p.uf)
             emit_rows<true, true>(p, r, b, row);
@@ -797,26 +805,29 @@ int launch_step(lbm3_ctx* ctx) {
 }
 
 // The launch shape of a context whose user sets none.  A block spends seg_z + 3
-// planes' time (the halo planes and the first loads), so the segments that are
-// best make the blocks of an SM times that the smallest.  At 18 rows an SM holds
-// one block; at 10 rows two, which then take 1.45 times as long as one alone.
-// With a uniform velocity 18 rows win where both fill the chip (fewer halo
-// rows: 256^3 575 against 622 us, 150x97x61 43 against 45 us); a velocity field
-// needs the second block to hide the longer chains (256^3 791 against 724 us,
-// 220x200x180 425 against 355 us, 150x97x61 55 against 53 us).
+// planes' time (the halo planes and the first loads), so the best segments make
+// the blocks of an SM times that the least.  In units of a plane of 10 rows alone
+// on an SM, a plane of 18 rows takes 1.45, and a second block of 10 rows beside the
+// first 0.45 (0.75 with a velocity field, whose chains need more registers).
+// Measured, us per step at the best segments of 18 / 10 rows: uniform velocity
+// 256^3 504 / 485, 150x97x61 39 / 39, 64x50x40 16.5 / 14.5; velocity field 256^3
+// 655 / 788, 220x200x180 356 / 398, 150x97x61 49 / 49.
 void default_shape(const lbm3_params* p, int* rows, int* seg_z) {
-    *rows = p->velocity_field ? 10 : 18;
-    const long long tiles = (long long)((p->nx + TILE_IN - 1) / TILE_IN) * ((p->ny + *rows - 3) / (*rows - 2));
+    const double second = p->velocity_field ? 1.75 : 1.45;
     double best = -1.0;
-    for (int n = 1; n <= p->nz; ++n) {
-        const int seg = (p->nz + n - 1) / n;
-        if (n > 1 && seg == (p->nz + n - 2) / (n - 1)) continue;
-        const long long blocks = tiles * ((p->nz + seg - 1) / seg), per_sm = (blocks + 151) / 152;
-        const double load = p->velocity_field ? 1.45 * (double)(per_sm / 2) + (double)(per_sm % 2) : (double)per_sm;
-        const double cost = load * (seg + 3);
-        if (best < 0.0 || cost < best) {
-            best = cost;
-            *seg_z = seg;
+    for (int r : {10, 18}) {
+        const long long tiles = (long long)((p->nx + TILE_IN - 1) / TILE_IN) * ((p->ny + r - 3) / (r - 2));
+        for (int n = 1; n <= p->nz; ++n) {
+            const int seg = (p->nz + n - 1) / n;
+            if (n > 1 && seg == (p->nz + n - 2) / (n - 1)) continue;
+            const long long blocks = tiles * ((p->nz + seg - 1) / seg), per_sm = (blocks + 151) / 152;
+            const double load = r == 18 ? 1.45 * (double)per_sm : second * (double)(per_sm / 2) + (double)(per_sm % 2);
+            const double cost = load * (seg + 3);
+            if (best < 0.0 || cost < best) {
+                best = cost;
+                *rows = r;
+                *seg_z = seg;
+            }
         }
     }
 }
@@ -880,12 +891,15 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
         axis_factors(p->u[i], fac[i][0], fac[i][1], fac[i][2]);
     }
     auto both = [](double v) { return make_float2((float)v, (float)v); };
-    for (int k = 0; k < 3; ++k)
-        for (int e = 0; e < 3; ++e) kp.fx[k][e] = both(fac[0][k][e]);
+    const double ux = p->u[0];
+    kp.fx[0] = both(0.5 * (1.0 / 3.0 + ux * ux));
+    kp.fx[1] = both(2.0 * ux);
+    kp.fx[2] = both(0.5 * ux * ux);
+    kp.fx[3] = both(0.5 * ux);
     for (int c = 0; c < 3; ++c)
         for (int b = 0; b < 3; ++b) {
             kp.aa[c][b] = both(fac[1][0][b] * fac[2][0][c]);
-            kp.cc[c][b] = both(fac[1][2][b] * fac[2][2][c]);
+            kp.cc[c][b] = both(0.5 * fac[1][2][b] * fac[2][2][c]);
             kp.bc[c][b] = both(fac[1][1][b] * fac[2][2][c]);
             kp.cb[c][b] = both(fac[1][2][b] * fac[2][1][c]);
         }

@@ -125,8 +125,9 @@ __device__ __forceinline__ void lds(const float* p, float (&v)[N]) {
 // 128 bytes a cycle like any other, so a k costs (2 RO + 4 RS) / 4 cycles of
 // the SM for RO RS / 4 cycles of FMAs), at the few warps these sizes give an
 // SM.  Measured on GB300: an epoch of 1024 samples (this kernel and k_wgrad)
-// 37 us with <2, 2, 256> (8 samples a block, 128 blocks), 41 with <4, 2, 128>
-// and <4, 1, 256>, 504 before with one launch per layer and direction; a scan
+// 40 us with <2, 2, 256> (8 samples a block, 128 blocks), 44 with <4, 2, 128>
+// and <4, 1, 256>, 504 before with one launch per layer and direction (37 since
+// k_wgrad's copies got cheaper); a scan
 // of 11,776 samples, copies included, 70 us with <4, 5, 512>, 74 with
 // <8, 5, 256>, 193 before.
 template <int RO, int RS, int NT, bool BACKWARD>
