@@ -208,9 +208,24 @@ int sm_count() {
     return nsm > 0 ? nsm : 1;
 }
 
+// Rows per tile of the tile-parallel step, given the tiles that 4 .. 8 rows make.
+// A tile's time grows slowly with its rows and an SM holds three, so: the fewest
+// rows that leave one tile to an SM, else 4 if those fit at once, else the fewest
+// that do, else 8.  us per step at 4 / 5 / 6 / 7 / 8 rows: 128 x 128 fixed velocity
+// 3.7 3.9 3.9 4.0 4.4, 200 x 100 5.9 5.6 5.8 6.0 6.1, 256 x 128 7.2 6.9 7.3 6.2 6.3,
+// 301 x 167 BF16 6.3 7.0 7.6 8.2 7.0, 400 x 200 11.3 11.3 9.4 9.8 10.2, 512 x 256
+// 15.6 14.1 14.2 13.5 13.6, 800 x 400 30.6 28.2 27.0 25.9 24.5.
+template <class Tiles>
+int tile_rows(Tiles tiles, int nsm) {
+    for (int rows = 4; rows <= 8; ++rows)
+        if (tiles(rows) <= nsm) return rows;
+    for (int rows = 4; rows <= 8; ++rows)
+        if (tiles(rows) <= 3 * (int64_t)nsm) return rows;
+    return 8;
+}
+
 // Launch shape of a run whose user has not set one.
-//  * Up to 14 tiles of 32 x 8 per SM: the tile-parallel step, 4 rows a tile
-//    while those fit the chip at once (three blocks per SM), else 8.  Measured
+//  * Up to 14 tiles of 32 x 8 per SM: the tile-parallel step.  Measured
 //    on GB300 (FP32 coupled, us per step, against 128-wide strips of 32 rows
 //    before and the best sweep shape): 128 x 128 4.9 / 57.0 / 10.9, 512 x 256
 //    13.3 / 58.4 / 14.6, 1024 x 512 36.9 / 59.0 / 35.6; 2048 x 1024 128 / 136
@@ -240,7 +255,7 @@ lbm::FusedShape default_shape(const lbm::KParams& kp, int st) {
     }
     const int64_t strips = (kp.nx + 31) / 32;
     if (strips * ((kp.ny + 7) / 8) <= 14 * (int64_t)nsm)
-        best.tile = strips * ((kp.ny + 3) / 4) <= 3 * (int64_t)nsm ? 4 : 8;
+        best.tile = tile_rows([&](int rows) { return strips * ((kp.ny + rows - 1) / rows); }, nsm);
     return best;
 }
 
@@ -949,13 +964,13 @@ lbm::FusedShape batch_default_shape(const lbm_params* params, int nruns) {
             best.seg = seg;
         }
     }
-    int64_t tiles4 = 0, tiles8 = 0;
-    for (int r = 0; r < nruns; ++r) {
-        const int64_t strips = (params[r].nx + 31) / 32;
-        tiles4 += strips * ((params[r].ny + 3) / 4);
-        tiles8 += strips * ((params[r].ny + 7) / 8);
-    }
-    if (tiles8 <= 14 * (int64_t)nsm) best.tile = tiles4 <= 3 * (int64_t)nsm ? 4 : 8;
+    auto tiles = [&](int rows) {
+        int64_t n = 0;
+        for (int r = 0; r < nruns; ++r)
+            n += (int64_t)((params[r].nx + 31) / 32) * ((params[r].ny + rows - 1) / rows);
+        return n;
+    };
+    if (tiles(8) <= 14 * (int64_t)nsm) best.tile = tile_rows(tiles, nsm);
     return best;
 }
 

@@ -113,3 +113,12 @@ def test_batch_stall_hook_on_the_tile_step():
         assert np.isfinite(r.fields()["phi"]).all()
     s.close()
     b.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(201, 101), (399, 203), (257, 127)])  # 5, 6 and 7 rows a tile
+@pytest.mark.parametrize("walls,dtype", [(0, lbm.LBM_F32), (1, lbm.LBM_F32), (1, lbm.LBM_F16S)])
+def test_tile_step_of_other_heights_equals_sweep(nx, ny, walls, dtype):
+    a = run(nx, ny, dtype, walls, False, 1.0, 20)
+    b = run(nx, ny, dtype, walls, False, 1.0, 20, shape=(128, 16))
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
