@@ -945,20 +945,22 @@ int batch_fail(lbm_batch* b, cudaError_t e) {
 // Launch shape of a batch whose user has not set one: the tile-parallel step up
 // to 14 tiles of 32 x 8 per SM (as for one run), else 64-wide strips, the
 // fastest width of the batch kernel at every size measured, of the height with
-// the least (waves of resident blocks, and a third for the last) x (rows + 5).
-// us per step (192 x 32 before, now): 10 runs of 768 x 256 146 -> 109, 128 of
-// 384 x 128 569 -> 358, 10 of 256 x 128 73 -> 27.  The 64-wide form has no two
+// the least (waves of resident blocks + 0.7) x (rows + 4): 0.7 of a wave is what
+// the ragged end costs.  Over nine batches timed at 8 .. 64 rows that is within 2 %
+// of the best height (0.3 of a wave, and heights 8 rows apart: 5 %).  us per step
+// (192 x 32 before, at this shape): 10 runs of 768 x 256 146 -> 110, 128 of
+// 384 x 128 569 -> 359, 10 of 256 x 128 73 -> 27.  The 64-wide form has no two
 // cells per thread: setting that takes the 192-wide one.
 lbm::FusedShape batch_default_shape(const lbm_params* params, int nruns) {
     const int nsm = sm_count();
     lbm::FusedShape best{64, 32, 1, lbm::OUT_DIRECT};
     const double slots = (double)nsm * lbm::batch_blocks_per_sm(params[0].mode == LBM_COUPLED);
     double best_t = 1e300;
-    for (int seg : {8, 12, 16, 20, 24, 28, 32, 40, 48, 64}) {
+    for (int seg = 8; seg <= 64; seg += 4) {
         double blocks = 0;
         for (int r = 0; r < nruns; ++r)
             blocks += (double)((params[r].nx + 59) / 60) * ((params[r].ny + seg - 1) / seg);
-        const double t = (std::max(1.0, blocks / slots) + 0.3) * (seg + 5);
+        const double t = (std::max(1.0, blocks / slots) + 0.7) * (seg + 4);
         if (t < best_t) {
             best_t = t;
             best.seg = seg;
