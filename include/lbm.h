@@ -171,7 +171,8 @@ int lbm_get_populations(lbm_ctx *ctx, double *f, double *h, double *g);
  * [9][ny][nx]; NULL leaves that lattice unchanged).  Synchronous. */
 int lbm_set_populations(lbm_ctx *ctx, const double *f, const double *h, const double *g);
 
-/* FP64 reductions over the current state into *out (see lbm_diag).
+/* Reductions over the current state into *out (see lbm_diag): sums of the
+ * fixed-point values, exact, and FP64 from there; deterministic.
  * Synchronous.  Returns LBM_OK even when out->status reports non-finite cells. */
 int lbm_diagnostics(lbm_ctx *ctx, lbm_diag *out);
 
