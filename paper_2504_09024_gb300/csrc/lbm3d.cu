@@ -30,7 +30,9 @@
 // integers a uniform region is an exact fixed point.)
 //
 // A cell whose zeroth moment leaves (-4, 4) sends FX_BAD in all its
-// populations.  Populations are formed again when they are asked for: those of
+// populations, and a cell that receives FX_BAD gets it as its zeroth moment, so it
+// is out of range in turn.  (The sums do not say so by themselves: an even number
+// of FX_BAD adds up to nothing.)  Populations are formed again when they are asked for: those of
 // the state from the moments one step back (the other buffer), those of the
 // initial state from the fields it was made of, which the context keeps.  The
 // sums alone say phi, c and the totals, unless a population may have been out
@@ -46,7 +48,10 @@
 // the moments of plane k + 1 are on their way to registers meanwhile.  The
 // exchange buffer and the phi plane alternate between two copies, so one
 // barrier per plane suffices.  Halo rows form only the populations that enter
-// the tile.
+// the tile.  The loop forms populations as if every cell were valid; a block that
+// met one that is not goes over its cells once more at its end (mark_invalid).
+// (Bits of invalid cells exchanged in the loop with the populations cost 8 to 10 %
+// of a step in which nothing is invalid.)
 //
 // What bounds it: instruction issue (58-73 % of the slots, DRAM at a fifth of its
 // rate) at the 18 to 20 warps an SM that the registers allow.  256^3 at the library's
@@ -145,6 +150,11 @@ __device__ __forceinline__ void emit27(const T (&Ax)[3], const T (&Bx)[3], const
 
 __device__ __forceinline__ float fx_to_f(int v) { return (float)v * FX_INV; }
 
+// Both zeroth moments inside (-4, 4).
+__device__ __forceinline__ bool valid(int2 s) {
+    return fabsf(fx_to_f(s.x)) < S_MAX && fabsf(fx_to_f(s.y)) < S_MAX;
+}
+
 // What the gradient needs of one plane of phi around a cell: phi smoothed over
 // the plane, and its smoothed differences along x and y (twice the derivative).
 // Differences of equal values are exactly zero.
@@ -204,7 +214,7 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
         r.k[i] = lbm::vfma(w, lbm::vfma(q, f2(__fmul_rn(g[i], inv)), -a), a);
         big += fabsf(r.k[i].x) + fabsf(r.k[i].y);  // NaN stays NaN
     }
-    r.ok = fabsf(phi) < S_MAX && fabsf(c) < S_MAX;
+    r.ok = valid(m[0]);
     // Uniform |u| < 1/2: over the 27 neighbours the A products add up to 1 and those of
     // B and C to at most 3.2 a component, so |sum| < 4 + 3.2 * 0.3.  A field with
     // |u| <= 1/4, each neighbour its own: 2.3 and 3.5, so |sum| < 2 * 2.3 + 3.5 * 0.3.
@@ -292,7 +302,37 @@ constexpr int k3_ring_words() { return (ROWS + 2) * RING_W; }
 template <int ROWS>
 constexpr int k3_xchg_words() { return 24 * ROWS * TILE_W; }  // 6 x uint4 a cell
 template <int ROWS>
-constexpr int k3_smem() { return 4 * 2 * (k3_ring_words<ROWS>() + k3_xchg_words<ROWS>()); }
+constexpr int k3_ahead_words() { return 11 * ROWS * TILE_W; }  // 4 x int2 and 3 x float a cell
+template <int ROWS>
+constexpr int k3_smem(bool field) {
+    return 4 * (2 * (k3_ring_words<ROWS>() + k3_xchg_words<ROWS>()) + (field ? k3_ahead_words<ROWS>() : 0));
+}
+
+// Asynchronous copy of 4 or 8 bytes into shared memory.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(BYTES)
+                 : "memory");
+}
+
+// FX_BAD for the zeroth moments of the block's cells next to an invalid cell of
+// `src`.  A function of its own, so that the step's loop keeps no registers for it.
+template <int ROWS>
+__device__ __noinline__ void mark_invalid(const K3Params& p, const int* __restrict__ src, int* __restrict__ dst) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int x = blockIdx.x * TILE_IN + tx - 1, y = blockIdx.y * (ROWS - 2) + ty - 1;
+    if (tx < 1 || tx > TILE_IN || x >= p.nx || ty < 1 || ty > ROWS - 2 || y >= p.ny) return;
+    const int z0 = blockIdx.z * p.seg_z, z1 = min(p.nz, z0 + p.seg_z);
+    for (int z = z0; z < z1; ++z) {
+        bool bad = false;
+        for (int n = 0; n < Q27 && !bad; ++n) {
+            const int sx = wrapi(x + n % 3 - 1, p.nx), sy = wrapi(y + n / 3 % 3 - 1, p.ny), sz = wrapi(z + n / 9 - 1, p.nz);
+            bad = !valid(reinterpret_cast<const int2*>(src)[4 * p.nxny * sz + sy * p.nx + sx]);
+        }
+        if (bad) reinterpret_cast<int2*>(dst)[4 * p.nxny * z + y * p.nx + x] = make_int2(FX_BAD, FX_BAD);
+    }
+}
 
 template <int ROWS, bool UFIELD>
 __global__ void __launch_bounds__(ROWS * 32, k3_min_blocks<ROWS>())
@@ -342,6 +382,8 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         for (int i = 0; i < 3; ++i) u[i] = UFIELD ? __ldg(q + i * p.N) : p.u[i];
     };
 
+    __shared__ int met_invalid;
+    if (threadIdx.x == 0) met_invalid = 0;
     int zc = wrapi(z0 - 1, p.nz);  // the plane of k
     fetch(wrapi(z0 - 2, p.nz), 0);
     fetch(zc, 1);
@@ -356,15 +398,30 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
     fetch(zn, 0);
     __syncthreads();
 
+    // The moments and the velocity of the thread's cell in the next plane.  A uniform
+    // velocity leaves registers to have the moments loaded into; with a field they come
+    // by way of shared memory (live through the emission, some were spilled, and a
+    // spilled one waits there for its load: 655 us a step at 256^3, now 600).
+    int2* ahead = reinterpret_cast<int2*>(ring + 2 * RING) + threadIdx.x;    // [4][NT]
+    float* ahead_u = ring + 2 * RING + 8 * NT + threadIdx.x;                 // [3][NT]
+    auto load_ahead = [&](int z) {
+        const int2* q = reinterpret_cast<const int2*>(src + z * pstride) + cell;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) cp_async<8>(ahead + i * NT, q + (size_t)i * nxny);
+        const float* v = p.uf + (long long)z * nxny + cell;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) cp_async<4>(ahead_u + i * NT, v + i * p.N);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
     // Sums on their way, of f and h: `part` of plane k - 1 (complete but for what
     // comes from plane k), `up` of plane k (what came from plane k - 1).
     uint2 part[4] = {}, up[3] = {};
     int slot = 0;
     for (int k = z0 - 1; k <= z1; ++k) {
         int2 mn[4];
-        float un[3];
-        moments(zn, mn);
-        velocity(zn, un);
+        if constexpr (UFIELD) load_ahead(zn);
+        else moments(zn, mn);
         const int* q = src + zp * pstride;
         const int f0 = __ldg(q + 2 * o0), f1 = __ldg(q + 2 * o1);
 
@@ -374,45 +431,40 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         if (ty <= last + 1) {
             hi = plane(slot);
             const Collision r = collide<UFIELD>(p, m, lo, mid, hi, u);
-            if (!r.tame) *wild = 1;
-            auto emit = [&](auto bad) {
-                constexpr bool BAD = decltype(bad)::value;
-                uint2 moved = make_uint2(0u, 0u);
-                // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
-                auto across = [&](int b) {
-                    emit_rows<UFIELD, BAD>(p, r, b, [&](int c, uint2 total, uint2 v1, uint2 v2) {
-                        moved = moved + total;
-                        const uint2 t1 = from_left(v1), t2 = from_right(v2);
-                        const uint2 s = (total - v1 - v2) + t1 + t2, d = t1 - t2;
-                        x[(2 * c + b - 1) * PLANE] = make_uint4(s.x, d.x, s.y, d.y);
-                    });
-                };
-                if (ty <= last) across(1);
-                if (ty >= 1) across(2);
-                if (inner) {
-                    uint2 r1, r2;
-                    emit_rows<UFIELD, BAD>(p, r, 0, [&](int c, uint2 total, uint2 v1, uint2 v2) {
-                        const uint2 t1 = from_left(v1), t2 = from_right(v2);
-                        if (c == 0) {  // the rest population, once the other 26 are known
-                            moved = moved + (v1 + v2);
-                            r1 = t1;
-                            r2 = t2;
-                        } else {
-                            moved = moved + total;
-                            s0[c] = (total - v1 - v2) + t1 + t2;
-                            d0[c] = t1 - t2;
-                        }
-                    });
-                    uint2 rest = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
-                    if (BAD && !r.ok) rest = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
-                    s0[0] = rest + r1 + r2;
-                    d0[0] = r1 - r2;
-                }
+            uint2 moved = make_uint2(0u, 0u);
+            // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
+            auto across = [&](int b) {
+                emit_rows<UFIELD, false>(p, r, b, [&](int c, uint2 total, uint2 v1, uint2 v2) {
+                    moved = moved + total;
+                    const uint2 t1 = from_left(v1), t2 = from_right(v2);
+                    const uint2 s = (total - v1 - v2) + t1 + t2, d = t1 - t2;
+                    x[(2 * c + b - 1) * PLANE] = make_uint4(s.x, d.x, s.y, d.y);
+                });
             };
-            if (__all_sync(0xffffffffu, r.ok))
-                emit(std::false_type{});
-            else
-                emit(std::true_type{});
+            if (ty <= last) across(1);
+            if (ty >= 1) across(2);
+            if (inner) {
+                uint2 r1, r2;
+                emit_rows<UFIELD, false>(p, r, 0, [&](int c, uint2 total, uint2 v1, uint2 v2) {
+                    const uint2 t1 = from_left(v1), t2 = from_right(v2);
+                    if (c == 0) {  // the rest population, once the other 26 are known
+                        moved = moved + (v1 + v2);
+                        r1 = t1;
+                        r2 = t2;
+                    } else {
+                        moved = moved + total;
+                        s0[c] = (total - v1 - v2) + t1 + t2;
+                        d0[c] = t1 - t2;
+                    }
+                });
+                const uint2 rest = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
+                s0[0] = rest + r1 + r2;
+                d0[0] = r1 - r2;
+            }
+            if (!r.tame) {
+                *wild = 1;
+                if (!r.ok) met_invalid = 1;
+            }
         }
         ring[(slot ^ 1) * RING + threadIdx.x] = fx_to_f(f0);
         if (i1 < RING) ring[(slot ^ 1) * RING + i1] = fx_to_f(f1);
@@ -442,16 +494,21 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
             up[1] = JX[1];
             up[2] = JY[1];
         }
+        if constexpr (UFIELD) asm volatile("cp.async.wait_group 0;" ::: "memory");
         slot ^= 1;
         lo = mid;
         mid = hi;
         zn = zp;
         zp = next(zp);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m[i] = mn[i];
+        for (int i = 0; i < 4; ++i) m[i] = UFIELD ? ahead[i * NT] : mn[i];
+        if constexpr (UFIELD) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) u[i] = un[i];
+            for (int i = 0; i < 3; ++i) u[i] = ahead_u[i * NT];
+        }
     }
+    __syncthreads();
+    if (met_invalid) mark_invalid<ROWS>(p, src, dst);
 }
 
 // The fields an initial state is made of (velocity null: uniform u).
@@ -518,9 +575,10 @@ __global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state
                 uf[i * N + cell] = (float)v;
             }
         uint2 m[4] = {};
-        bool bad = false;
+        bool bad_f = false, bad_h = false;
         equilibrium(p, in, cell, [&](int q, int f, int h) {
-            bad |= f == FX_BAD || h == FX_BAD;
+            bad_f |= f == FX_BAD;
+            bad_h |= h == FX_BAD;
             const int e[3] = {q % 3, (q / 3) % 3, q / 9};
             const uint2 v = make_uint2((uint32_t)f, (uint32_t)h);
             m[0] = m[0] + v;
@@ -530,10 +588,12 @@ __global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state
                 if (e[i] == 2) m[1 + i] = m[1 + i] - v;
             }
         });
+        if (bad_f) m[0].x = (uint32_t)FX_BAD;
+        if (bad_h) m[0].y = (uint32_t)FX_BAD;
         uint2* o = reinterpret_cast<uint2*>(state) + (cell / p.nxny) * 4 * p.nxny + cell % p.nxny;
 #pragma unroll
         for (int i = 0; i < 4; ++i) o[i * p.nxny] = m[i];
-        if (bad) *wild = 1;
+        if (bad_f || bad_h) *wild = 1;
     }
 }
 
@@ -767,9 +827,9 @@ int grid_1d(long long n, int threads) {
 template <int ROWS>
 cudaError_t allow_smem(bool field) {
     return field ? cudaFuncSetAttribute(k3_step<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        k3_smem<ROWS>())
+                                        k3_smem<ROWS>(true))
                  : cudaFuncSetAttribute(k3_step<ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        k3_smem<ROWS>());
+                                        k3_smem<ROWS>(false));
 }
 
 int launch_step(lbm3_ctx* ctx) {
@@ -781,18 +841,18 @@ int launch_step(lbm3_ctx* ctx) {
               (kp.nz + ctx->seg_z - 1) / ctx->seg_z);
     const int src = ctx->cur, dst = 1 - ctx->cur;
     const bool field = kp.uf != nullptr;
-    auto go = [&](auto kern, int threads, int smem) {
-        kern<<<grid, threads, smem, ctx->stream>>>(p, ctx->buf[src], ctx->buf[dst], ctx->wild);
+    auto go = [&](auto kern, int smem) {
+        kern<<<grid, rows * 32, smem, ctx->stream>>>(p, ctx->buf[src], ctx->buf[dst], ctx->wild);
     };
     switch (rows) {
         case 6:
-            field ? go(k3_step<6, true>, 6 * 32, k3_smem<6>()) : go(k3_step<6, false>, 6 * 32, k3_smem<6>());
+            field ? go(k3_step<6, true>, k3_smem<6>(true)) : go(k3_step<6, false>, k3_smem<6>(false));
             break;
         case 10:
-            field ? go(k3_step<10, true>, 10 * 32, k3_smem<10>()) : go(k3_step<10, false>, 10 * 32, k3_smem<10>());
+            field ? go(k3_step<10, true>, k3_smem<10>(true)) : go(k3_step<10, false>, k3_smem<10>(false));
             break;
         case 18:
-            field ? go(k3_step<18, true>, 18 * 32, k3_smem<18>()) : go(k3_step<18, false>, 18 * 32, k3_smem<18>());
+            field ? go(k3_step<18, true>, k3_smem<18>(true)) : go(k3_step<18, false>, k3_smem<18>(false));
             break;
         default:
             return LBM_ERR_INVALID_ARG;
