@@ -30,7 +30,8 @@
 // integers a uniform region is an exact fixed point.)
 //
 // A cell whose zeroth moment leaves (-4, 4) sends FX_BAD in all its
-// populations, and a cell that receives FX_BAD gets it as its zeroth moment, so it
+// populations; a single population below -8 is FX_BAD too, and one above 8 is cut
+// off there.  A cell that receives FX_BAD gets it as its zeroth moment, so it
 // is out of range in turn.  (The sums do not say so by themselves: an even number
 // of FX_BAD adds up to nothing.)  Populations are formed again when they are asked for: those of
 // the state from the moments one step back (the other buffer), those of the
@@ -48,8 +49,9 @@
 // the moments of plane k + 1 are on their way to registers meanwhile.  The
 // exchange buffer and the phi plane alternate between two copies, so one
 // barrier per plane suffices.  Halo rows form only the populations that enter
-// the tile.  The loop forms populations as if every cell were valid; a block that
-// met one that is not goes over its cells once more at its end (mark_invalid).
+// the tile.  The loop forms populations as if every cell were valid and every
+// population in range; a block that met others goes over its cells once more at
+// its end (settle_invalid).
 // (Bits of invalid cells exchanged in the loop with the populations cost 8 to 10 %
 // of a step in which nothing is invalid.)
 //
@@ -184,8 +186,13 @@ struct Collision {
     int2 s_fx;
     f2 s, k[3];
     float u[3];
+    float most, big, fast;  // the larger |s|, the sum of |k'| and (velocity field) the largest |u|
     bool ok;    // both zeroth moments inside (-4, 4)
     bool tame;  // no population can leave the fixed-point range, nor their sums 32 bits
+    // ok, and no population can leave the range: |A| <= 1.17, |B| <= 2 and |C| <= 1 up to |u| = 1
+    __device__ __forceinline__ bool safe() const {
+        return ok && fast <= 1.0f && __fmaf_rn(1.6f, most, 2.0f * big) < 7.9f * FX_ONE;
+    }
 };
 
 template <bool UFIELD>
@@ -215,6 +222,9 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
         big += fabsf(r.k[i].x) + fabsf(r.k[i].y);  // NaN stays NaN
     }
     r.ok = valid(m[0]);
+    r.most = fmaxf(fabsf(r.s.x), fabsf(r.s.y));
+    r.big = big;
+    r.fast = UFIELD ? fmaxf(fmaxf(fabsf(u[0]), fabsf(u[1])), fabsf(u[2])) : 0.f;
     // Uniform |u| < 1/2: over the 27 neighbours the A products add up to 1 and those of
     // B and C to at most 3.2 a component, so |sum| < 4 + 3.2 * 0.3.  A field with
     // |u| <= 1/4, each neighbour its own: 2.3 and 3.5, so |sum| < 2 * 2.3 + 3.5 * 0.3.
@@ -225,14 +235,20 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
     return r;
 }
 
+__device__ __forceinline__ uint2 operator+(uint2 a, uint2 b) { return make_uint2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ uint2 operator-(uint2 a, uint2 b) { return make_uint2(a.x - b.x, a.y - b.y); }
+
 // Populations (0, b, c), (1, b, c), (2, b, c) of both lattices, c = 0, 1, 2, as
 // row(c, total, v1, v2): v1 and v2 and the row's sum are rounded to the grid, and
 // v0 = total - v1 - v2.  With P = s A A, X = kx C C, R = ky B C + kz C B the row is
 //     total = P + R,  v1, v2 = E +- O,
 //     E = P (cs^2 + u^2)/2 + X u + R u^2/2,  O = (P + R) u/2 + X/2.
 // UFIELD takes the factors from the cell's velocity, otherwise they come with the
-// parameters.  The rest population is the caller's (v0 of b = c = 0).
-template <bool UFIELD, bool BAD, class Row>
+// parameters.  The rest population is the caller's (v0 of b = c = 0).  With CHECK,
+// v0 of a cell that is not safe() is rounded by itself, like v1 and v2 (the
+// conversion cuts off at the ends of the range, and its lower end is FX_BAD), and
+// all populations of a cell that is not ok are FX_BAD.
+template <bool UFIELD, bool CHECK, class Row>
 __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r, int b, Row row) {
     float A[3][3], B[3][3], C[3][3];  // along y and z
     f2 th, u2x, uh2, uh;              // along x
@@ -275,15 +291,14 @@ __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r,
         }
         const f2 W = P + R, O = lbm::vfma(W, uh, X), E = lbm::vfma(P, th, lbm::vfma(X, u2x, R * uh2));
         auto grid = [&](f2 v) {
-            return BAD && !r.ok ? make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD)
-                                : make_uint2((uint32_t)__float2int_rn(v.x), (uint32_t)__float2int_rn(v.y));
+            return CHECK && !r.ok ? make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD)
+                                  : make_uint2((uint32_t)__float2int_rn(v.x), (uint32_t)__float2int_rn(v.y));
         };
-        row(c, grid(W), grid(E + O), grid(E - O));
+        const uint2 v1 = grid(E + O), v2 = grid(E - O);
+        row(c, CHECK && !r.safe() ? grid(lbm::vfma(f2(-2.0f), E, W)) + v1 + v2 : grid(W), v1, v2);
     }
 }
 
-__device__ __forceinline__ uint2 operator+(uint2 a, uint2 b) { return make_uint2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ uint2 operator-(uint2 a, uint2 b) { return make_uint2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ uint2 from_left(uint2 v) {
     return make_uint2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
 }
@@ -316,21 +331,88 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {
                  : "memory");
 }
 
-// FX_BAD for the zeroth moments of the block's cells next to an invalid cell of
-// `src`.  A function of its own, so that the step's loop keeps no registers for it.
+__device__ __forceinline__ int vel(int a) { return a == 0 ? 0 : a == 1 ? 1 : -1; }
+
+// The populations that a cell of a state sends out in a step: out(q, f, h).
+template <class Out>
+__device__ __forceinline__ void outgoing(const K3Params& p, const int* __restrict__ state, int x, int y, int z,
+                                         Out out) {
+    Plane pl[3];
+#pragma unroll
+    for (int dz = 0; dz < 3; ++dz) {
+        const int* q = state + 8 * p.nxny * wrapi(z + dz - 1, p.nz);
+        pl[dz] = plane_of([&](int dy, int dx) {
+            return fx_to_f(q[2 * ((long long)wrapi(y + dy, p.ny) * p.nx + wrapi(x + dx, p.nx))]);
+        });
+    }
+    const long long in = (long long)y * p.nx + x;
+    int2 m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = reinterpret_cast<const int2*>(state)[(4LL * z + i) * p.nxny + in];
+    float u[3] = {p.u[0], p.u[1], p.u[2]};
+    if (p.uf)
+        for (int i = 0; i < 3; ++i) u[i] = p.uf[i * p.N + z * p.nxny + in];
+    const Collision r = collide<true>(p, m, pl[0], pl[1], pl[2], u);
+    uint2 v[Q27], moved = make_uint2(0u, 0u);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        auto row = [&](int c, uint2 total, uint2 v1, uint2 v2) {
+            const int q = 3 * b + 9 * c;
+            v[q] = total - v1 - v2;
+            v[q + 1] = v1;
+            v[q + 2] = v2;
+            moved = moved + (q ? total : v1 + v2);
+        };
+        if (p.uf)
+            emit_rows<true, true>(p, r, b, row);
+        else
+            emit_rows<false, true>(p, r, b, row);
+    }
+    v[0] = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
+    if (!r.ok) v[0] = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
+#pragma unroll
+    for (int q = 0; q < Q27; ++q) out(q, (int)v[q].x, (int)v[q].y);
+}
+
+// What the step's loop leaves out, for a block that met invalid cells: FX_BAD for
+// the zeroth moments of cells that FX_BAD is sent to, by invalid cells of `src` and
+// (single: the block met cells that are not safe()) by others; for the latter all
+// sums are made once more, of the populations as they are cut off.  A function of
+// its own, and one that adds up in place: what it needs in registers costs the loop
+// up to 5 %.
 template <int ROWS>
-__device__ __noinline__ void mark_invalid(const K3Params& p, const int* __restrict__ src, int* __restrict__ dst) {
+__device__ __noinline__ void settle_invalid(const K3Params& p, const int* __restrict__ src, int* __restrict__ dst,
+                                            bool single) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int x = blockIdx.x * TILE_IN + tx - 1, y = blockIdx.y * (ROWS - 2) + ty - 1;
     if (tx < 1 || tx > TILE_IN || x >= p.nx || ty < 1 || ty > ROWS - 2 || y >= p.ny) return;
     const int z0 = blockIdx.z * p.seg_z, z1 = min(p.nz, z0 + p.seg_z);
     for (int z = z0; z < z1; ++z) {
-        bool bad = false;
-        for (int n = 0; n < Q27 && !bad; ++n) {
-            const int sx = wrapi(x + n % 3 - 1, p.nx), sy = wrapi(y + n / 3 % 3 - 1, p.ny), sz = wrapi(z + n / 9 - 1, p.nz);
-            bad = !valid(reinterpret_cast<const int2*>(src)[4 * p.nxny * sz + sy * p.nx + sx]);
+        bool bad_f = false, bad_h = false;
+        uint2* o = reinterpret_cast<uint2*>(dst) + 4 * p.nxny * z + y * p.nx + x;
+        if (single)
+            for (int i = 0; i < 4; ++i) o[i * p.nxny] = make_uint2(0u, 0u);
+        for (int want = 0; want < Q27; ++want) {
+            const int e[3] = {vel(want % 3), vel(want / 3 % 3), vel(want / 9)};
+            const int sx = wrapi(x - e[0], p.nx), sy = wrapi(y - e[1], p.ny), sz = wrapi(z - e[2], p.nz);
+            if (!valid(reinterpret_cast<const int2*>(src)[4 * p.nxny * sz + sy * p.nx + sx])) {
+                bad_f = bad_h = true;
+            } else if (single) {
+                outgoing(p, src, sx, sy, sz, [&](int q, int f, int h) {
+                    if (q != want) return;
+                    bad_f |= f == FX_BAD;
+                    bad_h |= h == FX_BAD;
+                    const uint2 v = make_uint2((uint32_t)f, (uint32_t)h);
+                    o[0] = o[0] + v;
+                    for (int i = 0; i < 3; ++i) {
+                        uint2* j = o + (i + 1) * p.nxny;
+                        *j = e[i] < 0 ? *j - v : e[i] ? *j + v : *j;
+                    }
+                });
+            }
         }
-        if (bad) reinterpret_cast<int2*>(dst)[4 * p.nxny * z + y * p.nx + x] = make_int2(FX_BAD, FX_BAD);
+        if (bad_f) o->x = (uint32_t)FX_BAD;
+        if (bad_h) o->y = (uint32_t)FX_BAD;
     }
 }
 
@@ -382,8 +464,8 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         for (int i = 0; i < 3; ++i) u[i] = UFIELD ? __ldg(q + i * p.N) : p.u[i];
     };
 
-    __shared__ int met_invalid;
-    if (threadIdx.x == 0) met_invalid = 0;
+    __shared__ int met_invalid, met_single;
+    if (threadIdx.x == 0) met_invalid = met_single = 0;
     int zc = wrapi(z0 - 1, p.nz);  // the plane of k
     fetch(wrapi(z0 - 2, p.nz), 0);
     fetch(zc, 1);
@@ -464,6 +546,7 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
             if (!r.tame) {
                 *wild = 1;
                 if (!r.ok) met_invalid = 1;
+                else if (!r.safe()) met_single = 1;
             }
         }
         ring[(slot ^ 1) * RING + threadIdx.x] = fx_to_f(f0);
@@ -508,7 +591,7 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         }
     }
     __syncthreads();
-    if (met_invalid) mark_invalid<ROWS>(p, src, dst);
+    if (met_invalid | met_single) settle_invalid<ROWS>(p, src, dst, met_single != 0);
 }
 
 // The fields an initial state is made of (velocity null: uniform u).
@@ -596,49 +679,6 @@ __global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state
         if (bad_f || bad_h) *wild = 1;
     }
 }
-
-// The populations that a cell of a state sends out in a step: out(q, f, h).
-template <class Out>
-__device__ __forceinline__ void outgoing(const K3Params& p, const int* __restrict__ state, int x, int y, int z,
-                                         Out out) {
-    Plane pl[3];
-#pragma unroll
-    for (int dz = 0; dz < 3; ++dz) {
-        const int* q = state + 8 * p.nxny * wrapi(z + dz - 1, p.nz);
-        pl[dz] = plane_of([&](int dy, int dx) {
-            return fx_to_f(q[2 * ((long long)wrapi(y + dy, p.ny) * p.nx + wrapi(x + dx, p.nx))]);
-        });
-    }
-    const long long in = (long long)y * p.nx + x;
-    int2 m[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) m[i] = reinterpret_cast<const int2*>(state)[(4LL * z + i) * p.nxny + in];
-    float u[3] = {p.u[0], p.u[1], p.u[2]};
-    if (p.uf)
-        for (int i = 0; i < 3; ++i) u[i] = p.uf[i * p.N + z * p.nxny + in];
-    const Collision r = collide<true>(p, m, pl[0], pl[1], pl[2], u);
-    uint2 v[Q27], moved = make_uint2(0u, 0u);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        auto row = [&](int c, uint2 total, uint2 v1, uint2 v2) {
-            const int q = 3 * b + 9 * c;
-            v[q] = total - v1 - v2;
-            v[q + 1] = v1;
-            v[q + 2] = v2;
-            moved = moved + (q ? total : v1 + v2);
-        };
-        if (p.uf)
-            emit_rows<true, true>(p, r, b, row);
-        else
-            emit_rows<false, true>(p, r, b, row);
-    }
-    v[0] = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
-    if (!r.ok) v[0] = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
-#pragma unroll
-    for (int q = 0; q < Q27; ++q) out(q, (int)v[q].x, (int)v[q].y);
-}
-
-__device__ __forceinline__ int vel(int a) { return a == 0 ? 0 : a == 1 ? 1 : -1; }
 
 // phi and c of a cell from its 27 incoming populations (NaN where one is
 // FX_BAD): of the initial fields (prev null), or sent by the state before.

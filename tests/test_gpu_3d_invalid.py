@@ -76,3 +76,80 @@ def test_invalid_cells_stay_invalid(cells, which, field, launch):
     again.step(3)
     clean.step(3)
     assert np.array_equal(clean.fields()["phi"], again.fields()["phi"]) and clean.sums()["nonfinite"] == 0
+
+
+def collided(shape, pops, u, W, M, D):
+    """Outgoing f populations of a state in FP64, [27] arrays, and the length of grad phi."""
+    nx, ny, nz = shape
+    E = np.array([tuple(v) for v in lbm3.lbm3_velocities()])
+    f = pops["f"]
+    s = f.sum(0)
+    j = [(E[:, i, None, None, None] * f).sum(0) for i in range(3)]
+    w1 = {-1: 1 / 6, 0: 2 / 3, 1: 1 / 6}
+    g = [0.0, 0.0, 0.0]
+    for e in E:
+        v = np.roll(s, tuple(-e[::-1]), (0, 1, 2))
+        for i in range(3):
+            g[i] = g[i] + 3 * w1[e[0]] * w1[e[1]] * w1[e[2]] * e[i] * v
+    size = np.sqrt(sum(a * a for a in g))
+    theta = 4 / W * (1 - s) * s
+    k = []
+    for i in range(3):
+        a = j[i] - u[i] * s
+        k.append(a + (M * theta * g[i] / np.maximum(size, 1e-30) - a) / (3 * M + 0.5))
+    fac = []
+    for v in u:
+        t = 1 / 3 + v * v
+        fac.append(({0: 1 - t, 1: (t + v) / 2, -1: (t - v) / 2}, {0: -2 * v, 1: v + 0.5, -1: v - 0.5},
+                    {0: 1 - v * v, 1: (v * v + v) / 2, -1: (v * v - v) / 2}))
+    (Ax, Bx, Cx), (Ay, By, Cy), (Az, Bz, Cz) = fac
+    return E, s, size, np.array([s * Ax[a] * Ay[b] * Az[c] + k[0] * Bx[a] * Cy[b] * Cz[c] + k[1] * Cx[a] * By[b] * Cz[c]
+                                 + k[2] * Cx[a] * Cy[b] * Bz[c] for a, b, c in E])
+
+
+@pytest.mark.parametrize("launch", [None, (6, 4), (10, 3), (18, 9)])
+def test_populations_that_leave_the_range(launch):
+    """phi = 1 (no interface flux) in a diverging velocity, W = 0.004: in the second
+    step theta reaches 80 and |k'| 23.  A population below -8 is invalid, one above 8
+    is cut off, whatever its velocity.  FP32 normals: phi to 2^-24, its gradient
+    above 1e-3, so k' to 23 * 4 * 2^-24 / 1e-3 = 6e-3 and populations to 1e-2."""
+    shape = nx, ny, nz = 34, 21, 9
+    Z, Y, X = np.meshgrid(np.arange(nz) + 0.5, np.arange(ny) + 0.5, np.arange(nx) + 0.5, indexing="ij")
+    wave = 2 * np.pi * (X / nx + Y / ny + Z / nz)
+    u = (0.1 * np.sin(2 * np.pi * X / nx), 0.1 * np.sin(2 * np.pi * Y / ny + 1.0), 0.05 * np.sin(wave))
+    phi, c = np.full((nz, ny, nx), 1.0), np.full((nz, ny, nx), 0.001)
+    W, M, D = 0.004, 1.0, 0.08
+    g = lbm3.Sim3(nx, ny, nz, W=W, M_phi=M, D_s=D, velocity_field=True)
+    g.init(phi, c, *u)
+    if launch:
+        lbm3.lbm3_set_launch_shape(g.ctx, *launch)
+    g.step(1)
+    E, s, size, want = collided(shape, g.pops(), u, W, M, D)
+    g.step(1)
+    got, f, sums = g.pops(), g.fields(), g.sums()
+    sent = np.array([np.roll(got["f"][q], tuple(-E[q][::-1]), (0, 1, 2)) for q in range(27)])
+    clear = size > 1e-3
+    assert clear.mean() > 0.8
+    low = high = still = 0
+    for q in range(27):
+        if not E[q].any():
+            continue
+        at = clear & (want[q] < -8 - 1e-2)
+        assert np.isnan(sent[q][at]).all()
+        low, still = low + at.sum(), still + (at.sum() if E[q][0] == 0 else 0)
+        at = clear & (want[q] > 8 + 1e-2)
+        assert (sent[q][at] == 8 - 2.0 ** -28).all()
+        high = high + at.sum()
+        at = clear & (np.abs(want[q]) < 8 - 1e-2)
+        assert np.abs(sent[q][at] - want[q][at]).max() < 1e-2
+    assert low > 200 and high > 200 and still > 200  # 326, 267 and 308 in FP64
+    # the rest population takes the remainder, modulo the range
+    left = (np.where(np.isnan(sent), -8.0, sent).sum(0) - s) / 16
+    assert (left == np.round(left)).all()
+    bad = np.isnan(got["f"]).any(0)
+    assert np.array_equal(np.isnan(f["phi"]), bad) and not np.isnan(f["c"]).any()
+    assert np.array_equal(f["phi"][~bad], got["f"].sum(0)[~bad]) and np.array_equal(f["c"], got["h"].sum(0))
+    assert sums["nonfinite"] == np.isnan(got["f"]).sum() and sums["sum_phi"] == np.nansum(got["f"])
+    # a cell that received one is invalid from then on
+    g.step(1)
+    assert np.isnan(g.fields()["phi"][spread(bad)]).all() and np.isnan(g.fields()["c"][spread(bad)]).all()
