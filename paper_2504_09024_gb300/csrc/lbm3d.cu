@@ -33,12 +33,15 @@
 // populations; a single population below -8 is FX_BAD too, and one above 8 is cut
 // off there.  A cell that receives FX_BAD gets it as its zeroth moment, so it
 // is out of range in turn.  (The sums do not say so by themselves: an even number
-// of FX_BAD adds up to nothing.)  Populations are formed again when they are asked for: those of
-// the state from the moments one step back (the other buffer), those of the
-// initial state from the fields it was made of, which the context keeps.  The
-// sums alone say phi, c and the totals, unless a population may have been out
-// of range; the step that saw such a cell raises the context's `wild` word,
-// and the outputs then look at every population.
+// of FX_BAD adds up to nothing.)
+//
+// Outputs.  phi and c are the zeroth moments.  Populations are formed again when
+// they are asked for: those of the state from the moments one step back (the other
+// buffer), those of the initial state from the fields it was made of, which the
+// context keeps.  A step writes its number into the `suspect` word of every plane
+// with a cell that is not certain to stay in range (Collision::tame): next to such a
+// plane the sums may have wrapped around, and in it populations may be invalid, so
+// there, and only there, fields and totals look at populations.
 //
 // Step kernel.  A block owns a 30 x (ROWS - 2) column of cells with a one-cell
 // halo (one warp per row of 32 columns) and marches through seg_z planes.  At
@@ -88,7 +91,6 @@ constexpr double FX_ONE_D = 268435456.0;
 constexpr double FX_INV_D = 1.0 / 268435456.0;
 constexpr int FX_BAD = (-2147483647 - 1);       // invalid population marker
 constexpr float S_MAX = 4.0f;                   // valid |zeroth moment|
-constexpr float K_TAME = 0.3f * FX_ONE;         // sum of |k'| up to which no population leaves the range
 constexpr int SUM_BLOCKS = 1024;
 constexpr int SUM_THREADS = 256;
 
@@ -108,6 +110,8 @@ struct K3Params {
     // both lanes
     float2 fx[4], aa[3][3], cc[3][3], bc[3][3], cb[3][3];
     const float* uf;  // per-cell velocity [3][N], or null for the uniform u
+    long long number;    // of the state that is written or read: steps since the initial one
+    long long* suspect;  // [nz + 1]: the last state that senders of a plane made suspect; of any plane
 };
 
 __host__ __device__ __forceinline__ int wrapi(int v, int n) {
@@ -178,6 +182,13 @@ __device__ __forceinline__ Plane plane_of(At at) {
                  __fsub_rn(m[2], m[0])};
 }
 
+// The largest magnitude (NaN if one is NaN).
+__device__ __forceinline__ float most_of(float a, float b, float c) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(fabsf(c)));
+    return r;
+}
+
 // A collision of both lattices (lane x: f, lane y: h), in fixed-point units:
 // zeroth moments, relaxed first-order central moments and the velocity.  Every
 // operation is written out (no contraction left to the compiler), so that the
@@ -186,12 +197,15 @@ struct Collision {
     int2 s_fx;
     f2 s, k[3];
     float u[3];
-    float most, big, fast;  // the larger |s|, the sum of |k'| and (velocity field) the largest |u|
-    bool ok;    // both zeroth moments inside (-4, 4)
-    bool tame;  // no population can leave the fixed-point range, nor their sums 32 bits
-    // ok, and no population can leave the range: |A| <= 1.17, |B| <= 2 and |C| <= 1 up to |u| = 1
+    float most, big, fast;  // the larger |s|, the largest |k'| and (velocity field) the largest |u|
+    bool tame;  // safe(), nor can the sums of what such cells send leave 32 bits
+    // both zeroth moments inside (-4, 4)
+    __device__ __forceinline__ bool ok() const { return most < S_MAX * FX_ONE; }
+    // and no population can leave the range: |A| <= 0.67, |B| <= 1 and |C| <= 1 up to |u| = 1/2,
+    // 1.17, 2 and 1 up to |u| = 1
     __device__ __forceinline__ bool safe() const {
-        return ok && fast <= 1.0f && __fmaf_rn(1.6f, most, 2.0f * big) < 7.9f * FX_ONE;
+        const bool half = fast <= 0.5f;
+        return ok() && fast <= 1.0f && __fmaf_rn(half ? 0.3f : 1.6f, most, (half ? 3.0f : 6.0f) * big) < 7.9f * FX_ONE;
     }
 };
 
@@ -213,25 +227,25 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
     const float thetac = __fmul_rn(__fmul_rn(__fmul_rn(p.c8W, c), __fsub_rn(p.phim, phi)), p.inv_dphi);
     const f2 q(__fmul_rn(p.M_phi, theta) * FX_ONE, __fmul_rn(p.D_s, thetac) * FX_ONE);
     const f2 w(p.w_kappa, p.w_chi);
-    float big = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const f2 a = lbm::vfma(f2(-u[i]), r.s, f2((float)m[i + 1].x, (float)m[i + 1].y));
         r.u[i] = u[i];
         r.k[i] = lbm::vfma(w, lbm::vfma(q, f2(__fmul_rn(g[i], inv)), -a), a);
-        big += fabsf(r.k[i].x) + fabsf(r.k[i].y);  // NaN stays NaN
     }
-    r.ok = valid(m[0]);
     r.most = fmaxf(fabsf(r.s.x), fabsf(r.s.y));
-    r.big = big;
-    r.fast = UFIELD ? fmaxf(fmaxf(fabsf(u[0]), fabsf(u[1])), fabsf(u[2])) : 0.f;
-    // Uniform |u| < 1/2: over the 27 neighbours the A products add up to 1 and those of
-    // B and C to at most 3.2 a component, so |sum| < 4 + 3.2 * 0.3.  A field with
-    // |u| <= 1/4, each neighbour its own: 2.3 and 3.5, so |sum| < 2 * 2.3 + 3.5 * 0.3.
-    r.tame = r.ok && big < K_TAME;
-    if (UFIELD)
-        r.tame = r.tame && fmaxf(fabsf(phi), fabsf(c)) < 2.0f &&
-                 fmaxf(fmaxf(fabsf(u[0]), fabsf(u[1])), fabsf(u[2])) <= 0.25f;
+    r.big = most_of(most_of(most_of(r.k[0].x, r.k[0].y, r.k[1].x), r.k[1].y, r.k[2].x), r.k[2].y, 0.f);
+    r.fast = UFIELD ? most_of(u[0], u[1], u[2]) : 0.f;
+    // What the 27 neighbours of a cell send it adds up to less than 8.  Uniform |u| < 1/2: the
+    // products of A add up to 1 and those of B and C to less than 3.2 a component, 4 + 3 * 3.2 *
+    // 0.4.  A field, where each neighbour has its own u and is of one kind or the other: 7.84, each
+    // product at its largest (test_range_bounds3.py).
+    if constexpr (UFIELD) {
+        const bool slow = r.fast <= 0.2f;
+        r.tame = r.fast <= 0.4f && r.most < (slow ? 2.1f : 1.1f) * FX_ONE && r.big < (slow ? 0.3f : 0.15f) * FX_ONE;
+    } else {
+        r.tame = r.ok() && r.big < 0.4f * FX_ONE;
+    }
     return r;
 }
 
@@ -291,7 +305,7 @@ __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r,
         }
         const f2 W = P + R, O = lbm::vfma(W, uh, X), E = lbm::vfma(P, th, lbm::vfma(X, u2x, R * uh2));
         auto grid = [&](f2 v) {
-            return CHECK && !r.ok ? make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD)
+            return CHECK && !r.ok() ? make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD)
                                   : make_uint2((uint32_t)__float2int_rn(v.x), (uint32_t)__float2int_rn(v.y));
         };
         const uint2 v1 = grid(E + O), v2 = grid(E - O);
@@ -369,7 +383,7 @@ __device__ __forceinline__ void outgoing(const K3Params& p, const int* __restric
             emit_rows<false, true>(p, r, b, row);
     }
     v[0] = make_uint2((uint32_t)r.s_fx.x, (uint32_t)r.s_fx.y) - moved;
-    if (!r.ok) v[0] = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
+    if (!r.ok()) v[0] = make_uint2((uint32_t)FX_BAD, (uint32_t)FX_BAD);
 #pragma unroll
     for (int q = 0; q < Q27; ++q) out(q, (int)v[q].x, (int)v[q].y);
 }
@@ -418,8 +432,7 @@ __device__ __noinline__ void settle_invalid(const K3Params& p, const int* __rest
 
 template <int ROWS, bool UFIELD>
 __global__ void __launch_bounds__(ROWS * 32, k3_min_blocks<ROWS>())
-k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __restrict__ dst,
-        int* __restrict__ wild) {
+k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __restrict__ dst) {
     extern __shared__ __align__(16) float smem[];
     constexpr int RING = k3_ring_words<ROWS>(), XCHG = k3_xchg_words<ROWS>(), NT = ROWS * 32;
     constexpr int PLANE = ROWS * TILE_W;
@@ -544,8 +557,8 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
                 d0[0] = r1 - r2;
             }
             if (!r.tame) {
-                *wild = 1;
-                if (!r.ok) met_invalid = 1;
+                p.suspect[wrapi(k, p.nz)] = p.suspect[p.nz] = p.number;
+                if (!r.ok()) met_invalid = 1;
                 else if (!r.safe()) met_single = 1;
             }
         }
@@ -645,7 +658,7 @@ __device__ __forceinline__ void equilibrium(const K3Params& p, const Seed& in, l
 
 // The state of the given fields, and a copy of the fields (see `Seed`).
 __global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state, double* __restrict__ keep,
-                        float* __restrict__ uf, int* __restrict__ wild) {
+                        float* __restrict__ uf) {
     const long long N = p.N;
     for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < N;
          cell += (long long)gridDim.x * blockDim.x) {
@@ -676,57 +689,67 @@ __global__ void k3_init(const K3Params p, const Seed in, int* __restrict__ state
         uint2* o = reinterpret_cast<uint2*>(state) + (cell / p.nxny) * 4 * p.nxny + cell % p.nxny;
 #pragma unroll
         for (int i = 0; i < 4; ++i) o[i * p.nxny] = m[i];
-        if (bad_f || bad_h) *wild = 1;
+        if (bad_f || bad_h) p.suspect[cell / p.nxny] = p.suspect[p.nz] = p.number;
     }
 }
 
-// phi and c of a cell from its 27 incoming populations (NaN where one is
-// FX_BAD): of the initial fields (prev null), or sent by the state before.
-__device__ __forceinline__ void fields_of_populations(const K3Params& p, const Seed& seed, const int* prev,
-                                                   long long cell, double* phi, double* c) {
-    long long sf = 0, sh = 0;
-    bool bf = false, bh = false;
-    auto add = [&](int f, int h) {
-        bf |= f == FX_BAD;
-        bh |= h == FX_BAD;
-        sf += f;
-        sh += h;
-    };
-    if (!prev) {
-        equilibrium(p, seed, cell, [&](int, int f, int h) { add(f, h); });
-    } else {
-        const int x = (int)(cell % p.nx), y = (int)((cell / p.nx) % p.ny), z = (int)(cell / p.nxny);
-        for (int want = 0; want < Q27; ++want)
-            outgoing(p, prev, wrapi(x - vel(want % 3), p.nx), wrapi(y - vel((want / 3) % 3), p.ny),
-                     wrapi(z - vel(want / 9), p.nz), [&](int q, int f, int h) {
-                         if (q == want) add(f, h);
-                     });
-    }
-    if (phi) phi[cell] = bf ? nan("") : (double)sf * FX_INV_D;
-    if (c) c[cell] = bh ? nan("") : (double)sh * FX_INV_D;
-}
-
-// phi and c of the state: exact integer sums, then FP64.
-__global__ void k3_fields(const K3Params p, const int* __restrict__ state, const int* __restrict__ wild,
-                          double* __restrict__ phi, double* __restrict__ c) {
-    if (*wild) return;
+// phi and c of the state: exact integer sums, then FP64 (NaN where a population is
+// FX_BAD).
+__global__ void k3_fields(const K3Params p, const int* __restrict__ state, double* __restrict__ phi,
+                          double* __restrict__ c) {
     const int nxny = (int)p.nxny;
     for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < p.N;
          cell += (long long)gridDim.x * blockDim.x) {
         const int2 s = reinterpret_cast<const int2*>(state)[cell + cell / nxny * 3 * nxny];
-        if (phi) phi[cell] = (double)s.x * FX_INV_D;
-        if (c) c[cell] = (double)s.y * FX_INV_D;
+        if (phi) phi[cell] = s.x == FX_BAD ? nan("") : (double)s.x * FX_INV_D;
+        if (c) c[cell] = s.y == FX_BAD ? nan("") : (double)s.y * FX_INV_D;
     }
 }
 
-// The same where a population may be invalid.  A kernel of its own: the code
-// that forms populations takes three times the registers.
-__global__ void k3_fields_wild(const K3Params p, const Seed seed, const int* prev, const int* __restrict__ wild,
-                               double* __restrict__ phi, double* __restrict__ c) {
-    if (!*wild) return;
-    for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < p.N;
-         cell += (long long)gridDim.x * blockDim.x)
-        fields_of_populations(p, seed, prev, cell, phi, c);
+// The same for the cells next to a suspect plane of `prev`, the state one step back,
+// whose sums may have wrapped around: multiples of 2^32 are added back.  The block
+// forms the populations of a tile and its halo once and adds them up coarsely, in
+// units of 2^6, which fits 32 bits; the state has the rest.
+constexpr int FT_X = 16, FT_Y = 8, FT_Z = 4, FT_N = FT_X * FT_Y * FT_Z;
+__global__ void __launch_bounds__(256) k3_fields_suspect(const K3Params p, const int* prev,
+                                                         const int* __restrict__ state, double* __restrict__ phi,
+                                                         double* __restrict__ c) {
+    if (p.suspect[p.nz] != p.number) return;
+    __shared__ int coarse[2][FT_N];
+    const int tiles_x = (p.nx + FT_X - 1) / FT_X, tiles_y = (p.ny + FT_Y - 1) / FT_Y, tiles_z = (p.nz + FT_Z - 1) / FT_Z;
+    for (long long tile = blockIdx.x; tile < (long long)tiles_x * tiles_y * tiles_z; tile += gridDim.x) {
+        const int x0 = (int)(tile % tiles_x) * FT_X, y0 = (int)(tile / tiles_x % tiles_y) * FT_Y,
+                  z0 = (int)(tile / tiles_x / tiles_y) * FT_Z;
+        const int plane = wrapi(z0 - 1 + (int)threadIdx.x, p.nz);
+        if (!__syncthreads_or(threadIdx.x < FT_Z + 2 && p.suspect[plane] == p.number)) continue;
+        for (int k = threadIdx.x; k < FT_N; k += 256) coarse[0][k] = coarse[1][k] = 0;
+        __syncthreads();
+        for (int k = threadIdx.x; k < (FT_X + 2) * (FT_Y + 2) * (FT_Z + 2); k += 256) {
+            const int lx = k % (FT_X + 2) - 1, ly = k / (FT_X + 2) % (FT_Y + 2) - 1, lz = k / (FT_X + 2) / (FT_Y + 2) - 1;
+            if (x0 + lx > p.nx || y0 + ly > p.ny || z0 + lz > p.nz) continue;
+            outgoing(p, prev, wrapi(x0 + lx, p.nx), wrapi(y0 + ly, p.ny), wrapi(z0 + lz, p.nz), [&](int q, int f, int h) {
+                const int rx = lx + vel(q % 3), ry = ly + vel((q / 3) % 3), rz = lz + vel(q / 9);
+                if (rx < 0 || rx >= FT_X || ry < 0 || ry >= FT_Y || rz < 0 || rz >= FT_Z) return;
+                const int at = (rz * FT_Y + ry) * FT_X + rx;
+                atomicAdd(&coarse[0][at], f >> 6);
+                atomicAdd(&coarse[1][at], h >> 6);
+            });
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < FT_N; k += 256) {
+            const int x = x0 + k % FT_X, y = y0 + k / FT_X % FT_Y, z = z0 + k / FT_X / FT_Y;
+            if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
+            const long long at = (long long)y * p.nx + x, cell = z * p.nxny + at;
+            const int2 s = reinterpret_cast<const int2*>(state)[4 * p.nxny * z + at];
+            // 27 populations lose less than 27 * 2^6 to the coarse units
+            auto whole = [](int sum, int in64) {
+                return (double)(sum + (((64LL * in64 - sum + 0xffffffffLL) >> 32) << 32)) * FX_INV_D;
+            };
+            if (phi && s.x != FX_BAD) phi[cell] = whole(s.x, coarse[0][k]);
+            if (c && s.y != FX_BAD) c[cell] = whole(s.y, coarse[1][k]);
+        }
+        __syncthreads();
+    }
 }
 
 // The state's populations as float64 [27][N] (NaN for FX_BAD): of the initial
@@ -768,21 +791,22 @@ __device__ __noinline__ void totals_of_populations(const K3Params& p, const Seed
 
 // Totals: sum f, sum h (exact, in integer units) and the FX_BAD count of the
 // state's populations (streaming is a permutation: those sent are those that
-// arrived).  Fixed grid and reduction order.
+// arrived, and a cell's add up to its zeroth moment unless its plane is suspect).
+// Fixed grid and reduction order.
 __global__ void __launch_bounds__(SUM_THREADS) k3_sum1(const K3Params p, const Seed seed,
                                                        const int* __restrict__ state, const int* prev,
-                                                       const int* __restrict__ wild,
                                                        long long* __restrict__ partial) {
     long long sf = 0, sh = 0, bad = 0;
-    const bool each = *wild != 0;
     const int nxny = (int)p.nxny;
+    const int* sent = prev ? prev : state;
     for (long long cell = blockIdx.x * (long long)SUM_THREADS + threadIdx.x; cell < p.N;
          cell += (long long)SUM_BLOCKS * SUM_THREADS) {
-        if (each) {
+        const long long z = cell / nxny;
+        if (p.suspect[z] == p.number) {
             totals_of_populations(p, seed, prev, cell, sf, sh, bad);
             continue;
         }
-        const int2 s = reinterpret_cast<const int2*>(state)[cell + cell / nxny * 3 * nxny];
+        const int2 s = reinterpret_cast<const int2*>(sent)[cell + z * 3 * nxny];
         sf += s.x;
         sh += s.y;
     }
@@ -826,7 +850,7 @@ struct lbm3_ctx {
     int* buf[2] = {nullptr, nullptr};    // states, [nz][4][ny][nx][2] fixed point: now and one step back
     float* uf = nullptr;                 // [3][N] prescribed velocity (velocity_field = 1)
     double* keep = nullptr;              // the initial fields, [2][N] or [5][N] with the velocity
-    int* wild = nullptr;                 // a population may have been out of range since the last init
+    long long* suspect = nullptr;        // see K3Params
     long long* partial = nullptr;        // 3 x SUM_BLOCKS partial sums
     double* result = nullptr;            // 3 totals
     int cur = 0;
@@ -855,6 +879,13 @@ Seed seed_of(const lbm3_ctx* ctx) {
     return s;
 }
 
+// The parameters of a kernel that reads the state.
+K3Params of_state(const lbm3_ctx* ctx) {
+    K3Params p = ctx->kp;
+    p.number = ctx->step;
+    return p;
+}
+
 // The state one step back, or null if the state is the initial one.
 const int* before(const lbm3_ctx* ctx) { return ctx->step ? ctx->buf[1 - ctx->cur] : nullptr; }
 
@@ -876,13 +907,14 @@ int launch_step(lbm3_ctx* ctx) {
     const K3Params& kp = ctx->kp;
     K3Params p = kp;
     p.seg_z = ctx->seg_z;
+    p.number = ctx->step + 1;
     const int rows = ctx->rows;
     dim3 grid((kp.nx + TILE_IN - 1) / TILE_IN, (kp.ny + rows - 3) / (rows - 2),
               (kp.nz + ctx->seg_z - 1) / ctx->seg_z);
     const int src = ctx->cur, dst = 1 - ctx->cur;
     const bool field = kp.uf != nullptr;
     auto go = [&](auto kern, int smem) {
-        kern<<<grid, rows * 32, smem, ctx->stream>>>(p, ctx->buf[src], ctx->buf[dst], ctx->wild);
+        kern<<<grid, rows * 32, smem, ctx->stream>>>(p, ctx->buf[src], ctx->buf[dst]);
     };
     switch (rows) {
         case 6:
@@ -1016,14 +1048,15 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
     const size_t keep_bytes = sizeof(double) * (p->velocity_field ? 5 : 2) * (size_t)kp.N;
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&ctx->buf[i], state_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->keep, keep_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->wild, sizeof(int));
+    const size_t suspect_bytes = sizeof(long long) * ((size_t)p->nz + 1);
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->suspect, suspect_bytes);
     if (e == cudaSuccess && p->velocity_field) e = cudaMalloc(&ctx->uf, sizeof(float) * 3 * (size_t)kp.N);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->partial, sizeof(long long) * 3 * SUM_BLOCKS);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->result, sizeof(double) * 3);
     // defined contents before the first init (the autotuner may step them)
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMemsetAsync(ctx->buf[i], 0, state_bytes, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->keep, 0, keep_bytes, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->wild, 0, sizeof(int), ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->suspect, 0xff, suspect_bytes, ctx->stream);
     if (e == cudaSuccess && ctx->uf) e = cudaMemsetAsync(ctx->uf, 0, sizeof(float) * 3 * (size_t)kp.N, ctx->stream);
     const bool field = p->velocity_field != 0;
     if (e == cudaSuccess) e = allow_smem<6>(field);
@@ -1036,6 +1069,7 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
         return rc;
     }
     kp.uf = ctx->uf;
+    kp.suspect = ctx->suspect;
     *out = ctx;
     return LBM_OK;
 }
@@ -1046,7 +1080,7 @@ void lbm3_destroy(lbm3_ctx* ctx) {
     for (int i = 0; i < 2; ++i) cudaFree(ctx->buf[i]);
     cudaFree(ctx->uf);
     cudaFree(ctx->keep);
-    cudaFree(ctx->wild);
+    cudaFree(ctx->suspect);
     cudaFree(ctx->partial);
     cudaFree(ctx->result);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
@@ -1066,12 +1100,12 @@ int lbm3_init_fields_device(lbm3_ctx* ctx, const double* phi, const double* c, c
         in.u[1] = uy;
         in.u[2] = uz;
     }
-    const cudaError_t e = cudaMemsetAsync(ctx->wild, 0, sizeof(int), ctx->stream);
+    const cudaError_t e =
+        cudaMemsetAsync(ctx->suspect, 0xff, sizeof(long long) * ((size_t)ctx->kp.nz + 1), ctx->stream);
     if (e != cudaSuccess) return fail(ctx, e);
     ctx->cur = 0;
-    k3_init<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, in, ctx->buf[0], ctx->keep, ctx->uf,
-                                                              ctx->wild);
     ctx->step = 0;
+    k3_init<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(of_state(ctx), in, ctx->buf[0], ctx->keep, ctx->uf);
     return fail(ctx, cudaGetLastError());
 }
 
@@ -1112,9 +1146,11 @@ int lbm3_step(lbm3_ctx* ctx, int64_t nsteps) {
 int lbm3_get_fields_device(lbm3_ctx* ctx, double* phi, double* c) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     if (!phi && !c) return LBM_OK;
-    k3_fields<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, ctx->buf[ctx->cur], ctx->wild, phi, c);
-    k3_fields_wild<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), before(ctx), ctx->wild,
-                                                                      phi, c);
+    const K3Params p = of_state(ctx);
+    k3_fields<<<grid_1d(p.N, 256), 256, 0, ctx->stream>>>(p, ctx->buf[ctx->cur], phi, c);
+    if (before(ctx))
+        k3_fields_suspect<<<grid_1d((p.N + 1) / 2, 256), 256, 0, ctx->stream>>>(p, before(ctx), ctx->buf[ctx->cur], phi,
+                                                                               c);
     return fail(ctx, cudaGetLastError());
 }
 
@@ -1157,8 +1193,8 @@ int lbm3_get_populations(lbm3_ctx* ctx, double* f, double* h) {
 
 int lbm3_sums(lbm3_ctx* ctx, double out[3]) {
     if (!ctx || !out) return LBM_ERR_INVALID_ARG;
-    k3_sum1<<<SUM_BLOCKS, SUM_THREADS, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), ctx->buf[ctx->cur], before(ctx),
-                                                         ctx->wild, ctx->partial);
+    k3_sum1<<<SUM_BLOCKS, SUM_THREADS, 0, ctx->stream>>>(of_state(ctx), seed_of(ctx), ctx->buf[ctx->cur],
+                                                         before(ctx), ctx->partial);
     k3_sum2<<<1, SUM_THREADS, 0, ctx->stream>>>(ctx->partial, ctx->result);
     int rc = fail(ctx, cudaGetLastError());
     if (rc == LBM_OK)

@@ -153,3 +153,59 @@ def test_populations_that_leave_the_range(launch):
     # a cell that received one is invalid from then on
     g.step(1)
     assert np.isnan(g.fields()["phi"][spread(bad)]).all() and np.isnan(g.fields()["c"][spread(bad)]).all()
+
+
+def timed(nx, u, spike=False):
+    """us of phi and c into device arrays after two steps with a velocity field of size u."""
+    import torch
+    z = torch.arange(nx, dtype=torch.float64, device="cuda") + 0.5 - nx / 2
+    r = torch.sqrt(z[:, None, None] ** 2 + z[None, :, None] ** 2 + z[None, None, :] ** 2)
+    zeta = nx / 4 - r
+    phi, c = 0.5 + 0.5 * torch.tanh(zeta / 2), 0.3 / torch.cosh(zeta / 2) ** 2
+    if spike:
+        phi[nx // 3, 5, 7] = 5.0
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        stream.wait_stream(torch.cuda.default_stream())
+        g = lbm3.Sim3(nx, nx, nx, W=4.0, M_phi=0.05, D_s=0.08, velocity_field=True, stream=stream.cuda_stream)
+        lbm3.lbm3_init_fields_device(g.ctx, phi, c, *(torch.full_like(phi, v) for v in (u, -u, 0.0)))
+        g.step(2)
+        out = torch.empty((2,) + phi.shape, dtype=torch.float64, device="cuda")
+        best = 1e30
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            lbm3.lbm3_get_fields_device(g.ctx, out[0], out[1])
+            b.record()
+            b.synchronize()
+            best = min(best, 1e3 * a.elapsed_time(b))
+    g.sums()
+    g.close()
+    return best
+
+
+def test_outputs_of_fast_and_of_partly_invalid_runs_stay_cheap():
+    """Populations are formed again only next to planes that call for it, and then once
+    each: a velocity of 0.35 costs nothing, one invalid cell three planes of 128, and a
+    velocity that no bound holds for (0.7) the populations of every cell once."""
+    usual = timed(128, 0.05)
+    assert timed(128, 0.35) < 3 * usual
+    assert timed(128, 0.05, spike=True) < 5 * usual
+    assert timed(128, 0.7) < 60 * usual
+
+
+@pytest.mark.parametrize("shape", [(5, 5, 5), (33, 17, 9), (16, 8, 4)])
+def test_sums_of_populations_that_leave_32_bits(shape):
+    """A converging velocity of 0.45 where c is 3.9: the populations that meet in a
+    cell are in range and their sum is not; c is the sum all the same."""
+    nx, ny, nz = shape
+    Z, Y, X = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    u = tuple(-0.45 * np.sign(a - n // 2) for a, n in ((X, nx), (Y, ny), (Z, nz)))
+    phi, c = np.full((nz, ny, nx), 0.5), np.full((nz, ny, nx), 3.9)
+    g = lbm3.Sim3(nx, ny, nz, W=4.0, M_phi=0.05, D_s=0.08, velocity_field=True)
+    g.init(phi, c, *u)
+    g.step(1)
+    f, p, s = g.fields(), g.pops(), g.sums()
+    assert f["c"].max() > 10.0
+    assert np.array_equal(f["c"], p["h"].sum(0)) and np.array_equal(f["phi"], p["f"].sum(0))
+    assert s["sum_c"] == p["h"].sum() and s["nonfinite"] == 0
