@@ -68,6 +68,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -949,10 +950,11 @@ void default_shape(const lbm3_params* p, int* rows, int* seg_z) {
     double best = -1.0;
     for (int r : {10, 18}) {
         const long long tiles = (long long)((p->nx + TILE_IN - 1) / TILE_IN) * ((p->ny + r - 3) / (r - 2));
-        for (int n = 1; n <= p->nz; ++n) {
-            const int seg = (p->nz + n - 1) / n;
-            if (n > 1 && seg == (p->nz + n - 2) / (n - 1)) continue;
-            const long long blocks = tiles * ((p->nz + seg - 1) / seg), per_sm = (blocks + 151) / 152;
+        // the distinct heights of nz planes in n segments, each with its smallest n (about
+        // 2 sqrt(nz) of them)
+        for (int n = 1, seg = 0; seg != 1; n = (int)((seg - 2LL + p->nz) / std::max(seg - 1, 1))) {
+            seg = (int)((n - 1LL + p->nz) / n);
+            const long long blocks = tiles * ((seg - 1LL + p->nz) / seg), per_sm = (blocks + 151) / 152;
             const double load = r == 18 ? 1.45 * (double)per_sm : second * (double)(per_sm / 2) + (double)(per_sm % 2);
             const double cost = load * (seg + 3);
             if (best < 0.0 || cost < best) {
