@@ -60,7 +60,7 @@ extern "C" {
 #endif
 
 /* nx * ny * nz may not exceed this (2^30 cells need 86 GB of the GPU's memory,
- * 129 GB with a velocity field), and 27 * nx * ny must stay below 2^31 (offsets
+ * 125 GB with a velocity field), and 27 * nx * ny must stay below 2^31 (offsets
  * inside a plane are 32-bit). */
 #define LBM3_MAX_CELLS 1073741824LL
 

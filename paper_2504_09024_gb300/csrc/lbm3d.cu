@@ -855,6 +855,7 @@ struct lbm3_ctx {
     long long* partial = nullptr;        // 3 x SUM_BLOCKS partial sums
     double* result = nullptr;            // 3 totals
     int cur = 0;
+    int sms = 1;
     int rows = 10, seg_z = 64;
     int64_t step = 0;
     int pending_error = LBM_OK;
@@ -890,9 +891,17 @@ K3Params of_state(const lbm3_ctx* ctx) {
 // The state one step back, or null if the state is the initial one.
 const int* before(const lbm3_ctx* ctx) { return ctx->step ? ctx->buf[1 - ctx->cur] : nullptr; }
 
-int grid_1d(long long n, int threads) {
-    long long b = (n + threads - 1) / threads;
-    return (int)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
+int grid_1d(const lbm3_ctx* ctx, long long n, int threads) {
+    const long long b = (n + threads - 1) / threads;
+    return (int)std::min(std::max(b, 1LL), 16LL * ctx->sms);
+}
+
+int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();  // (creating the context will report it)
+    return n > 0 ? n : 1;
 }
 
 // Shared memory above 48 KB has to be asked for, once per kernel and device.
@@ -945,7 +954,7 @@ int launch_step(lbm3_ctx* ctx) {
 // Measured, us per step at the best segments of 18 / 10 rows: uniform velocity
 // 256^3 504 / 485, 150x97x61 39 / 39, 64x50x40 16.5 / 14.5; velocity field 256^3
 // 655 / 788, 220x200x180 356 / 398, 150x97x61 49 / 49.
-void default_shape(const lbm3_params* p, int* rows, int* seg_z) {
+void default_shape(const lbm3_params* p, int sms, int* rows, int* seg_z) {
     const double second = p->velocity_field ? 1.75 : 1.45;
     double best = -1.0;
     for (int r : {10, 18}) {
@@ -954,7 +963,7 @@ void default_shape(const lbm3_params* p, int* rows, int* seg_z) {
         // 2 sqrt(nz) of them)
         for (int n = 1, seg = 0; seg != 1; n = (int)((seg - 2LL + p->nz) / std::max(seg - 1, 1))) {
             seg = (int)((n - 1LL + p->nz) / n);
-            const long long blocks = tiles * ((seg - 1LL + p->nz) / seg), per_sm = (blocks + 151) / 152;
+            const long long blocks = tiles * ((seg - 1LL + p->nz) / seg), per_sm = (blocks + sms - 1) / sms;
             const double load = r == 18 ? 1.45 * (double)per_sm : second * (double)(per_sm / 2) + (double)(per_sm % 2);
             const double cost = load * (seg + 3);
             if (best < 0.0 || cost < best) {
@@ -1038,7 +1047,8 @@ int lbm3_create(const lbm3_params* p, void* stream, lbm3_ctx** out) {
             kp.cb[c][b] = both(fac[1][2][b] * fac[2][1][c]);
         }
     kp.uf = nullptr;
-    default_shape(p, &ctx->rows, &ctx->seg_z);
+    ctx->sms = sm_count();
+    default_shape(p, ctx->sms, &ctx->rows, &ctx->seg_z);
     cudaError_t e = cudaSuccess;
     if (stream) {
         ctx->stream = (cudaStream_t)stream;
@@ -1107,7 +1117,7 @@ int lbm3_init_fields_device(lbm3_ctx* ctx, const double* phi, const double* c, c
     if (e != cudaSuccess) return fail(ctx, e);
     ctx->cur = 0;
     ctx->step = 0;
-    k3_init<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(of_state(ctx), in, ctx->buf[0], ctx->keep, ctx->uf);
+    k3_init<<<grid_1d(ctx, ctx->kp.N, 256), 256, 0, ctx->stream>>>(of_state(ctx), in, ctx->buf[0], ctx->keep, ctx->uf);
     return fail(ctx, cudaGetLastError());
 }
 
@@ -1149,9 +1159,9 @@ int lbm3_get_fields_device(lbm3_ctx* ctx, double* phi, double* c) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     if (!phi && !c) return LBM_OK;
     const K3Params p = of_state(ctx);
-    k3_fields<<<grid_1d(p.N, 256), 256, 0, ctx->stream>>>(p, ctx->buf[ctx->cur], phi, c);
+    k3_fields<<<grid_1d(ctx, p.N, 256), 256, 0, ctx->stream>>>(p, ctx->buf[ctx->cur], phi, c);
     if (before(ctx))
-        k3_fields_suspect<<<grid_1d((p.N + 1) / 2, 256), 256, 0, ctx->stream>>>(p, before(ctx), ctx->buf[ctx->cur], phi,
+        k3_fields_suspect<<<grid_1d(ctx, (p.N + 1) / 2, 256), 256, 0, ctx->stream>>>(p, before(ctx), ctx->buf[ctx->cur], phi,
                                                                                c);
     return fail(ctx, cudaGetLastError());
 }
@@ -1174,7 +1184,7 @@ int lbm3_get_fields(lbm3_ctx* ctx, double* phi, double* c) {
 int lbm3_get_populations_device(lbm3_ctx* ctx, double* f, double* h) {
     if (!ctx) return LBM_ERR_INVALID_ARG;
     if (!f && !h) return LBM_OK;
-    k3_pops<<<grid_1d(ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), before(ctx), f, h);
+    k3_pops<<<grid_1d(ctx, ctx->kp.N, 256), 256, 0, ctx->stream>>>(ctx->kp, seed_of(ctx), before(ctx), f, h);
     return fail(ctx, cudaGetLastError());
 }
 
