@@ -303,7 +303,8 @@ lbm_ctx *lbm_batch_run(lbm_batch *b, int32_t run);
 int lbm_batch_step(lbm_batch *b, int64_t nsteps);
 
 /* Wait for the batch stream; reports a pending CUDA error or an expired
- * bounded wait (LBM_ERR_TIMEOUT) of a batched step. */
+ * bounded wait (LBM_ERR_TIMEOUT) of a batched step or of a call on one of the
+ * batch's runs. */
 int lbm_batch_synchronize(lbm_batch *b);
 
 /* Form of the batched step (LBM_BATCH_PERSISTENT, the default, or

@@ -66,7 +66,8 @@ struct lbm_ctx {
     int st = lbm::ST_F32;
     float* pop16_alloc[2] = {nullptr, nullptr};
     unsigned* dstep = nullptr;  // step counter of the stochastic roundings
-    int* derr = nullptr;    // device flag: a bounded wait expired
+    int* derr = nullptr;    // device flag: a bounded wait expired (a batch's run: one of the batch's)
+    bool own_err = true;    // derr is this context's to free
     int pending_error = LBM_OK;
 };
 
@@ -499,7 +500,7 @@ void lbm_destroy(lbm_ctx* ctx) {
     cudaFree(ctx->stage);
     cudaFree(ctx->dwords);
     cudaFree(ctx->dresult);
-    cudaFree(ctx->derr);
+    if (ctx->own_err) cudaFree(ctx->derr);
     cudaFree(ctx->pop16_alloc[0]);
     cudaFree(ctx->pop16_alloc[1]);
     cudaFree(ctx->dstep);
@@ -912,7 +913,8 @@ struct lbm_batch {
     int dev = 0;                        // the device the batch was created on
     unsigned** dctrs = nullptr;         // the runs' step counters (device array)
     lbm::KParams* hkp = nullptr;        // the runs' parameters the graphs were built with
-    int* derr = nullptr;
+    int* derr = nullptr;                // flags: of the batched steps, then of every run (1 + nruns)
+    int* herr = nullptr;                // host copy
     int parity = 0;
     bool desc_valid = false;
     cudaGraphExec_t graph[GRAPH_CHUNKS][2] = {};
@@ -1199,7 +1201,8 @@ int lbm_batch_create(const lbm_params* params, int32_t nruns, void* stream, lbm_
     b->hdesc = (lbm::RunDesc*)std::calloc((size_t)nruns, sizeof(lbm::RunDesc));
     b->hkp = (lbm::KParams*)std::calloc((size_t)nruns, sizeof(lbm::KParams));
     b->htab = (lbm::BatchTable*)std::calloc((size_t)b->ntab, sizeof(lbm::BatchTable));
-    if (!b->runs || !b->hdesc || !b->hkp || !b->htab) {
+    b->herr = (int*)std::calloc((size_t)nruns + 1, sizeof(int));
+    if (!b->runs || !b->hdesc || !b->hkp || !b->htab || !b->herr) {
         lbm_batch_destroy(b);
         return LBM_ERR_NOMEM;
     }
@@ -1238,7 +1241,7 @@ int lbm_batch_create(const lbm_params* params, int32_t nruns, void* stream, lbm_
     b->slot0 = lbm::batch_params_alloc(b->dev, nruns);
     if (b->slot0 < 0) b->form = LBM_BATCH_CHAINS;
     cudaError_t e = cudaMalloc(&b->ddesc, sizeof(lbm::RunDesc) * (size_t)nruns);
-    if (e == cudaSuccess) e = cudaMalloc(&b->derr, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->derr, sizeof(int) * ((size_t)nruns + 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->dctrs, sizeof(unsigned*) * (size_t)nruns);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->dctrs, hctrs, sizeof(unsigned*) * (size_t)nruns, cudaMemcpyHostToDevice);
@@ -1248,7 +1251,14 @@ int lbm_batch_create(const lbm_params* params, int32_t nruns, void* stream, lbm_
         lbm_batch_destroy(b);
         return LBM_ERR_NOMEM;
     }
-    cudaMemset(b->derr, 0, sizeof(int));
+    cudaMemset(b->derr, 0, sizeof(int) * ((size_t)nruns + 1));
+    // the runs' own launches (fields, diagnostics, a run stepped alone) raise flags that
+    // lbm_batch_synchronize sees too
+    for (int r = 0; r < nruns; ++r) {
+        cudaFree(b->runs[r]->derr);
+        b->runs[r]->derr = b->derr + 1 + r;
+        b->runs[r]->own_err = false;
+    }
     b->shape = batch_default_shape(params, nruns);
     for (int r = 0; r < nruns; ++r) {
         const int rc = set_shape(b->runs[r], batch_chain_shape(b, r));
@@ -1276,6 +1286,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     std::free(b->hdesc);
     std::free(b->hkp);
     std::free(b->htab);
+    std::free(b->herr);
     cudaFree(b->ddesc);
     cudaFree(b->dctrs);
     cudaFree(b->derr);
@@ -1353,11 +1364,13 @@ int lbm_batch_synchronize(lbm_batch* b) {
     if (!b) return LBM_ERR_INVALID_ARG;
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return batch_fail(b, e);
-    int timed_out = 0;
-    e = cudaMemcpy(&timed_out, b->derr, sizeof(int), cudaMemcpyDeviceToHost);
+    const size_t bytes = sizeof(int) * ((size_t)b->nruns + 1);
+    e = cudaMemcpy(b->herr, b->derr, bytes, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return batch_fail(b, e);
+    int timed_out = 0;
+    for (int r = 0; r <= b->nruns && !timed_out; ++r) timed_out = b->herr[r];
     if (timed_out) {
-        cudaMemset(b->derr, 0, sizeof(int));
+        cudaMemset(b->derr, 0, bytes);
         b->pending_error = LBM_OK;
         return timed_out == 1 ? LBM_ERR_TIMEOUT : LBM_ERR_CUDA;
     }
