@@ -252,9 +252,10 @@ int lbm_debug_stall_next_step(lbm_ctx *ctx);
  * and keeps the fastest shape.  Candidates (TMA kernel): (tile_x, cells per
  * thread) in {(128, 1), (192, 1), (64, 1), (128, 2), (192, 2)} with both
  * store modes for FP32 storage, and (128 or 192, 1 or 2) staged for 16-bit
- * storage, and the small-grid step (kept with the fastest sweep
- * shape, which is what is reported); FUSED: tile_x 128.  seg_y in {8, 16, 32, 64, 128} plus the values
- * that fill one and two waves of resident blocks.  Needs one extra device buffer the size of a population
+ * storage, and the small-grid step with 4 to 8 rows a tile (kept with the
+ * fastest sweep shape, which is what is reported); FUSED: tile_x 128.  seg_y in
+ * {8, 16, 32, 64, 128} plus the values that fill one and two waves of resident
+ * blocks.  The shape the context comes with is a candidate too.  Needs one extra device buffer the size of a population
  * buffer while it runs.  Outputs (nullable): chosen shape and its time per
  * step in milliseconds.  Synchronous.
  * Errors: INVALID_ARG (steps < 1), UNSUPPORTED (split kernel), NOMEM, CUDA,
@@ -330,8 +331,9 @@ int lbm_batch_get_launch_shape(const lbm_batch *b, int32_t *tile_x, int32_t *seg
 /* Autotuner of the batched step: the persistent form over (tile_x, cells
  * per thread, store mode) in {(64, 1, direct), (128, 1, direct), (192, 1,
  * direct), (64, 1, staged), (128, 1, staged), (128, 2, staged)} x seg_y in
- * {16, 24, 32, 40, 48, 56, 64, 80} and the small-grid step; the chains form with every run's shape from
- * lbm_autotune on one run of each grid size, and with the shapes (192, 38,
+ * {16, 24, 32, 40, 48, 56, 64, 80} and the small-grid step with 4 to 8 rows a
+ * tile; the form and shapes the batch comes with; the chains form with every
+ * run's shape from lbm_autotune on one run of each grid size, and with the shapes (192, 38,
  * 1, direct), (128, 32, 1, direct) and (192, 38, 2, direct) for every run;
  * the fastest form and shapes are kept.  Every candidate is timed over `steps` rounded up to whole 32-step
  * graphs after one graph of warm-up, and the state, step counts and buffer

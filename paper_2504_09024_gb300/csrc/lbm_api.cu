@@ -1543,6 +1543,11 @@ int lbm_autotune(lbm_ctx* ctx, int32_t steps, int32_t* tile_x, int32_t* seg_y,
         sync_step_ctr(ctx);
         return ms / steps;
     };
+    // the shape it comes with, so that tuning never makes a run slower; the sweep's best
+    // shape is kept beside a tile-parallel step that wins (the getters report it)
+    if (ce == cudaSuccess) best = time_shape(shape0);
+    lbm::FusedShape sweep = shape0;
+    double sweep_best = shape0.tile ? 1e300 : best;
     for (int a = 0; a < ncand && ce == cudaSuccess && rc == LBM_OK; ++a) {
         const int bx = cand[a][0], cpt = cand[a][1], out = cand[a][2];
         const int per_sm = ctx->kernel != LBM_KERNEL_TMA
@@ -1553,24 +1558,30 @@ int lbm_autotune(lbm_ctx* ctx, int32_t steps, int32_t* tile_x, int32_t* seg_y,
         for (int k = 0; k < ns && ce == cudaSuccess && rc == LBM_OK; ++k) {
             const lbm::FusedShape sh{bx, segs[k], cpt, out};
             const double ms = time_shape(sh);
-            if (rc == LBM_OK && ms < best) {
-                best = ms;
-                best_shape = sh;
+            if (rc == LBM_OK && ms < sweep_best) {
+                sweep_best = ms;
+                sweep = sh;
             }
         }
     }
-    // the tile-parallel step, beside the best sweep shape (which is what the
-    // shape getters report and what setting it again selects: the same bits)
-    for (int tile : {4, 8}) {
+    int tile = shape0.tile;
+    if (sweep_best < best) {
+        best = sweep_best;
+        tile = 0;
+    }
+    for (int rows = 4; rows <= 8; ++rows) {
         if (ctx->kernel != LBM_KERNEL_TMA || ce != cudaSuccess || rc != LBM_OK) break;
-        lbm::FusedShape sh = best_shape;
-        sh.tile = tile;
+        if (rows == shape0.tile) continue;
+        lbm::FusedShape sh = sweep;
+        sh.tile = rows;
         const double ms = time_shape(sh);
         if (rc == LBM_OK && ms < best) {
             best = ms;
-            best_shape = sh;
+            tile = rows;
         }
     }
+    best_shape = sweep;
+    best_shape.tile = tile;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(snap);
@@ -1605,6 +1616,8 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
         std::free(best_runs);
         return LBM_ERR_NOMEM;
     }
+    // (the runs' own shapes, kept while the batch as it came is the best)
+    for (int r = 0; r < b->nruns; ++r) best_runs[r] = b->runs[r]->shape;
     cudaError_t ce = cudaSuccess;
     auto bytes_of = [&](int r) {
         const lbm_ctx* c = b->runs[r];
@@ -1645,10 +1658,18 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
     };
     const int form0 = b->form;
     const lbm::FusedShape shape0 = b->shape;
-    lbm::FusedShape best_shape = shape0;
     int best_form = form0;
     double best = 1e300;
-    // persistent form (when the batch holds parameter-bank slots)
+    // the form and shapes it comes with, so that tuning never makes a batch slower
+    if (ce == cudaSuccess) rc = time_it(best);
+    bool as_it_came = true;
+    // persistent form (when the batch holds parameter-bank slots): the sweep's best shape,
+    // and the rows of a tile-parallel step that wins beside it
+    const bool tiles0 = form0 == LBM_BATCH_PERSISTENT && shape0.tile;
+    lbm::FusedShape sweep = shape0;
+    double sweep_best = form0 == LBM_BATCH_PERSISTENT && !shape0.tile ? best : 1e300;
+    double best_persistent = form0 == LBM_BATCH_PERSISTENT ? best : 1e300;
+    int tile = form0 == LBM_BATCH_PERSISTENT ? shape0.tile : 0;
     b->form = LBM_BATCH_PERSISTENT;
     // block widths, cells per thread and store modes, each with a range of
     // tile heights (the tile count against the grid decides the last wave)
@@ -1661,26 +1682,35 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
             rc = batch_build_tiles(b);
             double ms = 0.0;
             if (rc == LBM_OK) rc = time_it(ms);
-            if (rc == LBM_OK && ms < best) {
-                best = ms;
-                best_form = LBM_BATCH_PERSISTENT;
-                best_shape = b->shape;
+            if (rc == LBM_OK && ms < sweep_best) {
+                sweep_best = ms;
+                sweep = b->shape;
             }
         }
     }
-    // the tile-parallel step, kept with the best sweep shape (reported)
-    for (int tile : {4, 8}) {
+    if (sweep_best < best_persistent) {
+        best_persistent = sweep_best;
+        tile = 0;
+    }
+    for (int rows = 4; rows <= 8; ++rows) {
         if (ncand == 0 || ce != cudaSuccess || rc != LBM_OK) break;
-        const lbm::FusedShape sweep = best_shape;
+        if (tiles0 && rows == shape0.tile) continue;
         b->shape = sweep;
-        b->shape.tile = tile;
+        b->shape.tile = rows;
         rc = batch_build_tiles(b);
         double ms = 0.0;
         if (rc == LBM_OK) rc = time_it(ms);
-        if (rc == LBM_OK && ms < best) {
-            best = ms;
-            best_shape = b->shape;
+        if (rc == LBM_OK && ms < best_persistent) {
+            best_persistent = ms;
+            tile = rows;
         }
+    }
+    lbm::FusedShape best_shape = sweep;
+    best_shape.tile = tile;
+    if (best_persistent < best) {
+        best = best_persistent;
+        best_form = LBM_BATCH_PERSISTENT;
+        as_it_came = false;
     }
     // chains form: every grid size tuned on its first run (the shape shared
     // by the runs of that size), then a few shapes common to all runs (with
@@ -1695,6 +1725,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
         if (rc == LBM_OK && ms < best) {
             best = ms;
             best_form = LBM_BATCH_CHAINS;
+            as_it_came = false;
             std::memcpy(best_runs, run_shape, sizeof(lbm::FusedShape) * (size_t)b->nruns);
         }
     };
@@ -1730,14 +1761,14 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps, int32_t* tile_x, int32_t* se
         std::free(best_runs);
         return ce != cudaSuccess ? batch_fail(b, ce) : rc;
     }
-    // keep the winner: the persistent shape always; the runs' own shapes
-    // are the winning chains shapes if the chains form won, else follow the
-    // persistent shape
+    // keep the winner: the persistent shape always; the runs' own shapes are as
+    // they were if nothing was faster, the winning chains shapes if the chains
+    // form won, else follow the persistent shape
     b->form = best_form;
     b->shape = best_shape;
     b->width_set = true;
     for (int r = 0; r < b->nruns && rc == LBM_OK; ++r)
-        rc = set_shape(b->runs[r], best_form == LBM_BATCH_CHAINS ? best_runs[r] : best_shape);
+        rc = set_shape(b->runs[r], as_it_came || best_form == LBM_BATCH_CHAINS ? best_runs[r] : best_shape);
     std::free(best_runs);
     if (rc == LBM_OK) rc = batch_build_tiles(b);
     if (rc != LBM_OK) return rc;
