@@ -73,8 +73,7 @@
 #include <cstdint>
 #include <cstring>
 #include <new>
-#include <type_traits>
-#include <vector>
+#include <utility>
 
 #include "lbm3.h"
 #include "lbm_vec.cuh"
@@ -1258,15 +1257,14 @@ int lbm3_get_launch_shape(const lbm3_ctx* ctx, int32_t* rows, int32_t* seg_z) {
 int lbm3_autotune(lbm3_ctx* ctx, int32_t steps, int32_t* rows_out, int32_t* seg_out, double* ms_out) {
     if (!ctx || steps < 1) return LBM_ERR_INVALID_ARG;
     Nvtx r("lbm3_autotune");
-    const int nz = ctx->kp.nz;
-    const int row_c[3] = {6, 10, 18};
-    std::vector<int> segs;
-    for (int s : {4, 8, 16, 32, 64, nz}) {
-        const int v = s < nz ? s : nz;
-        bool seen = false;
-        for (int t : segs) seen = seen || t == v;
-        if (!seen) segs.push_back(v);
-    }
+    // (rows, planes) worth a timing: the shape it comes with, then a ladder
+    std::pair<int, int> shapes[19] = {{ctx->rows, ctx->seg_z}};
+    int nshapes = 1;
+    for (int rows : {6, 10, 18})
+        for (int seg : {4, 8, 16, 32, 64, ctx->kp.nz}) {
+            const std::pair<int, int> sh{rows, std::min(seg, ctx->kp.nz)};
+            if (std::find(shapes, shapes + nshapes, sh) == shapes + nshapes) shapes[nshapes++] = sh;
+        }
     cudaEvent_t ev[2];
     if (cudaEventCreate(&ev[0]) != cudaSuccess) return fail(ctx, cudaGetLastError());
     if (cudaEventCreate(&ev[1]) != cudaSuccess) {
@@ -1276,31 +1274,29 @@ int lbm3_autotune(lbm3_ctx* ctx, int32_t steps, int32_t* rows_out, int32_t* seg_
     double best = -1.0;
     int best_rows = ctx->rows, best_seg = ctx->seg_z;
     int rc = LBM_OK;
-    for (int rows : row_c) {
-        for (int seg : segs) {
-            ctx->rows = rows;
-            ctx->seg_z = seg;
-            rc = launch_step(ctx);  // warm-up
-            if (rc != LBM_OK) break;
-            cudaEventRecord(ev[0], ctx->stream);
-            for (int s = 0; s < steps && rc == LBM_OK; ++s) rc = launch_step(ctx);
-            cudaEventRecord(ev[1], ctx->stream);
-            if (rc != LBM_OK) break;
-            cudaError_t e = cudaEventSynchronize(ev[1]);
-            if (e != cudaSuccess) {
-                rc = fail(ctx, e);
-                break;
-            }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, ev[0], ev[1]);
-            const double per = ms / steps;
-            if (best < 0.0 || per < best) {
-                best = per;
-                best_rows = rows;
-                best_seg = seg;
-            }
-        }
+    for (int k = 0; k < nshapes; ++k) {
+        const std::pair<int, int> sh = shapes[k];
+        ctx->rows = sh.first;
+        ctx->seg_z = sh.second;
+        rc = launch_step(ctx);  // warm-up
         if (rc != LBM_OK) break;
+        cudaEventRecord(ev[0], ctx->stream);
+        for (int s = 0; s < steps && rc == LBM_OK; ++s) rc = launch_step(ctx);
+        cudaEventRecord(ev[1], ctx->stream);
+        if (rc != LBM_OK) break;
+        cudaError_t e = cudaEventSynchronize(ev[1]);
+        if (e != cudaSuccess) {
+            rc = fail(ctx, e);
+            break;
+        }
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, ev[0], ev[1]);
+        const double per = ms / steps;
+        if (best < 0.0 || per < best) {
+            best = per;
+            best_rows = sh.first;
+            best_seg = sh.second;
+        }
     }
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2504_09024_gb300 import lbm, workloads as W
+from paper_2504_09024_gb300 import lbm, lbm3, workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +63,33 @@ def test_a_tuned_batch_is_not_slower(grids):
     assert tuned < 1.05 * alone
     for b in batches:
         b.close()
+
+
+def test_the_3d_tuner_times_the_shape_it_is_given():
+    """Three heights of tile, five of segment (4, 8, 16, 32 and all 40 planes), and the
+    shape that was set, which is none of those; one warm-up step each."""
+    g = lbm3.Sim3(40, 30, 40)
+    lbm3.lbm3_set_launch_shape(g.ctx, 10, 13)
+    lbm3.lbm3_autotune(g.ctx, 3)
+    assert g.t == (3 * 5 + 1) * (3 + 1)
+    lbm3.lbm3_set_launch_shape(g.ctx, 18, 40)
+    before = g.t
+    lbm3.lbm3_autotune(g.ctx, 3)
+    assert g.t - before == 3 * 5 * (3 + 1)
+    g.close()
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 256), (150, 97, 61)])
+def test_a_tuned_3d_run_is_not_slower(shape):
+    nx, ny, nz = shape
+    s = torch.cuda.Stream()
+    runs = [lbm3.Sim3(nx, ny, nz, u=(0.02, -0.013, 0.009), stream=s.cuda_stream) for _ in range(2)]
+    lbm3.lbm3_autotune(runs[1].ctx, 20)
+    z = torch.zeros((nz, ny, nx), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    for r in runs:
+        lbm3.lbm3_init_fields_device(r.ctx, z, z, None, None, None)
+    alone, tuned = median_us(runs, s, steps=40)
+    assert tuned < 1.05 * alone
+    for r in runs:
+        r.close()
