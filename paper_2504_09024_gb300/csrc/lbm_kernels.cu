@@ -500,43 +500,52 @@ __global__ void k_init_pre(KParams p, const float* __restrict__ F, float* __rest
     }
 }
 
-// a + b = s + e exactly (Knuth's TwoSum).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 // Deviation form of nine slots: returns their sum S rounded to fixed point (scale:
-// a power of two, inv its reciprocal) and d_q = u_q - w_q S.  In pairs of floats,
-// 48 bits: FP64 instructions issue at two lanes a cycle and SM, and ninety of them
-// a cell made the kernel 140 us at 1024 x 512; now 27.5.
+// a power of two, inv its reciprocal) and d_q = u_q - w_q S, as FP64 gives them
+// (the slots added in their order, each d_q by one fused multiply-add).  FP64
+// instructions issue at two lanes a cycle and SM, and those of a cell made the kernel
+// 140 us at 1024 x 512, so it is done in 64-bit whole numbers, in units of 2^-27
+// of the fixed point's: w_1 = 4 w_5 is whole there, and so are slots of ordinary
+// size.  Exact sums and products below 2^53 are what FP64 has, too; the few cells
+// for which that is not so, or whose S is so close to a tie that the rounding of
+// the FP64 sum could decide it, take FP64 itself: 38 us.  (Pairs of floats, 27 us,
+// lose bits where a slot all but cancels its share.)
 __device__ __forceinline__ int deviations(const float (&u)[9], float scale, float inv, float (&d)[9]) {
-    float hi = 0.0f, lo = 0.0f;
+    constexpr long long W1 = 14913081;  // 2^27 w_1
+    static_assert((float)W1 / 134217728.0f == wq(1) && wq(5) * 4.0f == wq(1), "weights in these units");
+    const float one = scale * 134217728.0f, unit = inv / 134217728.0f;
+    bool none = true, whole = true;  // S is certainly 0; certainly exact
+    long long U[9], sum = 0;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        float e;
-        two_sum(hi, u[q], hi, e);
-        lo += e;
+        const float f = u[q] * one;
+        none = none && fabsf(f) < 7.0e6f;  // 9 of them: 0.47 of a fixed-point unit
+        whole = whole && fabsf(f) < 7.2e16f && truncf(f) == f;  // below 2^56
+        U[q] = __float2ll_rn(f);
+        sum += U[q];
     }
-    // hi + lo to the nearest unit, ties to even
-    const float A = hi * scale;
-    int S = FX_INVALID;
-    if (fabsf(A) <= (float)FX_RANGE) {
-        const int iA = __float2int_rn(A);
-        const float rem = __fadd_rn(__fsub_rn(A, (float)iA), lo * scale), fl = floorf(rem);
-        const int n = iA + (int)fl;
-        S = n + (rem - fl > 0.5f || (rem - fl == 0.5f && (n & 1)));
-        if (abs(S) > FX_RANGE) S = FX_INVALID;
+    // eight roundings to 53 bits of sums below 9 * 2^56: less than 2^10 units
+    const long long S64 = (sum + (1 << 26)) >> 27;
+    whole = whole && abs((int)(sum & 0x7ffffff) - (1 << 26)) > 1024 && llabs(S64) <= FX_RANGE;
+    int S = (int)S64;
+    if (none || (whole && S == 0)) {  // (with the sign of a zero)
+#pragma unroll
+        for (int q = 1; q < 9; ++q) d[q] = u[q];
+        return 0;
     }
-    const float Sh = (float)S, Sl = (float)(S - (S == FX_INVALID ? S : (int)Sh));
 #pragma unroll
     for (int q = 1; q < 9; ++q) {
-        const float w = wq(q) * inv;  // exact
-        const float P = __fmul_rn(w, Sh), e = __fmaf_rn(w, Sl, __fmaf_rn(w, Sh, -P));
-        float s, t;
-        two_sum(u[q], -P, s, t);
-        d[q] = S == FX_INVALID ? __int_as_float(0x7fc00000) : __fadd_rn(s, __fsub_rn(t, e));
+        const long long D = (q <= 4 ? U[q] : 4 * U[q]) - W1 * S;
+        whole = whole && llabs(D) < 1LL << 53;
+        d[q] = __ll2float_rn(D) * (q <= 4 ? unit : 0.25f * unit);
+    }
+    if (!whole) {
+        double s = 0.0;
+        for (int q = 0; q < 9; ++q) s += (double)u[q];
+        S = fx_from_double(s, scale);
+        const double Sr = fx_to_double(S, scale);
+#pragma unroll
+        for (int q = 1; q < 9; ++q) d[q] = (float)__fma_rn(-(double)wq(q), Sr, (double)u[q]);
     }
     return S;
 }
