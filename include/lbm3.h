@@ -103,9 +103,8 @@ int lbm3_init_fields(lbm3_ctx *ctx, const double *phi, const double *c, const do
 int lbm3_init_fields_device(lbm3_ctx *ctx, const double *phi, const double *c,
                             const double *ux, const double *uy, const double *uz);
 
-/* Advance nsteps >= 0 time steps, one kernel launch per step: streaming
- * phi and c, the normal and theta, theta_c, both collisions and streaming.
- * Asynchronous. */
+/* Advance nsteps >= 0 time steps, one kernel launch per step: the normal of phi,
+ * theta and theta_c, both collisions, and streaming.  Asynchronous. */
 int lbm3_step(lbm3_ctx *ctx, int64_t nsteps);
 
 /* phi = sum f and c = sum h of the current state (post-streaming

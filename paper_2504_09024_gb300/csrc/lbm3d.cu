@@ -20,9 +20,10 @@
 // s = sum a and j = sum e a of the incoming populations, and those four sums
 // are all that is kept between steps: int32 fixed point in units of 2^-28,
 // words 2 (((z * 4 + m) * ny + y) * nx + x) (f) and the next (h), m = s, jx, jy, jz.
-// A step forms the 27 outgoing populations of a cell in registers, rounds each
-// to the 2^-28 grid (the rest population takes the integer remainder of s, so
-// sum f and sum h are conserved exactly) and adds them into the sums of the
+// A step forms the 27 outgoing populations of a cell in registers, rounded to the
+// 2^-28 grid (of a row along x its sum and its two moving populations are rounded,
+// the third is what is left; the rest population takes the integer remainder of s,
+// so sum f and sum h are conserved exactly), and adds them into the sums of the
 // cells they stream to; the sums are exact in integers, so the state is the
 // one that storing all 54 populations gives, at 64 bytes a cell and step
 // instead of 432.  (With FP32 storage every cell of a uniform region makes the
@@ -49,7 +50,8 @@
 // added by shuffles, along y through shared memory, along z in registers, and
 // the moments of plane k - 1 are then complete and stored.  phi of plane k + 2
 // (with a second halo cell for the gradient) is on its way to shared memory and
-// the moments of plane k + 1 are on their way to registers meanwhile.  The
+// the moments of plane k + 1 are on their way to registers (or by way of shared
+// memory, k3_ahead) meanwhile.  The
 // exchange buffer and the phi plane alternate between two copies, so one
 // barrier per plane suffices.  Halo rows form only the populations that enter
 // the tile.  The loop forms populations as if every cell were valid and every
@@ -63,8 +65,9 @@
 // shape: 1980 us a step with all populations stored; in moments 600 us with a
 // uniform velocity and 784 with a field; f and h in packed FP32 instructions (lane
 // x: f, lane y: h) and 16-byte words across rows 575 and 724; a row's two moving
-// populations and its sum instead of three populations (emit_rows) 504 and 655.
-// The 64 bytes a cell take 160 us.
+// populations and its sum instead of three populations (emit_rows) 504 and 655;
+// the next plane by way of shared memory 503 and 591.  The 64 bytes a cell take
+// 160 us.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -197,7 +200,7 @@ struct Collision {
     int2 s_fx;
     f2 s, k[3];
     float u[3];
-    float most, big, fast;  // the larger |s|, the largest |k'| and (velocity field) the largest |u|
+    float most, big, fast;  // the larger |s|, the largest |k'| (or |s|/10), a field's largest |u|
     bool tame;  // safe(), nor can the sums of what such cells send leave 32 bits
     // both zeroth moments inside (-4, 4)
     __device__ __forceinline__ bool ok() const { return most < S_MAX * FX_ONE; }
@@ -234,7 +237,7 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
         r.k[i] = lbm::vfma(w, lbm::vfma(q, f2(__fmul_rn(g[i], inv)), -a), a);
     }
     r.most = fmaxf(fabsf(r.s.x), fabsf(r.s.y));
-    r.big = most_of(most_of(most_of(r.k[0].x, r.k[0].y, r.k[1].x), r.k[1].y, r.k[2].x), r.k[2].y, 0.f);
+    r.big = most_of(most_of(most_of(r.k[0].x, r.k[0].y, r.k[1].x), r.k[1].y, r.k[2].x), r.k[2].y, 0.1f * r.most);
     r.fast = UFIELD ? most_of(u[0], u[1], u[2]) : 0.f;
     // What the 27 neighbours of a cell send it adds up to less than 8.  Uniform |u| < 1/2: the
     // products of A add up to 1 and those of B and C to less than 3.2 a component, 4 + 3 * 3.2 *
@@ -244,7 +247,7 @@ __device__ __forceinline__ Collision collide(const K3Params& p, const int2 (&m)[
         const bool slow = r.fast <= 0.2f;
         r.tame = r.fast <= 0.4f && r.most < (slow ? 2.1f : 1.1f) * FX_ONE && r.big < (slow ? 0.3f : 0.15f) * FX_ONE;
     } else {
-        r.tame = r.ok() && r.big < 0.4f * FX_ONE;
+        r.tame = r.big < 0.4f * FX_ONE;  // and |s| below 4
     }
     return r;
 }
@@ -321,7 +324,7 @@ __device__ __forceinline__ uint2 from_right(uint2 v) {
 }
 
 // Resident blocks per SM the register budget is sized for: 80 registers a
-// thread at 6 rows (80 to 176 bytes of spill), 96 at 10 and 18 (up to 44).
+// thread at 6 rows (about 90 bytes of spill), 96 at 10 and 18 (up to 20).
 template <int ROWS>
 constexpr int k3_min_blocks() { return ROWS == 6 ? 4 : ROWS == 10 ? 2 : 1; }
 
@@ -330,11 +333,16 @@ template <int ROWS>
 constexpr int k3_ring_words() { return (ROWS + 2) * RING_W; }
 template <int ROWS>
 constexpr int k3_xchg_words() { return 24 * ROWS * TILE_W; }  // 6 x uint4 a cell
-template <int ROWS>
-constexpr int k3_ahead_words() { return 11 * ROWS * TILE_W; }  // 4 x int2 and 3 x float a cell
-template <int ROWS>
-constexpr int k3_smem(bool field) {
-    return 4 * (2 * (k3_ring_words<ROWS>() + k3_xchg_words<ROWS>()) + (field ? k3_ahead_words<ROWS>() : 0));
+// Whether the next plane's moments (and velocity) come by way of shared memory: live
+// in registers through the emission, some are spilled, and a spilled one waits there
+// for its load.  us a step at 256^3, in registers and this way: field, 18 rows 655 and
+// 592, 10 rows (48 planes) 790 and 579; uniform, 18 rows 525 and 518, 10 rows 503 and 507.
+template <int ROWS, bool UFIELD>
+constexpr bool k3_ahead() { return UFIELD || ROWS == 18; }
+template <int ROWS, bool UFIELD>
+constexpr int k3_smem() {  // ahead: 4 x int2 and, with a field, 3 x float a cell
+    return 4 * (2 * (k3_ring_words<ROWS>() + k3_xchg_words<ROWS>()) +
+                (k3_ahead<ROWS, UFIELD>() ? (UFIELD ? 11 : 8) * ROWS * TILE_W : 0));
 }
 
 // Asynchronous copy of 4 or 8 bytes into shared memory.
@@ -493,19 +501,19 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
     fetch(zn, 0);
     __syncthreads();
 
-    // The moments and the velocity of the thread's cell in the next plane.  A uniform
-    // velocity leaves registers to have the moments loaded into; with a field they come
-    // by way of shared memory (live through the emission, some were spilled, and a
-    // spilled one waits there for its load: 655 us a step at 256^3, now 600).
+    // The moments and the velocity of the thread's cell in the next plane.
+    constexpr bool AHEAD = k3_ahead<ROWS, UFIELD>();
     int2* ahead = reinterpret_cast<int2*>(ring + 2 * RING) + threadIdx.x;    // [4][NT]
     float* ahead_u = ring + 2 * RING + 8 * NT + threadIdx.x;                 // [3][NT]
     auto load_ahead = [&](int z) {
         const int2* q = reinterpret_cast<const int2*>(src + z * pstride) + cell;
 #pragma unroll
         for (int i = 0; i < 4; ++i) cp_async<8>(ahead + i * NT, q + (size_t)i * nxny);
-        const float* v = p.uf + (long long)z * nxny + cell;
+        if constexpr (UFIELD) {
+            const float* v = p.uf + (long long)z * nxny + cell;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) cp_async<4>(ahead_u + i * NT, v + i * p.N);
+            for (int i = 0; i < 3; ++i) cp_async<4>(ahead_u + i * NT, v + i * p.N);
+        }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
@@ -515,7 +523,7 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
     int slot = 0;
     for (int k = z0 - 1; k <= z1; ++k) {
         int2 mn[4];
-        if constexpr (UFIELD) load_ahead(zn);
+        if constexpr (AHEAD) load_ahead(zn);
         else moments(zn, mn);
         const int* q = src + zp * pstride;
         const int f0 = __ldg(q + 2 * o0), f1 = __ldg(q + 2 * o1);
@@ -526,6 +534,11 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         if (ty <= last + 1) {
             hi = plane(slot);
             const Collision r = collide<UFIELD>(p, m, lo, mid, hi, u);
+            if (!r.tame) {
+                p.suspect[wrapi(k, p.nz)] = p.suspect[p.nz] = p.number;
+                if (!r.ok()) met_invalid = 1;
+                else if (!r.safe()) met_single = 1;
+            }
             uint2 moved = make_uint2(0u, 0u);
             // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
             auto across = [&](int b) {
@@ -556,11 +569,6 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
                 s0[0] = rest + r1 + r2;
                 d0[0] = r1 - r2;
             }
-            if (!r.tame) {
-                p.suspect[wrapi(k, p.nz)] = p.suspect[p.nz] = p.number;
-                if (!r.ok()) met_invalid = 1;
-                else if (!r.safe()) met_single = 1;
-            }
         }
         ring[(slot ^ 1) * RING + threadIdx.x] = fx_to_f(f0);
         if (i1 < RING) ring[(slot ^ 1) * RING + i1] = fx_to_f(f1);
@@ -590,14 +598,14 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
             up[1] = JX[1];
             up[2] = JY[1];
         }
-        if constexpr (UFIELD) asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if constexpr (AHEAD) asm volatile("cp.async.wait_group 0;" ::: "memory");
         slot ^= 1;
         lo = mid;
         mid = hi;
         zn = zp;
         zp = next(zp);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m[i] = UFIELD ? ahead[i * NT] : mn[i];
+        for (int i = 0; i < 4; ++i) m[i] = AHEAD ? ahead[i * NT] : mn[i];
         if constexpr (UFIELD) {
 #pragma unroll
             for (int i = 0; i < 3; ++i) u[i] = ahead_u[i * NT];
@@ -907,9 +915,9 @@ int sm_count() {
 template <int ROWS>
 cudaError_t allow_smem(bool field) {
     return field ? cudaFuncSetAttribute(k3_step<ROWS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        k3_smem<ROWS>(true))
+                                        k3_smem<ROWS, true>())
                  : cudaFuncSetAttribute(k3_step<ROWS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        k3_smem<ROWS>(false));
+                                        k3_smem<ROWS, false>());
 }
 
 int launch_step(lbm3_ctx* ctx) {
@@ -927,13 +935,13 @@ int launch_step(lbm3_ctx* ctx) {
     };
     switch (rows) {
         case 6:
-            field ? go(k3_step<6, true>, k3_smem<6>(true)) : go(k3_step<6, false>, k3_smem<6>(false));
+            field ? go(k3_step<6, true>, k3_smem<6, true>()) : go(k3_step<6, false>, k3_smem<6, false>());
             break;
         case 10:
-            field ? go(k3_step<10, true>, k3_smem<10>(true)) : go(k3_step<10, false>, k3_smem<10>(false));
+            field ? go(k3_step<10, true>, k3_smem<10, true>()) : go(k3_step<10, false>, k3_smem<10, false>());
             break;
         case 18:
-            field ? go(k3_step<18, true>, k3_smem<18>(true)) : go(k3_step<18, false>, k3_smem<18>(false));
+            field ? go(k3_step<18, true>, k3_smem<18, true>()) : go(k3_step<18, false>, k3_smem<18, false>());
             break;
         default:
             return LBM_ERR_INVALID_ARG;
@@ -949,10 +957,11 @@ int launch_step(lbm3_ctx* ctx) {
 // planes' time (the halo planes and the first loads), so the best segments make
 // the blocks of an SM times that the least.  In units of a plane of 10 rows alone
 // on an SM, a plane of 18 rows takes 1.45, and a second block of 10 rows beside the
-// first 0.45 (0.75 with a velocity field, whose chains need more registers).
-// Measured, us per step at the best segments of 18 / 10 rows: uniform velocity
-// 256^3 504 / 485, 150x97x61 39 / 39, 64x50x40 16.5 / 14.5; velocity field 256^3
-// 655 / 788, 220x200x180 356 / 398, 150x97x61 49 / 49.
+// first 0.45 (0.75 with a velocity field).  Measured, us per step at the shape this
+// takes / at the best segments of 18 / of 10 rows: uniform velocity 256^3 503 / 518 /
+// 487, 150x97x61 39 / 39 / 39, 64x50x40 14.4 / 16.5 / 14.5; velocity field 256^3 591 /
+// 591 / 579, 220x200x180 326 / 305 / 293, 150x97x61 45 / 45 / 47.  (With a field it
+// weighs 10 rows as they were before the moments came by way of shared memory.)
 void default_shape(const lbm3_params* p, int sms, int* rows, int* seg_z) {
     const double second = p->velocity_field ? 1.75 : 1.45;
     double best = -1.0;
