@@ -228,8 +228,8 @@ int tile_rows(Tiles tiles, int nsm) {
 // Launch shape of a run whose user has not set one.
 //  * Up to 14 tiles of 32 x 8 per SM: the tile-parallel step.  Measured
 //    on GB300 (FP32 coupled, us per step, against 128-wide strips of 32 rows
-//    before and the best sweep shape): 128 x 128 4.9 / 57.0 / 10.9, 512 x 256
-//    13.3 / 58.4 / 14.6, 1024 x 512 36.9 / 59.0 / 35.6; 2048 x 1024 128 / 136
+//    before and the best sweep shape): 128 x 128 5.3 / 57.0 / 15.5, 512 x 256
+//    13.6 / 58.4 / 17.3, 1024 x 512 38.3 / 59.0 / 35.7; 2048 x 1024 128 / 136
 //    / 96, so larger grids take the sweep.
 //  * The sweep: the height that fills the chip with one wave of strips, of the
 //    width whose (rows + 5) x (time of a row at full residency) is least

@@ -1253,8 +1253,9 @@ void launch_field_stats(const KParams& p, const double* phi, const double* c, co
 // ---------------------------------------------------------------------------
 // 4-connected components of {phi > level}, periodic in x, and in y without walls
 // ---------------------------------------------------------------------------
-// Union-find on the cells: label[k] <= k points towards the smallest cell of k's
-// tree.  Cells start pointing at the first cell of their run within 32 aligned
+// Union-find on the cells, joined by atomic minima (Playne and Hawick, "A New
+// Algorithm for Parallel Connected-Component Labelling on GPUs", IEEE TPDS 29(6),
+// 2018): label[k] <= k points towards the smallest cell of k's tree.  Cells start pointing at the first cell of their run within 32 aligned
 // columns; then every run is joined to its neighbours, each pair of runs once.
 // Components = trees at the start - joins.  Bound by the latency of the chains of
 // loads and atomics.  (Propagating the least label sweep by sweep, with a host
