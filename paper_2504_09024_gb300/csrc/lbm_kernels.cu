@@ -508,21 +508,24 @@ __global__ void k_init_pre(KParams p, const float* __restrict__ F, float* __rest
 // of the fixed point's: w_1 = 4 w_5 is whole there, and so are slots of ordinary
 // size.  Exact sums and products below 2^53 are what FP64 has, too; the few cells
 // for which that is not so, or whose S is so close to a tie that the rounding of
-// the FP64 sum could decide it, take FP64 itself: 38 us.  (Pairs of floats, 27 us,
+// the FP64 sum could decide it, take FP64 itself: 34 us.  (Pairs of floats, 27 us,
 // lose bits where a slot all but cancels its share.)
 __device__ __forceinline__ int deviations(const float (&u)[9], float scale, float inv, float (&d)[9]) {
     constexpr long long W1 = 14913081;  // 2^27 w_1
     static_assert((float)W1 / 134217728.0f == wq(1) && wq(5) * 4.0f == wq(1), "weights in these units");
     const float one = scale * 134217728.0f, unit = inv / 134217728.0f;
     bool none = true, whole = true;  // S is certainly 0; certainly exact
-    long long U[9], sum = 0;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const float f = u[q] * one;
-        none = none && fabsf(f) < 7.0e6f;  // 9 of them: 0.47 of a fixed-point unit
-        whole = whole && fabsf(f) < 7.2e16f && truncf(f) == f;  // below 2^56
-        U[q] = __float2ll_rn(f);
-        sum += U[q];
+    for (int q = 0; q < 9; ++q) none = none && fabsf(u[q] * one) < 7.0e6f;  // 9 of them: 0.47 of a fixed-point unit
+    long long U[9], sum = 0;
+    if (!none) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const float f = u[q] * one;
+            whole = whole && fabsf(f) < 7.2e16f && truncf(f) == f;  // below 2^56
+            U[q] = __float2ll_rn(f);
+            sum += U[q];
+        }
     }
     // eight roundings to 53 bits of sums below 9 * 2^56: less than 2^10 units
     const long long S64 = (sum + (1 << 26)) >> 27;
