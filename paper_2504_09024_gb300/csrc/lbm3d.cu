@@ -56,7 +56,7 @@
 // barrier per plane suffices.  Halo rows form only the populations that enter
 // the tile.  The loop forms populations as if every cell were valid and every
 // population in range; a block that met others goes over its cells once more at
-// its end (settle_invalid).
+// its end (settle).
 // (Bits of invalid cells exchanged in the loop with the populations cost 8 to 10 %
 // of a step in which nothing is invalid.)
 //
@@ -66,7 +66,7 @@
 // uniform velocity and 784 with a field; f and h in packed FP32 instructions (lane
 // x: f, lane y: h) and 16-byte words across rows 575 and 724; a row's two moving
 // populations and its sum instead of three populations (emit_rows) 504 and 655;
-// the next plane by way of shared memory 503 and 591.  The 64 bytes a cell take
+// the next plane by way of shared memory 503 and 602.  The 64 bytes a cell take
 // 160 us.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -204,11 +204,22 @@ struct Collision {
     bool tame;  // safe(), nor can the sums of what such cells send leave 32 bits
     // both zeroth moments inside (-4, 4)
     __device__ __forceinline__ bool ok() const { return most < S_MAX * FX_ONE; }
-    // and no population can leave the range: |A| <= 0.67, |B| <= 1 and |C| <= 1 up to |u| = 1/2,
-    // 1.17, 2 and 1 up to |u| = 1
+    // and no population can leave the range: uniform |u| < 1/2 |A| <= 0.67, |B| <= 1 and |C| <= 1;
+    // a field's by the largest factor of each axis
+    template <bool UFIELD>
     __device__ __forceinline__ bool safe() const {
-        const bool half = fast <= 0.5f;
-        return ok() && fast <= 1.0f && __fmaf_rn(half ? 0.3f : 1.6f, most, (half ? 3.0f : 6.0f) * big) < 7.9f * FX_ONE;
+        if constexpr (!UFIELD) return ok() && __fmaf_rn(0.3f, most, 3.0f * big) < 7.9f * FX_ONE;
+        float a = 1.0f, b[3], c[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float v = fabsf(u[i]), v2 = __fmul_rn(v, v), m = __fadd_rn(v2, v);
+            a = __fmul_rn(a, fmaxf(fmaxf(2.0f / 3.0f, __fadd_rn(v2, -2.0f / 3.0f)), __fmul_rn(0.5f, __fadd_rn(1.0f / 3.0f, m))));
+            b[i] = fmaxf(2.0f * v, __fadd_rn(v, 0.5f));
+            c[i] = fmaxf(fmaxf(1.0f, __fadd_rn(v2, -1.0f)), 0.5f * m);
+        }
+        const float k = __fmaf_rn(__fmul_rn(b[0], c[1]), c[2],
+                                  __fmaf_rn(__fmul_rn(c[0], b[1]), c[2], __fmul_rn(__fmul_rn(c[0], c[1]), b[2])));
+        return ok() && __fmaf_rn(a, most, __fmul_rn(k, big)) < 7.9f * FX_ONE;
     }
 };
 
@@ -312,7 +323,7 @@ __device__ __forceinline__ void emit_rows(const K3Params& p, const Collision& r,
                                   : make_uint2((uint32_t)__float2int_rn(v.x), (uint32_t)__float2int_rn(v.y));
         };
         const uint2 v1 = grid(E + O), v2 = grid(E - O);
-        row(c, CHECK && !r.safe() ? grid(lbm::vfma(f2(-2.0f), E, W)) + v1 + v2 : grid(W), v1, v2);
+        row(c, CHECK && !r.template safe<UFIELD>() ? grid(lbm::vfma(f2(-2.0f), E, W)) + v1 + v2 : grid(W), v1, v2);
     }
 }
 
@@ -336,7 +347,7 @@ constexpr int k3_xchg_words() { return 24 * ROWS * TILE_W; }  // 6 x uint4 a cel
 // Whether the next plane's moments (and velocity) come by way of shared memory: live
 // in registers through the emission, some are spilled, and a spilled one waits there
 // for its load.  us a step at 256^3, in registers and this way: field, 18 rows 655 and
-// 592, 10 rows (48 planes) 790 and 579; uniform, 18 rows 525 and 518, 10 rows 503 and 507.
+// 602, 10 rows (48 planes) 790 and 576; uniform, 18 rows 525 and 516, 10 rows 503 and 507.
 template <int ROWS, bool UFIELD>
 constexpr bool k3_ahead() { return UFIELD || ROWS == 18; }
 template <int ROWS, bool UFIELD>
@@ -396,15 +407,19 @@ __device__ __forceinline__ void outgoing(const K3Params& p, const int* __restric
     for (int q = 0; q < Q27; ++q) out(q, (int)v[q].x, (int)v[q].y);
 }
 
-// What the step's loop leaves out, for a block that met invalid cells: FX_BAD for
+// What the step's loop leaves out, for a block that met cells that are not tame: the
+// word of `suspect` for the whole box (from every such cell, stores to the one word
+// took longer than the step); and (invalid: the block met invalid ones) FX_BAD for
 // the zeroth moments of cells that FX_BAD is sent to, by invalid cells of `src` and
 // (single: the block met cells that are not safe()) by others; for the latter all
 // sums are made once more, of the populations as they are cut off.  A function of
 // its own, and one that adds up in place: what it needs in registers costs the loop
 // up to 5 %.
 template <int ROWS>
-__device__ __noinline__ void settle_invalid(const K3Params& p, const int* __restrict__ src, int* __restrict__ dst,
-                                            bool single) {
+__device__ __noinline__ void settle(const K3Params& p, const int* __restrict__ src, int* __restrict__ dst,
+                                    bool invalid, bool single) {
+    if (threadIdx.x == 0) p.suspect[p.nz] = p.number;
+    if (!invalid && !single) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int x = blockIdx.x * TILE_IN + tx - 1, y = blockIdx.y * (ROWS - 2) + ty - 1;
     if (tx < 1 || tx > TILE_IN || x >= p.nx || ty < 1 || ty > ROWS - 2 || y >= p.ny) return;
@@ -485,8 +500,8 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         for (int i = 0; i < 3; ++i) u[i] = UFIELD ? __ldg(q + i * p.N) : p.u[i];
     };
 
-    __shared__ int met_invalid, met_single;
-    if (threadIdx.x == 0) met_invalid = met_single = 0;
+    __shared__ int met_suspect, met_invalid, met_single;
+    if (threadIdx.x == 0) met_suspect = met_invalid = met_single = 0;
     int zc = wrapi(z0 - 1, p.nz);  // the plane of k
     fetch(wrapi(z0 - 2, p.nz), 0);
     fetch(zc, 1);
@@ -535,9 +550,10 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
             hi = plane(slot);
             const Collision r = collide<UFIELD>(p, m, lo, mid, hi, u);
             if (!r.tame) {
-                p.suspect[wrapi(k, p.nz)] = p.suspect[p.nz] = p.number;
+                p.suspect[wrapi(k, p.nz)] = p.number;
+                met_suspect = 1;
                 if (!r.ok()) met_invalid = 1;
-                else if (!r.safe()) met_single = 1;
+                else if (!r.template safe<UFIELD>()) met_single = 1;
             }
             uint2 moved = make_uint2(0u, 0u);
             // populations of y velocity +1 (b = 1) and -1 (b = 2): to the other rows
@@ -612,7 +628,7 @@ k3_step(const __grid_constant__ K3Params p, const int* __restrict__ src, int* __
         }
     }
     __syncthreads();
-    if (met_invalid | met_single) settle_invalid<ROWS>(p, src, dst, met_single != 0);
+    if (met_suspect) settle<ROWS>(p, src, dst, met_invalid != 0, met_single != 0);
 }
 
 // The fields an initial state is made of (velocity null: uniform u).
@@ -958,9 +974,9 @@ int launch_step(lbm3_ctx* ctx) {
 // the blocks of an SM times that the least.  In units of a plane of 10 rows alone
 // on an SM, a plane of 18 rows takes 1.45, and a second block of 10 rows beside the
 // first 0.45 (0.75 with a velocity field).  Measured, us per step at the shape this
-// takes / at the best segments of 18 / of 10 rows: uniform velocity 256^3 503 / 518 /
-// 487, 150x97x61 39 / 39 / 39, 64x50x40 14.4 / 16.5 / 14.5; velocity field 256^3 591 /
-// 591 / 579, 220x200x180 326 / 305 / 293, 150x97x61 45 / 45 / 47.  (With a field it
+// takes / at the best segments of 18 / of 10 rows: uniform velocity 256^3 503 / 516 /
+// 487, 150x97x61 39 / 39 / 39, 64x50x40 14.4 / 16.5 / 14.5; velocity field 256^3 602 /
+// 602 / 576, 220x200x180 331 / 305 / 293, 150x97x61 47 / 47 / 47.  (With a field it
 // weighs 10 rows as they were before the moments came by way of shared memory.)
 void default_shape(const lbm3_params* p, int sms, int* rows, int* seg_z) {
     const double second = p->velocity_field ? 1.75 : 1.45;

@@ -33,15 +33,15 @@ def bound(kinds, e):
     return s + k
 
 
-largest_of = {v: largest(v) for v in (0.2, 0.4, 0.5, 1.0)}
+largest_of = {v: largest(v) for v in (0.2, 0.4)}
 
 
 def test_tame_cells_of_a_field_add_up_in_range():
     kinds = [(0.2, 2.1, 0.3), (0.4, 1.1, 0.15)]
     total = sum(bound(kinds, e) for e in VEL)
     assert 7.5 < total < 7.9
-    # and they are safe(): 0.3 |s| + 3 max |k'| below 7.9
-    assert all(0.3 * m + 3 * b < 7.9 for _, m, b in kinds)
+    # and they are safe()
+    assert all(safe_bound((v, v, v), m, k) < 7.9 for v, m, k in kinds)
 
 
 def test_tame_cells_of_a_uniform_velocity_add_up_in_range():
@@ -51,11 +51,26 @@ def test_tame_cells_of_a_uniform_velocity_add_up_in_range():
         k = sum(abs(F[0][1][a] * F[1][2][b] * F[2][2][c]) + abs(F[0][2][a] * F[1][1][b] * F[2][2][c])
                 + abs(F[0][2][a] * F[1][2][b] * F[2][1][c]) for a, b, c in VEL)
         assert 4.0 * s + 0.4 * k < 7.9
-    assert 0.3 * 4 + 3 * 0.4 < 7.9
+    # and they are safe(), there with constants: |A| <= 2/3, |B| <= 1, |C| <= 1
+    assert (2 / 3) ** 3 < 0.3 and 0.3 * 4.0 + 3 * 0.4 < 7.9
+
+
+def safe_bound(u, most, big):
+    """As in Collision::safe(): the largest factor of each axis."""
+    v = np.abs(u)
+    a = np.maximum(np.maximum(2 / 3, v * v - 2 / 3), (1 / 3 + v * v + v) / 2)
+    b = np.maximum(2 * v, v + 0.5)
+    c = np.maximum(np.maximum(1, v * v - 1), (v * v + v) / 2)
+    return most * a.prod() + big * (b[0] * c[1] * c[2] + c[0] * b[1] * c[2] + c[0] * c[1] * b[2])
 
 
 def test_safe_cells_send_populations_in_range():
-    for v, per_s, per_k in ((0.5, 0.3, 3.0), (1.0, 1.6, 6.0)):
-        A, B, C = largest_of[v]
-        assert max(A.values()) ** 3 <= per_s
-        assert 3 * max(B.values()) * max(C.values()) ** 2 <= per_k + 1e-12
+    rng = np.random.default_rng(3)
+    for _ in range(2000):
+        u = rng.uniform(-2, 2, 3) * rng.choice([0.1, 1.0], 3)
+        most, big = rng.uniform(0, 4), rng.uniform(0, 3)
+        s, k = most * rng.choice([-1, 1]), big * rng.choice([-1, 1], 3)
+        (Ax, Bx, Cx), (Ay, By, Cy), (Az, Bz, Cz) = (factors(v) for v in u)
+        largest_sent = max(abs(s * Ax[a] * Ay[b] * Az[c] + k[0] * Bx[a] * Cy[b] * Cz[c] + k[1] * Cx[a] * By[b] * Cz[c]
+                               + k[2] * Cx[a] * Cy[b] * Bz[c]) for a, b, c in VEL)
+        assert largest_sent <= safe_bound(u, most, big) * (1 + 1e-12)
