@@ -1185,8 +1185,9 @@ int lbm3_get_fields_device(lbm3_ctx* ctx, double* phi, double* c) {
     const K3Params p = of_state(ctx);
     k3_fields<<<grid_1d(ctx, p.N, 256), 256, 0, ctx->stream>>>(p, ctx->buf[ctx->cur], phi, c);
     if (before(ctx))
-        k3_fields_suspect<<<grid_1d(ctx, (p.N + 1) / 2, 256), 256, 0, ctx->stream>>>(p, before(ctx), ctx->buf[ctx->cur], phi,
-                                                                               c);
+        // (four blocks an SM: usually they find nothing to do)
+        k3_fields_suspect<<<std::min(grid_1d(ctx, p.N, FT_N), 4 * ctx->sms), 256, 0, ctx->stream>>>(
+            p, before(ctx), ctx->buf[ctx->cur], phi, c);
     return fail(ctx, cudaGetLastError());
 }
 
