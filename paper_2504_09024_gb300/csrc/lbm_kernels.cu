@@ -505,18 +505,25 @@ __global__ void k_init_pre(KParams p, const float* __restrict__ F, float* __rest
 // (the slots added in their order, each d_q by one fused multiply-add).  FP64
 // instructions issue at two lanes a cycle and SM, and those of a cell made the kernel
 // 140 us at 1024 x 512, so it is done in 64-bit whole numbers, in units of 2^-27
-// of the fixed point's: w_1 = 4 w_5 is whole there, and so are slots of ordinary
-// size.  Exact sums and products below 2^53 are what FP64 has, too; the few cells
-// for which that is not so, or whose S is so close to a tie that the rounding of
-// the FP64 sum could decide it, take FP64 itself: 34 us.  (Pairs of floats, 27 us,
-// lose bits where a slot all but cancels its share.)
+// of the fixed point's, or 2^-47 where all slots are small: w_1 = 4 w_5 is whole
+// there, and so are the slots of nearly all cells.  Exact sums and products below
+// 2^53 are what FP64 has, too; the cells for which that is not so, or whose S is so
+// close to a tie that the rounding of the FP64 sum could decide it, take FP64
+// itself: 32 us.  (Pairs of floats, 27 us, lose bits where a slot all but cancels
+// its share.)
 __device__ __forceinline__ int deviations(const float (&u)[9], float scale, float inv, float (&d)[9]) {
     constexpr long long W1 = 14913081;  // 2^27 w_1
     static_assert((float)W1 / 134217728.0f == wq(1) && wq(5) * 4.0f == wq(1), "weights in these units");
-    const float one = scale * 134217728.0f, unit = inv / 134217728.0f;
-    bool none = true, whole = true;  // S is certainly 0; certainly exact
+    float one = scale * 134217728.0f, unit = inv / 134217728.0f;
+    bool none = true, fine = true, whole = true;  // S is certainly 0; slots are below 16 units; certainly exact
 #pragma unroll
-    for (int q = 0; q < 9; ++q) none = none && fabsf(u[q] * one) < 7.0e6f;  // 9 of them: 0.47 of a fixed-point unit
+    for (int q = 0; q < 9; ++q) {
+        const float f = fabsf(u[q] * one);
+        none = none && f < 7.0e6f;  // 9 of them: 0.47 of a fixed-point unit
+        fine = fine && f < 2.1e9f;  // below 2^31
+    }
+    const int more = fine ? 20 : 0;
+    if (fine) one *= 1048576.0f, unit *= 1.0f / 1048576.0f;
     long long U[9], sum = 0;
     if (!none) {
 #pragma unroll
@@ -528,17 +535,19 @@ __device__ __forceinline__ int deviations(const float (&u)[9], float scale, floa
         }
     }
     // eight roundings to 53 bits of sums below 9 * 2^56: less than 2^10 units
-    const long long S64 = (sum + (1 << 26)) >> 27;
-    whole = whole && abs((int)(sum & 0x7ffffff) - (1 << 26)) > 1024 && llabs(S64) <= FX_RANGE;
+    const long long half = 1LL << (26 + more);
+    const long long S64 = (sum + half) >> (27 + more);
+    whole = whole && llabs((sum & (2 * half - 1)) - half) > 1024 && llabs(S64) <= FX_RANGE;
     int S = (int)S64;
     if (none || (whole && S == 0)) {  // (with the sign of a zero)
 #pragma unroll
         for (int q = 1; q < 9; ++q) d[q] = u[q];
         return 0;
     }
+    const long long T = W1 * S << more;  // below 2^57
 #pragma unroll
     for (int q = 1; q < 9; ++q) {
-        const long long D = (q <= 4 ? U[q] : 4 * U[q]) - W1 * S;
+        const long long D = (q <= 4 ? U[q] : 4 * U[q]) - T;
         whole = whole && llabs(D) < 1LL << 53;
         d[q] = __ll2float_rn(D) * (q <= 4 ? unit : 0.25f * unit);
     }

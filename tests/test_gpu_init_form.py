@@ -26,6 +26,8 @@ def populations(kind, shape, rng):
     if kind == "tail":       # a tail that dies out, zeros of both signs among it
         v = w * 10.0 ** rng.uniform(-44, -9, shape)
         return (v * rng.choice([0.0, -0.0, 1.0, 1.0, 1.3], (9,) + shape)).astype(np.float32)
+    if kind == "foot":       # the foot of a profile: sums of a fixed-point unit to a few thousand
+        return (w * 10.0 ** rng.uniform(-10, -5, shape) * (1 + 0.1 * rng.standard_normal((9,) + shape))).astype(np.float32)
     if kind == "ties":       # sums at and next to half a unit: slot 8 carries what is missing
         f = (w * rng.uniform(0.1, 1.0, shape)).astype(np.float32)
         units = f[:8].astype(np.float64).sum(0) * 2.0 ** 29
@@ -48,7 +50,7 @@ def stored(f):
     return S, wide.astype(np.float64).astype(np.float32)
 
 
-@pytest.mark.parametrize("kind", ["interface", "bulk", "tail", "ties", "any"])
+@pytest.mark.parametrize("kind", ["interface", "bulk", "foot", "tail", "ties", "any"])
 def test_stored_form_has_the_bits_of_fp64(kind, tmp_path):
     nx, ny = 509, 257
     rng = np.random.default_rng(7)
